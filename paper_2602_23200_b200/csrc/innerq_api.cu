@@ -367,8 +367,8 @@ int innerq_quantize_prefill(innerq_cache_t* c, const void* k, const void* v, int
   if (n < 0) return INNERQ_ERR_CUDA;
   c->N = n_tokens;
   // Nothing of a fresh prefill counts as settled: the first decode after it waits for its predecessors before it
-  // reads any packed chunk (the prefill kernels are ordinary launches, whose writes a dependent launch may rely on
-  // only after that wait).  The decode that follows then streams ahead again.
+  // reads anything of the cache, the norms included (the last prefill kernel may have written them just before, and a
+  // dependent launch may rely on that only after the wait).  The decode that follows then streams ahead again.
   c->N_safe = 0;
   c->reads_settled = 0;
   c->launches[0] = n;

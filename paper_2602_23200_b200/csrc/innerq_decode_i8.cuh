@@ -254,6 +254,7 @@ __device__ __forceinline__ void decode_i8_body(const Layout& L, const Counts& cn
   auto dep_wait_for_iteration = [&](int i) {
     if (c_lo + (i + 1) * CPI > a.safe_chunks) dep_wait();
   };
+  if (a.safe_chunks < 0) dep_wait();      // first decode after a prefill: the norms come from the kernel before this one
   // q and the key norms are requested first of all, ahead of the bulk copies below: behind several
   // hundred KB of queued chunk data per SM they would take microseconds to arrive.
   // Only requested here: nothing may USE the loaded values before the copies below are issued (a warp issues in

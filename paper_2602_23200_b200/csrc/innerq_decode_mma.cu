@@ -117,10 +117,11 @@ void decode_mma_set_ablation(int mask) { g_ablation = mask & 3; }
 
 // n_q > 1: q and out are [B, n_q, Hq, D], the partials of a launch's (up to) four rows per unit go to
 // multi_partials [U * 4][max_splits][kPartialStride]
-// N_safe: token count of the cache when its previous decode was launched (or it was prefilled): chunks packed by
-// then are not written by any kernel that can still be running.
+// N_safe: token count of the cache when its previous decode was launched (0: prefilled since): chunks packed by then
+// are not written by any kernel that can still be running.
 static int safe_chunks_for(const Layout& L, int N_safe, const Counts& cn_now) {
-  const Counts old = counts_for(L, N_safe < 0 ? 0 : N_safe);
+  if (N_safe <= 0) return -1;      // no decode since the prefill: nothing of the cache may be read ahead
+  const Counts old = counts_for(L, N_safe);
   const bool outer = L.grouping == 1;
   int s = (outer ? old.n_qk : old.n_qv) / kChunk;
   const int now = (outer ? cn_now.n_qk : cn_now.n_qv) / kChunk;

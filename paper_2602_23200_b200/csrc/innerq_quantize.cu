@@ -5,57 +5,7 @@
 
 namespace iq {
 
-// ------------------------------------------------------------------ key norm
-// absmax[u][c] = max_t |K[u][t][c]| as fp32 bit patterns (non-negative floats order like uints).
-__global__ void __launch_bounds__(256) k_absmax_kernel(const __half* __restrict__ K, int N, int rows_per_block,
-                                                       uint32_t* __restrict__ absmax) {
-  const int u = blockIdx.y;
-  const int t0 = blockIdx.x * rows_per_block;
-  const int t1 = min(N, t0 + rows_per_block);
-  const int cg = threadIdx.x & 15;      // 8 channels each
-  const int rg = threadIdx.x >> 4;      // 16 rows in flight
-  const uint4* base = reinterpret_cast<const uint4*>(K + (size_t)u * N * kD);
-  __half2 m[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) m[i] = __float2half2_rn(0.f);
-  for (int t = t0 + rg; t < t1; t += 16) {
-    uint4 v = __ldg(base + (size_t)t * 16 + cg);
-    const __half2* h = reinterpret_cast<const __half2*>(&v);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) m[i] = __hmax2(m[i], __habs2(h[i]));
-  }
-  __shared__ float red[16][kD];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    red[rg][cg * 8 + 2 * i] = __low2float(m[i]);
-    red[rg][cg * 8 + 2 * i + 1] = __high2float(m[i]);
-  }
-  __syncthreads();
-  if (threadIdx.x < kD) {
-    float v = 0.f;
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v = fmaxf(v, red[i][threadIdx.x]);
-    atomicMax(absmax + (size_t)u * kD + threadIdx.x, __float_as_uint(v));
-  }
-}
-
-// norm = sqrt(absmax), 0 -> 1  (Section "Per-channel Normalization of K"); the absmax word is replaced by the
-// reciprocal 1 / norm (correctly rounded) that the quantisers multiply keys with
-__global__ void finalize_norm_kernel(uint32_t* __restrict__ absmax, float* __restrict__ norm, int n) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) {
-    float n_ = __fsqrt_rn(__uint_as_float(absmax[i]));
-    n_ = n_ == 0.f ? 1.0f : n_;
-    norm[i] = n_;
-    absmax[i] = __float_as_uint(__fdiv_rn(1.0f, n_));
-  }
-}
-
 __global__ void fill_u32_kernel(uint32_t* p, uint32_t v, int n) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) p[i] = v;
-}
-__global__ void fill_float_kernel(float* p, float v, int n) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) p[i] = v;
 }
@@ -210,22 +160,6 @@ __global__ void zero_pages_kernel(Layout L, const unsigned char* __restrict__ ca
   const size_t n = L.page_bytes / 16;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
     dst[i] = make_uint4(0u, 0u, 0u, 0u);
-}
-
-// ------------------------------------------------------------------ window copies (prefill)
-// Copies tokens [t0, t1) of the input into the sink (t < w_sink) or the recent ring.
-__global__ void copy_window_kernel(Layout L, Store S, const __half* __restrict__ X, int N, int t0, int t1,
-                                   unsigned char* __restrict__ cache) {
-  const int u = blockIdx.y;
-  const int n = (t1 - t0) * 16;
-  __half* sink = reinterpret_cast<__half*>(cache + S.sink_off + (size_t)u * S.sink_stride);
-  __half* ring = reinterpret_cast<__half*>(cache + S.ring_off + (size_t)u * S.ring_stride);
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    int t = t0 + (i >> 4), piece = i & 15;
-    uint4 v = *reinterpret_cast<const uint4*>(X + ((size_t)u * N + t) * kD + piece * 8);
-    __half* dst = t < L.w_sink ? sink + (size_t)t * kD : ring + (size_t)((t - L.w_sink) % S.ring_cap) * kD;
-    *reinterpret_cast<uint4*>(dst + piece * 8) = v;
-  }
 }
 
 // ------------------------------------------------------------------ append (quantise-on-evict)
@@ -552,22 +486,11 @@ static inline int grid_for(int n, int per_block, int cap) {
 
 int launch_prefill(const Layout& L, unsigned char* cache, unsigned char* ws, const __half* K, const __half* V, int N,
                    cudaStream_t st) {
-  int launches = 0;
   const Counts cn = counts_for(L, N);
-  float* norm = reinterpret_cast<float*>(cache + L.norm_off);
-  const bool use_norm = L.k_normalize != 0 && L.k.kind != kNone;
-  if (use_norm && N > 0) {
-    uint32_t* absmax = reinterpret_cast<uint32_t*>(ws + L.ws_absmax_off);
-    if (cudaMemsetAsync(absmax, 0, (size_t)L.U * kD * 4, st) != cudaSuccess) return -1;
-    const int rows_per_block = 512;
-    dim3 g((N + rows_per_block - 1) / rows_per_block, L.U);
-    k_absmax_kernel<<<g, 256, 0, st>>>(K, N, rows_per_block, absmax);
-    finalize_norm_kernel<<<(L.U * kD + 255) / 256, 256, 0, st>>>(absmax, norm, L.U * kD);
-    launches += 2;
-  } else {
-    fill_float_kernel<<<(L.U * kD + 255) / 256, 256, 0, st>>>(norm, 1.0f, L.U * kD);
-    launches += 1;
-  }
+  if (L.grouping == 0 && N > 0) return launch_prefill_inner(L, cn, cache, ws, K, V, st);
+  // an empty cache, the unquantised cache (all windows), or the outer-grouped one (generic routines, no key norm)
+  int launches = launch_prefill_windows(L, cn, cache, K, V, st);
+  if (launches < 0) return -1;
   if (L.k.kind != kNone && L.k.code_kind != L.k.kind) {
     // chunk words of the outer-grouped cache are filled token by token with OR: they start from zero
     if (L.page_groups == 0) {
@@ -580,47 +503,20 @@ int launch_prefill(const Layout& L, unsigned char* cache, unsigned char* ws, con
         launches += 1;
       }
     }
-  }
-  const Store* stores[2] = {&L.k, &L.v};
-  const __half* srcs[2] = {K, V};
-  const int nq[2] = {cn.n_qk, cn.n_qv};
-  for (int i = 0; i < 2; ++i) {
-    const Store& S = *stores[i];
-    if (N == 0) break;
-    if (S.kind == kNone) {      // unquantised: the whole input goes to the "sink" array
-      Layout Lf = L;
-      Lf.w_sink = L.max_tokens;
-      copy_window_kernel<<<dim3(grid_for(N * 16, 256, 1024), L.U), 256, 0, st>>>(Lf, S, srcs[i], N, 0, N, cache);
-      launches += 1;
-      continue;
-    }
-    const bool nrm = use_norm && i == 0;
-    if (nq[i] > 0 && S.code_kind != S.kind) {      // outer-grouped comparison cache: generic routines, no key norm
+    const Store* stores[2] = {&L.k, &L.v};
+    const __half* srcs[2] = {K, V};
+    const int nq[2] = {cn.n_qk, cn.n_qv};
+    for (int i = 0; i < 2; ++i) {
+      const Store& S = *stores[i];
+      if (nq[i] <= 0) continue;
       if (S.kind == kRow)
         quantize_rows_generic_kernel<<<dim3(grid_for(nq[i], 4 * 8, 4096), L.U), 128, 0, st>>>(L, S, srcs[i], N, nq[i], cache);
       else
         quantize_blocks_generic_kernel<<<dim3(grid_for(nq[i] / L.G, 1, 8192), L.U), 128, 0, st>>>(L, S, srcs[i], N, nq[i],
                                                                                                cache);
       launches += 1;
-    } else if (nq[i] > 0) {
-      const float* inv_norm = nrm ? reinterpret_cast<const float*>(ws + L.ws_absmax_off) : nullptr;
-      if (launch_quantize_store_prefill(L, S, srcs[i], N, nq[i], cache, inv_norm, st) < 0) return -1;
-      launches += 1;
-    }
-    // fp16 windows: sink, then everything after the quantised middle
-    if (cn.n_sink > 0) {
-      copy_window_kernel<<<dim3(1, L.U), 256, 0, st>>>(L, S, srcs[i], N, 0, cn.n_sink, cache);
-      launches += 1;
-    }
-    const int t_rec = cn.n_sink + nq[i];
-    if (N > t_rec) {
-      copy_window_kernel<<<dim3(grid_for((N - t_rec) * 16, 256, 64), L.U), 256, 0, st>>>(L, S, srcs[i], N, t_rec, N, cache);
-      launches += 1;
     }
   }
-  // the counts the decode kernel compares with its own N (see append_unit)
-  fill_u32_kernel<<<(L.U + 255) / 256, 256, 0, st>>>(reinterpret_cast<uint32_t*>(cache + L.appended_off), (uint32_t)N, L.U);
-  launches += 1;
   return cudaGetLastError() == cudaSuccess ? launches : -1;
 }
 

@@ -1,5 +1,5 @@
-// Prefill quantisers: the middle tokens of every unit into the ROW store (groups of G channels inside a token,
-// Section "InnerQ" for keys) and the BLOCK store (per-channel groups of G tokens, values).
+// Prefill quantisers of the inner-grouped cache: the middle tokens of every unit into the ROW store (groups of G
+// channels inside a token, Section "InnerQ" for keys) and the BLOCK store (per-channel groups of G tokens, values).
 //
 // Both are built around one work item: 32 values of one group held in the registers of one thread (a group of
 // 64 or 128 values is 2 or 4 such threads, which exchange their minima / maxima and error sums).  The thread
@@ -8,6 +8,13 @@
 // rounded fp32 operations as in group_params / asym_code / sym_code, so stored bits do not depend on the kernel:
 // rounding to an integer is done by adding 1.5 * 2^23 (round-to-nearest-even at unit granularity, identical to
 // rintf for |t| < 2^22; codes are bounded by a few times 2^b), which leaves the code in the low mantissa bits.
+//
+// What bounds them: instruction issue (both read and write far below the HBM rate), so values are kept as PAIRS and
+// every add / multiply is one packed fp32x2 instruction, whose two halves are rounded exactly as the scalar ones.  A
+// packed instruction does not raise the fp32 rate, but it takes one issue slot for two operations, and the slots it
+// frees go to the conversions, minima / maxima and byte permutes.
+#include <type_traits>
+
 #include "innerq_device.cuh"
 #include "innerq_kernels.h"
 
@@ -16,51 +23,147 @@ namespace iq {
 namespace {
 
 constexpr float kMagic = 12582912.0f;       // 1.5 * 2^23
-constexpr int kSeg = 32;                    // values per thread
+constexpr int kSeg = 32;                    // values per thread and group
+constexpr int kRowsCtasPerSm = 4;           // of 128 threads and 128 registers (5 or 6 with fewer registers: +-1 %)
 
-struct SegCoder {
-  float z_a, inv_a, s_a, lo_a, hi_a;        // asymmetric: clamp bounds in the magic domain
-  float inv_s, s_s, off_s, lo_s, hi_s;      // symmetric (offset-binary): magic + 2^(b-1), bounds
-  __device__ __forceinline__ explicit SegCoder(const GroupParams& p) {
-    z_a = p.z_a; inv_a = p.inv_a; s_a = p.s_a; lo_a = kMagic; hi_a = kMagic + p.L;
-    inv_s = p.inv_s; s_s = p.s_s; off_s = kMagic + p.half; lo_s = off_s + p.q_lo; hi_s = off_s + p.q_hi;
+// ---- two fp32 values in a 64-bit register pair
+using F2 = unsigned long long;
+__device__ __forceinline__ F2 f2(float lo, float hi) {
+  F2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float2 unf2(F2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+  F2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+// Product rounded by itself, as a * b + (-0).  A mul.rn.f32x2 (or an fma with a literal -0) is contracted by the
+// assembler with a following packed add, although its scalar form never is, and that moves codes at rounding ties; so
+// the -0 comes from a kernel argument, whose value the assembler does not know.
+struct Mul2 {
+  F2 neg_zero;
+  __device__ __forceinline__ explicit Mul2(float nz) : neg_zero(f2(nz, nz)) {}
+  __device__ __forceinline__ F2 operator()(F2 a, F2 b) const { return fma2(a, b, neg_zero); }
+};
+
+// x / DEN for DEN = 1, 3, 7, 15, correctly rounded: the product with the rounded reciprocal, corrected by its
+// FMA-computed (hence exact) remainder, which is exact for divisors known in advance (Brisebarre, Muller and Raina,
+// "Accelerating correctly rounded floating-point division when the divisor is known in advance", 2004); the host test
+// tests/div_const_check.cpp goes through every mantissa of the four divisors.  Results below the normal range may be
+// one unit off: the callers round to fp16, where they are zero.
+template <int DEN> __device__ __forceinline__ float div_const(float x) {
+  if constexpr (DEN == 1) return x;
+  constexpr float r = 1.0f / (float)DEN;
+  const float q = __fmul_rn(x, r);
+  const float q1 = __fmaf_rn(__fmaf_rn(-(float)DEN, q, x), r, q);
+  return fabsf(q) < INFINITY ? q1 : q;      // an infinite (or NaN) quotient has no remainder
+}
+
+// group_params (innerq_device.cuh) with its divisions by constants and reciprocals in their cheaper correctly rounded
+// forms: the same bits.
+template <int BITS> __device__ __forceinline__ GroupParams seg_params(float mn, float mx, int sym_variant) {
+  GroupParams p;
+  constexpr int L = (1 << BITS) - 1, half = 1 << (BITS - 1);
+  p.L = (float)L;
+  p.half = (float)half;
+  p.sa_bits = f2h_bits(div_const<L>(__fsub_rn(mx, mn)));
+  p.z_bits = f2h_bits(mn);
+  p.s_a = h2f_bits(p.sa_bits);
+  p.z_a = h2f_bits(p.z_bits);
+  p.inv_a = p.s_a == 0.f ? 0.f : __frcp_rn(p.s_a);
+  const float am = fmaxf(fabsf(mn), fabsf(mx));
+  if (sym_variant == 0) {
+    p.ss_bits = f2h_bits(div_const<half - 1>(am));
+    p.q_lo = -(float)(half - 1);
+  } else {
+    p.ss_bits = f2h_bits(div_const<L>(am));
+    p.q_lo = -(float)half;
   }
-  // code plus magic (asymmetric) / plus magic + 2^(b-1) (symmetric): the low mantissa bits are the stored code.
-  // CLAMP = false leaves out the clamp to the code range, for groups where no_clip() holds.
-  template <bool CLAMP> __device__ __forceinline__ float asym(float x) const {
-    const float t = __fadd_rn(__fmul_rn(__fsub_rn(x, z_a), inv_a), kMagic);
-    return CLAMP ? fminf(fmaxf(t, lo_a), hi_a) : t;
+  p.q_hi = (float)(half - 1);
+  p.s_s = h2f_bits(p.ss_bits);
+  p.inv_s = p.s_s == 0.f ? 0.f : __frcp_rn(p.s_s);
+  return p;
+}
+
+// Clamp bounds of both candidates in the magic domain, and whether any value of the group can need them.
+struct Bounds {
+  float off_s, lo_s, hi_s, hi_a;            // symmetric: magic + 2^(b-1) and its bounds; asymmetric: [magic, hi_a]
+  bool no_clip;
+  __device__ __forceinline__ Bounds(Mul2 mul2, const GroupParams& p, float mn, float mx)
+      : off_s(kMagic + p.half), lo_s(off_s + p.q_lo), hi_s(off_s + p.q_hi), hi_a(kMagic + p.L) {
+    // Both coders are non-decreasing in x (each step is a correctly rounded monotone operation and the reciprocal
+    // scales are >= 0), so if the group's minimum and maximum land inside the code range, every value does.
+    const F2 ends = f2(mn, mx);
+    const float2 a = unf2(add2(mul2(add2(ends, f2(-p.z_a, -p.z_a)), f2(p.inv_a, p.inv_a)), f2(kMagic, kMagic)));
+    const float2 s = unf2(add2(mul2(ends, f2(p.inv_s, p.inv_s)), f2(off_s, off_s)));
+    no_clip = a.x >= kMagic && a.y <= hi_a && s.x >= lo_s && s.y <= hi_s;
   }
-  template <bool CLAMP> __device__ __forceinline__ float sym(float x) const {
-    const float t = __fadd_rn(__fmul_rn(x, inv_s), off_s);
-    return CLAMP ? fminf(fmaxf(t, lo_s), hi_s) : t;
+};
+
+// The coders for a pair of values whose parameters may differ (two channels) or not (two values of one group).
+// Asymmetric: ((x - z) * inv) + magic; symmetric: (x * inv) + (magic + 2^(b-1)): the low mantissa bits are the stored
+// code.  CLAMP = false leaves out the clamp to the code range, for groups where no_clip holds.
+struct PairCoder {
+  Mul2 mul2;
+  F2 nz_a, inv_a, ns_a, inv_s, off_s, noff_s, ns_s;
+  float2 hi_a, lo_s, hi_s;
+  __device__ __forceinline__ PairCoder(Mul2 mul, const GroupParams& p, const Bounds& b, const GroupParams& q, const Bounds& d)
+      : mul2(mul), nz_a(f2(-p.z_a, -q.z_a)), inv_a(f2(p.inv_a, q.inv_a)), ns_a(f2(-p.s_a, -q.s_a)), inv_s(f2(p.inv_s, q.inv_s)),
+        off_s(f2(b.off_s, d.off_s)), noff_s(f2(-b.off_s, -d.off_s)), ns_s(f2(-p.s_s, -q.s_s)),
+        hi_a(make_float2(b.hi_a, d.hi_a)), lo_s(make_float2(b.lo_s, d.lo_s)), hi_s(make_float2(b.hi_s, d.hi_s)) {}
+  static __device__ __forceinline__ F2 clamp2(F2 t, float2 lo, float2 hi) {
+    const float2 v = unf2(t);
+    return f2(fminf(fmaxf(v.x, lo.x), hi.x), fminf(fmaxf(v.y, lo.y), hi.y));
   }
-  // Both coders are non-decreasing in x (each step is a correctly rounded monotone operation and the reciprocal
-  // scales are >= 0), so if the group's minimum and maximum land inside the code range, every value does.
-  __device__ __forceinline__ bool no_clip(float mn, float mx) const {
-    return asym<false>(mn) >= lo_a && asym<false>(mx) <= hi_a && sym<false>(mn) >= lo_s && sym<false>(mx) <= hi_s;
+  // L1 reconstruction errors (signed) of both candidates: used only to pick the mode of a hybrid group
+  template <bool CLAMP> __device__ __forceinline__ float2 err_asym(F2 x) const {
+    const F2 d = add2(x, nz_a);
+    F2 t = add2(mul2(d, inv_a), f2(kMagic, kMagic));
+    if (CLAMP) t = clamp2(t, make_float2(kMagic, kMagic), hi_a);
+    return unf2(fma2(ns_a, add2(t, f2(-kMagic, -kMagic)), d));
   }
-  // L1 reconstruction errors of one value (used only to pick the mode of a hybrid group)
-  template <bool CLAMP> __device__ __forceinline__ float err_asym(float x) const {
-    return fabsf(__fmaf_rn(-s_a, asym<CLAMP>(x) - kMagic, __fsub_rn(x, z_a)));
-  }
-  template <bool CLAMP> __device__ __forceinline__ float err_sym(float x) const {
-    return fabsf(__fmaf_rn(-s_s, sym<CLAMP>(x) - off_s, x));
+  template <bool CLAMP> __device__ __forceinline__ float2 err_sym(F2 x) const {
+    F2 t = add2(mul2(x, inv_s), off_s);
+    if (CLAMP) t = clamp2(t, lo_s, hi_s);
+    return unf2(fma2(ns_s, add2(t, noff_s), x));
   }
 };
 
 // The coder of the chosen mode as one formula, clamp(((x - z) * inv) + off): symmetric is z = 0 (x - 0 is exact).
-struct ChosenCoder {
-  float z, inv, off, lo, hi;
-  __device__ __forceinline__ ChosenCoder(const SegCoder& c, bool asym)
-      : z(asym ? c.z_a : 0.f), inv(asym ? c.inv_a : c.inv_s), off(asym ? kMagic : c.off_s), lo(asym ? c.lo_a : c.lo_s),
-        hi(asym ? c.hi_a : c.hi_s) {}
-  // bits of (1.5 * 2^23 + code): 0x4B400000 + code
-  template <bool CLAMP> __device__ __forceinline__ uint32_t code_bits(float x) const {
-    const float t = __fadd_rn(__fmul_rn(__fsub_rn(x, z), inv), off);
-    return __float_as_uint(CLAMP ? fminf(fmaxf(t, lo), hi) : t);
+struct ChosenPair {
+  Mul2 mul2;
+  F2 nz, inv, off;
+  float2 lo, hi;
+  __device__ __forceinline__ ChosenPair(Mul2 mul, const GroupParams& p, const Bounds& b, bool asym_p, const GroupParams& q,
+                                        const Bounds& d, bool asym_q)
+      : mul2(mul), nz(f2(asym_p ? -p.z_a : 0.f, asym_q ? -q.z_a : 0.f)), inv(f2(asym_p ? p.inv_a : p.inv_s, asym_q ? q.inv_a : q.inv_s)),
+        off(f2(asym_p ? kMagic : b.off_s, asym_q ? kMagic : d.off_s)),
+        lo(make_float2(asym_p ? kMagic : b.lo_s, asym_q ? kMagic : d.lo_s)),
+        hi(make_float2(asym_p ? b.hi_a : b.hi_s, asym_q ? d.hi_a : d.hi_s)) {}
+  // bits of (1.5 * 2^23 + code) of both values: the low byte is the code
+  template <bool CLAMP> __device__ __forceinline__ uint2 code_bits(F2 x) const {
+    F2 t = add2(mul2(add2(x, nz), inv), off);
+    if (CLAMP) t = PairCoder::clamp2(t, lo, hi);
+    const float2 v = unf2(t);
+    return make_uint2(__float_as_uint(v.x), __float_as_uint(v.y));
   }
 };
+
+// low bytes of four code words as the four bytes of one word
+__device__ __forceinline__ uint32_t bytes4(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  return __byte_perm(__byte_perm(a, b, 0x0040), __byte_perm(c, d, 0x0040), 0x5410);
+}
 
 __device__ __forceinline__ float min3(float a, float b, float c) {
   float r;
@@ -72,390 +175,344 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
   return r;
 }
-// min / max of 32 registers (three-input min / max: two values per instruction)
-__device__ __forceinline__ void seg_minmax(const float (&x)[kSeg], float& mn, float& mx) {
-  float a = fminf(x[0], x[1]), b = fmaxf(x[0], x[1]);
-#pragma unroll
-  for (int e = 2; e < kSeg; e += 2) { a = min3(a, x[e], x[e + 1]); b = max3(b, x[e], x[e + 1]); }
-  mn = a; mx = b;
+
+// 3-bit codes in byte order (see row_pos_i8_3 / block_pos_i8_3): four codes in the bytes of w become the 2-bit plane's
+// bytes (bit position 0) and the 1-bit plane's bytes (bit 0); `odd` (the bit position of the segment is odd) picks the
+// split of a code between the planes.
+__device__ __forceinline__ void split_planes(uint32_t w, int odd, uint32_t& lo, uint32_t& hi) {
+  lo = (w >> odd) & 0x03030303u;
+  hi = (w >> (odd ? 0 : 2)) & 0x01010101u;
 }
 
-template <bool CLAMP>
-__device__ __forceinline__ void seg_errors(const SegCoder& sc, const float (&x)[kSeg], float& ea, float& es) {
-  float a0 = 0.f, a1 = 0.f, s0 = 0.f, s1 = 0.f;
+// Reduce-scatter by OR over the four lanes 4q .. 4q+3 of 2 * NJ words v[NH * j + h], j = 0..3 (h = 0..NH-1): lane
+// `pos` of the four ends up with the complete words of j = pos.
+template <int NH> __device__ __forceinline__ void quad_reduce_scatter(const uint32_t (&v)[4 * NH], int pos, uint32_t (&out)[NH]) {
+  uint32_t m[2 * NH];                          // step 1: keep the j of my parity (j = 2 i + (pos & 1))
 #pragma unroll
-  for (int e = 0; e < kSeg; e += 2) {
-    a0 += sc.template err_asym<CLAMP>(x[e]); a1 += sc.template err_asym<CLAMP>(x[e + 1]);
-    s0 += sc.template err_sym<CLAMP>(x[e]);  s1 += sc.template err_sym<CLAMP>(x[e + 1]);
-  }
-  ea = a0 + a1; es = s0 + s1;
-}
-
-constexpr uint32_t kMagicBits = 0x4B400000u;     // bit pattern of kMagic
-
-// Packs the 32 codes of a ROW-store segment into its local words (positions of segment 0, see the kernel).
-// Codes arrive as kMagicBits + code; with 2 or 4 bits the fields are filled by wrap-around adds of the shifted
-// patterns, the shifted kMagicBits being taken off at the end (a compile-time constant per word).
-template <int BITS, bool CLAMP>
-__device__ __forceinline__ void pack_row_segment(const ChosenCoder& cc, const float (&x)[kSeg], uint32_t (&lw)[4],
-                                                 uint32_t (&hw)[4]) {
-  constexpr int PB = BITS == 3 ? 2 : BITS, WM = PB == 2 ? 2 : 4;
-  uint32_t cw[4] = {0u, 0u, 0u, 0u};
+  for (int i = 0; i < 2; ++i)
 #pragma unroll
-  for (int i = 0; i < 4; ++i) { lw[i] = 0u; hw[i] = 0u; }
-#pragma unroll
-  for (int e = 0; e < kSeg; ++e) {
-    const uint32_t code = cc.template code_bits<CLAMP>(x[e]);
-    const BitPos lo = row_pos_plane(e, PB);            // constants: segment 0's positions
-    if constexpr (BITS == 3) {
-      const BitPos hi = row_pos_plane(e, 1);
-      lw[lo.word / WM] |= (code & 3u) << lo.bit;
-      hw[hi.word] |= ((code >> 2) & 1u) << hi.bit;
-    } else {
-      lw[lo.word / WM] += code << lo.bit;
-      cw[lo.word / WM] += kMagicBits << lo.bit;
+    for (int h = 0; h < NH; ++h) {
+      const uint32_t keep = (pos & 1) ? v[NH * (2 * i + 1) + h] : v[NH * (2 * i) + h];
+      const uint32_t give = (pos & 1) ? v[NH * (2 * i) + h] : v[NH * (2 * i + 1) + h];
+      m[NH * i + h] = keep | __shfl_xor_sync(0xffffffffu, give, 1);
     }
-  }
 #pragma unroll
-  for (int i = 0; i < 4; ++i) lw[i] -= cw[i];
-}
-
-// Same for a BLOCK-store segment (32 tokens of one channel; positions of channel 0).
-template <int BITS, bool CLAMP>
-__device__ __forceinline__ void pack_block_segment(const ChosenCoder& cc, const float (&x)[kSeg],
-                                                   uint32_t (&lw)[BITS == 4 ? 8 : 4], uint32_t (&hw)[4]) {
-  constexpr int PB = BITS == 3 ? 2 : BITS, NW = PB == 4 ? 8 : 4;
-  uint32_t cw[NW];
-#pragma unroll
-  for (int i = 0; i < NW; ++i) { lw[i] = 0u; cw[i] = 0u; }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) hw[i] = 0u;
-#pragma unroll
-  for (int t = 0; t < kSeg; ++t) {
-    const uint32_t code = cc.template code_bits<CLAMP>(x[t]);
-    const BitPos lo = block_pos_plane(t, 0, PB);       // constants: channel 0's positions
-    const int li = PB == 4 ? (lo.word >> 8) * 4 + ((lo.word >> 2) & 3) : (lo.word >> 2) & 3;   // (k-step,) tid4
-    if constexpr (BITS == 3) {
-      const BitPos hi = block_pos_plane(t, 0, 1);
-      lw[li] |= (code & 3u) << lo.bit;
-      hw[(hi.word >> 2) & 3] |= ((code >> 2) & 1u) << hi.bit;
-    } else {
-      lw[li] += code << lo.bit;
-      cw[li] += kMagicBits << lo.bit;
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < NW; ++i) lw[i] -= cw[i];
-}
-
-// Byte-order layout (Store::perm = 1, 2- or 4-bit codes).  ROW segment = 32 consecutive channels = one bit position of
-// 32 bytes of the row: the codes go to position 0 of 8 words here (index 2 * j + h, see row_pos_i8), the caller
-// places them in the row and shifts them to its position.
-template <int BITS, bool CLAMP>
-__device__ __forceinline__ void pack_row_segment_i8(const ChosenCoder& cc, const float (&x)[kSeg], uint32_t (&w8)[8]) {
-  uint32_t cw[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) { w8[i] = 0u; cw[i] = 0u; }
-#pragma unroll
-  for (int e = 0; e < kSeg; ++e) {
-    const uint32_t code = cc.template code_bits<CLAMP>(x[e]);
-    const BitPos p = row_pos_i8(e, BITS);               // constants: positions of channels 0..31 (bit position 0)
-    const int li = BITS == 4 ? 2 * (p.word >> 2) + (p.word & 1) : p.word;
-    w8[li] += code << p.bit;
-    cw[li] += kMagicBits << p.bit;
-  }
-#pragma unroll
-  for (int i = 0; i < 8; ++i) w8[i] -= cw[i];
-}
-// BLOCK segment = 32 tokens of one channel: bytes of the 8 words [j][half] of its fragment row (see block_pos_i8), at
-// bit position 0 here.  Word index: 2 * j + half.
-template <int BITS, bool CLAMP>
-__device__ __forceinline__ void pack_block_segment_i8(const ChosenCoder& cc, const float (&x)[kSeg], uint32_t (&w8)[8]) {
-  uint32_t cw[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) { w8[i] = 0u; cw[i] = 0u; }
-#pragma unroll
-  for (int t = 0; t < kSeg; ++t) {
-    const uint32_t code = cc.template code_bits<CLAMP>(x[t]);
-    const BitPos p = block_pos_i8(t, 0, BITS);          // constants: channel 0 (W = 0, gid = 0, position 0, rh = 0)
-    const int li = 2 * ((p.word >> 2) & 3) + ((p.word >> 1) & 1);      // 2 * j + half
-    w8[li] += code << p.bit;
-    cw[li] += kMagicBits << p.bit;
-  }
-#pragma unroll
-  for (int i = 0; i < 8; ++i) w8[i] -= cw[i];
-}
-
-// 3-bit codes in byte order (see row_pos_i8_3 / block_pos_i8_3): the 2-bit plane's words as above (bit position 0)
-// and the 1-bit plane's bits at bit 0 of their bytes; `odd` (bit position of the segment is odd) picks the split of
-// a code between the planes.  ROW: hw[h][j] = 1-bit plane word j, bits of row half h.
-template <bool CLAMP>
-__device__ __forceinline__ void pack_row_segment_i8_3(const ChosenCoder& cc, const float (&x)[kSeg], int odd,
-                                                      uint32_t (&w8)[8], uint32_t (&hw)[2][4]) {
-#pragma unroll
-  for (int i = 0; i < 8; ++i) { w8[i] = 0u; hw[i >> 2][i & 3] = 0u; }
-  const int sh_lo = odd, sh_hi = odd ? 0 : 2;
-#pragma unroll
-  for (int e = 0; e < kSeg; ++e) {
-    const uint32_t code = cc.template code_bits<CLAMP>(x[e]);      // kMagicBits + code: the low bits are the code
-    const int lw = e >> 2, j = lw & 3, h = lw >> 2, sh = 8 * (e & 3);
-    w8[2 * j + h] |= ((code >> sh_lo) & 3u) << sh;
-    hw[h][j] |= ((code >> sh_hi) & 1u) << sh;
-  }
-}
-// BLOCK: word index 2 * j + half in both planes.
-template <bool CLAMP>
-__device__ __forceinline__ void pack_block_segment_i8_3(const ChosenCoder& cc, const float (&x)[kSeg], int odd,
-                                                        uint32_t (&w8)[8], uint32_t (&h8)[8]) {
-#pragma unroll
-  for (int i = 0; i < 8; ++i) { w8[i] = 0u; h8[i] = 0u; }
-  const int sh_lo = odd, sh_hi = odd ? 0 : 2;
-#pragma unroll
-  for (int t = 0; t < kSeg; ++t) {
-    const uint32_t code = cc.template code_bits<CLAMP>(x[t]);
-    const int k = 4 * (t & 7) + (t >> 3), li = 2 * ((k & 15) >> 2) + (k >> 4), sh = 8 * (k & 3);
-    w8[li] |= ((code >> sh_lo) & 3u) << sh;
-    h8[li] |= ((code >> sh_hi) & 1u) << sh;
+  for (int h = 0; h < NH; ++h) {               // step 2: keep i = pos >> 1
+    const uint32_t keep = (pos & 2) ? m[NH + h] : m[h];
+    const uint32_t give = (pos & 2) ? m[h] : m[NH + h];
+    out[h] = keep | __shfl_xor_sync(0xffffffffu, give, 2);
   }
 }
 
-__device__ __forceinline__ void unpack8(const uint4& v, float* x) {
-  const __half2* h = reinterpret_cast<const __half2*>(&v);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float2 f = __half22float2(h[i]);
-    x[2 * i] = f.x; x[2 * i + 1] = f.y;
-  }
+// Key norm of one channel from the partial maxima [U][n_part][128]: sqrt(max |K|), 0 -> 1 (Section "Per-channel
+// Normalization of K").
+__device__ __forceinline__ float key_norm(const float* __restrict__ absmax, int n_part, int u, int c) {
+  const float* p = absmax + (size_t)u * n_part * kD + c;
+  float m = 0.f;
+#pragma unroll 8
+  for (int i = 0; i < n_part; ++i) m = fmaxf(m, __ldcg(p + (size_t)i * kD));
+  const float n = __fsqrt_rn(m);
+  return n == 0.f ? 1.0f : n;
+}
+
+// Chunk record ci (32 tokens) of a unit: chunk_rec_ptr with the group size's shift instead of divisions (a group has
+// 1 << sh chunks; the inner-grouped record starts with its chunks).
+__device__ __forceinline__ unsigned char* chunk_ptr(const Rec& rec, const Store& S, int ci, int sh) {
+  return group_ptr(rec, ci >> sh) + (ci & ((1 << sh) - 1)) * S.chunk_stride;
 }
 
 // ------------------------------------------------------------------ ROW store
 // A warp quantises 8 consecutive tokens per iteration: lane = 4 * (token in the batch) + segment, segment =
-// channels 32*seg .. 32*seg+31.  The 8 packed rows and their metadata entries are contiguous in the chunk record.
-// Positions of the segment's codes (see row_pos_plane): element e of segment 0 sits in local word j = tid4(e);
-// for segment seg the word index and the bit offset move by a per-plane amount that depends on seg only.
-template <int BITS, bool NORM, bool I8 = false>
-__global__ void __launch_bounds__(128) quantize_rows_prefill_kernel(Layout L, Store S, const __half* __restrict__ X, int N,
-                                                                    int n_q, unsigned char* __restrict__ cache,
-                                                                    const float* __restrict__ inv_norm) {
+// channels 32*seg .. 32*seg+31, which is one bit position (2, 3 bits: p = seg; 4 bits: nibble seg % 2 of row half
+// seg / 2) of the bytes of the packed row.  The four lanes of a token exchange their words so that each stores a
+// contiguous run of complete ones; the 8 packed rows and their metadata entries are contiguous in the chunk record.
+// (Through shared memory with an atomic OR per word instead: 22 more shared-memory operations per 32 values.)
+// CTA x of the grid takes the x-th part of all units' batches (a contiguous run, so every CTA ends at the same time
+// whatever the number of units), unit by unit.
+// NORM: the unit's key norm comes from `absmax`, n_part partial maxima per unit that prefill_first_kernel wrote; every
+// unit's norm is stored once.  The launch may start before that kernel has ended (griddepcontrol.wait).
+template <int BITS, bool NORM>
+__global__ void __launch_bounds__(128, kRowsCtasPerSm)
+quantize_rows_prefill_kernel(const __grid_constant__ Layout L, const __half* __restrict__ X, int N, int n_q,
+                             unsigned char* __restrict__ cache, const float* __restrict__ absmax, int n_part, float neg_zero) {
+  const Mul2 mul2(neg_zero);
+  const Store& S = L.k;
   constexpr int RW = 4 * BITS;                // 32-bit words per packed row
-  constexpr int PB = BITS == 3 ? 2 : BITS;    // bits of the primary plane
-  __shared__ uint32_t stage_all[4][8 * RW];
-  const int u = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int seg = lane & 3, tk = lane >> 2;
-  const int gl = L.G >> 5;                    // lanes per group: 1, 2 or 4
-  uint32_t* stage = stage_all[warp];
-#pragma unroll
-  for (int k = 0; k < RW / 4; ++k) stage[lane + 32 * k] = 0u;
-  float inv[NORM ? kSeg : 1];
+  const int gl = L.G >> 5, sh = gl >> 1;      // lanes per group: 1, 2 or 4, and its logarithm
+  // reciprocal key norms: segment rows padded to 36 words, so that the four lanes of a token read different banks
+  __shared__ __align__(16) float inv_s[NORM ? 4 * 36 : 4];
   if constexpr (NORM) {
-    const float4* p = reinterpret_cast<const float4*>(inv_norm + (size_t)u * kD + kSeg * seg);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const float4 v = __ldg(p + k);
-      inv[4 * k] = v.x; inv[4 * k + 1] = v.y; inv[4 * k + 2] = v.z; inv[4 * k + 3] = v.w;
-    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    float* norm = reinterpret_cast<float*>(cache + L.norm_off);
+    for (int u = blockIdx.x; u < L.U; u += gridDim.x) norm[(size_t)u * kD + threadIdx.x] = key_norm(absmax, n_part, u, threadIdx.x);
   }
-  // where this segment's local words go inside the row, and by how much its fields are shifted
-  constexpr int WM = PB == 2 ? 2 : 4;        // row words between consecutive local words
-  const int w_add = PB == 2 ? (seg >> 1) : seg;
-  const int sh_lo = PB == 2 ? 8 * (seg & 1) : 0, sh_hi = 4 * seg;
-  const Rec rec = unit_rec(L, cache, u);
-  const __half* Xu = X + ((size_t)u * N + L.w_sink) * kD + kSeg * seg;
   const int n_batches = (n_q + 7) >> 3;
-  const int stride = gridDim.x * 4;
-  int bi = blockIdx.x * 4 + warp;
-  uint4 raw[4];
-  if (bi < n_batches) {
-    const uint4* src = reinterpret_cast<const uint4*>(Xu + (size_t)min(bi * 8 + tk, n_q - 1) * kD);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) raw[k] = __ldg(src + k);
-  }
-  for (; bi < n_batches; bi += stride) {
-    const int i0 = bi * 8;
-    float x[kSeg];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) unpack8(raw[k], x + 8 * k);
-    if (bi + stride < n_batches) {            // next batch's rows are requested before this one is worked on
-      const uint4* src = reinterpret_cast<const uint4*>(Xu + (size_t)min((bi + stride) * 8 + tk, n_q - 1) * kD);
+  const long long total = (long long)L.U * n_batches;
+  long long at = total * blockIdx.x / gridDim.x;
+  const long long end = total * (blockIdx.x + 1) / gridDim.x;
+  while (at < end) {
+    const int u = (int)(at / n_batches);
+    int bi = (int)(at - (long long)u * n_batches) + warp;
+    const int b_end = (int)(end - (long long)u * n_batches < n_batches ? end - (long long)u * n_batches : n_batches);
+    at = (long long)(u + 1) * n_batches;
+    if constexpr (NORM) {
+      __syncthreads();                          // the previous unit's norms are no longer read
+      inv_s[(threadIdx.x >> 5) * 36 + (threadIdx.x & 31)] = __fdiv_rn(1.0f, key_norm(absmax, n_part, u, threadIdx.x));
+      __syncthreads();
+    }
+    const Rec rec = unit_rec(L, cache, u);
+    const __half* Xu = X + ((size_t)u * N + L.w_sink) * kD + kSeg * seg;
+    uint4 raw[4];
+    if (bi < b_end) {
+      const uint4* src = reinterpret_cast<const uint4*>(Xu + (size_t)min(bi * 8 + tk, n_q - 1) * kD);
 #pragma unroll
       for (int k = 0; k < 4; ++k) raw[k] = __ldg(src + k);
     }
-    if constexpr (NORM) {
+    for (; bi < b_end; bi += 4) {
+      const int i0 = bi * 8;
+      F2 x[kSeg / 2];
 #pragma unroll
-      for (int e = 0; e < kSeg; ++e) x[e] = __fmul_rn(x[e], inv[e]);
-    }
-    float mn, mx;
-    seg_minmax(x, mn, mx);
-    for (int o = 1; o < gl; o <<= 1) {
-      mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    }
-    const GroupParams p = group_params(mn, mx, fmaxf(fabsf(mn), fabsf(mx)), BITS, L.sym_variant);
-    const SegCoder sc(p);
-    const bool no_clip = sc.no_clip(mn, mx);        // the same for all lanes of a group
-    bool asym = S.mode == 1;
-    if (S.mode == 2) {
-      float ea, es;
-      if (no_clip) seg_errors<false>(sc, x, ea, es);
-      else seg_errors<true>(sc, x, ea, es);
+      for (int k = 0; k < 4; ++k) {
+        const __half2* h = reinterpret_cast<const __half2*>(&raw[k]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float2 v = __half22float2(h[i]);
+          x[4 * k + i] = f2(v.x, v.y);
+        }
+      }
+      if (bi + 4 < b_end) {                     // next batch's rows are requested before this one is worked on
+        const uint4* src = reinterpret_cast<const uint4*>(Xu + (size_t)min((bi + 4) * 8 + tk, n_q - 1) * kD);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) raw[k] = __ldg(src + k);
+      }
+      if constexpr (NORM) {
+#pragma unroll
+        for (int e = 0; e < kSeg / 4; ++e) {
+          const float4 v = *reinterpret_cast<const float4*>(inv_s + seg * 36 + 4 * e);
+          x[2 * e] = mul2(x[2 * e], f2(v.x, v.y));
+          x[2 * e + 1] = mul2(x[2 * e + 1], f2(v.z, v.w));
+        }
+      }
+      float mn, mx;                             // three-input min / max: two values per instruction
+      {
+        const float2 v = unf2(x[0]);
+        mn = fminf(v.x, v.y); mx = fmaxf(v.x, v.y);
+#pragma unroll
+        for (int e = 1; e < kSeg / 2; ++e) {
+          const float2 w = unf2(x[e]);
+          mn = min3(mn, w.x, w.y); mx = max3(mx, w.x, w.y);
+        }
+      }
       for (int o = 1; o < gl; o <<= 1) {
-        ea += __shfl_xor_sync(0xffffffffu, ea, o);
-        es += __shfl_xor_sync(0xffffffffu, es, o);
+        mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
       }
-      asym = ea < es;
-    }
-    const ChosenCoder cc(sc, asym);
-    uint32_t* row = stage + tk * RW;
-    if constexpr (I8 && BITS == 3) {
-      uint32_t w8[8], hw[2][4];
-      if (no_clip) pack_row_segment_i8_3<false>(cc, x, seg & 1, w8, hw);
-      else pack_row_segment_i8_3<true>(cc, x, seg & 1, w8, hw);
-      __syncwarp();                                        // the stage is zero and no longer being read
-      const int b0 = hi_bit_i8(seg, 0), b1 = hi_bit_i8(seg, 1);
+      const GroupParams p = seg_params<BITS>(mn, mx, L.sym_variant);
+      const Bounds bd(mul2, p, mn, mx);               // the same for all lanes of a group
+      bool asym = S.mode == 1;
+      if (S.mode == 2) {
+        const PairCoder pc(mul2, p, bd, p, bd);
+        float2 ea = make_float2(0.f, 0.f), es = make_float2(0.f, 0.f);
+        auto sums = [&](auto clamp) {
 #pragma unroll
-      for (int jj = 0; jj < 8; ++jj) atomicOr(&row[jj], w8[jj] << (2 * seg));
-#pragma unroll
-      for (int jj = 0; jj < 4; ++jj) atomicOr(&row[8 + jj], (hw[0][jj] << b0) | (hw[1][jj] << b1));
-    } else if constexpr (I8) {
-      uint32_t w8[8];
-      if (no_clip) pack_row_segment_i8<BITS, false>(cc, x, w8);
-      else pack_row_segment_i8<BITS, true>(cc, x, w8);
-      __syncwarp();                                        // the stage is zero and no longer being read
-#pragma unroll
-      for (int jj = 0; jj < 8; ++jj) {
-        if constexpr (BITS == 2) atomicOr(&row[jj], w8[jj] << (2 * seg));
-        else atomicOr(&row[4 * (jj >> 1) + 2 * (seg >> 1) + (jj & 1)], w8[jj] << (4 * (seg & 1)));
+          for (int e = 0; e < kSeg / 2; ++e) {
+            const float2 a = pc.template err_asym<decltype(clamp)::value>(x[e]), s = pc.template err_sym<decltype(clamp)::value>(x[e]);
+            ea.x += fabsf(a.x); ea.y += fabsf(a.y);
+            es.x += fabsf(s.x); es.y += fabsf(s.y);
+          }
+        };
+        if (bd.no_clip) sums(std::false_type{});
+        else sums(std::true_type{});
+        float a = ea.x + ea.y, s = es.x + es.y;
+        for (int o = 1; o < gl; o <<= 1) {
+          a += __shfl_xor_sync(0xffffffffu, a, o);
+          s += __shfl_xor_sync(0xffffffffu, s, o);
+        }
+        asym = a < s;
       }
-    } else {
-      uint32_t lw[4], hw[4];
-      if (no_clip) pack_row_segment<BITS, false>(cc, x, lw, hw);
-      else pack_row_segment<BITS, true>(cc, x, lw, hw);
-      __syncwarp();                                        // the stage is zero and no longer being read
+      uint32_t w8[8];                           // [2 * j + h]: bytes 16 h + 4 j .. + 3 of the segment's bit position
+      {
+        const ChosenPair cc(mul2, p, bd, asym, p, bd, asym);
+        auto codes = [&](auto clamp) {
 #pragma unroll
-      for (int jj = 0; jj < 4; ++jj) {
-        atomicOr(&row[WM * jj + w_add], lw[jj] << sh_lo);
-        if constexpr (BITS == 3) atomicOr(&row[row_hi_plane_word() + jj], hw[jj] << sh_hi);
+          for (int lw = 0; lw < 8; ++lw) {
+            const uint2 a = cc.template code_bits<decltype(clamp)::value>(x[2 * lw]), b = cc.template code_bits<decltype(clamp)::value>(x[2 * lw + 1]);
+            w8[2 * (lw & 3) + (lw >> 2)] = bytes4(a.x, a.y, b.x, b.y);
+          }
+        };
+        if (bd.no_clip) codes(std::false_type{});
+        else codes(std::true_type{});
       }
-    }
-    const int i = i0 + tk;
-    if (i < n_q && (lane & (gl - 1)) == 0)
-      store_meta(row_meta_ptr(rec, S, i0), (size_t)tk * S.n_groups + (seg >> (gl >> 1)), S.meta_bytes, group_meta(p, asym));
-    __syncwarp();
-    uint32_t* dst = reinterpret_cast<uint32_t*>(row_code_ptr(rec, S, i0));
+      __syncwarp();
+      const int i = i0 + tk;
+      unsigned char* chunk = chunk_ptr(rec, S, i0 / kChunk, sh);
+      const int in_chunk = (i0 % kChunk) + tk;
+      uint32_t* row = reinterpret_cast<uint32_t*>(chunk + S.code_in_rec) + in_chunk * RW;
+      if constexpr (BITS == 4) {
+        // segments 2q, 2q + 1 are the nibbles of the same 8 words: each of the two lanes keeps the words of two j
+        const int half = seg >> 1, odd = seg & 1;
+        uint32_t o4[4];
 #pragma unroll
-    for (int k = 0; k < RW / 4; ++k) {
-      const int idx = lane + 32 * k;
-      if (i0 + idx / RW < n_q) dst[idx] = stage[idx];
-      stage[idx] = 0u;
+        for (int k = 0; k < 8; ++k) w8[k] <<= 4 * odd;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const uint32_t keep = odd ? w8[4 + k] : w8[k], give = odd ? w8[k] : w8[4 + k];
+          o4[k] = keep | __shfl_xor_sync(0xffffffffu, give, 1);
+        }
+        if (i < n_q) {
+          *reinterpret_cast<uint2*>(row + 4 * (2 * odd) + 2 * half) = make_uint2(o4[0], o4[1]);
+          *reinterpret_cast<uint2*>(row + 4 * (2 * odd + 1) + 2 * half) = make_uint2(o4[2], o4[3]);
+        }
+      } else {
+        uint32_t o2[2];
+        if constexpr (BITS == 3) {
+          const int b0 = hi_bit_i8(seg, 0), b1 = hi_bit_i8(seg, 1);
+          uint32_t h4[4], o1[1];
+#pragma unroll
+          for (int jj = 0; jj < 4; ++jj) {
+            uint32_t lo0, hi0, lo1, hi1;
+            split_planes(w8[2 * jj], seg & 1, lo0, hi0);
+            split_planes(w8[2 * jj + 1], seg & 1, lo1, hi1);
+            w8[2 * jj] = lo0; w8[2 * jj + 1] = lo1;
+            h4[jj] = (hi0 << b0) | (hi1 << b1);
+          }
+          quad_reduce_scatter<1>(h4, seg, o1);
+          if (i < n_q) row[8 + seg] = o1[0];
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) w8[k] <<= 2 * seg;
+        quad_reduce_scatter<2>(w8, seg, o2);
+        if (i < n_q) *reinterpret_cast<uint2*>(row + 2 * seg) = make_uint2(o2[0], o2[1]);
+      }
+      if (i < n_q && (lane & (gl - 1)) == 0)
+        store_meta(chunk + S.meta_in_rec, (in_chunk << (2 - sh)) + (seg >> sh), S.meta_bytes, group_meta(p, asym));
     }
   }
 }
 
 // ------------------------------------------------------------------ BLOCK store
-// A CTA of 64 * (G / 32) threads quantises one group of G tokens x 128 channels per iteration: thread
-// (channel pair cp, chunk k) owns tokens 32k .. 32k+31 of channels 2cp and 2cp+1, read straight from global memory
-// (one 32-bit load per token: a warp reads 128 contiguous bytes of each token row).  The two channels of a pair
-// are the two row halves of one MMA fragment row pair, so between them they fill whole words of the packed chunk
-// and no staging or atomics are needed (3-bit: the 1-bit plane's words are shared with the neighbouring pair).
-template <int BITS, bool NORM, bool I8 = false>
-__global__ void __launch_bounds__(256) quantize_blocks_prefill_kernel(Layout L, Store S, const __half* __restrict__ X,
-                                                                      int N, int n_q, unsigned char* __restrict__ cache,
-                                                                      const float* __restrict__ inv_norm) {
-  constexpr int PB = BITS == 3 ? 2 : BITS;
-  constexpr int NW = PB == 4 ? 8 : 4;
-  extern __shared__ __align__(16) unsigned char smem_q[];
-  const int G = L.G, CH = G >> 5;
-  float4* red = reinterpret_cast<float4*>(smem_q);                               // [CH][128]: mn, mx, ea, es
-  const int u = blockIdx.y, tid = threadIdx.x, cp = tid & 63, k = tid >> 6, c0 = 2 * cp;
-  float inv[2] = {1.0f, 1.0f};
-  if constexpr (NORM) { inv[0] = inv_norm[(size_t)u * kD + c0]; inv[1] = inv_norm[(size_t)u * kD + c0 + 1]; }
-  const Rec rec = unit_rec(L, cache, u);
-  const __half* Xu = X + ((size_t)u * N + L.w_sink) * kD + c0;
-  // positions (see block_pos_plane): fragment coordinates of the pair (row halves rh = 0, 1)
-  const int m = 4 * (c0 >> 6) + ((c0 >> 1) & 3), gid = (c0 >> 3) & 7;
-  const int base_lo = (m >> 2) * 128 + 16 * gid + (m & 3);                        // + 4 * tid4 (+ 256 * k-step for 4 bits)
-  const int base_hi = chunk_hi_plane_word() + 16 * gid + (m >> 1);
-  for (int j = blockIdx.x; j < n_q / G; j += gridDim.x) {
-    uint32_t raw[kSeg];
-    const __half* src = Xu + ((size_t)j * G + kSeg * k) * kD;
+// 64 * (G / 32) threads quantise one group of G tokens x 128 channels, a CTA of 256 threads 4 / (G / 32) groups at a
+// time: thread (channel pair cp, chunk k) owns tokens 32k .. 32k+31 of channels 2cp and 2cp+1, read straight from global
+// memory (one 32-bit load per token: a warp reads 128 contiguous bytes of each token row).  A pair of values is the two
+// channels of one token.  The two channels are the two row halves of one MMA fragment row pair, and the pairs that
+// share words of the packed chunk are adjacent lanes, which exchange them and store 16 contiguous bytes each (3-bit:
+// the 1-bit plane's words are shared with the other channel half, a warp away).
+// CTA `part` of `n_parts` takes a contiguous run of all units' groups.
+constexpr int kBlocksSmemWords = 4 * 128 + 4 * 32;      // uint4: statistics of 4 chunks, 1-bit plane words of 4 chunks
+template <int BITS>
+__device__ __forceinline__ void quantize_blocks(const Layout& L, const __half* __restrict__ X, int N, int n_q,
+                                                unsigned char* __restrict__ cache, int part, int n_parts, uint4* smem_q,
+                                                Mul2 mul2) {
+  const Store& S = L.v;
+  const int G = L.G, CH = G >> 5, sh = CH >> 1, per_cta = 4 >> sh, n_groups = n_q / G;
+  const int tid = threadIdx.x, cp = tid & 63, k4 = tid >> 6, k = k4 & (CH - 1), c0 = 2 * cp;
+  float4* red_m = reinterpret_cast<float4*>(smem_q);                             // [4][64]: min, max of both channels
+  float4* red_e = red_m + 4 * 64;                                                // [4][64]: error sums of both channels
+  uint4* red_h = smem_q + 4 * 128;                                               // [4][32]: 1-bit plane words
+  const int m = 4 * (c0 >> 6) + ((c0 >> 1) & 3), gid = (c0 >> 3) & 7;             // fragment coordinates of the pair
+  const long long items = (long long)L.U * n_groups, steps = (items + per_cta - 1) / per_cta;
+  for (long long step = steps * part / n_parts; step < steps * (part + 1) / n_parts; ++step) {
+    long long item = step * per_cta + (k4 >> sh);
+    const bool valid = item < items;                        // the last step may have fewer groups than the CTA takes
+    if (!valid) item = items - 1;
+    const int u = (int)(item / n_groups), j = (int)(item - (long long)u * n_groups);
+    const __half* Xu = X + ((size_t)u * N + L.w_sink) * kD + c0;
+    F2 x[kSeg];
+    {
+      uint32_t raw[kSeg];
+      const __half* src = Xu + ((size_t)j * G + kSeg * k) * kD;
 #pragma unroll
-    for (int t = 0; t < kSeg; ++t) raw[t] = __ldg(reinterpret_cast<const uint32_t*>(src + (size_t)t * kD));
-    uint32_t wlo[NW], whi[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-    for (int i = 0; i < NW; ++i) wlo[i] = 0u;
-    [[maybe_unused]] uint32_t w16[2][8];      // byte order: words [rh][2 * j + half] of this channel pair, at its bit position
-    [[maybe_unused]] uint32_t h16[I8 && BITS == 3 ? 2 : 1][8];      // ... of the 1-bit plane of 3-bit codes
-    uint32_t meta2[2];
-    if (CH > 1 || (I8 && BITS == 3)) __syncthreads();       // the previous group's exchange words are no longer read
-#pragma unroll
-    for (int rh = 0; rh < 2; ++rh) {
-      float x[kSeg];
+      for (int t = 0; t < kSeg; ++t) raw[t] = __ldg(reinterpret_cast<const uint32_t*>(src + (size_t)t * kD));
 #pragma unroll
       for (int t = 0; t < kSeg; ++t) {
-        const __half2 h2 = *reinterpret_cast<const __half2*>(&raw[t]);
-        x[t] = rh ? __high2float(h2) : __low2float(h2);
-        if constexpr (NORM) x[t] = __fmul_rn(x[t], inv[rh]);
+        const float2 v = __half22float2(*reinterpret_cast<const __half2*>(&raw[t]));
+        x[t] = f2(v.x, v.y);
       }
-      float mn, mx;
-      seg_minmax(x, mn, mx);
-      if (CH > 1) {
-        red[k * 128 + c0 + rh] = make_float4(mn, mx, 0.f, 0.f);
-        __syncthreads();
-        for (int kk = 0; kk < CH; ++kk) {
-          const float4 o = red[kk * 128 + c0 + rh];
-          mn = fminf(mn, o.x); mx = fmaxf(mx, o.y);
-        }
-      }
-      const GroupParams p = group_params(mn, mx, fmaxf(fabsf(mn), fabsf(mx)), BITS, L.sym_variant);
-      const SegCoder sc(p);
-      const bool no_clip = sc.no_clip(mn, mx);
-      bool asym = S.mode == 1;
-      if (S.mode == 2) {
-        float ea, es;
-        if (no_clip) seg_errors<false>(sc, x, ea, es);
-        else seg_errors<true>(sc, x, ea, es);
-        if (CH > 1) {
-          red[k * 128 + c0 + rh].z = ea;
-          red[k * 128 + c0 + rh].w = es;
-          __syncthreads();
-          ea = 0.f; es = 0.f;
-          for (int kk = 0; kk < CH; ++kk) {
-            const float4 o = red[kk * 128 + c0 + rh];
-            ea += o.z; es += o.w;
-          }
-        }
-        asym = ea < es;
-      }
-      const ChosenCoder cc(sc, asym);
-      if constexpr (I8 && BITS == 3) {
-        if (no_clip) pack_block_segment_i8_3<false>(cc, x, cp & 1, w16[rh], h16[rh]);
-        else pack_block_segment_i8_3<true>(cc, x, cp & 1, w16[rh], h16[rh]);
-        const int sh_hi = hi_bit_i8(cp & 3, c0 >> 6);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) { w16[rh][i] <<= 2 * (cp & 3); h16[rh][i] <<= sh_hi; }
-      } else if constexpr (I8) {
-        if (no_clip) pack_block_segment_i8<BITS, false>(cc, x, w16[rh]);
-        else pack_block_segment_i8<BITS, true>(cc, x, w16[rh]);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) w16[rh][i] <<= BITS * (BITS == 2 ? cp & 3 : cp & 1);      // this pair's bit position
-      } else {
-        uint32_t lw[NW], hw[4];
-        if (no_clip) pack_block_segment<BITS, false>(cc, x, lw, hw);
-        else pack_block_segment<BITS, true>(cc, x, lw, hw);
-#pragma unroll
-        for (int i = 0; i < NW; ++i) wlo[i] |= lw[i] << (8 * rh);
-        if constexpr (BITS == 3) {
-#pragma unroll
-          for (int i = 0; i < 4; ++i) whi[i] |= hw[i] << (4 * (2 * (m & 1) + rh));
-        }
-      }
-      meta2[rh] = group_meta(p, asym);
     }
-    uint32_t* chunk = reinterpret_cast<uint32_t*>(block_code_ptr(rec, S, j * CH + k));
-    if constexpr (I8 && BITS == 4) {
+    float2 mn = unf2(x[0]), mx = mn;
+    {
+      const float2 v = unf2(x[1]);
+      mn.x = fminf(mn.x, v.x); mn.y = fminf(mn.y, v.y);
+      mx.x = fmaxf(mx.x, v.x); mx.y = fmaxf(mx.y, v.y);
+    }
+#pragma unroll
+    for (int t = 2; t < kSeg; t += 2) {
+      const float2 v = unf2(x[t]), w = unf2(x[t + 1]);
+      mn.x = min3(mn.x, v.x, w.x); mn.y = min3(mn.y, v.y, w.y);
+      mx.x = max3(mx.x, v.x, w.x); mx.y = max3(mx.y, v.y, w.y);
+    }
+    if (CH > 1) {
+      __syncthreads();                                       // the previous group's words are no longer read
+      red_m[k4 * 64 + cp] = make_float4(mn.x, mx.x, mn.y, mx.y);
+      __syncthreads();
+      for (int kk = 0; kk < CH; ++kk) {
+        const float4 o = red_m[(k4 - k + kk) * 64 + cp];
+        mn.x = fminf(mn.x, o.x); mx.x = fmaxf(mx.x, o.y);
+        mn.y = fminf(mn.y, o.z); mx.y = fmaxf(mx.y, o.w);
+      }
+    } else if (BITS == 3) {
+      __syncthreads();
+    }
+    const GroupParams p0 = seg_params<BITS>(mn.x, mx.x, L.sym_variant), p1 = seg_params<BITS>(mn.y, mx.y, L.sym_variant);
+    const Bounds b0(mul2, p0, mn.x, mx.x), b1(mul2, p1, mn.y, mx.y);
+    const bool no_clip = b0.no_clip && b1.no_clip;
+    bool asym0 = S.mode == 1, asym1 = asym0;
+    if (S.mode == 2) {
+      const PairCoder pc(mul2, p0, b0, p1, b1);
+      float2 a0 = make_float2(0.f, 0.f), a1 = a0, s0 = a0, s1 = a0;      // even / odd tokens
+      auto sums = [&](auto clamp) {
+        constexpr bool C = decltype(clamp)::value;
+#pragma unroll
+        for (int t = 0; t < kSeg; t += 2) {
+          const float2 ae = pc.template err_asym<C>(x[t]), ao = pc.template err_asym<C>(x[t + 1]);
+          a0.x += fabsf(ae.x); a0.y += fabsf(ae.y); a1.x += fabsf(ao.x); a1.y += fabsf(ao.y);
+          const float2 se = pc.template err_sym<C>(x[t]), so = pc.template err_sym<C>(x[t + 1]);
+          s0.x += fabsf(se.x); s0.y += fabsf(se.y); s1.x += fabsf(so.x); s1.y += fabsf(so.y);
+        }
+      };
+      if (no_clip) sums(std::false_type{});
+      else sums(std::true_type{});
+      float4 e = make_float4(a0.x + a1.x, s0.x + s1.x, a0.y + a1.y, s0.y + s1.y);
+      if (CH > 1) {
+        red_e[k4 * 64 + cp] = e;
+        __syncthreads();
+        e = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int kk = 0; kk < CH; ++kk) {
+          const float4 o = red_e[(k4 - k + kk) * 64 + cp];
+          e.x += o.x; e.y += o.y; e.z += o.z; e.w += o.w;
+        }
+      }
+      asym0 = e.x < e.y;
+      asym1 = e.z < e.w;
+    }
+    // codes of token t sit in byte t / 8 of word [2 * (t % 4) + (t % 8) / 4] (see block_pos_i8), at bit position 0 here
+    uint32_t w[2][8];
+    {
+      const ChosenPair cc(mul2, p0, b0, asym0, p1, b1, asym1);
+      auto codes = [&](auto clamp) {
+        constexpr bool C = decltype(clamp)::value;
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+          const uint2 a = cc.template code_bits<C>(x[t]), b = cc.template code_bits<C>(x[t + 8]),
+                      c = cc.template code_bits<C>(x[t + 16]), d = cc.template code_bits<C>(x[t + 24]);
+          w[0][2 * (t & 3) + (t >> 2)] = bytes4(a.x, b.x, c.x, d.x);
+          w[1][2 * (t & 3) + (t >> 2)] = bytes4(a.y, b.y, c.y, d.y);
+        }
+      };
+      if (no_clip) codes(std::false_type{});
+      else codes(std::true_type{});
+    }
+    const Rec rec = unit_rec(L, cache, u);
+    unsigned char* group = group_ptr(rec, j);
+    uint32_t* chunk = reinterpret_cast<uint32_t*>(group + k * S.chunk_stride + S.code_in_rec);
+    if constexpr (BITS == 4) {
       // The two channel pairs cp = 2q, 2q + 1 (adjacent lanes) fill the two nibbles of the same 16 words: after one
       // exchange lane `pos` holds the complete words of j = 2 pos, 2 pos + 1 (16 contiguous bytes each).
       const int pos = cp & 1, W = m >> 1;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) { w[0][i] <<= 4 * pos; w[1][i] <<= 4 * pos; }
 #pragma unroll
       for (int jj = 0; jj < 2; ++jj) {
         uint32_t f4[4];
@@ -463,114 +520,206 @@ __global__ void __launch_bounds__(256) quantize_blocks_prefill_kernel(Layout L, 
         for (int rh = 0; rh < 2; ++rh)
 #pragma unroll
           for (int half = 0; half < 2; ++half) {
-            const uint32_t keep = pos ? w16[rh][2 * (2 + jj) + half] : w16[rh][2 * jj + half];
-            const uint32_t give = pos ? w16[rh][2 * jj + half] : w16[rh][2 * (2 + jj) + half];
+            const uint32_t keep = pos ? w[rh][2 * (2 + jj) + half] : w[rh][2 * jj + half];
+            const uint32_t give = pos ? w[rh][2 * jj + half] : w[rh][2 * (2 + jj) + half];
             f4[2 * half + rh] = keep | __shfl_xor_sync(0xffffffffu, give, 1);
           }
-        *reinterpret_cast<uint4*>(chunk + W * 128 + (4 * gid + 2 * pos + jj) * 4) = make_uint4(f4[0], f4[1], f4[2], f4[3]);
+        if (valid) *reinterpret_cast<uint4*>(chunk + W * 128 + (4 * gid + 2 * pos + jj) * 4) = make_uint4(f4[0], f4[1], f4[2], f4[3]);
       }
-    } else if constexpr (I8) {
-      // The four channel pairs cp = 4q .. 4q+3 (adjacent lanes) fill the four bit positions of the same 16 words.
-      // Reduce-scatter by OR: after two exchange steps lane `pos` holds the complete words of j = pos (two halves,
-      // two row halves), which are 16 contiguous bytes of the chunk.
-      const int pos = cp & 3;
-      auto reduce_scatter = [&](const uint32_t (&w)[2][8]) {
-        uint32_t h8[2][4];                    // step 1: keep j of my parity (j = 2 * i + (pos & 1)), index [rh][2 * i + half]
+    } else {
+      // The four channel pairs cp = 4q .. 4q+3 (adjacent lanes) fill the four bit positions of the same 16 words:
+      // after two exchange steps lane `pos` holds the complete words of j = pos (two halves, two row halves), which
+      // are 16 contiguous bytes of the chunk.
+      const int pos = cp & 3, W = c0 >> 6;
+      uint32_t lo[16], out[4];                              // [4 * j + 2 * half + rh]: the word order in the chunk
+      [[maybe_unused]] uint32_t hi[16];
+      const int sh_hi = hi_bit_i8(pos, W);
 #pragma unroll
-        for (int rh = 0; rh < 2; ++rh)
+      for (int rh = 0; rh < 2; ++rh)
 #pragma unroll
-          for (int i = 0; i < 2; ++i)
-#pragma unroll
-            for (int half = 0; half < 2; ++half) {
-              const uint32_t keep = (pos & 1) ? w[rh][2 * (2 * i + 1) + half] : w[rh][2 * (2 * i) + half];
-              const uint32_t give = (pos & 1) ? w[rh][2 * (2 * i) + half] : w[rh][2 * (2 * i + 1) + half];
-              h8[rh][2 * i + half] = keep | __shfl_xor_sync(0xffffffffu, give, 1);
-            }
-        uint32_t f4[4];                       // step 2: keep i = pos >> 1; index 2 * half + rh (the word order in the chunk)
-#pragma unroll
-        for (int rh = 0; rh < 2; ++rh)
-#pragma unroll
-          for (int half = 0; half < 2; ++half) {
-            const uint32_t keep = (pos & 2) ? h8[rh][2 + half] : h8[rh][half];
-            const uint32_t give = (pos & 2) ? h8[rh][half] : h8[rh][2 + half];
-            f4[2 * half + rh] = keep | __shfl_xor_sync(0xffffffffu, give, 2);
+        for (int i = 0; i < 8; ++i) {
+          uint32_t l = w[rh][i];
+          if constexpr (BITS == 3) {
+            uint32_t h;
+            split_planes(w[rh][i], pos & 1, l, h);
+            hi[2 * i + rh] = h << sh_hi;
           }
-        return make_uint4(f4[0], f4[1], f4[2], f4[3]);
-      };
-      const int W = c0 >> 6;
-      *reinterpret_cast<uint4*>(chunk + W * 128 + (4 * gid + pos) * 4) = reduce_scatter(w16);
+          lo[2 * i + rh] = l << (2 * pos);
+        }
+      quad_reduce_scatter<4>(lo, pos, out);
+      if (valid) *reinterpret_cast<uint4*>(chunk + W * 128 + (4 * gid + pos) * 4) = make_uint4(out[0], out[1], out[2], out[3]);
       if constexpr (BITS == 3) {
         // 1-bit plane: the words of lane group gid hold the bits of both halves W of the channels, which two warps
         // of this chunk's 64 threads computed: the second hands its words to the first through shared memory
-        uint4* hx = reinterpret_cast<uint4*>(smem_q + (size_t)CH * 128 * 16) + k * 32 + (cp & 31);
-        const uint4 mine = reduce_scatter(h16);
+        uint4* hx = red_h + k4 * 32 + (cp & 31);
+        quad_reduce_scatter<4>(hi, pos, out);
+        const uint4 mine = make_uint4(out[0], out[1], out[2], out[3]);
         if (W == 1) *hx = mine;
         __syncthreads();
-        if (W == 0) {
+        if (W == 0 && valid) {
           const uint4 o = *hx;
           *reinterpret_cast<uint4*>(chunk + 256 + (4 * gid + pos) * 4) =
               make_uint4(mine.x | o.x, mine.y | o.y, mine.z | o.z, mine.w | o.w);
         }
       }
-    } else {
-#pragma unroll
-      for (int i = 0; i < NW; ++i) chunk[base_lo + 4 * (i & 3) + 256 * (i >> 2)] = wlo[i];
     }
-    if constexpr (BITS == 3 && !I8) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const uint32_t full = whi[i] | __shfl_xor_sync(0xffffffffu, whi[i], 1);   // the pair with the other m & 1
-        if ((cp & 1) == 0) chunk[base_hi + 4 * i] = full;
-      }
-    }
-    if (k == 0) {
-      store_meta(block_meta_ptr(rec, S, j), block_meta_index(c0), S.meta_bytes, meta2[0]);
-      store_meta(block_meta_ptr(rec, S, j), block_meta_index(c0 + 1), S.meta_bytes, meta2[1]);
+    if (k == 0 && valid) {
+      store_meta(group + S.meta_in_rec, block_meta_index(c0), S.meta_bytes, group_meta(p0, asym0));
+      store_meta(group + S.meta_in_rec, block_meta_index(c0 + 1), S.meta_bytes, group_meta(p1, asym1));
     }
   }
+}
+
+// ------------------------------------------------------------------ key maxima, windows, counts
+// Part `part` of n_part of unit u's rows: maxima of |K| per channel, kept as floats.  One CTA of 256 threads: 16 lanes
+// of 8 channels each, 16 rows at a time.
+__device__ __forceinline__ void key_absmax_part(const __half* __restrict__ K, int N, int u, int part, int n_part,
+                                                float* __restrict__ out, float* red) {
+  const int t0 = (int)((long long)N * part / n_part), t1 = (int)((long long)N * (part + 1) / n_part);
+  const int cg = threadIdx.x & 15, rg = threadIdx.x >> 4;
+  const uint4* base = reinterpret_cast<const uint4*>(K + (size_t)u * N * kD) + cg;
+  __half2 m[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) m[i] = __float2half2_rn(0.f);
+  auto take = [&](const uint4& v) {
+    const __half2* h = reinterpret_cast<const __half2*>(&v);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) m[i] = __hmax2(m[i], __habs2(h[i]));
+  };
+  int t = t0 + rg;
+  for (; t + 16 * 7 < t1; t += 16 * 8) {      // eight rows per thread in flight
+    uint4 v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = __ldg(base + (size_t)(t + 16 * i) * 16);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) take(v[i]);
+  }
+  for (; t < t1; t += 16) take(__ldg(base + (size_t)t * 16));
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    red[rg * kD + cg * 8 + 2 * i] = __low2float(m[i]);
+    red[rg * kD + cg * 8 + 2 * i + 1] = __high2float(m[i]);
+  }
+  __syncthreads();
+  if (threadIdx.x < kD) {
+    float v = 0.f;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v = fmaxf(v, red[i * kD + threadIdx.x]);
+    out[((size_t)u * n_part + part) * kD + threadIdx.x] = v;
+  }
+}
+
+// The fp16 windows of both tensors (an unquantised cache: everything), the counts that the decode kernel compares with
+// its own N (see append_publish) and, unless the key quantiser computes them, the norms (1).  Thread `i` of `n`.
+__device__ __forceinline__ void copy_windows(const Layout& L, const Counts& cn, const __half* __restrict__ K,
+                                             const __half* __restrict__ V, unsigned char* __restrict__ cache, bool set_norm,
+                                             int i0, int n) {
+  const int N = cn.N;
+  uint32_t* counts = reinterpret_cast<uint32_t*>(cache + L.appended_off);
+  for (int i = i0; i < L.U; i += n) counts[i] = (uint32_t)N;
+  if (set_norm) {
+    float* norm = reinterpret_cast<float*>(cache + L.norm_off);
+    for (int i = i0; i < L.U * kD; i += n) norm[i] = 1.0f;
+  }
+#pragma unroll 1
+  for (int s = 0; s < 2; ++s) {
+    const Store& S = s ? L.v : L.k;
+    const __half* X = s ? V : K;
+    const int n_q = s ? cn.n_qv : cn.n_qk, per_unit = (N - n_q) * 16;      // 16-byte pieces of the tokens kept in fp16
+    for (long long i = i0; i < (long long)per_unit * L.U; i += n) {
+      const int u = (int)(i / per_unit), r = (int)(i - (long long)u * per_unit), w = r >> 4, piece = r & 15;
+      const int t = w < cn.n_sink ? w : w + n_q;
+      const bool sink = S.kind == kNone || t < L.w_sink;
+      unsigned char* dst = cache + (sink ? S.sink_off + (size_t)u * S.sink_stride + (size_t)t * kD * 2
+                                         : S.ring_off + (size_t)u * S.ring_stride + (size_t)((t - L.w_sink) % S.ring_cap) * kD * 2);
+      *reinterpret_cast<uint4*>(dst + piece * 16) = __ldg(reinterpret_cast<const uint4*>(X + ((size_t)u * N + t) * kD) + piece);
+    }
+  }
+}
+
+// First of the two launches of an inner-grouped prefill: everything that does not need the key norms.  Roles [0, n_max)
+// take the key maxima (n_part per unit), the next n_val the value groups, the rest the windows.  The first two are dealt
+// to alternate CTAs: the maxima wait for memory while the value groups beside them on the SM compute (32 units x 32768
+// tokens, 2 bits, G = 128: 164 us; one role after the other 177 us; as two launches 43 + 134 us).  A prompt of a few hundred tokens is bound by its launches, not by its kernels: ten
+// of them (clear, maxima, norms, two quantisers, four window copies, counts) took 42.6 us for 512 tokens of 8 heads.
+template <int VBITS>
+__global__ void __launch_bounds__(256, 2)
+prefill_first_kernel(const __grid_constant__ Layout L, const Counts cn, const __half* __restrict__ K,
+                     const __half* __restrict__ V, unsigned char* __restrict__ cache, float* __restrict__ absmax, int n_part,
+                     int n_max, int n_val, float neg_zero) {
+  __shared__ uint4 smem[kBlocksSmemWords];
+  static_assert(sizeof(smem) >= 16 * kD * sizeof(float), "the maxima's reduction fits");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  int b = blockIdx.x;
+  const int pairs = n_max < n_val ? n_max : n_val;
+  if (b < 2 * pairs) b = (b & 1) ? n_max + (b >> 1) : b >> 1;
+  else if (b < n_max + n_val) b = n_max > n_val ? b - pairs : n_max + (b - n_max);
+  if (b < n_max)
+    key_absmax_part(K, cn.N, b / n_part, b % n_part, n_part, absmax, reinterpret_cast<float*>(smem));
+  else if (b < n_max + n_val)
+    quantize_blocks<VBITS>(L, V, cn.N, cn.n_qv, cache, b - n_max, n_val, smem, Mul2(neg_zero));
+  else
+    copy_windows(L, cn, K, V, cache, n_max == 0, (b - n_max - n_val) * 256 + threadIdx.x, (gridDim.x - n_max - n_val) * 256);
+}
+
+__global__ void __launch_bounds__(256) prefill_windows_kernel(const __grid_constant__ Layout L, const Counts cn,
+                                                              const __half* __restrict__ K, const __half* __restrict__ V,
+                                                              unsigned char* __restrict__ cache) {
+  copy_windows(L, cn, K, V, cache, true, blockIdx.x * 256 + threadIdx.x, gridDim.x * 256);
+}
+
+int clamp_int(long long n, int lo, int hi) { return (int)(n < lo ? lo : (n > hi ? hi : n)); }
+
+int window_ctas(const Layout& L, const Counts& cn) {      // about four 16-byte pieces per thread
+  const long long pieces = (long long)L.U * 16 * (2 * cn.N - cn.n_qk - cn.n_qv) + L.U * kD;
+  return clamp_int((pieces + 1023) / 1024, 1, 148 * 8);
+}
+
+template <int KBITS>
+int launch_rows(const Layout& L, const Counts& cn, const __half* K, unsigned char* cache, const float* absmax, int n_part,
+                cudaStream_t st) {
+  // one wave of CTAs, each with at least two batches of 8 rows per warp; with norms at least one CTA (it stores them)
+  const long long batches = (long long)L.U * ((cn.n_qk + 7) / 8);
+  if (batches == 0 && !absmax) return 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(clamp_int((batches + 7) / 8, absmax ? (L.U < 148 ? L.U : 148) : 1, 148 * kRowsCtasPerSm));
+  cfg.blockDim = dim3(128); cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // see prefill_first_kernel
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = absmax ? 1 : 0;
+  const cudaError_t e =
+      absmax ? cudaLaunchKernelEx(&cfg, quantize_rows_prefill_kernel<KBITS, true>, L, K, cn.N, cn.n_qk, cache, absmax, n_part, -0.f)
+             : cudaLaunchKernelEx(&cfg, quantize_rows_prefill_kernel<KBITS, false>, L, K, cn.N, cn.n_qk, cache, absmax, n_part, -0.f);
+  return e == cudaSuccess ? 1 : -1;
 }
 
 }  // namespace
 
-static inline int grid_cap(int n, int cap) { return n < 1 ? 1 : (n > cap ? cap : n); }
-
-template <int BITS>
-static int launch_store_bits(const Layout& L, const Store& S, const __half* X, int N, int n_q, unsigned char* cache,
-                             const float* inv_norm, cudaStream_t st) {
-  if (S.kind == kRow) {
-    // a warp takes batches of 8 tokens; several batches per warp amortise its set-up (32 reciprocal norms)
-    const int n_batches = (n_q + 7) / 8;
-    const int per_unit = grid_cap((n_batches + 4 * 8 - 1) / (4 * 8), grid_cap(148 * 16 / L.U, 1 << 16));
-    dim3 grid(per_unit, L.U);
-    if (S.perm == 1) {
-      if (inv_norm) quantize_rows_prefill_kernel<BITS, true, true><<<grid, 128, 0, st>>>(L, S, X, N, n_q, cache, inv_norm);
-      else quantize_rows_prefill_kernel<BITS, false, true><<<grid, 128, 0, st>>>(L, S, X, N, n_q, cache, nullptr);
-      return cudaGetLastError() == cudaSuccess ? 1 : -1;
-    }
-    if (inv_norm) quantize_rows_prefill_kernel<BITS, true><<<grid, 128, 0, st>>>(L, S, X, N, n_q, cache, inv_norm);
-    else quantize_rows_prefill_kernel<BITS, false><<<grid, 128, 0, st>>>(L, S, X, N, n_q, cache, nullptr);
-  } else {
-    const int CH = L.G / kChunk;
-    // reduction words of groups spanning several chunks; 3-bit codes in byte order: exchange of the 1-bit plane's words
-    const int smem = CH * 128 * 16 + (BITS == 3 && S.perm == 1 ? CH * 32 * 16 : 0);
-    auto kern = inv_norm ? quantize_blocks_prefill_kernel<BITS, true> : quantize_blocks_prefill_kernel<BITS, false>;
-    if (S.perm == 1)
-      kern = inv_norm ? quantize_blocks_prefill_kernel<BITS, true, true> : quantize_blocks_prefill_kernel<BITS, false, true>;
-    const int n_groups = n_q / L.G;
-    dim3 grid(grid_cap(n_groups, grid_cap(148 * 16 / L.U, 1 << 16)), L.U);
-    kern<<<grid, 64 * CH, smem, st>>>(L, S, X, N, n_q, cache, inv_norm);
-  }
+int launch_prefill_windows(const Layout& L, const Counts& cn, unsigned char* cache, const __half* K, const __half* V,
+                           cudaStream_t st) {
+  prefill_windows_kernel<<<window_ctas(L, cn), 256, 0, st>>>(L, cn, K, V, cache);
   return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
 
-// Quantises rows / groups [0, n_q) of every unit of store S from the prefill input X ([U][N][128] fp16; the token
-// of row i is w_sink + i).  inv_norm: reciprocal key norms [U][128], or null for unnormalised values.
-int launch_quantize_store_prefill(const Layout& L, const Store& S, const __half* X, int N, int n_q, unsigned char* cache,
-                                  const float* inv_norm, cudaStream_t st) {
-  if (S.bits == 2) return launch_store_bits<2>(L, S, X, N, n_q, cache, inv_norm, st);
-  if (S.bits == 3) return launch_store_bits<3>(L, S, X, N, n_q, cache, inv_norm, st);
-  if (S.bits == 4) return launch_store_bits<4>(L, S, X, N, n_q, cache, inv_norm, st);
-  return -1;
+int launch_prefill_inner(const Layout& L, const Counts& cn, unsigned char* cache, unsigned char* ws, const __half* K,
+                         const __half* V, cudaStream_t st) {
+  float* absmax = L.k_normalize ? reinterpret_cast<float*>(ws + L.ws_partial_off) : nullptr;
+  // key maxima: about four CTAs per SM, at least 64 rows each; their results go where the decode keeps its split
+  // partials, which has max_splits rows of more than 128 floats per unit
+  static_assert(kPartialStride >= kD, "a row of partial maxima fits a split partial");
+  const int n_part = absmax ? clamp_int((cn.N + 63) / 64, 1, clamp_int((4 * 148 + L.U - 1) / L.U, 1, L.max_splits)) : 0;
+  const int n_max = n_part * L.U;
+  const long long steps = cn.n_qv > 0 ? ((long long)L.U * (cn.n_qv / L.G) * (L.G / kChunk) + 3) / 4 : 0;
+  const int n_val = clamp_int(steps, 0, 148 * 8);
+  const int grid = n_max + n_val + window_ctas(L, cn);
+  auto first = L.v.bits == 2 ? prefill_first_kernel<2> : L.v.bits == 3 ? prefill_first_kernel<3> : prefill_first_kernel<4>;
+  first<<<grid, 256, 0, st>>>(L, cn, K, V, cache, absmax, n_part, n_max, n_val, -0.f);
+  if (cudaGetLastError() != cudaSuccess) return -1;
+  const int rows = L.k.bits == 2   ? launch_rows<2>(L, cn, K, cache, absmax, n_part, st)
+                   : L.k.bits == 3 ? launch_rows<3>(L, cn, K, cache, absmax, n_part, st)
+                                   : launch_rows<4>(L, cn, K, cache, absmax, n_part, st);
+  return rows < 0 ? -1 : 1 + rows;
 }
 
 }  // namespace iq

@@ -70,6 +70,32 @@ def test_prefill_and_decode_inner(bits, G, mode, variant, N):
     check_decode(w, oc, gc, variants=(0, 1, 3, 4), splits=(0, 1, 3, 7))
 
 
+# Edges of the prefill quantisers: nothing / one row / one batch of 8 rows more or less quantised, one group more or
+# less, numbers of (unit, group) items that the CTAs do not divide evenly, caches without key norms, and values far from
+# zero in narrow groups (shift), whose rounded zero-point pushes codes out of range so that the clamping paths run.
+@pytest.mark.parametrize("kb,vb,G,N,batch,heads,norm,variant,shift", [
+    (2, 2, 32, 20, 1, 1, 1, 0, 0.0), (2, 2, 32, 21, 1, 3, 1, 0, 0.0), (3, 3, 32, 28, 1, 1, 1, 0, 0.0),
+    (4, 4, 32, 29, 5, 1, 1, 0, 0.0), (2, 3, 32, 52, 1, 37, 1, 0, 0.0), (3, 2, 64, 83, 1, 5, 1, 0, 0.0),
+    (4, 2, 64, 84, 3, 3, 1, 0, 0.0), (2, 4, 128, 148, 1, 7, 1, 0, 0.0), (3, 4, 128, 275, 1, 1, 1, 0, 0.0),
+    (2, 2, 32, 333, 1, 2, 0, 0, 0.0), (4, 3, 128, 2117, 1, 1, 0, 0, 0.0),
+    (2, 2, 32, 333, 1, 2, 1, 0, 700.0), (3, 3, 64, 333, 1, 2, 1, 1, -700.0), (4, 4, 128, 333, 1, 2, 0, 0, 700.0),
+    (2, 4, 32, 333, 1, 2, 0, 1, 3.0), (4, 2, 64, 9001, 1, 1, 1, 0, 0.0),
+])
+def test_prefill_edges(kb, vb, G, N, batch, heads, norm, variant, shift):
+    w = synth.tiny(n_tokens=N, group=G, k_bits=kb, v_bits=vb, batch=batch, n_kv_heads=heads, n_q_heads=heads, k_normalize=norm,
+                   sym_variant=variant)
+    K, V = synth.kv_all(w)
+    if shift:
+        K, V = (K * np.float16(0.1) + np.float16(shift)), (V * np.float16(0.1) + np.float16(shift))
+    oc = O.from_workload(w, max_tokens=N + 300)
+    gc = gpu_cache(w)
+    for _ in range(2):                     # the second prefill runs over the first one's workspace and cache
+        oc.prefill(K, V)
+        gc.innerq_quantize_prefill(dev(K), dev(V))
+        P.assert_export_equal(gc.innerq_cache_export(), oc.export(), O.INNER, G, True, True)
+        K, V = np.ascontiguousarray(K[..., ::-1, :]), np.ascontiguousarray(V[..., ::-1, :])
+
+
 @pytest.mark.parametrize("bits,G,N", [(2, 32, 333), (3, 64, 420), (4, 128, 541)])
 def test_prefill_and_decode_outer(bits, G, N):
     w = synth.tiny(n_tokens=N, group=G, k_bits=bits, v_bits=bits, grouping=O.OUTER, k_normalize=0,
