@@ -71,7 +71,7 @@ constexpr float kPScale = 65535.0f;          // p <= 1 as 16 bits: two unsigned 
 // streaming loop (scores taken as 0), bit 1 the value side's; all bytes are still streamed.
 // KB / VB: bits per key / value code (2, 3 or 4).
 template <int KB, int VB, int G, int KM, int VM, bool SPLIT, int CPI, bool PAGED = false, int ABL = 0>
-__device__ __forceinline__ void decode_i8_body(const Layout& L, const Counts& cn, const DecodeArgs& a, const int u,
+__device__ __forceinline__ void decode_i8_body(const Layout& L, const Counts& cn, const DecodeArgs& a, const int ux,
                                                const PageIds* ptab = nullptr) {
   using SL = StageLayout<KB, VB, G, KM, VM, CPI>;
   static_assert(KB >= 2 && KB <= 4 && VB >= 2 && VB <= 4, "2-, 3- and 4-bit codes");
@@ -90,15 +90,16 @@ __device__ __forceinline__ void decode_i8_body(const Layout& L, const Counts& cn
   const int gid = lane >> 2, j = lane & 3;
   const int split = blockIdx.y;
   if (split >= a.grid_y) return;      // batched launch: this sequence uses fewer grid rows than the longest one
-  const int b = u / L.Hkv, hkv = u % L.Hkv;
-  const int nh = min(SPLIT ? 1 : kHeads, L.r * a.n_q - a.head0);
+  int u = ux, pass = 0;               // ux = unit * passes + pass
+  if (!SPLIT && a.passes > 1) { u = ux / a.passes; pass = ux - u * a.passes; }
+  const int head0 = a.head0 + kHeads * pass;
+  const int nh = min(SPLIT ? 1 : kHeads, L.r * a.n_q - head0);
   // Row of q / out of column h of this launch: head h' = (head0 + h) % r of query token i = (head0 + h) / r
-  // (q, out: [B, n_q, Hq, D]; n_q = 1: the pass's heads are consecutive rows), and the row of its split partials.
+  // (q, out: [B, n_q, Hq, D]; n_q = 1: the pass's heads are consecutive rows).
   auto q_row = [&](int h) {
-    const int v = a.head0 + h, i = a.n_q > 1 ? v / L.r : 0;
+    const int b = u / L.Hkv, hkv = u - b * L.Hkv, v = head0 + h, i = a.n_q > 1 ? v / L.r : 0;
     return (b * a.n_q + i) * L.Hq + hkv * L.r + (v - i * L.r);
   };
-  const int prow0 = a.n_q > 1 ? u * kHeads : q_row(0);
   const int n_parts = a.grid_y;
   const bool fast = split < a.n_splits;
   // ---------------- this warp's work: tail tiles and a range of packed chunks ----------------------
@@ -277,6 +278,11 @@ __device__ __forceinline__ void decode_i8_body(const Layout& L, const Counts& cn
       dep_wait_for_iteration(s);
       if (lane == 0) issue(s);
     }
+  // What the end of the kernel needs of this waits in shared memory: kept in registers it pushes some of the streaming
+  // loop's into local memory, and worked out again there its divisions are on the critical path of the launch's end.
+  __shared__ int4 s_rows, s_end;      // rows of out; row of the split partials, unit, ticket field, heads
+  if (tid < kHeads) reinterpret_cast<int*>(&s_rows)[tid] = q_row(tid);
+  if (tid == 0) s_end = make_int4(a.n_q > 1 ? ux * kHeads : q_row(0), u, pass * a.ticket_bits, nh);
   float q_early[2], n_early[2];
 #pragma unroll
   for (int e = 0; e < 2; ++e) {
@@ -379,7 +385,7 @@ __device__ __forceinline__ void decode_i8_body(const Layout& L, const Counts& cn
     // ---- as owner of C-fragment columns 2j, 2j+1: head j, or in SPLIT (head 0, key group j)
     const int my_head = SPLIT ? 0 : j;
     // first absolute token position this lane's query row must not see (all tokens for the newest query)
-    const int pos_end = cn.n_sink + cn.n_qk + cn.n_k_recent - (a.n_q - 1 - (a.head0 + my_head) / L.r);
+    const int pos_end = cn.n_sink + cn.n_qk + cn.n_k_recent - (a.n_q - 1 - (head0 + my_head) / L.r);
     const float kfac = pow2i(qe_s[my_head]) * (1.0f / kQDigits);      // raw integer score sums -> log2-domain scores
     float Qg[SPLIT ? 1 : NG];
     if constexpr (SPLIT) {
@@ -755,6 +761,22 @@ __device__ __forceinline__ void decode_i8_body(const Layout& L, const Counts& cn
     // different phases, so it has to stay resident in the instruction cache.
 #pragma unroll 1
     for (int it = 0; it < n_iters; ++it) {
+      // The 16 bits of p are relative to the soft-max reference, so a long range loses its small ones: a launch that gives
+      // a warp several times the range it would have had (passes > 1) starts a fresh reference after every such range,
+      // between two value groups.  The reference is let down as far as the float sums, which grow by that power of two,
+      // stay below 2^40 (the sum of the head's p bounds the others); the next scores move it up to where they need it.
+      if (!SPLIT && (it & a.reset_mask) == a.reset_want) {
+        float l = l_part;
+        l += __shfl_xor_sync(0xffffffffu, l, 4);
+        l += __shfl_xor_sync(0xffffffffu, l, 8);
+        l += __shfl_xor_sync(0xffffffffu, l, 16);
+        const int room = min(40, max(0, 40 + 127 - (__float_as_int(l) >> 23)));
+        const float up = pow2i(room);
+        m_run -= (float)room;
+        l_part *= up;
+#pragma unroll
+        for (int m = 0; m < 8; ++m) { out_acc[m][0] *= up; out_acc[m][1] *= up; }
+      }
       const int st = it & (NST - 1);
       const uint32_t parity = (uint32_t)(it / NST) & 1u;
       if (!mbar_wait(bars_u32 + 8 * st, parity)) { failed = true; break; }
@@ -1087,8 +1109,9 @@ __device__ __forceinline__ void decode_i8_body(const Layout& L, const Counts& cn
       }
     }
     __syncthreads();
+    const int prow0 = s_end.x, nh_end = s_end.w;
     float* partials = a.partials;
-    for (int i = tid; i < nh * kD; i += kThreads) {
+    for (int i = tid; i < nh_end * kD; i += kThreads) {
       const int h = i >> 7, c = i & (kD - 1);
       float M = -INFINITY;
 #pragma unroll
@@ -1101,7 +1124,7 @@ __device__ __forceinline__ void decode_i8_body(const Layout& L, const Counts& cn
         num = fmaf(r_[c], wgt, num);
         den = fmaf(r_[kD + 1], wgt, den);
       }
-      float* P = partials + ((size_t)(prow0 + h) * L.max_splits + split) * kPartialStride;
+      float* P = partials + ((size_t)(prow0 + h) * a.part_stride + split) * kPartialStride;
       P[c] = num;
       if (c == 0) { P[kD] = M; P[kD + 1] = den; }
     }
@@ -1109,24 +1132,30 @@ __device__ __forceinline__ void decode_i8_body(const Layout& L, const Counts& cn
 
   // ---------------- cross-CTA merge: the last CTA of the unit to arrive combines all parts -----------
   __shared__ unsigned int s_ticket;
+  const int4 end = s_end;
   __syncthreads();                 // all partial writes of this CTA happen-before thread 0's ticket below
   if (tid == 0) {
     // release: publishes the whole CTA's partial (ordered before this thread by the barrier) with the ticket;
     // acquire: the CTA that draws the last ticket sees every other CTA's partial
     unsigned int t;
-    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;"
-                 : "=r"(t) : "l"(reinterpret_cast<unsigned int*>(a.ws + L.ws_ticket_off) + u) : "memory");
-    s_ticket = t;
+    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], %2;"
+                 : "=r"(t)
+                 : "l"(reinterpret_cast<unsigned int*>(a.ws + L.ws_ticket_off) + end.y), "r"(1u << end.z)
+                 : "memory");
+    s_ticket = (t >> end.z) & (0xffffffffu >> (32 - a.ticket_bits));
   }
   __syncthreads();
   if (s_ticket != a.grid_y - 1) return;
-  merge_parts(a.partials, reinterpret_cast<float*>(smem), a.out, nh, n_parts, prow0,
-              make_int4(q_row(0), q_row(1), q_row(2), q_row(3)), L.max_splits);
-  if (tid == 0) reinterpret_cast<unsigned int*>(a.ws + L.ws_ticket_off)[u] = 0u;   // ready for the next launch
+  merge_parts(a.partials, reinterpret_cast<float*>(smem), a.out, end.w, n_parts, end.x, s_rows, a.part_stride);
+  if (tid == 0) {                                                                  // ready for the next launch
+    unsigned int* ticket = reinterpret_cast<unsigned int*>(a.ws + L.ws_ticket_off) + end.y;
+    if (a.passes > 1) atomicSub(ticket, (unsigned int)a.grid_y << end.z);
+    else *ticket = 0u;
+  }
 }
 
 
-// One cache: block x = unit.
+// One cache: block x = (unit, pass).
 template <int KB, int VB, int G, int KM, int VM, bool SPLIT, int CPI, bool PAGED = false, int ABL = 0>
 __global__ void __launch_bounds__(kThreads, 2)
 decode_i8_kernel(const Layout L, const Counts cn, const DecodeArgs a) {
@@ -1138,12 +1167,12 @@ __global__ void __launch_bounds__(kThreads, 2)
 decode_i8_paged_kernel(const Layout L, const Counts cn, const DecodeArgs a, const __grid_constant__ PageIds P) {
   decode_i8_body<KB, VB, G, KM, VM, SPLIT, CPI, true>(L, cn, a, blockIdx.x, &P);
 }
-// Several caches of one configuration: block x = sequence * U + unit.
+// Several caches of one configuration: block x = (sequence, unit, pass).
 template <int KB, int VB, int G, int KM, int VM, bool SPLIT, int CPI, bool PAGED = false>
 __global__ void __launch_bounds__(kThreads, 2)
 decode_i8_batched_kernel(const __grid_constant__ Layout L, const __grid_constant__ SeqTable T) {
-  const int seq = blockIdx.x / L.U;
-  decode_i8_body<KB, VB, G, KM, VM, SPLIT, CPI, PAGED>(L, T.s[seq].cn, T.s[seq].a, blockIdx.x - seq * L.U);
+  const int per_seq = L.U * T.s[0].a.passes, seq = blockIdx.x / per_seq;
+  decode_i8_body<KB, VB, G, KM, VM, SPLIT, CPI, PAGED>(L, T.s[seq].cn, T.s[seq].a, blockIdx.x - seq * per_seq);
 }
 
 // ---- host side: the launchers of one metadata format (KM, VM) at every group size ---------------------------
@@ -1166,11 +1195,21 @@ int launch_i8_one_p(const Layout& L, const Counts& cn, DecodeArgs a, int n_split
     }
   }
   const int grid_y = fill_split_args<RU>(L, cn, a, false, n_splits, 0);
-  dim3 grid(L.U, grid_y);
+  a.reset_mask = 0; a.reset_want = 1;      // never
+  const int n_units = (cn.n_qv / kChunk + RU - 1) / RU;
+  const int ref_splits = std::min(a.ref_splits, (n_units + kWarps - 1) / kWarps);      // as in fill_split_args
+  if (ref_splits > a.n_splits) {
+    const int warps = kWarps * ref_splits;
+    int every = std::max(1, RU / CPI);      // a whole value group; then the largest power of two within the other range
+    while (2 * every <= n_units / warps * RU / CPI) every *= 2;
+    a.reset_mask = every - 1; a.reset_want = 0;
+  }
   int launches = 0;
-  const int step = SPLIT ? 1 : kHeads;
-  for (int h0 = 0; h0 < L.r * a.n_q; h0 += step) {
+  const int rows = L.r * a.n_q, step = SPLIT ? 1 : kHeads, per = a.passes;
+  for (int h0 = 0; h0 < rows; h0 += step * per) {
     a.head0 = h0;
+    a.passes = std::min(per, (rows - h0 + step - 1) / step);
+    const dim3 grid(L.U * a.passes, grid_y);
     // launched as a programmatic dependent of whatever precedes it in the stream (see the kernel's dep_wait)
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid; cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kSmem; cfg.stream = st;
@@ -1232,16 +1271,17 @@ int launch_i8_batched_p(const Layout& L, SeqTable& T, int n_seqs, int n_splits, 
   int grid_y = 1;
   for (int i = 0; i < n_seqs; ++i) {
     int want = chunks[i] > 0 ? (int)((chunks[i] + lo - 1) / lo) : 1;
-    if (want > L.max_splits) want = L.max_splits;
+    if (want > T.s[i].a.row_cap) want = T.s[i].a.row_cap;
     if (want > 128) want = 128;
     const int gy = fill_split_args<RU>(L, T.s[i].cn, T.s[i].a, false, want, 0);
     if (gy > grid_y) grid_y = gy;
   }
-  dim3 grid(n_seqs * L.U, grid_y);
   int launches = 0;
-  const int step = SPLIT ? 1 : kHeads;
-  for (int h0 = 0; h0 < L.r; h0 += step) {
-    for (int i = 0; i < n_seqs; ++i) T.s[i].a.head0 = h0;
+  const int step = SPLIT ? 1 : kHeads, per = T.s[0].a.passes;
+  for (int h0 = 0; h0 < L.r; h0 += step * per) {
+    const int passes = std::min(per, (L.r - h0 + step - 1) / step);
+    for (int i = 0; i < n_seqs; ++i) { T.s[i].a.head0 = h0; T.s[i].a.passes = passes; }
+    const dim3 grid(n_seqs * L.U * passes, grid_y);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid; cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kSmem; cfg.stream = st;
     cudaLaunchAttribute attr[1];

@@ -1,6 +1,8 @@
 // Host side of the fused decode kernel over the packed InnerQ cache: picks the kernel family of the cache's
 // packed format and fills the launch parameters.  The kernels are in innerq_decode_i8.cuh (inner-grouped caches,
 // one translation unit per format: innerq_decode_mma_k*v*_m*.cu) and innerq_decode_mma.cuh (outer-grouped caches).
+#include <algorithm>
+
 #include "innerq_decode_mma.h"
 #include "innerq_kernels.h"
 
@@ -76,6 +78,28 @@ int default_splits(const Layout& L, int n_units_total) {
   return n_splits;
 }
 
+// Groups of four query rows that one launch takes (passes), and what follows from it.  All of them go into one launch,
+// up to eight (more: launches of equal size): one start, one end and one read of the records from HBM instead of one per
+// group.  Fewer where the split count does not fit: with p passes a pass has 32 / p bits of a unit's ticket word to
+// count its CTAs in and, with several query tokens (whose partials live in scratch of four rows per unit), 1 / p of a
+// row's split partials.
+int fill_pass_args(const Layout& L, DecodeArgs& a, int n_splits) {
+  const int total = (L.r * a.n_q + 3) / 4, launches = (total + 7) / 8;
+  int per = (total + launches - 1) / launches;
+  auto by_ticket = [&](int p) { return p == 1 ? L.max_splits : std::min(L.max_splits, (1 << (32 / p)) - 1); };
+  auto by_part = [&](int p) { return a.n_q > 1 ? L.max_splits / p : L.max_splits; };
+  auto fits = [&](int p) {
+    if (n_splits > 0) return n_splits <= std::min(by_ticket(p), by_part(p));      // the caller's choice
+    return std::min(default_splits(L, L.U * p), by_part(p)) <= by_ticket(p);
+  };
+  while (per > 1 && !fits(per)) --per;
+  a.passes = per;
+  a.ticket_bits = 32 / per;
+  a.row_cap = std::min(by_ticket(per), by_part(per));
+  a.part_stride = by_part(per);
+  return per;
+}
+
 }  // namespace
 
 bool decode_mma_supported(const Layout& L) { return format_launcher(L) != nullptr; }
@@ -103,6 +127,10 @@ int launch_decode_mma_batched(const Layout& L, int n, const unsigned char* const
     fill_count_args(L, e.cn, e.a);
     e.a.safe_chunks = safe_chunks_for(L, Ns_safe[i], e.cn);
     e.a.n_q = 1;
+    e.a.passes = 1;      // more than four query heads per KV head: one launch per four
+    e.a.ticket_bits = 32;
+    e.a.row_cap = e.a.part_stride = L.max_splits;
+    e.a.ref_splits = e.a.reset_mask = 0; e.a.reset_want = 1;
     e.a.ablation = g_ablation;
     e.a.partials = reinterpret_cast<float*>(wss[i] + L.ws_partial_off);
     e.a.pages_host = nullptr;      // paged caches: a batched launch reads every cache's table from its buffer
@@ -115,8 +143,8 @@ int launch_decode_mma_batched(const Layout& L, int n, const unsigned char* const
 void decode_mma_set_chunks_per_iter(int n) { g_chunks_per_iter = (n == 1 || n == 2) ? n : 0; }
 void decode_mma_set_ablation(int mask) { g_ablation = mask & 3; }
 
-// n_q > 1: q and out are [B, n_q, Hq, D], the partials of a launch's (up to) four rows per unit go to
-// multi_partials [U * 4][max_splits][kPartialStride]
+// n_q > 1: q and out are [B, n_q, Hq, D], the partials of a launch's rows go to multi_partials, which holds
+// [U * 4][max_splits][kPartialStride]: with p passes [U * p * 4][max_splits / p]
 // N_safe: token count of the cache when its previous decode was launched (0: prefilled since): chunks packed by then
 // are not written by any kernel that can still be running.
 static int safe_chunks_for(const Layout& L, int N_safe, const Counts& cn_now) {
@@ -134,20 +162,25 @@ int launch_decode_mma(const Layout& L, const unsigned char* cache, unsigned char
   const FormatLauncher launch = format_launcher(L);
   if (!launch) return -2;
   const Counts cn = counts_for(L, N);
-  if (n_splits <= 0) n_splits = default_splits(L, L.U);
+  if (n_q < 1 || (n_q > 1 && !multi_partials)) return -1;
   if (n_splits > L.max_splits) n_splits = L.max_splits;
   if (n_splits > 128) n_splits = 128;            // slots of the merge tables in shared memory
   DecodeArgs a;
+  a.n_q = n_q;
+  const int per = fill_pass_args(L, a, n_splits);
+  a.ref_splits = a.reset_mask = 0; a.reset_want = 1;
+  if (n_splits <= 0) {
+    n_splits = default_splits(L, L.U * per);
+    if (per > 1) a.ref_splits = default_splits(L, L.U);
+  }
   a.cache = cache; a.ws = ws; a.q = q; a.out = out;
   a.n_splits = n_splits;
   fill_count_args(L, cn, a);
   a.safe_chunks = safe_chunks_for(L, N_safe, cn);
-  a.n_q = n_q;
   a.ablation = g_ablation;
   a.partials = n_q > 1 ? multi_partials : reinterpret_cast<float*>(ws + L.ws_partial_off);
   a.pages_host = pages_host;
   a.n_pages_host = n_pages_host;
-  if (n_q < 1 || (n_q > 1 && !multi_partials)) return -1;
   return launch(L, cn, a, n_splits, g_chunks_per_iter, st);
 }
 

@@ -29,13 +29,20 @@ struct DecodeArgs {
                          // before this kernel waits for its predecessors (programmatic dependent launch); -1: no
                          // decode since the prefill, wait before anything of the cache is read (norms included)
   int head0;             // first query row (within the KV head's r * n_q) handled by this launch
+  int passes;            // groups of four query rows per unit in this launch: block x = (unit, pass), pass p takes the rows
+                         // head0 + 4 p ..; the passes of a unit read the same records at the same time, through L2
+  int ticket_bits;       // every pass counts its arriving CTAs in its own field of the unit's ticket word
+  int row_cap;           // most grid rows: what a ticket field and part_stride hold
+  int part_stride;       // split partials per query row in `partials`
+  int ref_splits;        // > 0: the split count whose ranges the soft-max references follow (see kernel), else 0
+  int reset_mask, reset_want;   // ... a warp takes a fresh reference at iterations it with (it & mask) == want
   int n_q;               // consecutive query tokens per sequence (1: plain decode).  Row v = i * r + h of a KV head is
                          // head h of query token i; q / out are [B, n_q, Hq, D]; query i does not see the newest
                          // n_q - 1 - i tokens (all of them outside the chunks where keys AND values are packed)
   int ablation;          // timing experiments only (results are then wrong on purpose): bit 0 leaves out the key side's
                          // unpack + MMA work of the streaming loop (scores are taken as 0), bit 1 the value side's
-  float* partials;       // split partials [rows][max_splits][kPartialStride]: row = global query head (n_q == 1) or
-                         // unit * 4 + column of the launch (n_q > 1)
+  float* partials;       // split partials [rows][part_stride][kPartialStride]: row = global query head (n_q == 1) or
+                         // (unit, pass) * 4 + column of the launch (n_q > 1)
   // HOST side only (paged caches): the cache's page list, which the launcher copies into the kernel's parameter
   // space when it fits (PageIds), so that no copy of a CTA waits for a look-up in the table in device memory
   const uint32_t* pages_host;

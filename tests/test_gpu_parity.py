@@ -348,6 +348,31 @@ def test_multi_query_decode(grouping, r, G, bits, n_q):
     assert gc.innerq_read_device_error() == 0
 
 
+# Several groups of four query rows in one launch (and, beyond eight groups, in several): query heads and query tokens, key
+# rows whose length falls and rises by 2^+-10 along the context, so that the soft-max references of a warp's range move
+# both ways, peaked and flat parts of the context in one range.
+@pytest.mark.parametrize("r,n_q,G,kb,vb,N", [(8, 1, 32, 2, 2, 3001), (9, 1, 64, 3, 3, 2900), (16, 1, 128, 4, 4, 3001),
+                                             (4, 5, 32, 4, 2, 3001), (4, 9, 64, 2, 2, 2500), (1, 33, 128, 2, 2, 3001),
+                                             (5, 3, 32, 3, 2, 700), (8, 2, 64, 4, 3, 150)])
+@pytest.mark.parametrize("grouping", [O.INNER, O.OUTER])
+def test_many_query_rows_in_one_launch(grouping, r, n_q, G, kb, vb, N):
+    if grouping == O.OUTER:
+        kb = vb = 2 if kb < 4 else 4
+    w = synth.tiny(n_tokens=N, group=G, k_bits=kb, v_bits=vb, batch=1, n_kv_heads=2, n_q_heads=2 * r, w_recent=64, grouping=grouping,
+                   k_normalize=int(grouping == O.INNER), **({} if grouping == O.INNER else dict(k_mode=O.ASYM, v_mode=O.ASYM)))
+    K, V = synth.kv_all(w)
+    K = (K * np.exp2(10.0 * np.cos(np.arange(N) / 300.0) - 8.0)[None, None, :, None]).astype(np.float16)
+    oc, gc = O.from_workload(w, max_tokens=N + 300), gpu_cache(w)
+    oc.prefill(K, V)
+    gc.innerq_quantize_prefill(dev(K), dev(V))
+    q = np.stack([synth.query(w, i) for i in range(n_q)], axis=1)
+    ref = oc.decode_multi(q)
+    for _ in range(2):
+        out = gc.innerq_decode_attention_multi(dev(q)) if n_q > 1 else gc.innerq_decode_attention(dev(q[:, 0]))[:, None]
+        P.assert_outputs_close(out.cpu().numpy(), ref, f"r={r} n_q={n_q}")
+    assert gc.innerq_read_device_error() == 0
+
+
 def test_multi_query_short_contexts_and_limits():
     from paper_2602_23200_b200 import binding as B
     # everything in the windows: even sink tokens are masked by position
