@@ -195,6 +195,43 @@ def _dev_ptr(t, name: str, shape, device=None) -> int:
     return t.data_ptr()
 
 
+class _Fast:
+    """The same two checks for the calls of a decode step, which a model makes per layer and token: at 30 layers the
+    general forms above cost more host time (4-5 us a call of 12) than the kernels take on short contexts.  One attribute
+    read per property, in the order that lets a valid tensor through with the fewest; whatever does not pass goes to the
+    general form, which raises (or accepts) it.  Nothing is remembered from call to call."""
+    ready = False
+
+    @classmethod
+    def load(cls):
+        import torch
+        cls.f16, cls.empty = torch.float16, torch.empty_like
+        cls.get_device = staticmethod(torch.cuda.current_device)
+        cls.get_stream = staticmethod(lambda i: torch.cuda.current_stream(i).cuda_stream)
+        # the functions behind those two, without the Stream object and the lazy-initialisation check (a cache exists)
+        for name, attr in (("_cuda_getDevice", "get_device"), ("_cuda_getCurrentRawStream", "get_stream")):
+            if hasattr(torch._C, name):
+                setattr(cls, attr, staticmethod(getattr(torch._C, name)))
+        cls.ready = True
+
+
+def _stream_of(stream, device) -> int:
+    index = device.index
+    if stream is None and _Fast.get_device() == index:
+        return _Fast.get_stream(index)
+    return _stream_ptr(stream, device)
+
+
+def _ptr_of(t, name: str, shape, device) -> int:
+    """`shape`: a tuple."""
+    try:
+        if t.dtype is _Fast.f16 and t.shape == shape and t.get_device() == device.index and t.is_contiguous():
+            return t.data_ptr()
+    except AttributeError:
+        pass
+    return _dev_ptr(t, name, shape, device)
+
+
 def _handles(caches):
     if not caches or any(not isinstance(c, InnerQCache) for c in caches):
         raise TypeError("caches must be a non-empty sequence of InnerQCache objects")
@@ -205,23 +242,26 @@ def _handles(caches):
 def innerq_append_token_batched(caches, k_new, v_new, stream=None):
     """Appends one token to every cache of the list (same configuration, own lengths): k_new, v_new are
     fp16 [n, batch, n_kv_heads, head_dim] device tensors, row i for caches[i]."""
-    c = caches[0].cfg
-    shape = (len(caches), c.batch, c.n_kv_heads, c.head_dim)
-    _check(lib().innerq_append_token_batched(_handles(caches), len(caches), _dev_ptr(k_new, "k_new", shape, caches[0].device),
-                                             _dev_ptr(v_new, "v_new", shape, caches[0].device), _stream_ptr(stream, caches[0].device)),
-           "innerq_append_token_batched")
+    c, n = caches[0], len(caches)
+    handles = _handles(caches)
+    shape = (n,) + c._kv_shape
+    st = _lib.innerq_append_token_batched(handles, n, _ptr_of(k_new, "k_new", shape, c.device), _ptr_of(v_new, "v_new", shape, c.device),
+                                          _stream_of(stream, c.device))
+    if st < 0:
+        _check(st, "innerq_append_token_batched")
 
 
 def innerq_decode_attention_batched(caches, q, out=None, stream=None):
     """Decode attention for every cache of the list over its own tokens: q fp16 [n, batch, n_q_heads, head_dim]."""
-    import torch
-    c = caches[0].cfg
-    shape = (len(caches), c.batch, c.n_q_heads, c.head_dim)
+    c, n = caches[0], len(caches)
+    handles = _handles(caches)
+    shape = (n,) + c._q_shape
+    q_ptr = _ptr_of(q, "q", shape, c.device)
     if out is None:
-        out = torch.empty(shape, dtype=torch.float16, device=caches[0].device)
-    _check(lib().innerq_decode_attention_batched(_handles(caches), len(caches), _dev_ptr(q, "q", shape, caches[0].device),
-                                                 _dev_ptr(out, "out", shape, caches[0].device), _stream_ptr(stream, caches[0].device)),
-           "innerq_decode_attention_batched")
+        out = _Fast.empty(q)
+    st = _lib.innerq_decode_attention_batched(handles, n, q_ptr, _ptr_of(out, "out", shape, c.device), _stream_of(stream, c.device))
+    if st < 0:
+        _check(st, "innerq_decode_attention_batched")
     return out
 
 
@@ -255,6 +295,10 @@ class InnerQCache:
                                                        _stream_ptr(stream, self.device), C.byref(h)),
                        "innerq_cache_create_paged")
         self._h = h
+        self._kv_shape = (cfg.batch, cfg.n_kv_heads, cfg.head_dim)
+        self._q_shape = (cfg.batch, cfg.n_q_heads, cfg.head_dim)
+        if not _Fast.ready:
+            _Fast.load()
 
     # ---- paged caches
     def innerq_cache_pages_for(self, n_tokens: int) -> int:
@@ -308,26 +352,32 @@ class InnerQCache:
         return self.cfg.batch * self.cfg.n_kv_heads
 
     def innerq_quantize_prefill(self, k, v, stream=None):
-        c = self.cfg
+        batch, heads, dim = self._kv_shape
         n = int(k.shape[2]) if k.dim() == 4 else -1
-        shape = (c.batch, c.n_kv_heads, n, c.head_dim)
-        kp, vp = (_dev_ptr(k, "k", shape, self.device), _dev_ptr(v, "v", shape, self.device)) if n > 0 else (k.data_ptr(), v.data_ptr())
-        _check(lib().innerq_quantize_prefill(self._h, kp, vp, n, _stream_ptr(stream, self.device)), "innerq_quantize_prefill")
+        shape = (batch, heads, n, dim)
+        kp, vp = (_ptr_of(k, "k", shape, self.device), _ptr_of(v, "v", shape, self.device)) if n > 0 else (k.data_ptr(), v.data_ptr())
+        st = _lib.innerq_quantize_prefill(self._h, kp, vp, n, _stream_of(stream, self.device))
+        if st < 0:
+            _check(st, "innerq_quantize_prefill")
 
     def innerq_append_token(self, k_new, v_new, stream=None):
-        c = self.cfg
-        shape = (c.batch, c.n_kv_heads, c.head_dim)
-        _check(lib().innerq_append_token(self._h, _dev_ptr(k_new, "k_new", shape, self.device), _dev_ptr(v_new, "v_new", shape, self.device),
-                                         _stream_ptr(stream, self.device)), "innerq_append_token")
+        device = self.device
+        st = _lib.innerq_append_token(self._h, _ptr_of(k_new, "k_new", self._kv_shape, device),
+                                      _ptr_of(v_new, "v_new", self._kv_shape, device), _stream_of(stream, device))
+        if st < 0:
+            _check(st, "innerq_append_token")
 
     def innerq_decode_attention(self, q, out=None, stream=None):
-        import torch
-        c = self.cfg
-        shape = (c.batch, c.n_q_heads, c.head_dim)
+        device = self.device
+        q_ptr = _ptr_of(q, "q", self._q_shape, device)
         if out is None:
-            out = torch.empty(shape, dtype=torch.float16, device=self.device)
-        _check(lib().innerq_decode_attention(self._h, _dev_ptr(q, "q", shape, self.device), _dev_ptr(out, "out", shape, self.device),
-                                             _stream_ptr(stream, self.device)), "innerq_decode_attention")
+            out = _Fast.empty(q)
+            out_ptr = out.data_ptr()
+        else:
+            out_ptr = _ptr_of(out, "out", self._q_shape, device)
+        st = _lib.innerq_decode_attention(self._h, q_ptr, out_ptr, _stream_of(stream, device))
+        if st < 0:
+            _check(st, "innerq_decode_attention")
         return out
 
     # The two calls of a decode step with addresses instead of tensors, for loops that have validated their buffers
@@ -381,19 +431,18 @@ class InnerQCache:
         caller synchronises the stream before reading `out_host`.  The device staging buffer the C call needs
         is a torch allocation made here on first use."""
         import torch
-        c = self.cfg
-        kv_shape, q_shape = (c.batch, c.n_kv_heads, c.head_dim), (c.batch, c.n_q_heads, c.head_dim)
+        c, kv_shape, q_shape = self.cfg, self._kv_shape, self._q_shape
         for t, name, shape in ((k_new_host, "k_new_host", kv_shape), (v_new_host, "v_new_host", kv_shape),
                                (q_host, "q_host", q_shape), (out_host, "out_host", q_shape)):
-            if not (isinstance(t, torch.Tensor) and not t.is_cuda and t.dtype == torch.float16 and t.is_contiguous()
-                    and tuple(t.shape) == shape):
+            if not (isinstance(t, torch.Tensor) and not t.is_cuda and t.dtype is torch.float16 and t.shape == shape
+                    and t.is_contiguous()):
                 raise TypeError(f"{name} must be a contiguous host fp16 tensor of shape {shape}")
         if getattr(self, "_staging", None) is None:
             n = C.c_size_t()
             _check(lib().innerq_step_staging_bytes(C.byref(c), C.byref(n)), "innerq_step_staging_bytes")
             self._staging = torch.empty(n.value, dtype=torch.uint8, device=self.device)
-        _check(lib().innerq_decode_step_host(self._h, k_new_host.data_ptr(), v_new_host.data_ptr(), q_host.data_ptr(),
-                                             out_host.data_ptr(), self._staging.data_ptr(), _stream_ptr(stream, self.device)),
+        _check(_lib.innerq_decode_step_host(self._h, k_new_host.data_ptr(), v_new_host.data_ptr(), q_host.data_ptr(),
+                                            out_host.data_ptr(), self._staging.data_ptr(), _stream_of(stream, self.device)),
                "innerq_decode_step_host")
 
     def innerq_set_decode_options(self, n_splits: int = 0, variant: int = 0):
