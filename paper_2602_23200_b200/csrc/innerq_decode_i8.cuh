@@ -94,11 +94,15 @@ __device__ __forceinline__ void decode_i8_body(const Layout& L, const Counts& cn
   if (!SPLIT && a.passes > 1) { u = ux / a.passes; pass = ux - u * a.passes; }
   const int head0 = a.head0 + kHeads * pass;
   const int nh = min(SPLIT ? 1 : kHeads, L.r * a.n_q - head0);
-  // Row of q / out of column h of this launch: head h' = (head0 + h) % r of query token i = (head0 + h) / r
+  // Row of q / out of column h of a pass: head h' = (head0 + h) % r of query token i = (head0 + h) / r
   // (q, out: [B, n_q, Hq, D]; n_q = 1: the pass's heads are consecutive rows).
-  auto q_row = [&](int h) {
-    const int b = u / L.Hkv, hkv = u - b * L.Hkv, v = head0 + h, i = a.n_q > 1 ? v / L.r : 0;
+  auto q_row_of = [&](int unit, int first, int h) {
+    if (a.n_q == 1) return unit * L.r + first + h;
+    const int b = unit / L.Hkv, hkv = unit - b * L.Hkv, v = first + h, i = v / L.r;
     return (b * a.n_q + i) * L.Hq + hkv * L.r + (v - i * L.r);
+  };
+  auto q_row = [&](int h) {
+    return q_row_of(u, head0, h);
   };
   const int n_parts = a.grid_y;
   const bool fast = split < a.n_splits;
@@ -278,11 +282,8 @@ __device__ __forceinline__ void decode_i8_body(const Layout& L, const Counts& cn
       dep_wait_for_iteration(s);
       if (lane == 0) issue(s);
     }
-  // What the end of the kernel needs of this waits in shared memory: kept in registers it pushes some of the streaming
-  // loop's into local memory, and worked out again there its divisions are on the critical path of the launch's end.
-  __shared__ int4 s_rows, s_end;      // rows of out; row of the split partials, unit, ticket field, heads
-  if (tid < kHeads) reinterpret_cast<int*>(&s_rows)[tid] = q_row(tid);
-  if (tid == 0) s_end = make_int4(a.n_q > 1 ? ux * kHeads : q_row(0), u, pass * a.ticket_bits, nh);
+  __shared__ int s_head0;      // for the end of the kernel: a register of its own would cost the streaming loop one
+  if (!SPLIT && tid == 0) s_head0 = head0;
   float q_early[2], n_early[2];
 #pragma unroll
   for (int e = 0; e < 2; ++e) {
@@ -759,312 +760,318 @@ __device__ __forceinline__ void decode_i8_body(const Layout& L, const Counts& cn
 
     // The loop body is deliberately not unrolled over iterations: two CTAs of eight warps walk it at
     // different phases, so it has to stay resident in the instruction cache.
+    //
+    // The 16 bits of p are relative to the soft-max reference, so a long range loses its small ones: a launch that gives a
+    // warp several times the range it would have had (passes > 1) starts a fresh reference after every such range
+    // (reset_iters iterations, whole value groups).  An outer loop, because a test in the loop body costs every launch
+    // 0.8 % (4 x 8 KV heads x 131072 tokens, 2 bits: 62.3 us instead of 61.7).
+    int it = 0;
+    for (int it_end = !SPLIT && a.reset_iters > 0 ? min(n_iters, a.reset_iters) : n_iters;;) {
 #pragma unroll 1
-    for (int it = 0; it < n_iters; ++it) {
-      // The 16 bits of p are relative to the soft-max reference, so a long range loses its small ones: a launch that gives
-      // a warp several times the range it would have had (passes > 1) starts a fresh reference after every such range,
-      // between two value groups.  The reference is let down as far as the float sums, which grow by that power of two,
-      // stay below 2^40 (the sum of the head's p bounds the others); the next scores move it up to where they need it.
-      if (!SPLIT && (it & a.reset_mask) == a.reset_want) {
-        float l = l_part;
-        l += __shfl_xor_sync(0xffffffffu, l, 4);
-        l += __shfl_xor_sync(0xffffffffu, l, 8);
-        l += __shfl_xor_sync(0xffffffffu, l, 16);
-        const int room = min(40, max(0, 40 + 127 - (__float_as_int(l) >> 23)));
-        const float up = pow2i(room);
-        m_run -= (float)room;
-        l_part *= up;
-#pragma unroll
-        for (int m = 0; m < 8; ++m) { out_acc[m][0] *= up; out_acc[m][1] *= up; }
-      }
-      const int st = it & (NST - 1);
-      const uint32_t parity = (uint32_t)(it / NST) & 1u;
-      if (!mbar_wait(bars_u32 + 8 * st, parity)) { failed = true; break; }
-      const unsigned char* sp = ring + st * SL::kBytes;
-      const int ci0 = c_lo + it * CPI;                           // first chunk of this iteration (unit-relative)
-      const bool last_valid = CPI == 1 || (it * CPI + 1 < n_chunks_w);   // odd chunk count: the last half is empty
+      for (; it < it_end; ++it) {
+        const int st = it & (NST - 1);
+        const uint32_t parity = (uint32_t)(it / NST) & 1u;
+        if (!mbar_wait(bars_u32 + 8 * st, parity)) { failed = true; break; }
+        const unsigned char* sp = ring + st * SL::kBytes;
+        const int ci0 = c_lo + it * CPI;                           // first chunk of this iteration (unit-relative)
+        const bool last_valid = CPI == 1 || (it * CPI + 1 < n_chunks_w);   // odd chunk count: the last half is empty
 
-      // ---------------- raw scores: CPI * 2 m-tiles of 16 tokens -------------------------------------
-      // With several key groups per token and several heads per pass, the four lanes of a quad need the decoder
-      // parameters of the same (row, group) entries: lane = row decodes its row's NG entries once, the warp exchanges
-      // them through its side area (free between the value groups' ends), each lane reads its two rows per m-tile.
-      if constexpr (kShareKMeta && !(ABL & 1)) {
+        // ---------------- raw scores: CPI * 2 m-tiles of 16 tokens -------------------------------------
+        // With several key groups per token and several heads per pass, the four lanes of a quad need the decoder
+        // parameters of the same (row, group) entries: lane = row decodes its row's NG entries once, the warp exchanges
+        // them through its side area (free between the value groups' ends), each lane reads its two rows per m-tile.
+        if constexpr (kShareKMeta && !(ABL & 1)) {
+#pragma unroll
+          for (int cc = 0; cc < CPI; ++cc) {
+            if (cc > 0 && !last_valid) continue;
+            const unsigned char* kmb = sp + SL::off(cc) + SL::kOffKMeta + lane * (NG * KM);
+            float* dst = reinterpret_cast<float*>(side) + cc * (kChunk * NG * 2) + lane * (NG * 2);
+            float sz[2 * NG];
+            if constexpr (KM == 4) {
+              uint32_t mw[NG];
+              if constexpr (NG == 4) {
+                const uint4 t = *reinterpret_cast<const uint4*>(kmb);
+                mw[0] = t.x; mw[1] = t.y; mw[2] = t.z; mw[3] = t.w;
+              } else {
+                const uint2 t = *reinterpret_cast<const uint2*>(kmb);
+                mw[0] = t.x; mw[1] = t.y;
+              }
+#pragma unroll
+              for (int g = 0; g < NG; ++g) decode_fast(mw[g], neg_half, sz[2 * g], sz[2 * g + 1]);
+            } else {
+              uint32_t hw[NG / 2];
+              if constexpr (NG == 4) {
+                const uint2 t = *reinterpret_cast<const uint2*>(kmb);
+                hw[0] = t.x; hw[1] = t.y;
+              } else {
+                hw[0] = *reinterpret_cast<const uint32_t*>(kmb);
+              }
+#pragma unroll
+              for (int g = 0; g < NG; ++g) {
+                sz[2 * g] = h2f_bits((hw[g >> 1] >> (16 * (g & 1))) & 0x7FFFu);
+                sz[2 * g + 1] = neg_half * sz[2 * g];
+              }
+            }
+#pragma unroll
+            for (int g = 0; g < NG; g += 2)
+              *reinterpret_cast<float4*>(dst + 2 * g) = make_float4(sz[2 * g], sz[2 * g + 1], sz[2 * g + 2], sz[2 * g + 3]);
+          }
+          __syncwarp();
+        }
+        float sc[CPI][2][2];
+#pragma unroll
+        for (int cc = 0; cc < CPI; ++cc) {
+          if (cc > 0 && !last_valid) {      // nothing there: this warp's range ends in the middle of the iteration
+            sc[cc][0][0] = sc[cc][0][1] = sc[cc][1][0] = sc[cc][1][1] = -INFINITY;
+            continue;
+          }
+          const uint32_t* kc = reinterpret_cast<const uint32_t*>(sp + SL::off(cc));
+          const uint32_t* km = reinterpret_cast<const uint32_t*>(sp + SL::off(cc) + SL::kOffKMeta);
+#pragma unroll
+          for (int mt = 0; mt < 2; ++mt) {
+            if constexpr (ABL & 1) sc[cc][mt][0] = sc[cc][mt][1] = 0.f;      // timing experiment: no key side
+            else if constexpr (kShareKMeta)
+              k_mtile(std::true_type{}, kc, side + cc * (kChunk * NG * 2), 16 * mt, sc[cc][mt][0], sc[cc][mt][1]);
+            else k_mtile(std::false_type{}, kc, km, 16 * mt, sc[cc][mt][0], sc[cc][mt][1]);
+          }
+        }
+        if constexpr (kShareKMeta && !(ABL & 1)) __syncwarp();      // the side area goes back to the value groups' ends
+
+        // ---------------- online softmax (log2 domain; raw scores are in integer units: times kfac) -----
+        // The reference m_run of the running sums is an INTEGER that no score so far exceeds (the ceiling of the
+        // largest one when it last moved): p = 2^(s - m_run) <= 1 fills the 16 bits of its integer image, and a move of
+        // the reference rescales the integer accumulators of the open value group by an exact shift.
+        float cmax = -INFINITY;
+#pragma unroll
+        for (int cc = 0; cc < CPI; ++cc)
+          cmax = fmaxf(cmax, fmaxf(fmaxf(sc[cc][0][0], sc[cc][0][1]), fmaxf(sc[cc][1][0], sc[cc][1][1])));
+        float m_new = m_run;
+        if (__any_sync(0xffffffffu, cmax * kfac > m_run)) {
+          cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, 4));
+          cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, 8));
+          cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, 16));
+          m_new = fmaxf(m_run, ceilf(cmax * kfac));
+          const float alpha = ex2_approx(m_run - m_new);     // 2^-k exactly; 0 on the first iteration (m_run = -inf)
+          l_part *= alpha;
+          psum *= alpha;
+#pragma unroll
+          for (int m = 0; m < 8; ++m) { out_acc[m][0] *= alpha; out_acc[m][1] *= alpha; }
+          if constexpr (!kFreshEveryChunk && !kStaticSlots) {      // (else no value group is open between iterations)
+            // sums of the open value group: (256 hi + lo) >> k, the bits that leave hi carried into lo (they weigh 256)
+            const int k = m_run == -INFINITY ? 23 : min(23, (int)(m_new - m_run));
+            const int keep = k < 23 ? -1 : 0, low = (1 << k) - 1;
+#pragma unroll
+            for (int m = 0; m < 8; ++m)
+#pragma unroll
+              for (int rh = 0; rh < 2; ++rh) {
+                const int hi = (accg[m][2 * rh] - kMagicU) & keep, lo = (accg[m][2 * rh + 1] - kMagicU) & keep;
+                accg[m][2 * rh] = kMagicU + (hi >> k);
+                accg[m][2 * rh + 1] = kMagicU + ((lo + ((hi & low) << 8)) >> k);
+              }
+          }
+        }
+        m_run = m_new;
+
 #pragma unroll
         for (int cc = 0; cc < CPI; ++cc) {
           if (cc > 0 && !last_valid) continue;
-          const unsigned char* kmb = sp + SL::off(cc) + SL::kOffKMeta + lane * (NG * KM);
-          float* dst = reinterpret_cast<float*>(side) + cc * (kChunk * NG * 2) + lane * (NG * 2);
-          float sz[2 * NG];
-          if constexpr (KM == 4) {
-            uint32_t mw[NG];
-            if constexpr (NG == 4) {
-              const uint4 t = *reinterpret_cast<const uint4*>(kmb);
-              mw[0] = t.x; mw[1] = t.y; mw[2] = t.z; mw[3] = t.w;
-            } else {
-              const uint2 t = *reinterpret_cast<const uint2*>(kmb);
-              mw[0] = t.x; mw[1] = t.y;
-            }
+          const int ci = ci0 + cc;
+          const uint32_t* vc = reinterpret_cast<const uint32_t*>(sp + SL::off(cc) + SL::kOffVCodes);
+          const uint32_t* vm = reinterpret_cast<const uint32_t*>(sp + SL::off(cc) + SL::kRec);
+          // slot: position of this chunk's value group in the SPLIT window / position of the chunk in its group
+          // (kStaticSlots: an iteration is exactly one value group, so the position is the chunk's index in the iteration)
+          const int slot = SPLIT ? (ci - c_lo) & (WIN - 1) : (kStaticSlots ? cc : ci % CH);
+          const bool group_start = slot == 0;
+          // the first MMA of a sum takes the constant as its accumulator input instead of registers set up for it
+          const bool init_here = kFreshEveryChunk || (kStaticSlots && cc == 0);
+          const bool group_end = SPLIT ? (slot == WIN - 1 || (it == n_iters - 1 && (cc == CPI - 1 || !last_valid)))
+                                       : (slot == CH - 1);
+          if (!kFreshEveryChunk && !kStaticSlots && group_start) {
 #pragma unroll
-            for (int g = 0; g < NG; ++g) decode_fast(mw[g], neg_half, sz[2 * g], sz[2 * g + 1]);
-          } else {
-            uint32_t hw[NG / 2];
-            if constexpr (NG == 4) {
-              const uint2 t = *reinterpret_cast<const uint2*>(kmb);
-              hw[0] = t.x; hw[1] = t.y;
-            } else {
-              hw[0] = *reinterpret_cast<const uint32_t*>(kmb);
-            }
+            for (int m = 0; m < 8; ++m)
 #pragma unroll
-            for (int g = 0; g < NG; ++g) {
-              sz[2 * g] = h2f_bits((hw[g >> 1] >> (16 * (g & 1))) & 0x7FFFu);
-              sz[2 * g + 1] = neg_half * sz[2 * g];
-            }
+              for (int e = 0; e < 4; ++e) accg[m][e] = kMagicU;
           }
+          // ---------------- probabilities as 16-bit integers, two base-256 digits -------------------------
+          // This lane's four tokens of the chunk are rows gid + 8 i (i = 2 mt + h), which the value chunk stores at
+          // k = 4 gid + i: its digit words are exactly one B register of the lanes that need them.
+          uint32_t Pb[4];
+          float psum_c = 0.f;
 #pragma unroll
-          for (int g = 0; g < NG; g += 2)
-            *reinterpret_cast<float4*>(dst + 2 * g) = make_float4(sz[2 * g], sz[2 * g + 1], sz[2 * g + 2], sz[2 * g + 3]);
+          for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const float p = ex2_approx(fmaf(sc[cc][mt][h], kfac, -m_new));
+              psum_c += p;
+              Pb[2 * mt + h] = __float_as_uint(fmaf(p, kPScale, kMagicUf));      // low 16 bits: rint(p * 65535)
+            }
+          l_part += psum_c;
+          if constexpr (SPLIT) psum += (j == slot) ? psum_c : 0.f;
+          else psum += psum_c;
+          const uint32_t x01 = prmt(Pb[0], Pb[1], 0x5140u), x23 = prmt(Pb[2], Pb[3], 0x5140u);   // (lo0, lo1, hi0, hi1)
+          const uint32_t Plo = prmt(x01, x23, 0x5410u), Phi = prmt(x01, x23, 0x7632u);
+          const uint32_t h0 = __shfl_sync(0xffffffffu, Phi, src0), l0 = __shfl_sync(0xffffffffu, Plo, src0);
+          const uint32_t h1 = __shfl_sync(0xffffffffu, Phi, src1), l1 = __shfl_sync(0xffffffffu, Plo, src1);
+          uint32_t b0 = (gid & 1) ? l0 : h0, b1 = (gid & 1) ? l1 : h1;
+          if (SPLIT && (gid >> 1) != slot) { b0 = 0u; b1 = 0u; }      // column pair of this chunk's window slot only
+
+          // ---------------- values: 8 m-tiles of 16 channels x one k-step of 32 tokens --------------------
+          if constexpr (!(ABL & 2) && VB == 3) {
+            // 3-bit codes: word sets W = 0, 1 of the 2-bit plane (as with 2-bit codes) and one set of the 1-bit plane,
+            // as it is for W = 0 and shifted by one for W = 1
+            const uint4 l0 = *reinterpret_cast<const uint4*>(vc + lane * 4);
+            const uint4 l1 = *reinterpret_cast<const uint4*>(vc + 128 + lane * 4);
+            const uint4 h4 = *reinterpret_cast<const uint4*>(vc + 256 + lane * 4);
+            const uint32_t lw[2][4] = {{l0.x, l0.y, l0.z, l0.w}, {l1.x, l1.y, l1.z, l1.w}};
+            const uint32_t hw[4] = {h4.x, h4.y, h4.z, h4.w};
+#pragma unroll
+            for (int W = 0; W < 2; ++W) {
+              uint32_t we[4], wo[4];
+#pragma unroll
+              for (int r = 0; r < 4; ++r) {
+                const uint32_t ze = W ? hw[r] >> 1 : hw[r], zo = W ? hw[r] << 1 : hw[r];
+                we[r] = (lw[W][r] & 0x33333333u) | (ze & 0xCCCCCCCCu);
+                wo[r] = (lw[W][r] & 0xCCCCCCCCu) | (zo & 0x33333333u);
+              }
+#pragma unroll
+              for (int pos = 0; pos < 4; ++pos) {
+                const uint32_t mk = (pos & 1) ? (0x0E0E0E0Eu << (4 * (pos >> 1))) : (0x07070707u << (4 * (pos >> 1)));
+                const uint32_t* src = (pos & 1) ? wo : we;
+                if (init_here)
+                  imma_uu_init(accg[4 * W + pos], src[0] & mk, src[1] & mk, src[2] & mk, src[3] & mk, b0, b1, kMagicU);
+                else
+                  imma_uu(accg[4 * W + pos], src[0] & mk, src[1] & mk, src[2] & mk, src[3] & mk, b0, b1);
+              }
+            }
+          } else if constexpr (!(ABL & 2) && VB == 4) {
+            // 4-bit codes: word set W = m / 2 (four words: the roles a0 .. a3), nibble m % 2
+#pragma unroll
+            for (int W = 0; W < 4; ++W) {
+              const uint4 v = *reinterpret_cast<const uint4*>(vc + W * 128 + lane * 4);
+#pragma unroll
+              for (int pos = 0; pos < 2; ++pos) {
+                const uint32_t mk = pos ? 0xF0F0F0F0u : 0x0F0F0F0Fu;
+                if (init_here)
+                  imma_uu_init(accg[2 * W + pos], v.x & mk, v.y & mk, v.z & mk, v.w & mk, b0, b1, kMagicU);
+                else
+                  imma_uu(accg[2 * W + pos], v.x & mk, v.y & mk, v.z & mk, v.w & mk, b0, b1);
+              }
+            }
+          } else if constexpr (!(ABL & 2)) {
+            const uint4 v0 = *reinterpret_cast<const uint4*>(vc + lane * 4);
+            const uint4 v1 = *reinterpret_cast<const uint4*>(vc + 128 + lane * 4);
+            const uint32_t vw[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
+#pragma unroll
+            for (int W = 0; W < 2; ++W)
+#pragma unroll
+              for (int pos = 0; pos < 4; ++pos) {
+                const uint32_t mk = 0x03030303u << (2 * pos);
+                if (init_here)
+                  imma_uu_init(accg[4 * W + pos], vw[4 * W] & mk, vw[4 * W + 1] & mk, vw[4 * W + 2] & mk, vw[4 * W + 3] & mk,
+                               b0, b1, kMagicU);
+                else
+                  imma_uu(accg[4 * W + pos], vw[4 * W] & mk, vw[4 * W + 1] & mk, vw[4 * W + 2] & mk, vw[4 * W + 3] & mk, b0, b1);
+              }
+          }
+
+          // ---------------- end of a value group: apply scale / zero-point once per channel -----------
+          const bool chunk_valid = cc == 0 || last_valid;
+          if constexpr (SPLIT) {
+            // keep this group's metadata for the end of the window (the stage will be refilled)
+            if (chunk_valid && lane * 16 < SL::kVMeta)
+              *reinterpret_cast<uint4*>(side + slot * (SL::kVMeta / 4) + lane * 4) = *reinterpret_cast<const uint4*>(vm + lane * 4);
+          }
+          if (group_end && chunk_valid) {
+            if constexpr (SPLIT) __syncwarp();
+            float pg = psum;
+            pg += __shfl_xor_sync(0xffffffffu, pg, 4);
+            pg += __shfl_xor_sync(0xffffffffu, pg, 8);
+            pg += __shfl_xor_sync(0xffffffffu, pg, 16);
+            pg *= kPScale;                                // out_acc is in units of 1 / kPScale
+            const uint32_t* vmg = SPLIT ? side + j * (SL::kVMeta / 4) : vm;    // this group's entries (slot j's in SPLIT)
+            // code sum of fragment row (m, rh): m-tile m sits at bit position m % 4 of its words (weight 4^(m % 4);
+            // 3-bit fields: 1, 2, 16, 32), with 4-bit codes in nibble m % 2
+            auto acc_sum = [&](int m, int rh) {
+              return vdigits(accg[m][2 * rh], accg[m][2 * rh + 1],
+                             VB == 2 ? pow2i(-2 * (m & 3)) : VB == 4 ? pow2i(-4 * (m & 1)) : pow2i(-(2 * (m & 2) + (m & 1))));
+            };
+            if constexpr (!SPLIT && VM == 4) {
+              // The four lanes of a quad need the same 16 entries: every lane decodes 4 of the group's 128 once, the
+              // warp exchanges (scale, zero-point) pairs through its side area (rows of 16 pairs, padded to 36 words
+              // so that the 128-bit reads of the eight lane groups fall into different banks), each lane reads its 16.
+              float* ds = reinterpret_cast<float*>(side);
+              {
+                const uint4 mw = *reinterpret_cast<const uint4*>(vmg + lane * 4);
+                const uint32_t mws[4] = {mw.x, mw.y, mw.z, mw.w};
+                float sz[8];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) decode_fast(mws[e], neg_half_v, sz[2 * e], sz[2 * e + 1]);
+                float* dst = ds + (lane >> 2) * 36 + (lane & 3) * 8;       // entries 4*lane .. 4*lane+3 = row lane/4
+                *reinterpret_cast<float4*>(dst) = make_float4(sz[0], sz[1], sz[2], sz[3]);
+                *reinterpret_cast<float4*>(dst + 4) = make_float4(sz[4], sz[5], sz[6], sz[7]);
+              }
+              __syncwarp();
+              const float4* row = reinterpret_cast<const float4*>(ds + gid * 36);
+#pragma unroll
+              for (int q8 = 0; q8 < 8; ++q8) {
+                const float4 v = row[q8];                                   // entries 2*q8, 2*q8 + 1: (s, z, s, z)
+                const int m = q8;                                           // entry idx = 2 * m + rh
+                out_acc[m][0] = fmaf(v.x, acc_sum(m, 0), fmaf(v.y, pg, out_acc[m][0]));
+                out_acc[m][1] = fmaf(v.z, acc_sum(m, 1), fmaf(v.w, pg, out_acc[m][1]));
+              }
+              __syncwarp();                                                 // the side area is reused at the next group end
+            } else if constexpr (VM == 4) {
+              const uint4* vm4 = reinterpret_cast<const uint4*>(vmg + gid * 16);
+#pragma unroll
+              for (int q4 = 0; q4 < 4; ++q4) {
+                const uint4 mw = vm4[q4];
+                const uint32_t mws[4] = {mw.x, mw.y, mw.z, mw.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                  const int idx = q4 * 4 + e, m = idx >> 1, rh = idx & 1;    // fragment row (m, rh) of lane group gid
+                  float s_, z_;
+                  decode_fast(mws[e], neg_half_v, s_, z_);
+                  out_acc[m][rh] = fmaf(s_, acc_sum(m, rh), fmaf(z_, pg, out_acc[m][rh]));
+                }
+              }
+            } else {
+              const uint4* vm4 = reinterpret_cast<const uint4*>(reinterpret_cast<const uint16_t*>(vmg) + gid * 16);
+#pragma unroll
+              for (int q4 = 0; q4 < 2; ++q4) {
+                const uint4 mw = vm4[q4];
+                const uint32_t mws[4] = {mw.x, mw.y, mw.z, mw.w};
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                  const int idx = q4 * 8 + e, m = idx >> 1, rh = idx & 1;
+                  const float s_ = h2f_bits((uint16_t)((mws[e >> 1] >> (16 * (e & 1))) & 0x7FFFu));
+                  out_acc[m][rh] = fmaf(s_, acc_sum(m, rh), fmaf(neg_half_v * s_, pg, out_acc[m][rh]));
+                }
+              }
+            }
+            psum = 0.f;
+          }
         }
+
         __syncwarp();
-      }
-      float sc[CPI][2][2];
-#pragma unroll
-      for (int cc = 0; cc < CPI; ++cc) {
-        if (cc > 0 && !last_valid) {      // nothing there: this warp's range ends in the middle of the iteration
-          sc[cc][0][0] = sc[cc][0][1] = sc[cc][1][0] = sc[cc][1][1] = -INFINITY;
-          continue;
-        }
-        const uint32_t* kc = reinterpret_cast<const uint32_t*>(sp + SL::off(cc));
-        const uint32_t* km = reinterpret_cast<const uint32_t*>(sp + SL::off(cc) + SL::kOffKMeta);
-#pragma unroll
-        for (int mt = 0; mt < 2; ++mt) {
-          if constexpr (ABL & 1) sc[cc][mt][0] = sc[cc][mt][1] = 0.f;      // timing experiment: no key side
-          else if constexpr (kShareKMeta)
-            k_mtile(std::true_type{}, kc, side + cc * (kChunk * NG * 2), 16 * mt, sc[cc][mt][0], sc[cc][mt][1]);
-          else k_mtile(std::false_type{}, kc, km, 16 * mt, sc[cc][mt][0], sc[cc][mt][1]);
+        if (it + NST < n_iters) {
+          dep_wait_for_iteration(it + NST);
+          if (lane == 0) issue(st);
         }
       }
-      if constexpr (kShareKMeta && !(ABL & 1)) __syncwarp();      // the side area goes back to the value groups' ends
-
-      // ---------------- online softmax (log2 domain; raw scores are in integer units: times kfac) -----
-      // The reference m_run of the running sums is an INTEGER that no score so far exceeds (the ceiling of the
-      // largest one when it last moved): p = 2^(s - m_run) <= 1 fills the 16 bits of its integer image, and a move of
-      // the reference rescales the integer accumulators of the open value group by an exact shift.
-      float cmax = -INFINITY;
+      if (SPLIT || it >= n_iters || failed) break;
+      // The reference is let down as far as the float sums, which grow by that power of two, stay below 2^40 (the sum of
+      // the head's p bounds the others); the next scores move it up to where they need it.
+      it_end = min(n_iters, it_end + a.reset_iters);
+      float l = l_part;
+      l += __shfl_xor_sync(0xffffffffu, l, 4);
+      l += __shfl_xor_sync(0xffffffffu, l, 8);
+      l += __shfl_xor_sync(0xffffffffu, l, 16);
+      const int room = min(40, max(0, 40 + 127 - (__float_as_int(l) >> 23)));
+      const float up = pow2i(room);
+      m_run -= (float)room;
+      l_part *= up;
 #pragma unroll
-      for (int cc = 0; cc < CPI; ++cc)
-        cmax = fmaxf(cmax, fmaxf(fmaxf(sc[cc][0][0], sc[cc][0][1]), fmaxf(sc[cc][1][0], sc[cc][1][1])));
-      float m_new = m_run;
-      if (__any_sync(0xffffffffu, cmax * kfac > m_run)) {
-        cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, 4));
-        cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, 8));
-        cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, 16));
-        m_new = fmaxf(m_run, ceilf(cmax * kfac));
-        const float alpha = ex2_approx(m_run - m_new);     // 2^-k exactly; 0 on the first iteration (m_run = -inf)
-        l_part *= alpha;
-        psum *= alpha;
-#pragma unroll
-        for (int m = 0; m < 8; ++m) { out_acc[m][0] *= alpha; out_acc[m][1] *= alpha; }
-        if constexpr (!kFreshEveryChunk && !kStaticSlots) {      // (else no value group is open between iterations)
-          // sums of the open value group: (256 hi + lo) >> k, the bits that leave hi carried into lo (they weigh 256)
-          const int k = m_run == -INFINITY ? 23 : min(23, (int)(m_new - m_run));
-          const int keep = k < 23 ? -1 : 0, low = (1 << k) - 1;
-#pragma unroll
-          for (int m = 0; m < 8; ++m)
-#pragma unroll
-            for (int rh = 0; rh < 2; ++rh) {
-              const int hi = (accg[m][2 * rh] - kMagicU) & keep, lo = (accg[m][2 * rh + 1] - kMagicU) & keep;
-              accg[m][2 * rh] = kMagicU + (hi >> k);
-              accg[m][2 * rh + 1] = kMagicU + ((lo + ((hi & low) << 8)) >> k);
-            }
-        }
-      }
-      m_run = m_new;
-
-#pragma unroll
-      for (int cc = 0; cc < CPI; ++cc) {
-        if (cc > 0 && !last_valid) continue;
-        const int ci = ci0 + cc;
-        const uint32_t* vc = reinterpret_cast<const uint32_t*>(sp + SL::off(cc) + SL::kOffVCodes);
-        const uint32_t* vm = reinterpret_cast<const uint32_t*>(sp + SL::off(cc) + SL::kRec);
-        // slot: position of this chunk's value group in the SPLIT window / position of the chunk in its group
-        // (kStaticSlots: an iteration is exactly one value group, so the position is the chunk's index in the iteration)
-        const int slot = SPLIT ? (ci - c_lo) & (WIN - 1) : (kStaticSlots ? cc : ci % CH);
-        const bool group_start = slot == 0;
-        // the first MMA of a sum takes the constant as its accumulator input instead of registers set up for it
-        const bool init_here = kFreshEveryChunk || (kStaticSlots && cc == 0);
-        const bool group_end = SPLIT ? (slot == WIN - 1 || (it == n_iters - 1 && (cc == CPI - 1 || !last_valid)))
-                                     : (slot == CH - 1);
-        if (!kFreshEveryChunk && !kStaticSlots && group_start) {
-#pragma unroll
-          for (int m = 0; m < 8; ++m)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) accg[m][e] = kMagicU;
-        }
-        // ---------------- probabilities as 16-bit integers, two base-256 digits -------------------------
-        // This lane's four tokens of the chunk are rows gid + 8 i (i = 2 mt + h), which the value chunk stores at
-        // k = 4 gid + i: its digit words are exactly one B register of the lanes that need them.
-        uint32_t Pb[4];
-        float psum_c = 0.f;
-#pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const float p = ex2_approx(fmaf(sc[cc][mt][h], kfac, -m_new));
-            psum_c += p;
-            Pb[2 * mt + h] = __float_as_uint(fmaf(p, kPScale, kMagicUf));      // low 16 bits: rint(p * 65535)
-          }
-        l_part += psum_c;
-        if constexpr (SPLIT) psum += (j == slot) ? psum_c : 0.f;
-        else psum += psum_c;
-        const uint32_t x01 = prmt(Pb[0], Pb[1], 0x5140u), x23 = prmt(Pb[2], Pb[3], 0x5140u);   // (lo0, lo1, hi0, hi1)
-        const uint32_t Plo = prmt(x01, x23, 0x5410u), Phi = prmt(x01, x23, 0x7632u);
-        const uint32_t h0 = __shfl_sync(0xffffffffu, Phi, src0), l0 = __shfl_sync(0xffffffffu, Plo, src0);
-        const uint32_t h1 = __shfl_sync(0xffffffffu, Phi, src1), l1 = __shfl_sync(0xffffffffu, Plo, src1);
-        uint32_t b0 = (gid & 1) ? l0 : h0, b1 = (gid & 1) ? l1 : h1;
-        if (SPLIT && (gid >> 1) != slot) { b0 = 0u; b1 = 0u; }      // column pair of this chunk's window slot only
-
-        // ---------------- values: 8 m-tiles of 16 channels x one k-step of 32 tokens --------------------
-        if constexpr (!(ABL & 2) && VB == 3) {
-          // 3-bit codes: word sets W = 0, 1 of the 2-bit plane (as with 2-bit codes) and one set of the 1-bit plane,
-          // as it is for W = 0 and shifted by one for W = 1
-          const uint4 l0 = *reinterpret_cast<const uint4*>(vc + lane * 4);
-          const uint4 l1 = *reinterpret_cast<const uint4*>(vc + 128 + lane * 4);
-          const uint4 h4 = *reinterpret_cast<const uint4*>(vc + 256 + lane * 4);
-          const uint32_t lw[2][4] = {{l0.x, l0.y, l0.z, l0.w}, {l1.x, l1.y, l1.z, l1.w}};
-          const uint32_t hw[4] = {h4.x, h4.y, h4.z, h4.w};
-#pragma unroll
-          for (int W = 0; W < 2; ++W) {
-            uint32_t we[4], wo[4];
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-              const uint32_t ze = W ? hw[r] >> 1 : hw[r], zo = W ? hw[r] << 1 : hw[r];
-              we[r] = (lw[W][r] & 0x33333333u) | (ze & 0xCCCCCCCCu);
-              wo[r] = (lw[W][r] & 0xCCCCCCCCu) | (zo & 0x33333333u);
-            }
-#pragma unroll
-            for (int pos = 0; pos < 4; ++pos) {
-              const uint32_t mk = (pos & 1) ? (0x0E0E0E0Eu << (4 * (pos >> 1))) : (0x07070707u << (4 * (pos >> 1)));
-              const uint32_t* src = (pos & 1) ? wo : we;
-              if (init_here)
-                imma_uu_init(accg[4 * W + pos], src[0] & mk, src[1] & mk, src[2] & mk, src[3] & mk, b0, b1, kMagicU);
-              else
-                imma_uu(accg[4 * W + pos], src[0] & mk, src[1] & mk, src[2] & mk, src[3] & mk, b0, b1);
-            }
-          }
-        } else if constexpr (!(ABL & 2) && VB == 4) {
-          // 4-bit codes: word set W = m / 2 (four words: the roles a0 .. a3), nibble m % 2
-#pragma unroll
-          for (int W = 0; W < 4; ++W) {
-            const uint4 v = *reinterpret_cast<const uint4*>(vc + W * 128 + lane * 4);
-#pragma unroll
-            for (int pos = 0; pos < 2; ++pos) {
-              const uint32_t mk = pos ? 0xF0F0F0F0u : 0x0F0F0F0Fu;
-              if (init_here)
-                imma_uu_init(accg[2 * W + pos], v.x & mk, v.y & mk, v.z & mk, v.w & mk, b0, b1, kMagicU);
-              else
-                imma_uu(accg[2 * W + pos], v.x & mk, v.y & mk, v.z & mk, v.w & mk, b0, b1);
-            }
-          }
-        } else if constexpr (!(ABL & 2)) {
-          const uint4 v0 = *reinterpret_cast<const uint4*>(vc + lane * 4);
-          const uint4 v1 = *reinterpret_cast<const uint4*>(vc + 128 + lane * 4);
-          const uint32_t vw[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-#pragma unroll
-          for (int W = 0; W < 2; ++W)
-#pragma unroll
-            for (int pos = 0; pos < 4; ++pos) {
-              const uint32_t mk = 0x03030303u << (2 * pos);
-              if (init_here)
-                imma_uu_init(accg[4 * W + pos], vw[4 * W] & mk, vw[4 * W + 1] & mk, vw[4 * W + 2] & mk, vw[4 * W + 3] & mk,
-                             b0, b1, kMagicU);
-              else
-                imma_uu(accg[4 * W + pos], vw[4 * W] & mk, vw[4 * W + 1] & mk, vw[4 * W + 2] & mk, vw[4 * W + 3] & mk, b0, b1);
-            }
-        }
-
-        // ---------------- end of a value group: apply scale / zero-point once per channel -----------
-        const bool chunk_valid = cc == 0 || last_valid;
-        if constexpr (SPLIT) {
-          // keep this group's metadata for the end of the window (the stage will be refilled)
-          if (chunk_valid && lane * 16 < SL::kVMeta)
-            *reinterpret_cast<uint4*>(side + slot * (SL::kVMeta / 4) + lane * 4) = *reinterpret_cast<const uint4*>(vm + lane * 4);
-        }
-        if (group_end && chunk_valid) {
-          if constexpr (SPLIT) __syncwarp();
-          float pg = psum;
-          pg += __shfl_xor_sync(0xffffffffu, pg, 4);
-          pg += __shfl_xor_sync(0xffffffffu, pg, 8);
-          pg += __shfl_xor_sync(0xffffffffu, pg, 16);
-          pg *= kPScale;                                // out_acc is in units of 1 / kPScale
-          const uint32_t* vmg = SPLIT ? side + j * (SL::kVMeta / 4) : vm;    // this group's entries (slot j's in SPLIT)
-          // code sum of fragment row (m, rh): m-tile m sits at bit position m % 4 of its words (weight 4^(m % 4);
-          // 3-bit fields: 1, 2, 16, 32), with 4-bit codes in nibble m % 2
-          auto acc_sum = [&](int m, int rh) {
-            return vdigits(accg[m][2 * rh], accg[m][2 * rh + 1],
-                           VB == 2 ? pow2i(-2 * (m & 3)) : VB == 4 ? pow2i(-4 * (m & 1)) : pow2i(-(2 * (m & 2) + (m & 1))));
-          };
-          if constexpr (!SPLIT && VM == 4) {
-            // The four lanes of a quad need the same 16 entries: every lane decodes 4 of the group's 128 once, the
-            // warp exchanges (scale, zero-point) pairs through its side area (rows of 16 pairs, padded to 36 words
-            // so that the 128-bit reads of the eight lane groups fall into different banks), each lane reads its 16.
-            float* ds = reinterpret_cast<float*>(side);
-            {
-              const uint4 mw = *reinterpret_cast<const uint4*>(vmg + lane * 4);
-              const uint32_t mws[4] = {mw.x, mw.y, mw.z, mw.w};
-              float sz[8];
-#pragma unroll
-              for (int e = 0; e < 4; ++e) decode_fast(mws[e], neg_half_v, sz[2 * e], sz[2 * e + 1]);
-              float* dst = ds + (lane >> 2) * 36 + (lane & 3) * 8;       // entries 4*lane .. 4*lane+3 = row lane/4
-              *reinterpret_cast<float4*>(dst) = make_float4(sz[0], sz[1], sz[2], sz[3]);
-              *reinterpret_cast<float4*>(dst + 4) = make_float4(sz[4], sz[5], sz[6], sz[7]);
-            }
-            __syncwarp();
-            const float4* row = reinterpret_cast<const float4*>(ds + gid * 36);
-#pragma unroll
-            for (int q8 = 0; q8 < 8; ++q8) {
-              const float4 v = row[q8];                                   // entries 2*q8, 2*q8 + 1: (s, z, s, z)
-              const int m = q8;                                           // entry idx = 2 * m + rh
-              out_acc[m][0] = fmaf(v.x, acc_sum(m, 0), fmaf(v.y, pg, out_acc[m][0]));
-              out_acc[m][1] = fmaf(v.z, acc_sum(m, 1), fmaf(v.w, pg, out_acc[m][1]));
-            }
-            __syncwarp();                                                 // the side area is reused at the next group end
-          } else if constexpr (VM == 4) {
-            const uint4* vm4 = reinterpret_cast<const uint4*>(vmg + gid * 16);
-#pragma unroll
-            for (int q4 = 0; q4 < 4; ++q4) {
-              const uint4 mw = vm4[q4];
-              const uint32_t mws[4] = {mw.x, mw.y, mw.z, mw.w};
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                const int idx = q4 * 4 + e, m = idx >> 1, rh = idx & 1;    // fragment row (m, rh) of lane group gid
-                float s_, z_;
-                decode_fast(mws[e], neg_half_v, s_, z_);
-                out_acc[m][rh] = fmaf(s_, acc_sum(m, rh), fmaf(z_, pg, out_acc[m][rh]));
-              }
-            }
-          } else {
-            const uint4* vm4 = reinterpret_cast<const uint4*>(reinterpret_cast<const uint16_t*>(vmg) + gid * 16);
-#pragma unroll
-            for (int q4 = 0; q4 < 2; ++q4) {
-              const uint4 mw = vm4[q4];
-              const uint32_t mws[4] = {mw.x, mw.y, mw.z, mw.w};
-#pragma unroll
-              for (int e = 0; e < 8; ++e) {
-                const int idx = q4 * 8 + e, m = idx >> 1, rh = idx & 1;
-                const float s_ = h2f_bits((uint16_t)((mws[e >> 1] >> (16 * (e & 1))) & 0x7FFFu));
-                out_acc[m][rh] = fmaf(s_, acc_sum(m, rh), fmaf(neg_half_v * s_, pg, out_acc[m][rh]));
-              }
-            }
-          }
-          psum = 0.f;
-        }
-      }
-
-      __syncwarp();
-      if (it + NST < n_iters) {
-        dep_wait_for_iteration(it + NST);
-        if (lane == 0) issue(st);
-      }
+      for (int m = 0; m < 8; ++m) { out_acc[m][0] *= up; out_acc[m][1] *= up; }
     }
 
     // the partials and tickets written below are also shared with the previous decode
@@ -1109,7 +1116,8 @@ __device__ __forceinline__ void decode_i8_body(const Layout& L, const Counts& cn
       }
     }
     __syncthreads();
-    const int prow0 = s_end.x, nh_end = s_end.w;
+    const int first = SPLIT ? a.head0 : s_head0, nh_end = min(SPLIT ? 1 : kHeads, L.r * a.n_q - first);
+    const int prow0 = a.n_q > 1 ? ux * kHeads : q_row_of(u, first, 0);
     float* partials = a.partials;
     for (int i = tid; i < nh_end * kD; i += kThreads) {
       const int h = i >> 7, c = i & (kD - 1);
@@ -1132,7 +1140,8 @@ __device__ __forceinline__ void decode_i8_body(const Layout& L, const Counts& cn
 
   // ---------------- cross-CTA merge: the last CTA of the unit to arrive combines all parts -----------
   __shared__ unsigned int s_ticket;
-  const int4 end = s_end;
+  const int first = SPLIT ? a.head0 : s_head0, nh_end = min(SPLIT ? 1 : kHeads, L.r * a.n_q - first);
+  const int shift = SPLIT ? 0 : (first - a.head0) / kHeads * a.ticket_bits;      // this pass's field of the unit's ticket word
   __syncthreads();                 // all partial writes of this CTA happen-before thread 0's ticket below
   if (tid == 0) {
     // release: publishes the whole CTA's partial (ordered before this thread by the barrier) with the ticket;
@@ -1140,16 +1149,18 @@ __device__ __forceinline__ void decode_i8_body(const Layout& L, const Counts& cn
     unsigned int t;
     asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], %2;"
                  : "=r"(t)
-                 : "l"(reinterpret_cast<unsigned int*>(a.ws + L.ws_ticket_off) + end.y), "r"(1u << end.z)
+                 : "l"(reinterpret_cast<unsigned int*>(a.ws + L.ws_ticket_off) + u), "r"(1u << shift)
                  : "memory");
-    s_ticket = (t >> end.z) & (0xffffffffu >> (32 - a.ticket_bits));
+    s_ticket = SPLIT ? t : (t >> shift) & (0xffffffffu >> (32 - a.ticket_bits));
   }
   __syncthreads();
   if (s_ticket != a.grid_y - 1) return;
-  merge_parts(a.partials, reinterpret_cast<float*>(smem), a.out, end.w, n_parts, end.x, s_rows, a.part_stride);
+  merge_parts(a.partials, reinterpret_cast<float*>(smem), a.out, nh_end, n_parts,
+              a.n_q > 1 ? ux * kHeads : q_row_of(u, first, 0),
+              make_int4(q_row_of(u, first, 0), q_row_of(u, first, 1), q_row_of(u, first, 2), q_row_of(u, first, 3)), a.part_stride);
   if (tid == 0) {                                                                  // ready for the next launch
-    unsigned int* ticket = reinterpret_cast<unsigned int*>(a.ws + L.ws_ticket_off) + end.y;
-    if (a.passes > 1) atomicSub(ticket, (unsigned int)a.grid_y << end.z);
+    unsigned int* ticket = reinterpret_cast<unsigned int*>(a.ws + L.ws_ticket_off) + u;
+    if (!SPLIT && a.passes > 1) atomicSub(ticket, (unsigned int)a.grid_y << shift);
     else *ticket = 0u;
   }
 }
@@ -1195,15 +1206,10 @@ int launch_i8_one_p(const Layout& L, const Counts& cn, DecodeArgs a, int n_split
     }
   }
   const int grid_y = fill_split_args<RU>(L, cn, a, false, n_splits, 0);
-  a.reset_mask = 0; a.reset_want = 1;      // never
   const int n_units = (cn.n_qv / kChunk + RU - 1) / RU;
   const int ref_splits = std::min(a.ref_splits, (n_units + kWarps - 1) / kWarps);      // as in fill_split_args
-  if (ref_splits > a.n_splits) {
-    const int warps = kWarps * ref_splits;
-    int every = std::max(1, RU / CPI);      // a whole value group; then the largest power of two within the other range
-    while (2 * every <= n_units / warps * RU / CPI) every *= 2;
-    a.reset_mask = every - 1; a.reset_want = 0;
-  }
+  if (ref_splits > a.n_splits)      // the range units a warp would have had, as iterations (at least a whole value group)
+    a.reset_iters = std::max(1, std::max(1, n_units / (kWarps * ref_splits)) * RU / CPI);
   int launches = 0;
   const int rows = L.r * a.n_q, step = SPLIT ? 1 : kHeads, per = a.passes;
   for (int h0 = 0; h0 < rows; h0 += step * per) {

@@ -130,7 +130,7 @@ int launch_decode_mma_batched(const Layout& L, int n, const unsigned char* const
     e.a.passes = 1;      // more than four query heads per KV head: one launch per four
     e.a.ticket_bits = 32;
     e.a.row_cap = e.a.part_stride = L.max_splits;
-    e.a.ref_splits = e.a.reset_mask = 0; e.a.reset_want = 1;
+    e.a.ref_splits = e.a.reset_iters = 0;
     e.a.ablation = g_ablation;
     e.a.partials = reinterpret_cast<float*>(wss[i] + L.ws_partial_off);
     e.a.pages_host = nullptr;      // paged caches: a batched launch reads every cache's table from its buffer
@@ -168,7 +168,7 @@ int launch_decode_mma(const Layout& L, const unsigned char* cache, unsigned char
   DecodeArgs a;
   a.n_q = n_q;
   const int per = fill_pass_args(L, a, n_splits);
-  a.ref_splits = a.reset_mask = 0; a.reset_want = 1;
+  a.ref_splits = a.reset_iters = 0;
   if (n_splits <= 0) {
     n_splits = default_splits(L, L.U * per);
     if (per > 1) a.ref_splits = default_splits(L, L.U);

@@ -35,7 +35,7 @@ struct DecodeArgs {
   int row_cap;           // most grid rows: what a ticket field and part_stride hold
   int part_stride;       // split partials per query row in `partials`
   int ref_splits;        // > 0: the split count whose ranges the soft-max references follow (see kernel), else 0
-  int reset_mask, reset_want;   // ... a warp takes a fresh reference at iterations it with (it & mask) == want
+  int reset_iters;       // ... as loop iterations between two fresh references of a warp (0: none but the first)
   int n_q;               // consecutive query tokens per sequence (1: plain decode).  Row v = i * r + h of a KV head is
                          // head h of query token i; q / out are [B, n_q, Hq, D]; query i does not see the newest
                          // n_q - 1 - i tokens (all of them outside the chunks where keys AND values are packed)
