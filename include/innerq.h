@@ -217,8 +217,9 @@ int innerq_step_staging_bytes(const innerq_config_t* cfg, size_t* bytes);
  *   q, out        : device, fp16 [batch, n_q, n_q_heads, head_dim]; n_q = 1 is innerq_decode_attention.
  *   dev_scratch   : device, 256-byte aligned, at least innerq_multi_query_scratch_bytes(cfg) bytes; owned by the
  *                   caller, used only during the call (split partials of up to four query rows per KV head).
- * The rows of a KV head (its n_q * r query heads) are processed four per pass over the packed cache: with one
- * query head per KV head four query tokens share one pass, with four or more each token takes its own.
+ * The rows of a KV head (its n_q * r query heads) are processed in groups of four, up to eight groups in one launch that
+ * read the packed cache together: with one query head per KV head four query tokens share a group, with four or more
+ * each token takes its own.
  * Limits: the fused kernel only (packed inner- or outer-grouped cache in a format it supports; decode variant
  * 0 or 2); the n_q - 1 newest tokens must all lie outside the token range in which keys AND values are packed
  * (always true for n_q - 1 <= w_recent once the windows are full).  Otherwise UNSUPPORTED, nothing launched.

@@ -87,7 +87,7 @@ struct Layout {
   size_t cache_bytes;
   // workspace
   size_t ws_partial_off;   // float [B*Hq][max_splits][kPartialStride]
-  size_t ws_absmax_off;    // uint32 [U][D]
+  size_t ws_absmax_off;    // [U][D] words, not used any more (the workspace keeps its size)
   size_t ws_ticket_off;    // uint32 [U]
   size_t workspace_bytes;
   // Paged record area (page_groups > 0): the group records of a cache live in pages of a pool that several caches
