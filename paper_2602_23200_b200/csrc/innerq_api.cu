@@ -7,6 +7,7 @@
 
 #include "../../include/innerq.h"
 #include "innerq_kernels.h"
+#include "innerq_split.h"
 
 using namespace iq;
 
@@ -146,10 +147,7 @@ void make_layout(const innerq_config_t& c, Layout& L, int page_tokens = 0) {
   L.k_normalize = (c.grouping == INNERQ_GROUPING_INNER && c.k_normalize) ? 1 : 0;
   L.max_tokens = c.max_tokens;
   L.sm_scale = c.sm_scale > 0.f ? c.sm_scale : 0.08838834764831845f;   // 1/sqrt(128)
-  // partial slots per query head: token-range splits plus one per 32 tokens of the fp16 tail
-  int ms = (4 * 148 + L.U - 1) / L.U;
-  ms = ms < 1 ? 1 : (ms > 64 ? 64 : ms);
-  L.max_splits = ms + (c.w_sink + c.w_recent + L.G + 31) / 32 + 1;
+  L.max_splits = max_splits_for(L.U, c.w_sink, c.w_recent, L.G);
   size_t off = 0;
   L.norm_off = off; off = align_up(off + (size_t)L.U * kD * 4, 256);
   L.appended_off = off; off = align_up(off + (size_t)L.U * 8, 256);      // counts [U], then append part tickets [U]

@@ -1205,7 +1205,7 @@ int launch_i8_one_p(const Layout& L, const Counts& cn, DecodeArgs a, int n_split
       table_in_params = true;
     }
   }
-  const int grid_y = fill_split_args<RU>(L, cn, a, false, n_splits, 0);
+  const int grid_y = fill_split_args(L, cn, a, RU, false, n_splits, 0);
   const int n_units = (cn.n_qv / kChunk + RU - 1) / RU;
   const int ref_splits = std::min(a.ref_splits, (n_units + kWarps - 1) / kWarps);      // as in fill_split_args
   if (ref_splits > a.n_splits)      // the range units a warp would have had, as iterations (at least a whole value group)
@@ -1279,7 +1279,7 @@ int launch_i8_batched_p(const Layout& L, SeqTable& T, int n_seqs, int n_splits, 
     int want = chunks[i] > 0 ? (int)((chunks[i] + lo - 1) / lo) : 1;
     if (want > T.s[i].a.row_cap) want = T.s[i].a.row_cap;
     if (want > 128) want = 128;
-    const int gy = fill_split_args<RU>(L, T.s[i].cn, T.s[i].a, false, want, 0);
+    const int gy = fill_split_args(L, T.s[i].cn, T.s[i].a, RU, false, want, 0);
     if (gy > grid_y) grid_y = gy;
   }
   int launches = 0;

@@ -1,8 +1,6 @@
 // Host side of the fused decode kernel over the packed InnerQ cache: picks the kernel family of the cache's
 // packed format and fills the launch parameters.  The kernels are in innerq_decode_i8.cuh (inner-grouped caches,
 // one translation unit per format: innerq_decode_mma_k*v*_m*.cu) and innerq_decode_mma.cuh (outer-grouped caches).
-#include <algorithm>
-
 #include "innerq_decode_mma.h"
 #include "innerq_kernels.h"
 
@@ -70,36 +68,6 @@ void fill_count_args(const Layout& L, const Counts& cn, DecodeArgs& a) {
   a.head0 = 0;
 }
 
-int default_splits(const Layout& L, int n_units_total) {
-  int n_splits = (2 * 148) / n_units_total;      // two resident CTAs per SM, one wave
-  if (n_splits < 1) n_splits = 1;
-  if (n_splits > L.max_splits) n_splits = L.max_splits;
-  if (n_splits > 128) n_splits = 128;            // slots of the merge tables in shared memory
-  return n_splits;
-}
-
-// Groups of four query rows that one launch takes (passes), and what follows from it.  All of them go into one launch,
-// up to eight (more: launches of equal size): one start, one end and one read of the records from HBM instead of one per
-// group.  Fewer where the split count does not fit: with p passes a pass has 32 / p bits of a unit's ticket word to
-// count its CTAs in and, with several query tokens (whose partials live in scratch of four rows per unit), 1 / p of a
-// row's split partials.
-int fill_pass_args(const Layout& L, DecodeArgs& a, int n_splits) {
-  const int total = (L.r * a.n_q + 3) / 4, launches = (total + 7) / 8;
-  int per = (total + launches - 1) / launches;
-  auto by_ticket = [&](int p) { return p == 1 ? L.max_splits : std::min(L.max_splits, (1 << (32 / p)) - 1); };
-  auto by_part = [&](int p) { return a.n_q > 1 ? L.max_splits / p : L.max_splits; };
-  auto fits = [&](int p) {
-    if (n_splits > 0) return n_splits <= std::min(by_ticket(p), by_part(p));      // the caller's choice
-    return std::min(default_splits(L, L.U * p), by_part(p)) <= by_ticket(p);
-  };
-  while (per > 1 && !fits(per)) --per;
-  a.passes = per;
-  a.ticket_bits = 32 / per;
-  a.row_cap = std::min(by_ticket(per), by_part(per));
-  a.part_stride = by_part(per);
-  return per;
-}
-
 }  // namespace
 
 bool decode_mma_supported(const Layout& L) { return format_launcher(L) != nullptr; }
@@ -163,16 +131,9 @@ int launch_decode_mma(const Layout& L, const unsigned char* cache, unsigned char
   if (!launch) return -2;
   const Counts cn = counts_for(L, N);
   if (n_q < 1 || (n_q > 1 && !multi_partials)) return -1;
-  if (n_splits > L.max_splits) n_splits = L.max_splits;
-  if (n_splits > 128) n_splits = 128;            // slots of the merge tables in shared memory
   DecodeArgs a;
   a.n_q = n_q;
-  const int per = fill_pass_args(L, a, n_splits);
-  a.ref_splits = a.reset_iters = 0;
-  if (n_splits <= 0) {
-    n_splits = default_splits(L, L.U * per);
-    if (per > 1) a.ref_splits = default_splits(L, L.U);
-  }
+  n_splits = plan_call(L, a, n_splits);
   a.cache = cache; a.ws = ws; a.q = q; a.out = out;
   a.n_splits = n_splits;
   fill_count_args(L, cn, a);

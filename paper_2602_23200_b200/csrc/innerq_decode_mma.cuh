@@ -35,7 +35,7 @@ namespace iq {
 
 namespace {
 
-constexpr int kWarps = 8;
+constexpr int kWarps = kSplitWarps;
 constexpr int kThreads = kWarps * 32;
 constexpr int kHeads = 4;              // query heads per pass (hi/lo columns: 8 mma columns)
 constexpr float kLog2e = 1.4426950408889634f;
@@ -1330,32 +1330,6 @@ decode_mma_batched_kernel(const __grid_constant__ Layout L, const __grid_constan
   decode_mma_body<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, PAGED>(L, T.s[seq].cn, T.s[seq].a, blockIdx.x - seq * per_seq);
 }
 
-// Split-dependent launch parameters of one cache for a grid of grid_y rows (0: choose it): how many of the rows
-// stream packed chunks, the range units per row, the tail tiles per row.  Returns grid_y.
-template <int RU>
-int fill_split_args(const Layout& L, const Counts& cn, DecodeArgs& a, bool outer, int n_splits, int grid_y) {
-  const int n_chunks = (outer ? cn.n_qk : cn.n_qv) / kChunk;
-  const int n_units = (n_chunks + RU - 1) / RU;
-  const int by_work = (n_units + kWarps - 1) / kWarps;      // at least one range unit per warp
-  if (n_splits > by_work) n_splits = by_work;
-  if (n_units == 0) n_splits = 0;
-  if (grid_y <= 0) {
-    // without packed chunks the CTAs only share the tail tiles (eight per CTA)
-    grid_y = n_splits > 0 ? n_splits : (a.n_tail_tiles + kWarps - 1) / kWarps;
-    if (grid_y < 1) grid_y = 1;
-    if (grid_y > a.row_cap) grid_y = a.row_cap;
-  }
-  if (n_splits > grid_y) n_splits = grid_y;
-  a.grid_y = grid_y;
-  a.n_splits = n_splits;
-  a.tail_cost_units = n_splits ? 1 : 0;     // a tail tile costs a warp about as much as one value group's chunks
-  const int virt = n_units + a.tail_cost_units * a.n_tail_tiles;
-  a.units_per_split = n_splits ? (virt + n_splits - 1) / n_splits : 0;
-  a.tiles_q0 = a.n_tail_tiles / grid_y;
-  a.tiles_rem = a.n_tail_tiles % grid_y;
-  return grid_y;
-}
-
 template <int KB, int VB, int G, int KM, int VM, bool SPLIT, int CPI, bool OUTER = false, bool PAGED = false>
 int launch_one_p(const Layout& L, const Counts& cn, DecodeArgs a, int n_splits, cudaStream_t st) {
   using SL = StageLayout<KB, VB, G, KM, VM, CPI>;
@@ -1374,7 +1348,7 @@ int launch_one_p(const Layout& L, const Counts& cn, DecodeArgs a, int n_splits, 
       table_in_params = true;
     }
   }
-  const int grid_y = fill_split_args<RU>(L, cn, a, OUTER, n_splits, 0);
+  const int grid_y = fill_split_args(L, cn, a, RU, OUTER, n_splits, 0);
   int launches = 0;
   const int rows = L.r * a.n_q, step = SPLIT ? 1 : kHeads, per = a.passes;
   for (int h0 = 0; h0 < rows; h0 += step * per) {
@@ -1449,7 +1423,7 @@ int launch_one_batched_p(const Layout& L, SeqTable& T, int n_seqs, int n_splits,
     int want = chunks[i] > 0 ? (int)((chunks[i] + lo - 1) / lo) : 1;
     if (want > T.s[i].a.row_cap) want = T.s[i].a.row_cap;
     if (want > 128) want = 128;
-    const int gy = fill_split_args<RU>(L, T.s[i].cn, T.s[i].a, OUTER, want, 0);
+    const int gy = fill_split_args(L, T.s[i].cn, T.s[i].a, RU, OUTER, want, 0);
     if (gy > grid_y) grid_y = gy;
   }
   int launches = 0;

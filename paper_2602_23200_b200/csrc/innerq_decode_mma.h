@@ -5,40 +5,22 @@
 #include <cuda_runtime.h>
 
 #include "innerq_layout.h"
+#include "innerq_split.h"
 
 namespace iq {
 
 // Launch parameters shared by every format's kernels (filled by launch_decode_mma).
-struct DecodeArgs {
+struct DecodeArgs : SplitArgs {
   const unsigned char* cache;
   unsigned char* ws;
   const __half* q;
   __half* out;
-  int grid_y;            // grid rows (blockIdx.y) that work on this cache: the launch's gridDim.y, or fewer for a
-                         // short sequence of a batched launch (the rows beyond it return at once)
-  int n_splits;          // CTAs per unit that stream packed chunks (blockIdx.y < n_splits <= grid_y)
-  int n_tail_tiles;      // tiles of 16 tokens outside the packed-K/packed-V range: skew tiles first, then fp16 tiles;
-                         // tile x belongs to CTA x % grid_y, warp (x / grid_y) % 8
-  int n_skew_tiles;      // of those, tiles whose keys are packed rows (values still fp16)
-  int tiles_q0, tiles_rem;   // n_tail_tiles / grid_y and n_tail_tiles % grid_y
   int k_ring_pos0, v_ring_pos0;   // ring slot of the oldest recent key token / oldest fp16 value token
-  int units_per_split;   // range units (max(value group, iteration) of chunks) per CTA, before the tail discount
-  int tail_cost_units;   // a warp streams this many range units less per tail tile it handles (load balance)
   int safe_chunks;       // chunks [0, safe_chunks) of every unit were complete before the previous decode of this cache
                          // was launched: no kernel that may still be running writes them, so they are streamed
                          // before this kernel waits for its predecessors (programmatic dependent launch); -1: no
                          // decode since the prefill, wait before anything of the cache is read (norms included)
   int head0;             // first query row (within the KV head's r * n_q) handled by this launch
-  int passes;            // groups of four query rows per unit in this launch: block x = (unit, pass), pass p takes the rows
-                         // head0 + 4 p ..; the passes of a unit read the same records at the same time, through L2
-  int ticket_bits;       // every pass counts its arriving CTAs in its own field of the unit's ticket word
-  int row_cap;           // most grid rows: what a ticket field and part_stride hold
-  int part_stride;       // split partials per query row in `partials`
-  int ref_splits;        // > 0: the split count whose ranges the soft-max references follow (see kernel), else 0
-  int reset_iters;       // ... as loop iterations between two fresh references of a warp (0: none but the first)
-  int n_q;               // consecutive query tokens per sequence (1: plain decode).  Row v = i * r + h of a KV head is
-                         // head h of query token i; q / out are [B, n_q, Hq, D]; query i does not see the newest
-                         // n_q - 1 - i tokens (all of them outside the chunks where keys AND values are packed)
   int ablation;          // timing experiments only (results are then wrong on purpose): bit 0 leaves out the key side's
                          // unpack + MMA work of the streaming loop (scores are taken as 0), bit 1 the value side's
   float* partials;       // split partials [rows][part_stride][kPartialStride]: row = global query head (n_q == 1) or

@@ -373,6 +373,21 @@ def test_many_query_rows_in_one_launch(grouping, r, n_q, G, kb, vb, N):
     assert gc.innerq_read_device_error() == 0
 
 
+# Many units with short windows: a unit has fewer split partials (7) than the call has groups of query rows (8).
+@pytest.mark.parametrize("grouping", [O.INNER, O.OUTER])
+def test_multi_query_over_many_units(grouping):
+    inner = grouping == O.INNER
+    w = synth.tiny(batch=128, n_q_heads=16, n_kv_heads=4, n_tokens=230, group=32, w_sink=4, w_recent=64, grouping=grouping,
+                   k_normalize=int(inner), **({} if inner else dict(k_mode=O.ASYM, v_mode=O.ASYM)))
+    oc, gc, _, _ = run_prefill_both(w)
+    q = np.stack([synth.query(w, i) for i in range(8)], axis=1)
+    ref = oc.decode_multi(q)
+    for splits in (0, 1):
+        gc.innerq_set_decode_options(splits, 0)
+        P.assert_outputs_close(gc.innerq_decode_attention_multi(dev(q)).cpu().numpy(), ref, f"512 units, splits={splits}")
+    assert gc.innerq_read_device_error() == 0
+
+
 def test_multi_query_short_contexts_and_limits():
     from paper_2602_23200_b200 import binding as B
     # everything in the windows: even sink tokens are masked by position

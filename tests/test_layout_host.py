@@ -28,3 +28,11 @@ def test_division_by_the_quantisers_constants_is_correctly_rounded(tmp_path):
                     os.path.join(HERE, "div_const_check.cpp")], check=True)
     r = subprocess.run([exe], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout
+
+
+@pytest.mark.skipif(shutil.which("g++") is None, reason="needs a host C++ compiler")
+def test_every_launch_has_a_grid_whose_partials_and_tickets_fit(tmp_path):
+    exe = str(tmp_path / "host_split_check")
+    subprocess.run(["g++", "-std=c++17", "-O2", "-I", CSRC, "-o", exe, os.path.join(HERE, "host_split_check.cpp")], check=True)
+    r = subprocess.run([exe], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout
