@@ -133,7 +133,7 @@ int launch_decode_mma(const Layout& L, const unsigned char* cache, unsigned char
   if (n_q < 1 || (n_q > 1 && !multi_partials)) return -1;
   DecodeArgs a;
   a.n_q = n_q;
-  n_splits = plan_call(L, a, n_splits);
+  n_splits = plan_call(L, cn, a, L.grouping == 1, n_splits);
   a.cache = cache; a.ws = ws; a.q = q; a.out = out;
   a.n_splits = n_splits;
   fill_count_args(L, cn, a);

@@ -45,37 +45,72 @@ inline int default_splits(const Layout& L, int n_units_total) {
   return std::min(std::max(1, kCtaSlots / n_units_total), std::min(L.max_splits, 128));
 }
 
-// Groups of four query rows that one launch takes (passes), and what follows from it.  All of them go into one launch,
-// up to eight (more: launches of equal size): one start, one end and one read of the records from HBM instead of one per
-// group.  Fewer where the split count does not fit: with p passes a pass has 32 / p bits of a unit's ticket word to
-// count its CTAs in and, with several query tokens (whose partials live in scratch of four rows per unit), 1 / p of a
-// row's split partials, which has to be one at least (many units with short windows have fewer than eight).
-inline int fill_pass_args(const Layout& L, SplitArgs& a, int n_splits) {
-  const int total = (L.r * a.n_q + 3) / 4, launches = (total + 7) / 8;
-  int per = (total + launches - 1) / launches;
-  auto by_ticket = [&](int p) { return p == 1 ? L.max_splits : std::min(L.max_splits, (1 << (32 / p)) - 1); };
-  auto by_part = [&](int p) { return a.n_q > 1 ? L.max_splits / p : L.max_splits; };
-  auto fits = [&](int p) {
-    if (by_part(p) < 1) return false;
-    if (n_splits > 0) return n_splits <= std::min(by_ticket(p), by_part(p));      // the caller's choice
-    return std::min(default_splits(L, L.U * p), by_part(p)) <= by_ticket(p);
-  };
-  while (per > 1 && !fits(per)) --per;
-  a.passes = per;
-  a.ticket_bits = 32 / per;
-  a.row_cap = std::min(by_ticket(per), by_part(per));
-  a.part_stride = by_part(per);
-  return per;
+// Most grid rows of a launch of p passes: a pass counts its CTAs in 32 / p bits of a unit's ticket word and, with several
+// query tokens (whose partials live in scratch of four rows per unit), has 1 / p of a row's split partials.
+inline int partial_slots(const Layout& L, int n_q, int p) { return n_q > 1 ? L.max_splits / p : L.max_splits; }
+inline int most_rows(const Layout& L, int n_q, int p) {
+  const int by_ticket = p == 1 ? L.max_splits : std::min(L.max_splits, (1 << (32 / p)) - 1);
+  return std::min(by_ticket, partial_slots(L, n_q, p));
 }
 
-// The split of a call: passes and the split count (n_splits > 0: the caller's choice), which is returned.
-inline int plan_call(const Layout& L, SplitArgs& a, int n_splits) {
+// The split of a call: groups of four query rows per launch (passes), and the split count (n_splits > 0: the caller's
+// choice), which is returned.  All groups go into one launch, up to eight, with one wave of CTAs together: one start, one
+// end and one read of the records from HBM instead of one per group.  Two things can make that the slower choice, on long
+// contexts by up to a factor of two: a wave that leaves slots idle (40 units with five groups: one split each, 200 CTAs),
+// and few units whose partials do not hold enough splits for every group (one unit with eight groups: 8 of 37).  So the
+// launches that could be made (groups per launch, splits that fill one half wave more at a time) are compared by
+//   waves * (chunks per CTA + 18) + 20 per further launch,
+// in chunks (of 32 tokens, 0.16 us): 18 are a CTA's start and end; launches overlap, so the waves are those of all CTAs
+// together; a last half wave counts 0.65, its CTAs have an SM each.  Of what is within 4 % of the best, the fewest launches
+// and longest ranges (they leave most to the neighbours in a chain of calls).  Alone / in a chain, us, against one launch
+// per group and against always one wave: 40 units x 16384 tokens, r 4, n_q 5, 4 bits: 96.7 / 77.7, 109.7 / 95.7,
+// 116.0 / 79.6; 80 x 16384, r 8: 79.0 / 59.1, 81.6 / 62.4, 106.1 / 60.6; 1 x 524288, n_q 8: 118.4 / 81.5, 128.3 / 98.4,
+// 209.1 / 83.9.
+inline int plan_call(const Layout& L, const Counts& cn, SplitArgs& a, bool outer, int n_splits) {
+  const int total = (L.r * a.n_q + 3) / 4, ru = L.G / kChunk, n_chunks = (outer ? cn.n_qk : cn.n_qv) / kChunk;
   n_splits = std::min(n_splits, std::min(L.max_splits, 128));      // 128: slots of the merge tables in shared memory
-  const int per = fill_pass_args(L, a, n_splits);
-  a.ref_splits = a.reset_iters = 0;
-  if (n_splits > 0) return n_splits;
-  if (per > 1) a.ref_splits = default_splits(L, L.U);
-  return default_splits(L, L.U * per);
+  const bool chosen = n_splits > 0;
+  int best_p = 1, best_s = chosen ? n_splits : default_splits(L, L.U);
+  if (total > 1) {
+    struct { int p, s; float cost; } cand[8 * 12];
+    int n_cand = 0;
+    float least = 0.f;
+    const int by_work = std::max(1, ((n_chunks + ru - 1) / ru + kSplitWarps - 1) / kSplitWarps);      // see fill_split_args
+    auto add = [&](int p, int s) {
+      const int launches = (total + p - 1) / p, used = std::min(s, by_work);
+      const long long ctas = (long long)L.U * total * used;
+      const long long rest = ctas % kCtaSlots;
+      const float waves = (float)(ctas / kCtaSlots) + (rest == 0 ? 0.f : rest <= kCtaSlots / 2 ? 0.65f : 1.f);
+      const float cost = waves * ((float)n_chunks / (float)used + 18.f) + 20.f * (float)(launches - 1);
+      if (n_cand == 0 || cost < least) least = cost;
+      cand[n_cand++] = {p, s, cost};
+    };
+    for (int launches = (total + 7) / 8, last = 0; launches <= total; ++launches) {
+      const int p = (total + launches - 1) / launches;
+      if (p == last) continue;
+      last = p;
+      const int cap = most_rows(L, a.n_q, p);
+      if (cap < 1 || (chosen && n_splits > cap)) continue;
+      if (chosen) { best_p = p; break; }
+      const int one_wave = std::min(default_splits(L, L.U * p), cap), most = std::min(default_splits(L, L.U), cap);
+      add(p, one_wave);
+      for (int half = 3, s = one_wave; half <= 10; ++half) {
+        const int next = (int)((long long)half * (kCtaSlots / 2) / ((long long)L.U * p));
+        if (next <= s || next > most) continue;
+        add(p, s = next);
+      }
+      if (most > one_wave) add(p, most);
+    }
+    for (int i = 0; i < n_cand && !chosen; ++i)
+      if (cand[i].cost <= 1.04f * least) { best_p = cand[i].p; best_s = cand[i].s; break; }
+  }
+  a.passes = best_p;
+  a.ticket_bits = 32 / best_p;
+  a.row_cap = most_rows(L, a.n_q, best_p);
+  a.part_stride = partial_slots(L, a.n_q, best_p);
+  a.ref_splits = !chosen && best_p > 1 ? default_splits(L, L.U) : 0;
+  a.reset_iters = 0;
+  return best_s;
 }
 
 // Split-dependent launch parameters of one cache for a grid of grid_y rows (0: choose it): how many of the rows

@@ -1,6 +1,8 @@
 // Host check of csrc/innerq_split.h over the shapes that the library accepts (no GPU): every launch has a grid, its split
-// partials fit the memory they are given, its CTAs fit the ticket field that counts them, the tail tiles are all dealt.
+// partials fit the memory they are given, its CTAs fit the ticket field that counts them, the tail tiles are all dealt,
+// and groups of query rows share a launch only where that pays.
 // Prints one line per failed property and returns 1 if there were any.
+#include <cmath>
 #include <cstdio>
 
 #include "innerq_split.h"
@@ -26,19 +28,32 @@ int main() {
                 const Counts cn = counts_for(L, N);
                 SplitArgs a = {};
                 a.n_q = n_q;
-                const int n = plan_call(L, a, n_splits);
-                a.n_skew_tiles = (cn.n_qk - cn.n_qv + 15) / 16;
-                a.n_tail_tiles = a.n_skew_tiles + (cn.n_sink + cn.n_k_recent + 15) / 16;
-                ++calls;
+                const int n = plan_call(L, cn, a, false, n_splits);
                 auto check = [&](bool ok, const char* what) {
                   if (!ok && failures++ < 20)
                     std::printf("FAIL %s: units %d windows %d %d G %d r %d n_q %d splits %d N %d: passes %d row_cap %d\n", what, U,
                                 w[0], w[1], G, r, n_q, n_splits, N, a.passes, a.row_cap);
                   return ok;
                 };
+                // an explicit split count is kept as long as a launch of one group can hold it
+                check(n_splits == 0 || n == std::min(n_splits, std::min(L.max_splits, 128)), "the caller's splits");
+                a.n_skew_tiles = (cn.n_qk - cn.n_qv + 15) / 16;
+                a.n_tail_tiles = a.n_skew_tiles + (cn.n_sink + cn.n_k_recent + 15) / 16;
+                ++calls;
                 const bool cap = check(a.row_cap >= 1 && a.row_cap <= a.part_stride, "a row of the grid");
                 check(a.passes >= 1 && a.passes <= 8 && n >= 1, "passes");
                 check(a.part_stride * (n_q > 1 ? a.passes : 1) <= L.max_splits, "partials fit their memory");
+                if (n_splits == 0) {
+                  // what the launches take, in chunks per CTA slot (starts and ends: 18; a half wave has its SMs to itself):
+                  // never much more than with one launch per group of four rows
+                  const int total = (r * n_q + 3) / 4, units = (cn.n_qv / kChunk + G / kChunk - 1) / (G / kChunk);
+                  auto time = [&](int p, int s) {
+                    s = std::min(s, std::max(1, (units + 7) / 8));
+                    const double ctas = (double)U * total * s, full = std::floor(ctas / 296), rest = ctas - 296 * full;
+                    return (full + (rest == 0 ? 0 : rest <= 148 ? 0.65 : 1)) * (cn.n_qv / 32 / (double)s + 18) + 20 * ((total + p - 1) / p - 1);
+                  };
+                  check(time(a.passes, n) <= 1.05 * time(1, default_splits(L, U)), "time against one launch per group");
+                }
                 if (!cap) continue;      // the next function divides by the grid
                 const int grid = fill_split_args(L, cn, a, G / kChunk, false, n, 0);
                 check(grid >= 1 && grid <= a.row_cap && a.n_splits <= grid, "grid rows");
