@@ -1206,10 +1206,7 @@ int launch_i8_one_p(const Layout& L, const Counts& cn, DecodeArgs a, int n_split
     }
   }
   const int grid_y = fill_split_args(L, cn, a, RU, false, n_splits, 0);
-  const int n_units = (cn.n_qv / kChunk + RU - 1) / RU;
-  const int ref_splits = std::min(a.ref_splits, (n_units + kWarps - 1) / kWarps);      // as in fill_split_args
-  if (ref_splits > a.n_splits)      // the range units a warp would have had, as iterations (at least a whole value group)
-    a.reset_iters = std::max(1, std::max(1, n_units / (kWarps * ref_splits)) * RU / CPI);
+  fill_reference_args(cn, a, RU, CPI, false);
   int launches = 0;
   const int rows = L.r * a.n_q, step = SPLIT ? 1 : kHeads, per = a.passes;
   for (int h0 = 0; h0 < rows; h0 += step * per) {

@@ -274,7 +274,9 @@ __device__ __noinline__ void merge_parts(const float* __restrict__ partials, flo
 // group.  One chunk per iteration, four heads per pass.
 // ABL (timing experiments only, results wrong on purpose): bit 0 leaves out the key side's unpack + MMA work of the
 // streaming loop (scores taken as 0), bit 1 the value side's; all bytes are still streamed.
-template <int KB, int VB, int G, int KM, int VM, bool SPLIT, int CPI, bool OUTER = false, bool PAGED = false, int ABL = 0>
+// RENEW: the soft-max references are renewed along a warp's range (a.reset_iters > 0), an instance of its own: in the others
+// the registers that this takes cost 1-5 % (16 x 8 KV heads x 8192 tokens, 4 bits, G = 64: 37.4 us without, 38.4 with).
+template <int KB, int VB, int G, int KM, int VM, bool SPLIT, int CPI, bool OUTER = false, bool PAGED = false, int ABL = 0, bool RENEW = false>
 __device__ __forceinline__ void decode_mma_body(const Layout& L, const Counts& cn, const DecodeArgs& a, const int ux,
                                                 const PageIds* ptab = nullptr) {
   constexpr int KP = KB == 3 ? 2 : KB, VP = VB == 3 ? 2 : VB;     // bits of the primary code plane
@@ -934,267 +936,302 @@ __device__ __forceinline__ void decode_mma_body(const Layout& L, const Counts& c
     __syncwarp();
     if (lane == 0 && atomicAdd(&s_past_tail, 1u) == kWarps - 1) grid_launch_dependents();
 
+    // OUTER: value sum of fragment row (m, rh); G = 32: rows of lanes 16..31 belong to the m-tile's second group
+    [[maybe_unused]] auto outer_sum = [&](int m, int rh) {
+      return NG == 4 && (gid >> 2) != 0 ? accg[m][2 * rh + 1] : accg[m][2 * rh];
+    };
+
     // The loop body is deliberately not unrolled over iterations: two CTAs of eight warps walk it at
     // different phases, so it has to stay resident in the instruction cache.
+    //
+    // RENEW: p is an fp16 operand relative to the soft-max reference, the small ones of a long range are subnormal, and the
+    // tensor cores round every addition to their sums.  Where a warp has several times the range that it would have in a
+    // launch of one group (see fill_reference_args), both start afresh after every such range.  An outer loop: a test in
+    // the loop body costs these launches 4-7 % (64 units x 16384 tokens, r 8, 2 bits, G = 64: 66 us per call in a chain,
+    // 71 with the test).
+    int it = 0;
+    for (int it_end = RENEW ? min(n_iters, a.reset_iters) : n_iters;;) {
 #pragma unroll 1
-    for (int it = 0; it < n_iters; ++it) {
-      const int st = it & (NST - 1);
-      const uint32_t parity = (uint32_t)(it / NST) & 1u;
-      if (!mbar_wait(bars_u32 + 8 * st, parity)) { failed = true; break; }
-      const unsigned char* sp = ring + st * SL::kBytes;
-      const int ci0 = c_lo + it * CPI;                           // first chunk of this iteration (unit-relative)
-      const bool last_valid = CPI == 1 || (it * CPI + 1 < n_chunks_w);   // odd chunk count: the last half is empty
+      for (; it < it_end; ++it) {
+        const int st = it & (NST - 1);
+        const uint32_t parity = (uint32_t)(it / NST) & 1u;
+        if (!mbar_wait(bars_u32 + 8 * st, parity)) { failed = true; break; }
+        const unsigned char* sp = ring + st * SL::kBytes;
+        const int ci0 = c_lo + it * CPI;                           // first chunk of this iteration (unit-relative)
+        const bool last_valid = CPI == 1 || (it * CPI + 1 < n_chunks_w);   // odd chunk count: the last half is empty
 
-      // ---------------- raw scores: CPI * 2 m-tiles of 16 tokens -------------------------------------
-      float sc[CPI][2][2];
+        // ---------------- raw scores: CPI * 2 m-tiles of 16 tokens -------------------------------------
+        float sc[CPI][2][2];
 #pragma unroll
-      for (int cc = 0; cc < CPI; ++cc) {
-        if (cc > 0 && !last_valid) {      // nothing there: this warp's range ends in the middle of the iteration
-          sc[cc][0][0] = sc[cc][0][1] = sc[cc][1][0] = sc[cc][1][1] = -INFINITY;
-          continue;
-        }
-        // OUTER: a group's first chunk is preceded in the stage by the key group's metadata
-        const int lead = OUTER && ((ci0 + cc) & (CH - 1)) == 0 ? SL::kVMeta : 0;
-        if constexpr (OUTER) {
-          if (lead) outer_group(reinterpret_cast<const uint32_t*>(sp));
-        }
-        const uint32_t* kc = reinterpret_cast<const uint32_t*>(sp + lead + SL::off(cc));
-        const uint32_t* km = reinterpret_cast<const uint32_t*>(sp + lead + SL::off(cc) + SL::kOffKMeta);
-#pragma unroll
-        for (int mt = 0; mt < 2; ++mt) {
-          float sA = 0.f, sB = 0.f;
-          if constexpr (!(ABL & 1)) k_mtile(kc, km, 16 * mt, sA, sB);      // (else: timing experiment, no key side)
-          if constexpr (OUTER) {       // true log2-domain scores right away (the scaling changes from group to group)
-            sA = fmaf(sA, kfac_cur, kconst);
-            sB = fmaf(sB, kfac_cur, kconst);
+        for (int cc = 0; cc < CPI; ++cc) {
+          if (cc > 0 && !last_valid) {      // nothing there: this warp's range ends in the middle of the iteration
+            sc[cc][0][0] = sc[cc][0][1] = sc[cc][1][0] = sc[cc][1][1] = -INFINITY;
+            continue;
           }
-          const bool valid = cc == 0 || last_valid;
-          sc[cc][mt][0] = valid ? sA : -INFINITY;
-          sc[cc][mt][1] = valid ? sB : -INFINITY;
-        }
-      }
-
-      // ---------------- online softmax (log2 domain; raw scores still carry 1/kfac) -------------------
-      // The reference m_run of the running sums is any value within kLazy of the largest score so far, not the
-      // maximum itself: it only moves (with the cross-lane reduction and the rescaling that takes) when a score of
-      // this iteration exceeds it by more than kLazy, so p <= 2^kLazy and the usual iteration needs one vote.
-      constexpr float kLazy = OUTER ? 0.f : 4.f;
-      float cmax = -INFINITY;
+          // OUTER: a group's first chunk is preceded in the stage by the key group's metadata
+          const int lead = OUTER && ((ci0 + cc) & (CH - 1)) == 0 ? SL::kVMeta : 0;
+          if constexpr (OUTER) {
+            if (lead) outer_group(reinterpret_cast<const uint32_t*>(sp));
+          }
+          const uint32_t* kc = reinterpret_cast<const uint32_t*>(sp + lead + SL::off(cc));
+          const uint32_t* km = reinterpret_cast<const uint32_t*>(sp + lead + SL::off(cc) + SL::kOffKMeta);
 #pragma unroll
-      for (int cc = 0; cc < CPI; ++cc)
-        cmax = fmaxf(cmax, fmaxf(fmaxf(sc[cc][0][0], sc[cc][0][1]), fmaxf(sc[cc][1][0], sc[cc][1][1])));
-      const float kf = OUTER ? 1.0f : kfac;                    // what the raw scores still have to be multiplied by
-      float m_new = m_run;
-      if (__any_sync(0xffffffffu, cmax * kf > m_run + kLazy)) {
-        cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, 4));
-        cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, 8));
-        cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, 16));
-        m_new = fmaxf(m_run, cmax * kf);
-        const float alpha = ex2_approx(m_run - m_new);     // 0 on the first iteration (m_run = -inf)
-        l_part *= alpha;
-        psum *= alpha;
-        if constexpr (OUTER) {
-#pragma unroll
-          for (int g = 0; g < NG; ++g) zacc[g] *= alpha;
-        }
-#pragma unroll
-        for (int m = 0; m < 8; ++m) {
-          out_acc[m][0] *= alpha; out_acc[m][1] *= alpha;
-#pragma unroll
-          for (int e = 0; e < 4; ++e) accg[m][e] *= alpha;
-        }
-      }
-      m_run = m_new;
-
-#pragma unroll
-      for (int cc = 0; cc < CPI; ++cc) {
-        if (cc > 0 && !last_valid) continue;
-        const int ci = ci0 + cc;
-        const int lead = OUTER && (ci & (CH - 1)) == 0 ? SL::kVMeta : 0;
-        const uint32_t* vc = reinterpret_cast<const uint32_t*>(sp + lead + SL::off(cc) + SL::kOffVCodes);
-        const uint32_t* vm = reinterpret_cast<const uint32_t*>(sp + SL::off(cc) + SL::kRec);
-        // slot: position of this chunk's value group in the SPLIT window / position of the chunk in its group
-        const int slot = SPLIT ? (ci - c_lo) & (WIN - 1) : ci % CH;
-        const bool group_start = slot == 0;
-        const bool group_end = SPLIT ? (slot == WIN - 1 || (it == n_iters - 1 && (cc == CPI - 1 || !last_valid)))
-                                     : (slot == CH - 1);
-        constexpr bool kFreshEveryChunk = !SPLIT && !OUTER && CH == 1;   // then the first value mma takes a zero C
-        if (!OUTER && !kFreshEveryChunk && group_start) {
-#pragma unroll
-          for (int m = 0; m < 8; ++m)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) accg[m][e] = 0.f;
-        }
-        uint32_t Bps[NSET][2][2];
-        uint32_t (&Bp)[2][2] = Bps[0];
-        float psum_c = 0.f;
-#pragma unroll
-        for (int mt = 0; mt < 2; ++mt) {
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const float p = ex2_approx(fmaf(sc[cc][mt][h], kf, -m_new));
-            psum_c += p;
-            const int pos = VP == 2 ? 2 * mt + h : h;
-            if constexpr (OUTER) {
-              uint32_t pks[NSET];
-              outer_v_operand(reinterpret_cast<const uint32_t*>(sp + lead + SL::off(cc) + SL::kOffKMeta), 16 * mt + gid + 8 * h, p,
-                              pos, pks);
-#pragma unroll
-              for (int st_ = 0; st_ < NSET; ++st_) Bps[st_][mt][h] = movmatrix_trans(pks[st_]);
-              continue;
+          for (int mt = 0; mt < 2; ++mt) {
+            float sA = 0.f, sB = 0.f;
+            if constexpr (!(ABL & 1)) k_mtile(kc, km, 16 * mt, sA, sB);      // (else: timing experiment, no key side)
+            if constexpr (OUTER) {       // true log2-domain scores right away (the scaling changes from group to group)
+              sA = fmaf(sA, kfac_cur, kconst);
+              sB = fmaf(sB, kfac_cur, kconst);
             }
-            // p goes in as one fp16 (the lo column stays zero): its 2^-12 relative rounding is random per token and
-            // far inside the output tolerance, and it saves the hi/lo split of every probability
-            uint32_t pk = pack_half2_rn(p * pow2i(10 - VP * pos), 0.f);
-            if (SPLIT && j != slot) pk = 0u;                 // column pair of this chunk's window slot only
-            Bp[mt][h] = movmatrix_trans(pk);
+            const bool valid = cc == 0 || last_valid;
+            sc[cc][mt][0] = valid ? sA : -INFINITY;
+            sc[cc][mt][1] = valid ? sB : -INFINITY;
           }
         }
-        l_part += psum_c;
-        if constexpr (SPLIT) psum += (j == slot) ? psum_c : 0.f;
-        else psum += psum_c;
 
-        // ---------------- values: 8 m-tiles of 16 channels x 2 k-steps of 16 tokens ------------------
-        if constexpr (ABL & 2) {
-          // timing experiment: no value side
-        } else if constexpr (VP == 2) {
-          const uint4 v0 = *reinterpret_cast<const uint4*>(vc + lane * 4);
-          const uint4 v1 = *reinterpret_cast<const uint4*>(vc + 128 + lane * 4);
-          const uint32_t vw[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
+        // ---------------- online softmax (log2 domain; raw scores still carry 1/kfac) -------------------
+        // The reference m_run of the running sums is any value within kLazy of the largest score so far, not the
+        // maximum itself: it only moves (with the cross-lane reduction and the rescaling that takes) when a score of
+        // this iteration exceeds it by more than kLazy, so p <= 2^kLazy and the usual iteration needs one vote.
+        constexpr float kLazy = OUTER ? 0.f : 4.f;
+        float cmax = -INFINITY;
+#pragma unroll
+        for (int cc = 0; cc < CPI; ++cc)
+          cmax = fmaxf(cmax, fmaxf(fmaxf(sc[cc][0][0], sc[cc][0][1]), fmaxf(sc[cc][1][0], sc[cc][1][1])));
+        const float kf = OUTER ? 1.0f : kfac;                    // what the raw scores still have to be multiplied by
+        float m_new = m_run;
+        if (__any_sync(0xffffffffu, cmax * kf > m_run + kLazy)) {
+          cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, 4));
+          cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, 8));
+          cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, 16));
+          m_new = fmaxf(m_run, cmax * kf);
+          const float alpha = ex2_approx(m_run - m_new);     // 0 on the first iteration (m_run = -inf)
+          l_part *= alpha;
+          psum *= alpha;
+          if constexpr (OUTER) {
+#pragma unroll
+            for (int g = 0; g < NG; ++g) zacc[g] *= alpha;
+          }
 #pragma unroll
           for (int m = 0; m < 8; ++m) {
-            const uint32_t w0 = vw[m], w1 = vw[m] >> 8;
+            out_acc[m][0] *= alpha; out_acc[m][1] *= alpha;
 #pragma unroll
-            for (int ks = 0; ks < 2; ++ks) {
-              const uint32_t m0 = FV::kField << (2 * (2 * ks)), m1 = FV::kField << (2 * (2 * ks + 1));
-              if (kFreshEveryChunk && ks == 0) mma16816_z(accg[m], w0 & m0, w1 & m0, w0 & m1, w1 & m1, Bp[ks][0], Bp[ks][1]);
-              else mma16816(accg[m], w0 & m0, w1 & m0, w0 & m1, w1 & m1, Bps[NSET > 1 ? m >> 2 : 0][ks][0], Bps[NSET > 1 ? m >> 2 : 0][ks][1]);
-            }
-          }
-        } else {
-#pragma unroll
-          for (int ks = 0; ks < 2; ++ks) {
-#pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-              const uint4 v = *reinterpret_cast<const uint4*>(vc + ks * 256 + hh * 128 + lane * 4);
-              const uint32_t vw[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-              for (int mm = 0; mm < 4; ++mm) {
-                const uint32_t w0 = vw[mm], w1 = vw[mm] >> 8;
-                const uint32_t m0 = FV::kField, m1 = FV::kField << 4;
-                if (kFreshEveryChunk && ks == 0)
-                  mma16816_z(accg[hh * 4 + mm], w0 & m0, w1 & m0, w0 & m1, w1 & m1, Bp[ks][0], Bp[ks][1]);
-                else
-                  mma16816(accg[hh * 4 + mm], w0 & m0, w1 & m0, w0 & m1, w1 & m1, Bps[NSET > 1 ? hh : 0][ks][0], Bps[NSET > 1 ? hh : 0][ks][1]);
-              }
-            }
+            for (int e = 0; e < 4; ++e) accg[m][e] *= alpha;
           }
         }
+        m_run = m_new;
 
-        if constexpr (VB == 3 && !(ABL & 2)) {
-          // 1-bit plane (weight 4): 4 words per lane, word m/2 holds fields ((m%2)*2 + rh)*4 + 2*ks + kh
-          const uint4 hv = *reinterpret_cast<const uint4*>(vc + 256 + lane * 4);
-          const uint32_t hw[4] = {hv.x, hv.y, hv.z, hv.w};
-          uint32_t Bh[2][2];
 #pragma unroll
-          for (int ks = 0; ks < 2; ++ks)
+        for (int cc = 0; cc < CPI; ++cc) {
+          if (cc > 0 && !last_valid) continue;
+          const int ci = ci0 + cc;
+          const int lead = OUTER && (ci & (CH - 1)) == 0 ? SL::kVMeta : 0;
+          const uint32_t* vc = reinterpret_cast<const uint32_t*>(sp + lead + SL::off(cc) + SL::kOffVCodes);
+          const uint32_t* vm = reinterpret_cast<const uint32_t*>(sp + SL::off(cc) + SL::kRec);
+          // slot: position of this chunk's value group in the SPLIT window / position of the chunk in its group
+          const int slot = SPLIT ? (ci - c_lo) & (WIN - 1) : ci % CH;
+          const bool group_start = slot == 0;
+          const bool group_end = SPLIT ? (slot == WIN - 1 || (it == n_iters - 1 && (cc == CPI - 1 || !last_valid)))
+                                       : (slot == CH - 1);
+          constexpr bool kFreshEveryChunk = !SPLIT && !OUTER && CH == 1;   // then the first value mma takes a zero C
+          if (!OUTER && !kFreshEveryChunk && group_start) {
+#pragma unroll
+            for (int m = 0; m < 8; ++m)
+#pragma unroll
+              for (int e = 0; e < 4; ++e) accg[m][e] = 0.f;
+          }
+          uint32_t Bps[NSET][2][2];
+          uint32_t (&Bp)[2][2] = Bps[0];
+          float psum_c = 0.f;
+#pragma unroll
+          for (int mt = 0; mt < 2; ++mt) {
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-              const __half2 f = __float2half2_rn(pow2i(2 * ks + h + 2));      // 4^pos * 4 / 2^pos of the p fragment
-              const __half2 bb = __hmul2(*reinterpret_cast<const __half2*>(&Bp[ks][h]), f);
-              Bh[ks][h] = *reinterpret_cast<const uint32_t*>(&bb);
-            }
+              const float p = ex2_approx(fmaf(sc[cc][mt][h], kf, -m_new));
+              psum_c += p;
+              const int pos = VP == 2 ? 2 * mt + h : h;
+              if constexpr (OUTER) {
+                uint32_t pks[NSET];
+                outer_v_operand(reinterpret_cast<const uint32_t*>(sp + lead + SL::off(cc) + SL::kOffKMeta), 16 * mt + gid + 8 * h, p,
+                                pos, pks);
 #pragma unroll
-          for (int m = 0; m < 8; ++m) {
-            const uint32_t x0 = hw[m >> 1] >> (8 * (m & 1)), x1 = hw[m >> 1] >> (8 * (m & 1) + 4);
-#pragma unroll
-            for (int ks = 0; ks < 2; ++ks) {
-              const uint32_t h0 = 0x00010001u << (2 * ks), h1 = 0x00010001u << (2 * ks + 1);
-              mma16816(accg[m], x0 & h0, x1 & h0, x0 & h1, x1 & h1, Bh[ks][0], Bh[ks][1]);
+                for (int st_ = 0; st_ < NSET; ++st_) Bps[st_][mt][h] = movmatrix_trans(pks[st_]);
+                continue;
+              }
+              // p goes in as one fp16 (the lo column stays zero): its 2^-12 relative rounding is random per token and
+              // far inside the output tolerance, and it saves the hi/lo split of every probability
+              uint32_t pk = pack_half2_rn(p * pow2i(10 - VP * pos), 0.f);
+              if (SPLIT && j != slot) pk = 0u;                 // column pair of this chunk's window slot only
+              Bp[mt][h] = movmatrix_trans(pk);
             }
           }
-        }
+          l_part += psum_c;
+          if constexpr (SPLIT) psum += (j == slot) ? psum_c : 0.f;
+          else psum += psum_c;
 
-        // ---------------- end of a value group: apply scale / zero-point once per channel -----------
-        const bool chunk_valid = cc == 0 || last_valid;
-        if constexpr (SPLIT) {
-          // keep this group's metadata for the end of the window (the stage will be refilled)
-          if (chunk_valid && lane * 16 < SL::kVMeta)
-            *reinterpret_cast<uint4*>(side + slot * (SL::kVMeta / 4) + lane * 4) = *reinterpret_cast<const uint4*>(vm + lane * 4);
-        }
-        if (!OUTER && group_end && chunk_valid) {
-          if constexpr (SPLIT) __syncwarp();
-          float pg = psum;
-          pg += __shfl_xor_sync(0xffffffffu, pg, 4);
-          pg += __shfl_xor_sync(0xffffffffu, pg, 8);
-          pg += __shfl_xor_sync(0xffffffffu, pg, 16);
-          pg *= 0x1p-14f;                               // accumulators carry p * 2^10 * 2^-24
-          const uint32_t* vmg = SPLIT ? side + j * (SL::kVMeta / 4) : vm;    // this group's entries (slot j's in SPLIT)
-          // The value sums of a lane sit in the even accumulator columns (p enters as one fp16 per token, the lo
-          // column of its pair is zero), except in the outer-grouped variant.
-          auto acc_sum = [&](int m, int rh) { return OUTER ? accg[m][2 * rh] + accg[m][2 * rh + 1] : accg[m][2 * rh]; };
-          if constexpr (!SPLIT && VM == 4) {
-            // The four lanes of a quad need the same 16 entries: every lane decodes 4 of the group's 128 once, the
-            // warp exchanges (scale, zero-point) pairs through its side area (rows of 16 pairs, padded to 36 words
-            // so that the 128-bit reads of the eight lane groups fall into different banks), each lane reads its 16.
-            float* ds = reinterpret_cast<float*>(side);
-            {
-              const uint4 mw = *reinterpret_cast<const uint4*>(vmg + lane * 4);
-              const uint32_t mws[4] = {mw.x, mw.y, mw.z, mw.w};
-              float sz[8];
+          // ---------------- values: 8 m-tiles of 16 channels x 2 k-steps of 16 tokens ------------------
+          if constexpr (ABL & 2) {
+            // timing experiment: no value side
+          } else if constexpr (VP == 2) {
+            const uint4 v0 = *reinterpret_cast<const uint4*>(vc + lane * 4);
+            const uint4 v1 = *reinterpret_cast<const uint4*>(vc + 128 + lane * 4);
+            const uint32_t vw[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
 #pragma unroll
-              for (int e = 0; e < 4; ++e) decode_fast(mws[e], neg_half_v, sz[2 * e], sz[2 * e + 1]);
-              float* dst = ds + (lane >> 2) * 36 + (lane & 3) * 8;       // entries 4*lane .. 4*lane+3 = row lane/4
-              *reinterpret_cast<float4*>(dst) = make_float4(sz[0], sz[1], sz[2], sz[3]);
-              *reinterpret_cast<float4*>(dst + 4) = make_float4(sz[4], sz[5], sz[6], sz[7]);
-            }
-            __syncwarp();
-            const float4* row = reinterpret_cast<const float4*>(ds + gid * 36);
+            for (int m = 0; m < 8; ++m) {
+              const uint32_t w0 = vw[m], w1 = vw[m] >> 8;
 #pragma unroll
-            for (int q8 = 0; q8 < 8; ++q8) {
-              const float4 v = row[q8];                                   // entries 2*q8, 2*q8 + 1: (s, z, s, z)
-              const int m = q8;                                           // entry idx = 2 * m + rh
-              out_acc[m][0] = fmaf(v.x, acc_sum(m, 0), fmaf(v.y, pg, out_acc[m][0]));
-              out_acc[m][1] = fmaf(v.z, acc_sum(m, 1), fmaf(v.w, pg, out_acc[m][1]));
-            }
-            __syncwarp();                                                 // the side area is reused at the next group end
-          } else if constexpr (VM == 4) {
-            const uint4* vm4 = reinterpret_cast<const uint4*>(vmg + gid * 16);
-#pragma unroll
-            for (int q4 = 0; q4 < 4; ++q4) {
-              const uint4 mw = vm4[q4];
-              const uint32_t mws[4] = {mw.x, mw.y, mw.z, mw.w};
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                const int idx = q4 * 4 + e, m = idx >> 1, rh = idx & 1;    // fragment row (m, rh) of lane group gid
-                float s_, z_;
-                decode_fast(mws[e], neg_half_v, s_, z_);
-                out_acc[m][rh] = fmaf(s_, acc_sum(m, rh), fmaf(z_, pg, out_acc[m][rh]));
+              for (int ks = 0; ks < 2; ++ks) {
+                const uint32_t m0 = FV::kField << (2 * (2 * ks)), m1 = FV::kField << (2 * (2 * ks + 1));
+                if (kFreshEveryChunk && ks == 0) mma16816_z(accg[m], w0 & m0, w1 & m0, w0 & m1, w1 & m1, Bp[ks][0], Bp[ks][1]);
+                else mma16816(accg[m], w0 & m0, w1 & m0, w0 & m1, w1 & m1, Bps[NSET > 1 ? m >> 2 : 0][ks][0], Bps[NSET > 1 ? m >> 2 : 0][ks][1]);
               }
             }
           } else {
-            const uint4* vm4 = reinterpret_cast<const uint4*>(reinterpret_cast<const uint16_t*>(vmg) + gid * 16);
 #pragma unroll
-            for (int q4 = 0; q4 < 2; ++q4) {
-              const uint4 mw = vm4[q4];
-              const uint32_t mws[4] = {mw.x, mw.y, mw.z, mw.w};
+            for (int ks = 0; ks < 2; ++ks) {
 #pragma unroll
-              for (int e = 0; e < 8; ++e) {
-                const int idx = q4 * 8 + e, m = idx >> 1, rh = idx & 1;
-                const float s_ = h2f_bits((uint16_t)((mws[e >> 1] >> (16 * (e & 1))) & 0x7FFFu));
-                out_acc[m][rh] = fmaf(s_, acc_sum(m, rh), fmaf(neg_half_v * s_, pg, out_acc[m][rh]));
+              for (int hh = 0; hh < 2; ++hh) {
+                const uint4 v = *reinterpret_cast<const uint4*>(vc + ks * 256 + hh * 128 + lane * 4);
+                const uint32_t vw[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int mm = 0; mm < 4; ++mm) {
+                  const uint32_t w0 = vw[mm], w1 = vw[mm] >> 8;
+                  const uint32_t m0 = FV::kField, m1 = FV::kField << 4;
+                  if (kFreshEveryChunk && ks == 0)
+                    mma16816_z(accg[hh * 4 + mm], w0 & m0, w1 & m0, w0 & m1, w1 & m1, Bp[ks][0], Bp[ks][1]);
+                  else
+                    mma16816(accg[hh * 4 + mm], w0 & m0, w1 & m0, w0 & m1, w1 & m1, Bps[NSET > 1 ? hh : 0][ks][0], Bps[NSET > 1 ? hh : 0][ks][1]);
+                }
               }
             }
           }
-          psum = 0.f;
+
+          if constexpr (VB == 3 && !(ABL & 2)) {
+            // 1-bit plane (weight 4): 4 words per lane, word m/2 holds fields ((m%2)*2 + rh)*4 + 2*ks + kh
+            const uint4 hv = *reinterpret_cast<const uint4*>(vc + 256 + lane * 4);
+            const uint32_t hw[4] = {hv.x, hv.y, hv.z, hv.w};
+            uint32_t Bh[2][2];
+#pragma unroll
+            for (int ks = 0; ks < 2; ++ks)
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                const __half2 f = __float2half2_rn(pow2i(2 * ks + h + 2));      // 4^pos * 4 / 2^pos of the p fragment
+                const __half2 bb = __hmul2(*reinterpret_cast<const __half2*>(&Bp[ks][h]), f);
+                Bh[ks][h] = *reinterpret_cast<const uint32_t*>(&bb);
+              }
+#pragma unroll
+            for (int m = 0; m < 8; ++m) {
+              const uint32_t x0 = hw[m >> 1] >> (8 * (m & 1)), x1 = hw[m >> 1] >> (8 * (m & 1) + 4);
+#pragma unroll
+              for (int ks = 0; ks < 2; ++ks) {
+                const uint32_t h0 = 0x00010001u << (2 * ks), h1 = 0x00010001u << (2 * ks + 1);
+                mma16816(accg[m], x0 & h0, x1 & h0, x0 & h1, x1 & h1, Bh[ks][0], Bh[ks][1]);
+              }
+            }
+          }
+
+          // ---------------- end of a value group: apply scale / zero-point once per channel -----------
+          const bool chunk_valid = cc == 0 || last_valid;
+          if constexpr (SPLIT) {
+            // keep this group's metadata for the end of the window (the stage will be refilled)
+            if (chunk_valid && lane * 16 < SL::kVMeta)
+              *reinterpret_cast<uint4*>(side + slot * (SL::kVMeta / 4) + lane * 4) = *reinterpret_cast<const uint4*>(vm + lane * 4);
+          }
+          if (!OUTER && group_end && chunk_valid) {
+            if constexpr (SPLIT) __syncwarp();
+            float pg = psum;
+            pg += __shfl_xor_sync(0xffffffffu, pg, 4);
+            pg += __shfl_xor_sync(0xffffffffu, pg, 8);
+            pg += __shfl_xor_sync(0xffffffffu, pg, 16);
+            pg *= 0x1p-14f;                               // accumulators carry p * 2^10 * 2^-24
+            const uint32_t* vmg = SPLIT ? side + j * (SL::kVMeta / 4) : vm;    // this group's entries (slot j's in SPLIT)
+            // The value sums of a lane sit in the even accumulator columns (p enters as one fp16 per token, the lo
+            // column of its pair is zero), except in the outer-grouped variant.
+            auto acc_sum = [&](int m, int rh) { return OUTER ? accg[m][2 * rh] + accg[m][2 * rh + 1] : accg[m][2 * rh]; };
+            if constexpr (!SPLIT && VM == 4) {
+              // The four lanes of a quad need the same 16 entries: every lane decodes 4 of the group's 128 once, the
+              // warp exchanges (scale, zero-point) pairs through its side area (rows of 16 pairs, padded to 36 words
+              // so that the 128-bit reads of the eight lane groups fall into different banks), each lane reads its 16.
+              float* ds = reinterpret_cast<float*>(side);
+              {
+                const uint4 mw = *reinterpret_cast<const uint4*>(vmg + lane * 4);
+                const uint32_t mws[4] = {mw.x, mw.y, mw.z, mw.w};
+                float sz[8];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) decode_fast(mws[e], neg_half_v, sz[2 * e], sz[2 * e + 1]);
+                float* dst = ds + (lane >> 2) * 36 + (lane & 3) * 8;       // entries 4*lane .. 4*lane+3 = row lane/4
+                *reinterpret_cast<float4*>(dst) = make_float4(sz[0], sz[1], sz[2], sz[3]);
+                *reinterpret_cast<float4*>(dst + 4) = make_float4(sz[4], sz[5], sz[6], sz[7]);
+              }
+              __syncwarp();
+              const float4* row = reinterpret_cast<const float4*>(ds + gid * 36);
+#pragma unroll
+              for (int q8 = 0; q8 < 8; ++q8) {
+                const float4 v = row[q8];                                   // entries 2*q8, 2*q8 + 1: (s, z, s, z)
+                const int m = q8;                                           // entry idx = 2 * m + rh
+                out_acc[m][0] = fmaf(v.x, acc_sum(m, 0), fmaf(v.y, pg, out_acc[m][0]));
+                out_acc[m][1] = fmaf(v.z, acc_sum(m, 1), fmaf(v.w, pg, out_acc[m][1]));
+              }
+              __syncwarp();                                                 // the side area is reused at the next group end
+            } else if constexpr (VM == 4) {
+              const uint4* vm4 = reinterpret_cast<const uint4*>(vmg + gid * 16);
+#pragma unroll
+              for (int q4 = 0; q4 < 4; ++q4) {
+                const uint4 mw = vm4[q4];
+                const uint32_t mws[4] = {mw.x, mw.y, mw.z, mw.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                  const int idx = q4 * 4 + e, m = idx >> 1, rh = idx & 1;    // fragment row (m, rh) of lane group gid
+                  float s_, z_;
+                  decode_fast(mws[e], neg_half_v, s_, z_);
+                  out_acc[m][rh] = fmaf(s_, acc_sum(m, rh), fmaf(z_, pg, out_acc[m][rh]));
+                }
+              }
+            } else {
+              const uint4* vm4 = reinterpret_cast<const uint4*>(reinterpret_cast<const uint16_t*>(vmg) + gid * 16);
+#pragma unroll
+              for (int q4 = 0; q4 < 2; ++q4) {
+                const uint4 mw = vm4[q4];
+                const uint32_t mws[4] = {mw.x, mw.y, mw.z, mw.w};
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                  const int idx = q4 * 8 + e, m = idx >> 1, rh = idx & 1;
+                  const float s_ = h2f_bits((uint16_t)((mws[e >> 1] >> (16 * (e & 1))) & 0x7FFFu));
+                  out_acc[m][rh] = fmaf(s_, acc_sum(m, rh), fmaf(neg_half_v * s_, pg, out_acc[m][rh]));
+                }
+              }
+            }
+            psum = 0.f;
+          }
+        }
+
+        __syncwarp();
+        if (it + NST < n_iters) {
+          dep_wait_for_iteration(it + NST);
+          if (lane == 0) issue(st);
         }
       }
-
-      __syncwarp();
-      if (it + NST < n_iters) {
-        dep_wait_for_iteration(it + NST);
-        if (lane == 0) issue(st);
-      }
+      if (!RENEW || it >= n_iters || failed) break;
+      // The reference is let down as far as the float sums, which grow by that power of two, stay below 2^40 (the head's sum
+      // of p bounds the others); the next scores move it up to where they need it.
+      it_end = min(n_iters, it_end + a.reset_iters);
+      float l = l_part;
+      l += __shfl_xor_sync(0xffffffffu, l, 4);
+      l += __shfl_xor_sync(0xffffffffu, l, 8);
+      l += __shfl_xor_sync(0xffffffffu, l, 16);
+      const int room = min(40, max(0, 40 + 127 - (__float_as_int(l) >> 23)));
+      const float up = pow2i(room);
+      m_run -= (float)room;
+      l_part *= up;
+#pragma unroll
+      for (int g = 0; g < (OUTER ? NG : 1); ++g) zacc[g] *= up;
+#pragma unroll
+      for (int m = 0; m < 8; ++m)
+#pragma unroll
+        for (int rh = 0; rh < 2; ++rh) {
+          out_acc[m][rh] = (out_acc[m][rh] + outer_sum(m, rh) * pow2i(10 - VBASE)) * up;
+          accg[m][2 * rh] = accg[m][2 * rh + 1] = 0.f;
+        }
     }
 
     // the partials and tickets written below are also shared with the previous decode
@@ -1230,20 +1267,13 @@ __device__ __forceinline__ void decode_mma_body(const Layout& L, const Counts& c
         zacc[g] += __shfl_xor_sync(0xffffffffu, zacc[g], 8);
         zacc[g] += __shfl_xor_sync(0xffffffffu, zacc[g], 16);
       }
-      const bool up = (gid >> 2) != 0;                 // G = 32: rows of lanes 16..31 belong to the m-tile's second group
+      const bool up = (gid >> 2) != 0;                 // as in outer_sum
 #pragma unroll
       for (int m = 0; m < 8; ++m)
 #pragma unroll
         for (int rh = 0; rh < 2; ++rh) {
-          float sel, zz;
-          if constexpr (NG == 4) {
-            sel = up ? accg[m][2 * rh + 1] : accg[m][2 * rh];
-            zz = up ? zacc[2 * (m >> 2) + 1] : zacc[2 * (m >> 2)];
-          } else {
-            sel = accg[m][2 * rh];
-            zz = zacc[NG == 2 ? (m >> 2) : 0];
-          }
-          out_acc[m][rh] += sel * pow2i(10 - VBASE) + zz * 0x1p-14f;
+          const float zz = NG == 4 ? (up ? zacc[2 * (m >> 2) + 1] : zacc[2 * (m >> 2)]) : zacc[NG == 2 ? (m >> 2) : 0];
+          out_acc[m][rh] += outer_sum(m, rh) * pow2i(10 - VBASE) + zz * 0x1p-14f;
         }
     }
     __syncthreads();                                   // every warp is done with its ring
@@ -1309,17 +1339,17 @@ __device__ __forceinline__ void decode_mma_body(const Layout& L, const Counts& c
 }
 
 // One cache: block x = (unit, pass).
-template <int KB, int VB, int G, int KM, int VM, bool SPLIT, int CPI, bool OUTER = false, bool PAGED = false, int ABL = 0>
+template <int KB, int VB, int G, int KM, int VM, bool SPLIT, int CPI, bool OUTER = false, bool PAGED = false, int ABL = 0, bool RENEW = false>
 __global__ void __launch_bounds__(kThreads, 2)
 decode_mma_kernel(const Layout L, const Counts cn, const DecodeArgs a) {
-  decode_mma_body<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, PAGED, ABL>(L, cn, a, blockIdx.x);
+  decode_mma_body<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, PAGED, ABL, RENEW>(L, cn, a, blockIdx.x);
 }
 
 // One paged cache with its page table in the parameter space (read in place: no look-up in device memory).
-template <int KB, int VB, int G, int KM, int VM, bool SPLIT, int CPI, bool OUTER = false>
+template <int KB, int VB, int G, int KM, int VM, bool SPLIT, int CPI, bool OUTER = false, bool RENEW = false>
 __global__ void __launch_bounds__(kThreads, 2)
 decode_mma_paged_kernel(const Layout L, const Counts cn, const DecodeArgs a, const __grid_constant__ PageIds P) {
-  decode_mma_body<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, true>(L, cn, a, blockIdx.x, &P);
+  decode_mma_body<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, true, 0, RENEW>(L, cn, a, blockIdx.x, &P);
 }
 // Several caches of one configuration: block x = (sequence, unit, pass), the sequence's counts and parameters come
 // from its table entry (read in place from the parameter space).
@@ -1330,25 +1360,23 @@ decode_mma_batched_kernel(const __grid_constant__ Layout L, const __grid_constan
   decode_mma_body<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, PAGED>(L, T.s[seq].cn, T.s[seq].a, blockIdx.x - seq * per_seq);
 }
 
-template <int KB, int VB, int G, int KM, int VM, bool SPLIT, int CPI, bool OUTER = false, bool PAGED = false>
-int launch_one_p(const Layout& L, const Counts& cn, DecodeArgs a, int n_splits, cudaStream_t st) {
+template <int KB, int VB, int G, int KM, int VM, bool SPLIT, int CPI, bool OUTER, bool PAGED, bool RENEW>
+int launch_one_p(const Layout& L, const Counts& cn, DecodeArgs a, int grid_y, cudaStream_t st) {
   using SL = StageLayout<KB, VB, G, KM, VM, CPI>;
   constexpr int kSmem = SL::kCtaBytes;
-  constexpr int RU = SL::kCH;
   static std::atomic<unsigned long long> configured{0};
-  if (!opt_in_dynamic_smem(decode_mma_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, PAGED>, kSmem, configured)) return -1;
+  if (!opt_in_dynamic_smem(decode_mma_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, PAGED, 0, RENEW>, kSmem, configured)) return -1;
   // a paged cache whose page list fits the parameter space: the kernel that takes the table as a parameter
   [[maybe_unused]] PageIds ids;
   bool table_in_params = false;
   if constexpr (PAGED) {
     static std::atomic<unsigned long long> configured_p{0};
     if (a.pages_host && a.n_pages_host <= kParamPages) {
-      if (!opt_in_dynamic_smem(decode_mma_paged_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER>, kSmem, configured_p)) return -1;
+      if (!opt_in_dynamic_smem(decode_mma_paged_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, RENEW>, kSmem, configured_p)) return -1;
       for (int i = 0; i < a.n_pages_host; ++i) ids.id[i] = a.pages_host[i];
       table_in_params = true;
     }
   }
-  const int grid_y = fill_split_args(L, cn, a, RU, OUTER, n_splits, 0);
   int launches = 0;
   const int rows = L.r * a.n_q, step = SPLIT ? 1 : kHeads, per = a.passes;
   for (int h0 = 0; h0 < rows; h0 += step * per) {
@@ -1366,8 +1394,8 @@ int launch_one_p(const Layout& L, const Counts& cn, DecodeArgs a, int n_splits, 
     cudaError_t err;
     if constexpr (PAGED) {
       if (a.ablation) return -2;      // the timing instances exist for contiguous caches only
-      err = table_in_params ? cudaLaunchKernelEx(&cfg, decode_mma_paged_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER>, L, cn, a, ids)
-                            : cudaLaunchKernelEx(&cfg, decode_mma_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, PAGED>, L, cn, a);
+      err = table_in_params ? cudaLaunchKernelEx(&cfg, decode_mma_paged_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, RENEW>, L, cn, a, ids)
+                            : cudaLaunchKernelEx(&cfg, decode_mma_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, PAGED, 0, RENEW>, L, cn, a);
     } else if (a.ablation == 1 || a.ablation == 2) {
 #ifdef IQ_WITH_TIMING_INSTANCES      // defined by the translation units of the formats the latency study times
       static std::atomic<unsigned long long> configured_a1{0}, configured_a2{0};
@@ -1382,7 +1410,7 @@ int launch_one_p(const Layout& L, const Counts& cn, DecodeArgs a, int n_splits, 
       return -2;
 #endif
     } else {
-      err = cudaLaunchKernelEx(&cfg, decode_mma_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, PAGED>, L, cn, a);
+      err = cudaLaunchKernelEx(&cfg, decode_mma_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, PAGED, 0, RENEW>, L, cn, a);
     }
     if (err != cudaSuccess) return -1;
     ++launches;
@@ -1447,9 +1475,15 @@ int launch_one_batched_p(const Layout& L, SeqTable& T, int n_seqs, int n_splits,
 // Contiguous or paged record area: two instances of every kernel, so that the contiguous one carries none of the
 // page arithmetic.
 template <int KB, int VB, int G, int KM, int VM, bool SPLIT, int CPI, bool OUTER = false>
-int launch_one(const Layout& L, const Counts& cn, const DecodeArgs& a, int n_splits, cudaStream_t st) {
-  return L.page_groups > 0 ? launch_one_p<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, true>(L, cn, a, n_splits, st)
-                           : launch_one_p<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, false>(L, cn, a, n_splits, st);
+int launch_one(const Layout& L, const Counts& cn, DecodeArgs a, int n_splits, cudaStream_t st) {
+  constexpr int RU = StageLayout<KB, VB, G, KM, VM, CPI>::kCH;
+  const int grid_y = fill_split_args(L, cn, a, RU, OUTER, n_splits, 0);
+  fill_reference_args(cn, a, RU, CPI, OUTER);
+  if (a.reset_iters > 0 && !a.ablation)
+    return L.page_groups > 0 ? launch_one_p<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, true, true>(L, cn, a, grid_y, st)
+                             : launch_one_p<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, false, true>(L, cn, a, grid_y, st);
+  return L.page_groups > 0 ? launch_one_p<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, true, false>(L, cn, a, grid_y, st)
+                           : launch_one_p<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, false, false>(L, cn, a, grid_y, st);
 }
 template <int KB, int VB, int G, int KM, int VM, bool SPLIT, int CPI, bool OUTER = false>
 int launch_one_batched(const Layout& L, SeqTable& T, int n_seqs, int n_splits, cudaStream_t st) {

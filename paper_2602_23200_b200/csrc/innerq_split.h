@@ -30,7 +30,8 @@ struct SplitArgs {
   int row_cap;           // most grid rows: what a ticket field and part_stride hold
   int part_stride;       // split partials per query row in `partials`
   int ref_splits;        // > 0: the split count whose ranges the soft-max references follow (see kernel), else 0
-  int reset_iters;       // ... as loop iterations between two fresh references of a warp (0: none but the first)
+  int reset_iters;       // ... as loop iterations between two fresh references of a warp (0: none but the first); see
+                         // fill_reference_args
 };
 
 // Partial slots per query head: token-range splits (two waves of CTAs for all units, 64 at most) plus one per 32 tokens of
@@ -81,7 +82,9 @@ inline int plan_call(const Layout& L, const Counts& cn, SplitArgs& a, bool outer
       const long long ctas = (long long)L.U * total * used;
       const long long rest = ctas % kCtaSlots;
       const float waves = (float)(ctas / kCtaSlots) + (rest == 0 ? 0.f : rest <= kCtaSlots / 2 ? 0.65f : 1.f);
-      const float cost = waves * ((float)n_chunks / (float)used + 18.f) + 20.f * (float)(launches - 1);
+      // outer grouping: the instance that renews its references takes 3-5 % longer
+      const float slower = outer && used < std::min(default_splits(L, L.U), by_work) ? 1.08f : 1.f;
+      const float cost = waves * ((float)n_chunks / (float)used + 18.f) * slower + 20.f * (float)(launches - 1);
       if (n_cand == 0 || cost < least) least = cost;
       cand[n_cand++] = {p, s, cost};
     };
@@ -136,6 +139,15 @@ inline int fill_split_args(const Layout& L, const Counts& cn, SplitArgs& a, int 
   a.tiles_q0 = a.n_tail_tiles / grid_y;
   a.tiles_rem = a.n_tail_tiles % grid_y;
   return grid_y;
+}
+
+// Iterations (of cpi chunks) between two fresh soft-max references: where the groups of a call share the CTA slots, a warp's
+// range is several times what it would be in a launch of one group, and a reference for all of it would resolve p less; so
+// it is renewed after every range that the warp would have had (whole value groups, one at least).
+inline void fill_reference_args(const Counts& cn, SplitArgs& a, int ru, int cpi, bool outer) {
+  const int n_units = ((outer ? cn.n_qk : cn.n_qv) / kChunk + ru - 1) / ru;
+  const int ref_splits = std::min(a.ref_splits, (n_units + kSplitWarps - 1) / kSplitWarps);      // as in fill_split_args
+  a.reset_iters = ref_splits > a.n_splits ? std::max(1, std::max(1, n_units / (kSplitWarps * ref_splits)) * ru / cpi) : 0;
 }
 
 }  // namespace iq

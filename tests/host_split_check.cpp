@@ -1,15 +1,42 @@
 // Host check of csrc/innerq_split.h over the shapes that the library accepts (no GPU): every launch has a grid, its split
 // partials fit the memory they are given, its CTAs fit the ticket field that counts them, the tail tiles are all dealt,
 // and groups of query rows share a launch only where that pays.
-// Prints one line per failed property and returns 1 if there were any.
+// Prints one line per failed property and returns 1 if there were any.  With eight arguments it prints the plan of one call.
 #include <cmath>
 #include <cstdio>
+#include <cstdlib>
 
 #include "innerq_split.h"
 
 using namespace iq;
 
-int main() {
+namespace {
+
+// The plan of one call as "passes splits default_splits reset_iters(one chunk per iteration) reset_iters(two)".
+int print_plan(char** v) {
+  const int U = std::atoi(v[1]), r = std::atoi(v[2]), n_q = std::atoi(v[3]), w_sink = std::atoi(v[4]), w_recent = std::atoi(v[5]),
+            G = std::atoi(v[6]), N = std::atoi(v[7]);
+  const bool outer = std::atoi(v[8]) != 0;
+  Layout L = {};
+  L.U = U; L.r = r; L.G = G; L.w_sink = w_sink; L.w_recent = w_recent;
+  L.max_splits = max_splits_for(U, w_sink, w_recent, G);
+  L.k.kind = outer ? kBlock : kRow; L.v.kind = outer ? kRow : kBlock;
+  const Counts cn = counts_for(L, N);
+  SplitArgs a = {};
+  a.n_q = n_q;
+  const int n = plan_call(L, cn, a, outer, 0);
+  fill_split_args(L, cn, a, G / kChunk, outer, n, 0);
+  fill_reference_args(cn, a, G / kChunk, 1, outer);
+  const int one = a.reset_iters;
+  fill_reference_args(cn, a, G / kChunk, 2, outer);
+  std::printf("%d %d %d %d %d\n", a.passes, a.n_splits, default_splits(L, U), one, a.reset_iters);
+  return 0;
+}
+
+}  // namespace
+
+int main(int argc, char** argv) {
+  if (argc == 9) return print_plan(argv);
   long long failures = 0, calls = 0;
   const int windows[][2] = {{0, 0}, {4, 32}, {4, 64}, {0, 64}, {32, 96}, {4, 128}, {4, 256}, {64, 2000}};
   for (int U = 1; U <= 65535; U = U < 700 ? U + 1 : U * 5 / 4)
