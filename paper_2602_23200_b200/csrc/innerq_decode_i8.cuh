@@ -1304,7 +1304,8 @@ int launch_i8_batched_p(const Layout& L, SeqTable& T, int n_seqs, int n_splits, 
 template <int KB, int VB, int G, int KM, int VM, bool SPLIT>
 int launch_i8_cpi(const Layout& L, const Counts& cn, const DecodeArgs& a, int n_splits, int cpi, cudaStream_t st) {
   const bool paged = L.page_groups > 0;
-  if (cpi == 0 && G == 32 && cn.n_qv / kChunk < 4 * kWarps * (n_splits > 0 ? n_splits : 1)) cpi = 1;
+  // with several groups in a launch: as one of them alone, whose ranges the soft-max references follow
+  if (cpi == 0 && G == 32 && cn.n_qv / kChunk < 4 * kWarps * std::max(1, std::max(n_splits, a.ref_splits))) cpi = 1;
   if constexpr (KB == 2 && VB == 2) {
     if (cpi != 1)
       return paged ? launch_i8_one_p<KB, VB, G, KM, VM, SPLIT, 2, true>(L, cn, a, n_splits, st)

@@ -399,6 +399,9 @@ def split_plan(tmp_path_factory):
 # error varies by 1 / sqrt(2 n), 0.8 % or less.
 RENEWED = [  # grouping, bits, G, batch, KV heads, r, n_q, N, paged
     (O.OUTER, 4, 128, 1, 2, 4, 8, 65536, False), (O.OUTER, 2, 32, 1, 4, 4, 8, 20000, False), (O.OUTER, 4, 64, 1, 2, 4, 8, 40000, True),
+    # G = 32 with one chunk per iteration (as one group alone takes there) and with two, then three value group sizes
+    (O.INNER, 2, 32, 2, 8, 4, 8, 8192, False), (O.INNER, 2, 32, 5, 8, 16, 1, 8000, False), (O.INNER, 2, 64, 2, 8, 4, 5, 16384, True),
+    (O.INNER, 4, 64, 1, 8, 4, 5, 16384, False), (O.INNER, 3, 128, 1, 8, 4, 5, 16384, False), (O.INNER, 2, 128, 3, 8, 8, 1, 16384, False),
 ]
 
 
