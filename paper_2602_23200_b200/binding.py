@@ -258,7 +258,7 @@ def innerq_decode_attention_batched(caches, q, out=None, stream=None):
     shape = (n,) + c._q_shape
     q_ptr = _ptr_of(q, "q", shape, c.device)
     if out is None:
-        out = _Fast.empty(q)
+        out = c._out_like.new_empty(shape)
     st = _lib.innerq_decode_attention_batched(handles, n, q_ptr, _ptr_of(out, "out", shape, c.device), _stream_of(stream, c.device))
     if st < 0:
         _check(st, "innerq_decode_attention_batched")
@@ -297,6 +297,8 @@ class InnerQCache:
         self._h = h
         self._kv_shape = (cfg.batch, cfg.n_kv_heads, cfg.head_dim)
         self._q_shape = (cfg.batch, cfg.n_q_heads, cfg.head_dim)
+        # what a result looks like, whatever class or strides the query has (a view of the workspace, never written)
+        self._out_like = self._ws_buf[:2 * cfg.batch * cfg.n_q_heads * cfg.head_dim].view(torch.float16).view(self._q_shape)
         if not _Fast.ready:
             _Fast.load()
 
@@ -371,7 +373,7 @@ class InnerQCache:
         device = self.device
         q_ptr = _ptr_of(q, "q", self._q_shape, device)
         if out is None:
-            out = _Fast.empty(q)
+            out = _Fast.empty(self._out_like)
             out_ptr = out.data_ptr()
         else:
             out_ptr = _ptr_of(out, "out", self._q_shape, device)

@@ -546,6 +546,25 @@ def test_batched_calls_with_caches_that_hold_a_batch_themselves():
         P.assert_export_equal(gc.innerq_cache_export(), oc.export(), O.INNER, w.group)
 
 
+def test_result_is_a_plain_contiguous_tensor_whatever_the_query_is():
+    # a query may be a tensor subclass, or carry any stride on a dimension of one element; the result does not inherit it
+    import torch
+    from paper_2602_23200_b200 import binding as B
+
+    class Sub(torch.Tensor):
+        pass
+
+    w = synth.tiny(batch=1, n_q_heads=4, n_kv_heads=2, n_tokens=60)
+    oc, gc, _, _ = run_prefill_both(w)
+    q0 = dev(synth.query(w, 0))
+    want = gc.innerq_decode_attention(q0)
+    for q in (q0.as_subclass(Sub), torch.nn.Parameter(q0, requires_grad=False), torch.as_strided(q0, q0.shape, (0, 128, 1)),
+              torch.stack([q0, q0], 1)[:, 0]):
+        for out in (gc.innerq_decode_attention(q), B.innerq_decode_attention_batched([gc], q.unsqueeze(0))[0]):
+            assert type(out) is torch.Tensor and out.stride() == (4 * 128, 128, 1) and not out.requires_grad
+            assert torch.equal(out, want)
+
+
 def test_batched_calls_argument_checks():
     from paper_2602_23200_b200 import binding as B
     w = synth.tiny(batch=1, n_q_heads=2, n_kv_heads=2, n_tokens=50)
