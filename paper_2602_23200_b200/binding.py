@@ -198,14 +198,14 @@ def _dev_ptr(t, name: str, shape, device=None) -> int:
 class _Fast:
     """The same two checks for the calls of a decode step, which a model makes per layer and token: at 30 layers the
     general forms above cost more host time (4-5 us a call of 12) than the kernels take on short contexts.  One attribute
-    read per property, in the order that lets a valid tensor through with the fewest; whatever does not pass goes to the
-    general form, which raises (or accepts) it.  Nothing is remembered from call to call."""
+    read per property, in the order that lets a valid tensor through with the fewest; whatever does not pass (a subclass
+    among it) goes to the general form, which raises (or accepts) it.  Nothing is remembered from call to call."""
     ready = False
 
     @classmethod
     def load(cls):
         import torch
-        cls.f16, cls.empty = torch.float16, torch.empty_like
+        cls.tensor, cls.f16, cls.empty = torch.Tensor, torch.float16, torch.empty_like
         cls.get_device = staticmethod(torch.cuda.current_device)
         cls.get_stream = staticmethod(lambda i: torch.cuda.current_stream(i).cuda_stream)
         # the functions behind those two, without the Stream object and the lazy-initialisation check (a cache exists)
@@ -224,11 +224,8 @@ def _stream_of(stream, device) -> int:
 
 def _ptr_of(t, name: str, shape, device) -> int:
     """`shape`: a tuple."""
-    try:
-        if t.dtype is _Fast.f16 and t.shape == shape and t.get_device() == device.index and t.is_contiguous():
-            return t.data_ptr()
-    except AttributeError:
-        pass
+    if type(t) is _Fast.tensor and t.dtype is _Fast.f16 and t.shape == shape and t.get_device() == device.index and t.is_contiguous():
+        return t.data_ptr()
     return _dev_ptr(t, name, shape, device)
 
 

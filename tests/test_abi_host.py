@@ -125,3 +125,26 @@ def test_paged_sizes_without_gpu():
     with pytest.raises(B.InnerQError) as ei:
         B.innerq_paged_cache_bytes(B.make_config(synth.config2(), grouping=B.GROUPING_FP16), 1024)
     assert ei.value.status == -2
+
+
+def test_the_short_checks_of_a_step_let_only_tensors_through():
+    torch = pytest.importorskip("torch")
+    B._Fast.load()
+
+    class LooksLikeOne:
+        dtype, shape = torch.float16, torch.Size((2, 128))
+
+        def get_device(self):
+            return 0
+
+        def is_contiguous(self):
+            return True
+
+        def data_ptr(self):
+            return 4096
+
+    with pytest.raises(TypeError):
+        B._ptr_of(LooksLikeOne(), "q", (2, 128), torch.device("cuda", 0))
+    for t in (torch.zeros(2, 128, dtype=torch.float16), torch.zeros(2, 128), [0.0], None):
+        with pytest.raises(TypeError):
+            B._ptr_of(t, "q", (2, 128), torch.device("cuda", 0))
