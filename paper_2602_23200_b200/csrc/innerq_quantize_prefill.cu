@@ -13,6 +13,7 @@
 // every add / multiply is one packed fp32x2 instruction, whose two halves are rounded exactly as the scalar ones.  A
 // packed instruction does not raise the fp32 rate, but it takes one issue slot for two operations, and the slots it
 // frees go to the conversions, minima / maxima and byte permutes.
+#include <algorithm>
 #include <type_traits>
 
 #include "innerq_device.cuh"
@@ -24,6 +25,7 @@ namespace {
 
 constexpr float kMagic = 12582912.0f;       // 1.5 * 2^23
 constexpr int kSeg = 32;                    // values per thread and group
+constexpr int kCopies = 8;                  // 16-byte copies in flight per thread
 constexpr int kRowsCtasPerSm = 4;           // of 128 threads and 128 registers (5 or 6 with fewer registers: +-1 %)
 
 // ---- two fp32 values in a 64-bit register pair
@@ -609,12 +611,14 @@ __device__ __forceinline__ void key_absmax_part(const __half* __restrict__ K, in
   }
 }
 
-// The fp16 windows of both tensors (an unquantised cache: everything), the counts that the decode kernel compares with
-// its own N (see append_publish) and, unless the key quantiser computes them, the norms (1).  Thread `i` of `n`.
+// The fp16 windows of both tensors and the counts that the decode kernel compares with its own N (see append_publish), and
+// the norms (1) unless the key quantiser computes them.  CTA `part` of `n_parts`, 256 threads.  Bound by memory latency in
+// this kernel's two CTAs per SM: kCopies 16-byte pieces are in flight per thread, and stepping from piece to piece takes no
+// division.  (One piece at a time with its division: 600 units x 1000 tokens, all in the windows, 255 us; now 143.)
 __device__ __forceinline__ void copy_windows(const Layout& L, const Counts& cn, const __half* __restrict__ K,
                                              const __half* __restrict__ V, unsigned char* __restrict__ cache, bool set_norm,
-                                             int i0, int n) {
-  const int N = cn.N;
+                                             int part, int n_parts) {
+  const int N = cn.N, i0 = part * 256 + threadIdx.x, n = n_parts * 256;
   uint32_t* counts = reinterpret_cast<uint32_t*>(cache + L.appended_off);
   for (int i = i0; i < L.U; i += n) counts[i] = (uint32_t)N;
   if (set_norm) {
@@ -626,13 +630,35 @@ __device__ __forceinline__ void copy_windows(const Layout& L, const Counts& cn, 
     const Store& S = s ? L.v : L.k;
     const __half* X = s ? V : K;
     const int n_q = s ? cn.n_qv : cn.n_qk, per_unit = (N - n_q) * 16;      // 16-byte pieces of the tokens kept in fp16
-    for (long long i = i0; i < (long long)per_unit * L.U; i += n) {
-      const int u = (int)(i / per_unit), r = (int)(i - (long long)u * per_unit), w = r >> 4, piece = r & 15;
-      const int t = w < cn.n_sink ? w : w + n_q;
-      const bool sink = S.kind == kNone || t < L.w_sink;
-      unsigned char* dst = cache + (sink ? S.sink_off + (size_t)u * S.sink_stride + (size_t)t * kD * 2
-                                         : S.ring_off + (size_t)u * S.ring_stride + (size_t)((t - L.w_sink) % S.ring_cap) * kD * 2);
-      *reinterpret_cast<uint4*>(dst + piece * 16) = __ldg(reinterpret_cast<const uint4*>(X + ((size_t)u * N + t) * kD) + piece);
+    if (per_unit == 0) continue;
+    // piece r of unit u; a thread's next one is n pieces further on
+    const int step_u = n / per_unit, step_r = n - step_u * per_unit, ring0 = n_q % S.ring_cap;
+    int u = i0 / per_unit, r = i0 - u * per_unit;
+    while (u < L.U) {
+      uint4 x[kCopies];
+      uint4* to[kCopies];
+#pragma unroll
+      for (int k = 0; k < kCopies; ++k) {
+        to[k] = nullptr;
+        if (u < L.U) {
+          const int w = r >> 4;                                            // the w-th token kept in fp16
+          const bool sink = w < cn.n_sink;
+          x[k] = __ldg(reinterpret_cast<const uint4*>(X + ((size_t)u * N + (sink ? w : w + n_q)) * kD) + (r & 15));
+          int slot = w;
+          if (!sink) {                                                     // the recent tokens fit the ring: it wraps once
+            slot = ring0 + w - cn.n_sink;
+            if (slot >= S.ring_cap) slot -= S.ring_cap;
+          }
+          unsigned char* base = cache + (sink ? S.sink_off + (size_t)u * S.sink_stride : S.ring_off + (size_t)u * S.ring_stride);
+          to[k] = reinterpret_cast<uint4*>(base) + (size_t)slot * 16 + (r & 15);
+          u += step_u;
+          r += step_r;
+          if (r >= per_unit) { r -= per_unit; ++u; }
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < kCopies; ++k)
+        if (to[k]) *to[k] = x[k];
     }
   }
 }
@@ -659,19 +685,37 @@ prefill_first_kernel(const __grid_constant__ Layout L, const Counts cn, const __
   else if (b < n_max + n_val)
     quantize_blocks<VBITS>(L, V, cn.N, cn.n_qv, cache, b - n_max, n_val, smem, Mul2(neg_zero));
   else
-    copy_windows(L, cn, K, V, cache, n_max == 0, (b - n_max - n_val) * 256 + threadIdx.x, (gridDim.x - n_max - n_val) * 256);
+    copy_windows(L, cn, K, V, cache, n_max == 0, b - n_max - n_val, gridDim.x - n_max - n_val);
 }
 
+// The same for a cache that has nothing else to do here: empty, unquantised (everything goes to the sink array) or
+// outer-grouped (its quantisers are launches of their own).  Grid (share, unit, tensor), a kernel of few registers: full
+// occupancy hides the latency (32 units x 65536 tokens, unquantised: 320 us, 6.7 TB/s; as a role of the kernel above 354).
 __global__ void __launch_bounds__(256) prefill_windows_kernel(const __grid_constant__ Layout L, const Counts cn,
                                                               const __half* __restrict__ K, const __half* __restrict__ V,
                                                               unsigned char* __restrict__ cache) {
-  copy_windows(L, cn, K, V, cache, true, blockIdx.x * 256 + threadIdx.x, gridDim.x * 256);
+  const int u = blockIdx.y, N = cn.N;
+  const Store& S = blockIdx.z ? L.v : L.k;
+  const int n_q = blockIdx.z ? cn.n_qv : cn.n_qk;
+  if (blockIdx.x == 0 && blockIdx.z == 0) {
+    if (threadIdx.x < kD) reinterpret_cast<float*>(cache + L.norm_off)[(size_t)u * kD + threadIdx.x] = 1.0f;
+    if (threadIdx.x == kD) reinterpret_cast<uint32_t*>(cache + L.appended_off)[u] = (uint32_t)N;
+  }
+  const uint4* X = reinterpret_cast<const uint4*>((blockIdx.z ? V : K) + (size_t)u * N * kD);
+  uint4* sink = reinterpret_cast<uint4*>(cache + S.sink_off + (size_t)u * S.sink_stride);
+  uint4* ring = reinterpret_cast<uint4*>(cache + S.ring_off + (size_t)u * S.ring_stride);
+  const int n_sink = S.kind == kNone ? N : cn.n_sink, per_unit = (N - n_q) * 16;
+  for (int i = blockIdx.x * 256 + threadIdx.x; i < per_unit; i += gridDim.x * 256) {
+    const int w = i >> 4, piece = i & 15;
+    if (w < n_sink) sink[i] = __ldg(X + i);
+    else ring[(size_t)((w + n_q - n_sink) % S.ring_cap) * 16 + piece] = __ldg(X + (size_t)(w + n_q) * 16 + piece);
+  }
 }
 
 int clamp_int(long long n, int lo, int hi) { return (int)(n < lo ? lo : (n > hi ? hi : n)); }
 
-int window_ctas(const Layout& L, const Counts& cn) {      // about four 16-byte pieces per thread
-  const long long pieces = (long long)L.U * 16 * (2 * cn.N - cn.n_qk - cn.n_qv) + L.U * kD;
+int window_ctas(const Layout& L, const Counts& cn) {      // about four 16-byte pieces per thread, eight CTAs per SM at most
+  const long long pieces = (long long)L.U * 16 * (2ll * cn.N - cn.n_qk - cn.n_qv) + L.U * kD;
   return clamp_int((pieces + 1023) / 1024, 1, 148 * 8);
 }
 
@@ -698,7 +742,8 @@ int launch_rows(const Layout& L, const Counts& cn, const __half* K, unsigned cha
 
 int launch_prefill_windows(const Layout& L, const Counts& cn, unsigned char* cache, const __half* K, const __half* V,
                            cudaStream_t st) {
-  prefill_windows_kernel<<<window_ctas(L, cn), 256, 0, st>>>(L, cn, K, V, cache);
+  const int n_fp16 = cn.N - std::min(cn.n_qk, cn.n_qv);
+  prefill_windows_kernel<<<dim3(clamp_int((n_fp16 + 15) / 16, 1, 1024), L.U, 2), 256, 0, st>>>(L, cn, K, V, cache);
   return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
 
