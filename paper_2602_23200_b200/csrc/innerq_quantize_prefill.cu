@@ -614,7 +614,7 @@ __device__ __forceinline__ void key_absmax_part(const __half* __restrict__ K, in
 // The fp16 windows of both tensors and the counts that the decode kernel compares with its own N (see append_publish), and
 // the norms (1) unless the key quantiser computes them.  CTA `part` of `n_parts`, 256 threads.  Bound by memory latency in
 // this kernel's two CTAs per SM: kCopies 16-byte pieces are in flight per thread, and stepping from piece to piece takes no
-// division.  (One piece at a time with its division: 600 units x 1000 tokens, all in the windows, 255 us; now 143.)
+// division.  (One piece at a time with its division: 600 units x 1000 tokens, all in the windows, 260 us; now 136.)
 __device__ __forceinline__ void copy_windows(const Layout& L, const Counts& cn, const __half* __restrict__ K,
                                              const __half* __restrict__ V, unsigned char* __restrict__ cache, bool set_norm,
                                              int part, int n_parts) {
@@ -690,7 +690,7 @@ prefill_first_kernel(const __grid_constant__ Layout L, const Counts cn, const __
 
 // The same for a cache that has nothing else to do here: empty, unquantised (everything goes to the sink array) or
 // outer-grouped (its quantisers are launches of their own).  Grid (share, unit, tensor), a kernel of few registers: full
-// occupancy hides the latency (32 units x 65536 tokens, unquantised: 320 us, 6.7 TB/s; as a role of the kernel above 354).
+// occupancy hides the latency (32 units x 65536 tokens, unquantised: 316 us, 6.8 TB/s; as a role of the kernel above 354).
 __global__ void __launch_bounds__(256) prefill_windows_kernel(const __grid_constant__ Layout L, const Counts cn,
                                                               const __half* __restrict__ K, const __half* __restrict__ V,
                                                               unsigned char* __restrict__ cache) {

@@ -96,6 +96,28 @@ def test_prefill_edges(kb, vb, G, N, batch, heads, norm, variant, shift):
         K, V = np.ascontiguousarray(K[..., ::-1, :]), np.ascontiguousarray(V[..., ::-1, :])
 
 
+# The fp16 windows: fewer tokens than the sink holds, nothing but windows, windows of no, one and many tokens, and unit
+# counts at which a thread's next piece is units further on or less than a unit's pieces away.
+@pytest.mark.parametrize("grouping", [O.INNER, O.OUTER, O.FP16])
+@pytest.mark.parametrize("batch,heads,N,w_sink,w_recent", [(1, 2, 3, 4, 16), (1, 1, 4, 4, 0), (37, 8, 1, 4, 16), (41, 8, 150, 4, 130),
+                                                           (1, 2, 700, 5, 300), (2, 3, 900, 0, 1), (1, 1, 2500, 4, 2048)])
+def test_prefill_windows(grouping, batch, heads, N, w_sink, w_recent):
+    inner = grouping == O.INNER
+    w = synth.tiny(n_tokens=N, batch=batch, n_kv_heads=heads, n_q_heads=heads, w_sink=w_sink, w_recent=w_recent, grouping=grouping,
+                   k_normalize=int(inner), **({} if inner else dict(k_mode=O.ASYM, v_mode=O.ASYM)))
+    oc, gc, K, V = run_prefill_both(w, max_tokens=N + 40)
+    for _ in range(2):                     # the second prefill runs over the first one's windows
+        e = gc.innerq_cache_export()
+        if grouping == O.FP16:
+            for name, x in (("k_sink", K), ("v_sink", V)):
+                np.testing.assert_array_equal(np.asarray(e[name])[:, :N].view(np.float16), x.reshape(-1, N, 128))
+        else:
+            P.assert_export_equal(e, oc.export(), grouping, w.group, k_hybrid=inner, v_hybrid=inner)
+        K, V = K[..., ::-1, :].copy(), V[..., ::-1, :].copy()
+        oc.prefill(K, V)
+        gc.innerq_quantize_prefill(dev(K), dev(V))
+
+
 @pytest.mark.parametrize("bits,G,N", [(2, 32, 333), (3, 64, 420), (4, 128, 541)])
 def test_prefill_and_decode_outer(bits, G, N):
     w = synth.tiny(n_tokens=N, group=G, k_bits=bits, v_bits=bits, grouping=O.OUTER, k_normalize=0,
