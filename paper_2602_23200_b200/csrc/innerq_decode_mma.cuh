@@ -193,10 +193,11 @@ __device__ __forceinline__ bool append_count_is(const uint32_t* flag, uint32_t N
 }
 
 // Cross-CTA merge, run by the last CTA of a unit to finish: log-sum-exp combination of the n_parts partial results
-// (rows prow0 .. of kPartialStride floats: acc[128], max, sum) of nh query rows, fp16 results to rows orow of out.
+// (rows prow0 .. of part_stride partials of kPartialStride floats: acc[128], max, sum) of nh query rows, fp16 results to
+// rows orow of out.
 // Kept out of line so that its registers do not add to the streaming loop's.
 __device__ __noinline__ void merge_parts(const float* __restrict__ partials, float* wm, __half* __restrict__ out, int nh,
-                                         int n_parts, int prow0, int4 orow, int max_splits) {
+                                         int n_parts, int prow0, int4 orow, int part_stride) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // Warp w merges parts w, w + 8, ... (four parts per round of loads, lane l the channels 4l .. 4l+3, running
   // max / rescale as in the streaming loop), then the eight warp results are combined through shared memory.
@@ -205,7 +206,7 @@ __device__ __noinline__ void merge_parts(const float* __restrict__ partials, flo
 #pragma unroll 1
   for (int h = 0; h < nh; ++h) {
     float M = -INFINITY, den = 0.f, n0 = 0.f, n1 = 0.f, n2 = 0.f, n3 = 0.f;
-    const float* Ph = partials + (size_t)(prow0 + h) * max_splits * kPartialStride;
+    const float* Ph = partials + (size_t)(prow0 + h) * part_stride * kPartialStride;
 #pragma unroll 1
     for (int s0 = warp; s0 < n_parts; s0 += 4 * kWarps) {
       float4 v[4];
@@ -1351,13 +1352,13 @@ __global__ void __launch_bounds__(kThreads, 2)
 decode_mma_paged_kernel(const Layout L, const Counts cn, const DecodeArgs a, const __grid_constant__ PageIds P) {
   decode_mma_body<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, true, 0, RENEW>(L, cn, a, blockIdx.x, &P);
 }
-// Several caches of one configuration: block x = (sequence, unit, pass), the sequence's counts and parameters come
+// Several caches of one configuration: block x = sequence * U + unit, the sequence's counts and parameters come
 // from its table entry (read in place from the parameter space).
 template <int KB, int VB, int G, int KM, int VM, bool SPLIT, int CPI, bool OUTER = false, bool PAGED = false>
 __global__ void __launch_bounds__(kThreads, 2)
 decode_mma_batched_kernel(const __grid_constant__ Layout L, const __grid_constant__ SeqTable T) {
-  const int per_seq = L.U * T.s[0].a.passes, seq = blockIdx.x / per_seq;
-  decode_mma_body<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, PAGED>(L, T.s[seq].cn, T.s[seq].a, blockIdx.x - seq * per_seq);
+  const int seq = blockIdx.x / L.U;
+  decode_mma_body<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, PAGED>(L, T.s[seq].cn, T.s[seq].a, blockIdx.x - seq * L.U);
 }
 
 template <int KB, int VB, int G, int KM, int VM, bool SPLIT, int CPI, bool OUTER, bool PAGED, bool RENEW>
@@ -1455,11 +1456,10 @@ int launch_one_batched_p(const Layout& L, SeqTable& T, int n_seqs, int n_splits,
     if (gy > grid_y) grid_y = gy;
   }
   int launches = 0;
-  const int step = SPLIT ? 1 : kHeads, per = T.s[0].a.passes;
-  for (int h0 = 0; h0 < L.r; h0 += step * per) {
-    const int passes = std::min(per, (L.r - h0 + step - 1) / step);
-    for (int i = 0; i < n_seqs; ++i) { T.s[i].a.head0 = h0; T.s[i].a.passes = passes; }
-    const dim3 grid(n_seqs * L.U * passes, grid_y);
+  const dim3 grid(n_seqs * L.U, grid_y);
+  const int step = SPLIT ? 1 : kHeads;
+  for (int h0 = 0; h0 < L.r; h0 += step) {      // one launch per group of query rows
+    for (int i = 0; i < n_seqs; ++i) T.s[i].a.head0 = h0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid; cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kSmem; cfg.stream = st;
     cudaLaunchAttribute attr[1];
