@@ -56,62 +56,72 @@ inline int most_rows(const Layout& L, int n_q, int p) {
 
 // The split of a call: groups of four query rows per launch (passes), and the split count (n_splits > 0: the caller's
 // choice), which is returned.  All groups go into one launch, up to eight, with one wave of CTAs together: one start, one
-// end and one read of the records from HBM instead of one per group.  Two things can make that the slower choice, on long
-// contexts by up to a factor of two: a wave that leaves slots idle (40 units with five groups: one split each, 200 CTAs),
-// and few units whose partials do not hold enough splits for every group (one unit with eight groups: 8 of 37).  So the
-// launches that could be made (groups per launch, splits that fill one half wave more at a time) are compared by
-//   waves * (chunks per CTA + 18) + 20 per further launch,
-// in chunks (of 32 tokens, 0.16 us): 18 are a CTA's start and end; launches overlap, so the waves are those of all CTAs
-// together; a last half wave counts 0.65, its CTAs have an SM each.  Of what is within 4 % of the best, the fewest launches
-// and longest ranges (they leave most to the neighbours in a chain of calls).  Alone / in a chain, us, against one launch
-// per group and against always one wave: 40 units x 16384 tokens, r 4, n_q 5, 4 bits: 96.7 / 77.7, 109.7 / 95.7,
-// 116.0 / 79.6; 80 x 16384, r 8: 79.0 / 59.1, 81.6 / 62.4, 106.1 / 60.6; 1 x 524288, n_q 8: 118.4 / 81.5, 128.3 / 98.4,
-// 209.1 / 83.9.
+// end and one read of the records from HBM instead of one per group.  Two things can make that slower for a call that runs
+// alone than one launch per group, on long contexts by up to a factor of two: a wave that leaves slots idle (40 units with
+// five groups: one split each, 200 CTAs), and few units whose partials do not hold enough splits for every group (one unit
+// with eight groups: 8 of 37).  Time alone, in chunks (of 32 tokens, 0.16 us):
+//   waves * (chunks per CTA + 18) + 14 per further launch
+// with 18 for a CTA's start and end; launches overlap, so the waves are those of all CTAs together; a last half wave counts
+// 0.65, its CTAs have an SM each.  Where that is less with one launch per group, the launches that could be made (groups
+// per launch, splits that fill half a wave more at a time) are compared, and of those within 6 % of the best the fewest
+// launches and longest ranges are taken: they leave most to the neighbours in a chain of calls.
+// Alone / in a chain, us: one launch per group; always one wave; chosen.  40 units x 16384 tokens, r 4, n_q 5, 4 bits:
+// 109.7 / 95.7; 116.0 / 79.6; 96.7 / 77.7.  80 x 16384, r 8: 81.6 / 62.4; 106.1 / 60.6; 79.0 / 59.1.  1 x 524288, n_q 8:
+// 128.3 / 98.4; 209.1 / 83.9; 107.5 / 83.7.
 inline int plan_call(const Layout& L, const Counts& cn, SplitArgs& a, bool outer, int n_splits) {
   const int total = (L.r * a.n_q + 3) / 4, ru = L.G / kChunk, n_chunks = (outer ? cn.n_qk : cn.n_qv) / kChunk;
+  const int alone = default_splits(L, L.U);                        // splits of a launch of one group
   n_splits = std::min(n_splits, std::min(L.max_splits, 128));      // 128: slots of the merge tables in shared memory
   const bool chosen = n_splits > 0;
-  int best_p = 1, best_s = chosen ? n_splits : default_splits(L, L.U);
-  if (total > 1) {
-    struct { int p, s; float cost; } cand[8 * 12];
-    int n_cand = 0;
-    float least = 0.f;
+  auto one_wave = [&](int p) { return std::min(default_splits(L, L.U * p), most_rows(L, a.n_q, p)); };
+  auto holds = [&](int p) {      // a launch of p groups has the partials and ticket bits for its splits
+    if (partial_slots(L, a.n_q, p) < 1) return false;
+    if (chosen) return n_splits <= most_rows(L, a.n_q, p);
+    return std::min(default_splits(L, L.U * p), partial_slots(L, a.n_q, p)) == one_wave(p);
+  };
+  const int fewest = (total + 7) / 8;
+  int best_p = (total + fewest - 1) / fewest;
+  while (best_p > 1 && !holds(best_p)) --best_p;
+  int best_s = chosen ? n_splits : one_wave(best_p);
+  if (!chosen && best_p > 1) {
     const int by_work = std::max(1, ((n_chunks + ru - 1) / ru + kSplitWarps - 1) / kSplitWarps);      // see fill_split_args
-    auto add = [&](int p, int s) {
-      const int launches = (total + p - 1) / p, used = std::min(s, by_work);
-      const long long ctas = (long long)L.U * total * used;
-      const long long rest = ctas % kCtaSlots;
+    auto time = [&](int p, int s) {
+      const int used = std::min(s, by_work);
+      const long long ctas = (long long)L.U * total * used, rest = ctas % kCtaSlots;
       const float waves = (float)(ctas / kCtaSlots) + (rest == 0 ? 0.f : rest <= kCtaSlots / 2 ? 0.65f : 1.f);
-      // outer grouping: the instance that renews its references takes 3-5 % longer
-      const float slower = outer && used < std::min(default_splits(L, L.U), by_work) ? 1.08f : 1.f;
-      const float cost = waves * ((float)n_chunks / (float)used + 18.f) * slower + 20.f * (float)(launches - 1);
-      if (n_cand == 0 || cost < least) least = cost;
-      cand[n_cand++] = {p, s, cost};
+      // outer grouping: the instance that renews its references takes 3-8 % longer
+      const float slower = outer && used < std::min(alone, by_work) ? 1.05f : 1.f;
+      return waves * ((float)n_chunks / (float)used + 18.f) * slower + 14.f * (float)((total + p - 1) / p - 1);
     };
-    for (int launches = (total + 7) / 8, last = 0; launches <= total; ++launches) {
-      const int p = (total + launches - 1) / launches;
-      if (p == last) continue;
-      last = p;
-      const int cap = most_rows(L, a.n_q, p);
-      if (cap < 1 || (chosen && n_splits > cap)) continue;
-      if (chosen) { best_p = p; break; }
-      const int one_wave = std::min(default_splits(L, L.U * p), cap), most = std::min(default_splits(L, L.U), cap);
-      add(p, one_wave);
-      for (int half = 3, s = one_wave; half <= 10; ++half) {
-        const int next = (int)((long long)half * (kCtaSlots / 2) / ((long long)L.U * p));
-        if (next <= s || next > most) continue;
-        add(p, s = next);
+    if (time(best_p, best_s) > time(1, alone)) {
+      struct { int p, s; float t; } cand[8 * 12];
+      int n = 0;
+      float least = time(1, alone);
+      auto add = [&](int p, int s) {
+        cand[n] = {p, s, time(p, s)};
+        least = std::min(least, cand[n++].t);
+      };
+      for (int launches = fewest, last = 0; launches <= total; ++launches) {
+        const int p = (total + launches - 1) / launches;
+        if (p == last || most_rows(L, a.n_q, p) < 1) continue;
+        last = p;
+        const int most = std::min(alone, most_rows(L, a.n_q, p));
+        add(p, one_wave(p));
+        for (int half = 3; half <= 10; ++half) {
+          const int s = (int)((long long)half * (kCtaSlots / 2) / ((long long)L.U * p));
+          if (s > cand[n - 1].s && s < most) add(p, s);
+        }
+        if (most > cand[n - 1].s) add(p, most);
       }
-      if (most > one_wave) add(p, most);
+      for (int i = n - 1; i >= 0; --i)
+        if (cand[i].t <= 1.06f * least) { best_p = cand[i].p; best_s = cand[i].s; }
     }
-    for (int i = 0; i < n_cand && !chosen; ++i)
-      if (cand[i].cost <= 1.04f * least) { best_p = cand[i].p; best_s = cand[i].s; break; }
   }
   a.passes = best_p;
   a.ticket_bits = 32 / best_p;
   a.row_cap = most_rows(L, a.n_q, best_p);
   a.part_stride = partial_slots(L, a.n_q, best_p);
-  a.ref_splits = !chosen && best_p > 1 ? default_splits(L, L.U) : 0;
+  a.ref_splits = !chosen && total > 1 ? alone : 0;
   a.reset_iters = 0;
   return best_s;
 }
@@ -143,11 +153,16 @@ inline int fill_split_args(const Layout& L, const Counts& cn, SplitArgs& a, int 
 
 // Iterations (of cpi chunks) between two fresh soft-max references: where the groups of a call share the CTA slots, a warp's
 // range is several times what it would be in a launch of one group, and a reference for all of it would resolve p less; so
-// it is renewed after every range that the warp would have had (whole value groups, one at least).
+// it is renewed after every range that the warp would have had (whole value groups, one at least).  Outer grouping, where
+// that takes an instance of its own: only if the ranges are longer, and the nearest number of groups (a renewal there costs
+// as much as a tenth of an iteration with its group).
 inline void fill_reference_args(const Counts& cn, SplitArgs& a, int ru, int cpi, bool outer) {
   const int n_units = ((outer ? cn.n_qk : cn.n_qv) / kChunk + ru - 1) / ru;
   const int ref_splits = std::min(a.ref_splits, (n_units + kSplitWarps - 1) / kSplitWarps);      // as in fill_split_args
-  a.reset_iters = ref_splits > a.n_splits ? std::max(1, std::max(1, n_units / (kSplitWarps * ref_splits)) * ru / cpi) : 0;
+  const bool renew = ref_splits > 0 && (outer ? ref_splits > a.n_splits : ref_splits >= a.n_splits);
+  const int per_warp = kSplitWarps * ref_splits;
+  const int units = renew ? std::max(1, (n_units + (outer ? per_warp / 2 : 0)) / per_warp) : 0;
+  a.reset_iters = renew ? std::max(1, units * ru / cpi) : 0;
 }
 
 }  // namespace iq

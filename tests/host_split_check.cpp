@@ -77,9 +77,9 @@ int main(int argc, char** argv) {
                   auto time = [&](int p, int s) {
                     s = std::min(s, std::max(1, (units + 7) / 8));
                     const double ctas = (double)U * total * s, full = std::floor(ctas / 296), rest = ctas - 296 * full;
-                    return (full + (rest == 0 ? 0 : rest <= 148 ? 0.65 : 1)) * (cn.n_qv / 32 / (double)s + 18) + 20 * ((total + p - 1) / p - 1);
+                    return (full + (rest == 0 ? 0 : rest <= 148 ? 0.65 : 1)) * (cn.n_qv / 32 / (double)s + 18) + 14 * ((total + p - 1) / p - 1);
                   };
-                  check(time(a.passes, n) <= 1.05 * time(1, default_splits(L, U)), "time against one launch per group");
+                  check(time(a.passes, n) <= 1.07 * time(1, default_splits(L, U)), "time against one launch per group");
                 }
                 if (!cap) continue;      // the next function divides by the grid
                 const int grid = fill_split_args(L, cn, a, G / kChunk, false, n, 0);
