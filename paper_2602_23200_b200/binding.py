@@ -197,22 +197,36 @@ def _dev_ptr(t, name: str, shape, device=None) -> int:
 
 class _Fast:
     """The same two checks for the calls of a decode step, which a model makes per layer and token: at 30 layers the
-    general forms above cost more host time (4-5 us a call of 12) than the kernels take on short contexts.  One attribute
-    read per property, in the order that lets a valid tensor through with the fewest; whatever does not pass (a subclass
-    among it) goes to the general form, which raises (or accepts) it.  Nothing is remembered from call to call."""
+    general forms above cost more host time (4-5 us a call of 12) than the kernels take on short contexts.  One look-up per
+    property, in the order that lets a valid tensor through with the fewest; whatever does not pass (a subclass among it)
+    goes to the general form, which raises (or accepts) it.  Nothing is remembered from call to call."""
     ready = False
 
     @classmethod
     def load(cls):
         import torch
-        cls.tensor, cls.f16, cls.empty = torch.Tensor, torch.float16, torch.empty_like
+        cls.empty = torch.empty_like
         cls.get_device = staticmethod(torch.cuda.current_device)
         cls.get_stream = staticmethod(lambda i: torch.cuda.current_stream(i).cuda_stream)
         # the functions behind those two, without the Stream object and the lazy-initialisation check (a cache exists)
         for name, attr in (("_cuda_getDevice", "get_device"), ("_cuda_getCurrentRawStream", "get_stream")):
             if hasattr(torch._C, name):
                 setattr(cls, attr, staticmethod(getattr(torch._C, name)))
+        global _ptr_of
+        _ptr_of = cls._make_ptr_of(torch.Tensor, torch.float16)
         cls.ready = True
+
+    @staticmethod
+    def _make_ptr_of(tensor, f16):
+        get_device, is_contiguous, data_ptr = tensor.get_device, tensor.is_contiguous, tensor.data_ptr
+
+        def ptr_of(t, name: str, shape, device) -> int:
+            """`shape`: a tuple."""
+            if type(t) is tensor and t.dtype is f16 and t.shape == shape and get_device(t) == device.index and is_contiguous(t):
+                return data_ptr(t)
+            return _dev_ptr(t, name, shape, device)
+
+        return ptr_of
 
 
 def _stream_of(stream, device) -> int:
@@ -222,11 +236,7 @@ def _stream_of(stream, device) -> int:
     return _stream_ptr(stream, device)
 
 
-def _ptr_of(t, name: str, shape, device) -> int:
-    """`shape`: a tuple."""
-    if type(t) is _Fast.tensor and t.dtype is _Fast.f16 and t.shape == shape and t.get_device() == device.index and t.is_contiguous():
-        return t.data_ptr()
-    return _dev_ptr(t, name, shape, device)
+_ptr_of = _dev_ptr      # until a cache exists: see _Fast.load
 
 
 def _handles(caches):
