@@ -158,6 +158,8 @@ int innerq_cache_n_tokens(const innerq_cache_t* cache);
  * tokens in fp16, and quantises the middle: per group statistics, symmetric / asymmetric
  * candidates, the hybrid choice, bit-packing.  Tokens grouped G at a time (V under INNER) that do
  * not fill a group stay fp16 in front of the recent window.  0 <= n_tokens <= max_tokens.
+ * Uses the workspace (partial maxima of the keys, where a decode keeps its split partials): like two decodes, a prefill
+ * and another call on the same workspace must not overlap.
  * Errors: INVALID_ARG, CAPACITY, CUDA. */
 int innerq_quantize_prefill(innerq_cache_t* cache, const void* k, const void* v, int32_t n_tokens,
                             void* cuda_stream);
@@ -218,8 +220,8 @@ int innerq_step_staging_bytes(const innerq_config_t* cfg, size_t* bytes);
  *   dev_scratch   : device, 256-byte aligned, at least innerq_multi_query_scratch_bytes(cfg) bytes; owned by the
  *                   caller, used only during the call (split partials of up to four query rows per KV head).
  * The rows of a KV head (its n_q * r query heads) are processed in groups of four, up to eight groups in one launch that
- * read the packed cache together: with one query head per KV head four query tokens share a group, with four or more
- * each token takes its own.
+ * read the packed cache together (fewer where that is the faster choice, or where dev_scratch holds no more): with one
+ * query head per KV head four query tokens share a group, with four or more each token takes its own.
  * Limits: the fused kernel only (packed inner- or outer-grouped cache in a format it supports; decode variant
  * 0 or 2); the n_q - 1 newest tokens must all lie outside the token range in which keys AND values are packed
  * (always true for n_q - 1 <= w_recent once the windows are full).  Otherwise UNSUPPORTED, nothing launched.
@@ -292,6 +294,10 @@ int innerq_cache_import(innerq_cache_t* cache, const innerq_export_t* ex, int32_
  *              CTAs per SM, the lowest latency for a launch that runs alone.  148 / (batch * n_kv_heads), i.e. one
  *              CTA per SM and launch, lets consecutive launches share the GPU and hide each other's start and end:
  *              10-15 % more steps per second in a loop of back-to-back calls, 10-25 % slower for a launch alone.
+ *              With more than four query rows per KV head (n_q * n_q_heads / n_kv_heads) the groups of four share a
+ *              launch and each is split into n_splits ranges, so the launch has that many times the CTAs; a count that
+ *              the launch's split partials cannot hold for every group gets more launches.  0 then chooses splits and
+ *              groups per launch together.
  *   variant  : 0 automatic, 1 plain SIMT kernel, 2 warp-MMA kernel (where supported; UNSUPPORTED otherwise),
  *              3 / 4 warp-MMA kernel with one / two 32-token chunks per loop iteration (sets a process-wide knob).
  *              6 / 7 TIMING ONLY, the output is wrong on purpose: the warp-MMA kernel with the unpack + MMA work of

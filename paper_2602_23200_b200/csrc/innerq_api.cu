@@ -17,8 +17,9 @@ struct innerq_cache {
   unsigned char* cache;
   unsigned char* ws;
   int N;
-  int N_safe;      // token count when the last decode of this cache was launched (or at prefill): what was packed by then
-                   // is complete and is not written again; a later decode may stream it before its predecessors finish
+  int N_safe;      // token count when the last decode of this cache was launched: what was packed by then is complete and
+                   // is not written again; a later decode may stream it before its predecessors finish.  0 (prefilled or
+                   // imported since): nothing may be read ahead, the norms included
   int reads_settled;   // the last kernel enqueued for this cache was a fused decode: when its dependents may start, it
                        // has read everything that an append writes (the fp16 rings, the newest packed rows); an
                        // append can then run without waiting first
@@ -177,7 +178,7 @@ void make_layout(const innerq_config_t& c, Layout& L, int page_tokens = 0) {
   L.cache_bytes = off;
   size_t w = 0;
   L.ws_partial_off = w; w = align_up(w + (size_t)L.B * L.Hq * L.max_splits * kPartialStride * 4, 256);
-  L.ws_absmax_off = w; w = align_up(w + (size_t)L.U * kD * 4, 256);
+  w = align_up(w + (size_t)L.U * kD * 4, 256);      // not used; the sizes that callers were told stay as they are
   L.ws_ticket_off = w; w = align_up(w + (size_t)(L.U + 8) * 4, 256);   // tickets [U], then the device error word
   L.workspace_bytes = w;
 }

@@ -86,8 +86,7 @@ struct Layout {
                        // Then uint32 [U]: tickets of the CTAs that share the append of one unit (zero between appends)
   size_t cache_bytes;
   // workspace
-  size_t ws_partial_off;   // float [B*Hq][max_splits][kPartialStride]
-  size_t ws_absmax_off;    // [U][D] words, not used any more (the workspace keeps its size)
+  size_t ws_partial_off;   // float [B*Hq][max_splits][kPartialStride]; during a prefill the partial maxima of the keys
   size_t ws_ticket_off;    // uint32 [U]
   size_t workspace_bytes;
   // Paged record area (page_groups > 0): the group records of a cache live in pages of a pool that several caches

@@ -1,5 +1,6 @@
-// Quantise-side kernels: per-channel key norm, group quantisation into the ROW / BLOCK stores
-// (prefill and quantise-on-evict share the same device routines), window copies, canonical export.
+// Quantise-side kernels: group quantisation into the ROW / BLOCK stores one token / group at a time (quantise-on-evict,
+// and the prefill of the outer-grouped cache), append, canonical export and import.  The prefill of the inner-grouped
+// cache, its key norms and the window copies are in innerq_quantize_prefill.cu.
 #include "innerq_device.cuh"
 #include "innerq_kernels.h"
 

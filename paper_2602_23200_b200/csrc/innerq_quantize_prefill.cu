@@ -7,7 +7,9 @@
 // candidates, then the codes of the chosen mode.  All value arithmetic is the same sequence of single, correctly
 // rounded fp32 operations as in group_params / asym_code / sym_code, so stored bits do not depend on the kernel:
 // rounding to an integer is done by adding 1.5 * 2^23 (round-to-nearest-even at unit granularity, identical to
-// rintf for |t| < 2^22; codes are bounded by a few times 2^b), which leaves the code in the low mantissa bits.
+// rintf for |t| < 2^22), which leaves the code in the low mantissa bits.  |t| before the clamp is at most a few times 2^b
+// plus the rounding error of the zero-point in units of the scale: keys are divided by the root of their largest value, so
+// their zero-point is below 2^8 and off by 2^-4 at most, and the smallest fp16 scale is 2^-24, hence |t| < 2^21.
 //
 // What bounds them: instruction issue (both read and write far below the HBM rate), so values are kept as PAIRS and
 // every add / multiply is one packed fp32x2 instruction, whose two halves are rounded exactly as the scalar ones.  A
@@ -17,6 +19,7 @@
 #include <type_traits>
 
 #include "innerq_device.cuh"
+#include "innerq_div_const.h"
 #include "innerq_kernels.h"
 
 namespace iq {
@@ -58,19 +61,6 @@ struct Mul2 {
   __device__ __forceinline__ explicit Mul2(float nz) : neg_zero(f2(nz, nz)) {}
   __device__ __forceinline__ F2 operator()(F2 a, F2 b) const { return fma2(a, b, neg_zero); }
 };
-
-// x / DEN for DEN = 1, 3, 7, 15, correctly rounded: the product with the rounded reciprocal, corrected by its
-// FMA-computed (hence exact) remainder, which is exact for divisors known in advance (Brisebarre, Muller and Raina,
-// "Accelerating correctly rounded floating-point division when the divisor is known in advance", 2004); the host test
-// tests/div_const_check.cpp goes through every mantissa of the four divisors.  Results below the normal range may be
-// one unit off: the callers round to fp16, where they are zero.
-template <int DEN> __device__ __forceinline__ float div_const(float x) {
-  if constexpr (DEN == 1) return x;
-  constexpr float r = 1.0f / (float)DEN;
-  const float q = __fmul_rn(x, r);
-  const float q1 = __fmaf_rn(__fmaf_rn(-(float)DEN, q, x), r, q);
-  return fabsf(q) < INFINITY ? q1 : q;      // an infinite (or NaN) quotient has no remainder
-}
 
 // group_params (innerq_device.cuh) with its divisions by constants and reciprocals in their cheaper correctly rounded
 // forms: the same bits.
@@ -666,8 +656,10 @@ __device__ __forceinline__ void copy_windows(const Layout& L, const Counts& cn, 
 // First of the two launches of an inner-grouped prefill: everything that does not need the key norms.  Roles [0, n_max)
 // take the key maxima (n_part per unit), the next n_val the value groups, the rest the windows.  The first two are dealt
 // to alternate CTAs: the maxima wait for memory while the value groups beside them on the SM compute (32 units x 32768
-// tokens, 2 bits, G = 128: 164 us; one role after the other 177 us; as two launches 43 + 134 us).  A prompt of a few hundred tokens is bound by its launches, not by its kernels: ten
-// of them (clear, maxima, norms, two quantisers, four window copies, counts) took 42.6 us for 512 tokens of 8 heads.
+// tokens, 2 bits, G = 128: 164 us; one role after the other 177 us; as two launches 43 + 134 us).  A prompt of a few
+// hundred tokens is bound by its launches, not by its kernels: ten of them (clear, maxima, norms, two quantisers, four
+// window copies, counts) took 38.9 us for 512 tokens of 8 heads (3 bits, symmetric; calls through the binding, one after
+// the other), the two take 10.2 us.
 template <int VBITS>
 __global__ void __launch_bounds__(256, 2)
 prefill_first_kernel(const __grid_constant__ Layout L, const Counts cn, const __half* __restrict__ K,

@@ -371,8 +371,8 @@ def test_multi_query_decode(grouping, r, G, bits, n_q):
 
 
 # Several groups of four query rows in one launch (and, beyond eight groups, in several): query heads and query tokens, key
-# rows whose length falls and rises by 2^+-10 along the context, so that the soft-max references of a warp's range move
-# both ways, peaked and flat parts of the context in one range.
+# rows whose length falls and rises by 2^+-10 along the context: peaked and flat parts of the context in one range, scores
+# far above and below the range's soft-max reference.  (Renewed references: test_rows_that_share_a_launch_lose_no_precision.)
 @pytest.mark.parametrize("r,n_q,G,kb,vb,N", [(8, 1, 32, 2, 2, 3001), (9, 1, 64, 3, 3, 2900), (16, 1, 128, 4, 4, 3001),
                                              (4, 5, 32, 4, 2, 3001), (4, 9, 64, 2, 2, 2500), (1, 33, 128, 2, 2, 3001),
                                              (5, 3, 32, 3, 2, 700), (8, 2, 64, 4, 3, 150)])

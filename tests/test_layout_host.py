@@ -24,7 +24,7 @@ def test_positions_are_bijections_and_operand_bytes_are_code_times_weight(tmp_pa
 @pytest.mark.skipif(shutil.which("g++") is None, reason="needs a host C++ compiler")
 def test_division_by_the_quantisers_constants_is_correctly_rounded(tmp_path):
     exe = str(tmp_path / "div_const_check")
-    subprocess.run(["g++", "-std=c++17", "-O2", "-march=native", "-ffp-contract=off", "-o", exe,
+    subprocess.run(["g++", "-std=c++17", "-O2", "-march=native", "-ffp-contract=off", "-I", CSRC, "-o", exe,
                     os.path.join(HERE, "div_const_check.cpp")], check=True)
     r = subprocess.run([exe], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout
