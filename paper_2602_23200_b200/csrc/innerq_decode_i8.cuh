@@ -284,9 +284,11 @@ __device__ __forceinline__ void decode_i8_body(const Layout& L, const Counts& cn
     }
   // What the end of the kernel needs of this waits in shared memory: in registers it would cost the streaming loop some,
   // worked out again there it is on the critical path of the launch's end (8 KV heads x 2000 to 32768 tokens, r 4, calls in
-  // a chain: 6.0 to 10.3 us, 0.1 us less this way).
+  // a chain: 6.0 to 10.3 us, 0.1 us less this way).  SPLIT has one query row: nothing to work out (32 heads x 30011 tokens,
+  // 0.1 us a step less without).
   __shared__ int4 s_end;      // row of the split partials, heads, ticket field, first query row
-  if (tid == 0) s_end = make_int4(a.n_q > 1 ? ux * kHeads : q_row(0), nh, SPLIT ? 0 : pass * a.ticket_bits, head0);
+  if (!SPLIT && tid == 0) s_end = make_int4(a.n_q > 1 ? ux * kHeads : q_row(0), nh, pass * a.ticket_bits, head0);
+  auto at_end = [&]() { return SPLIT ? make_int4(q_row_of(u, a.head0, 0), 1, 0, a.head0) : s_end; };
   float q_early[2], n_early[2];
 #pragma unroll
   for (int e = 0; e < 2; ++e) {
@@ -1120,7 +1122,7 @@ __device__ __forceinline__ void decode_i8_body(const Layout& L, const Counts& cn
       }
     }
     __syncthreads();
-    const int prow0 = s_end.x, nh_end = s_end.y;
+    const int prow0 = at_end().x, nh_end = at_end().y;
     float* partials = a.partials;
     for (int i = tid; i < nh_end * kD; i += kThreads) {
       const int h = i >> 7, c = i & (kD - 1);
@@ -1143,7 +1145,7 @@ __device__ __forceinline__ void decode_i8_body(const Layout& L, const Counts& cn
 
   // ---------------- cross-CTA merge: the last CTA of the unit to arrive combines all parts -----------
   __shared__ unsigned int s_ticket;
-  const int4 end = s_end;
+  const int4 end = at_end();
   __syncthreads();                 // all partial writes of this CTA happen-before thread 0's ticket below
   if (tid == 0) {
     // release: publishes the whole CTA's partial (ordered before this thread by the barrier) with the ticket;
