@@ -11,10 +11,10 @@
 // plus the rounding error of the zero-point in units of the scale: keys are divided by the root of their largest value, so
 // their zero-point is below 2^8 and off by 2^-4 at most, and the smallest fp16 scale is 2^-24, hence |t| < 2^21.
 //
-// What bounds them: instruction issue (both read and write far below the HBM rate), so values are kept as PAIRS and
-// every add / multiply is one packed fp32x2 instruction, whose two halves are rounded exactly as the scalar ones.  A
-// packed instruction does not raise the fp32 rate, but it takes one issue slot for two operations, and the slots it
-// frees go to the conversions, minima / maxima and byte permutes.
+// What bounds them: instruction issue (both read and write far below the HBM rate).  Values are kept as PAIRS and most
+// adds / multiplies are packed fp32x2 instructions, whose two halves are rounded exactly as the scalar ones.  A packed (or
+// half-precision pair) instruction occupies its pipe and the issue for two cycles, as two scalar ones do; it saves
+// instruction fetches and registers, not time.
 #include <algorithm>
 #include <type_traits>
 
@@ -152,9 +152,83 @@ struct ChosenPair {
   }
 };
 
-// low bytes of four code words as the four bytes of one word
-__device__ __forceinline__ uint32_t bytes4(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-  return __byte_perm(__byte_perm(a, b, 0x0040), __byte_perm(c, d, 0x0040), 0x5410);
+// Both candidates' L1 errors with fewer operations than PairCoder's, for the groups whose mode they settle beyond doubt
+// (quick_mode); the others get the sums above.  A segment's sums of one channel; packed and half-precision instructions
+// issue over two cycles, so what counts is operations: 11 per value above, 12.4 cycles measured.  32 units x 16384 tokens,
+// both tensors: 150 us before, 132 with 2 bits; 4 bits 151 and 138; groups that nothing but the sums above decides (equal
+// errors everywhere) cost 10 % more.
+//   2 bits: the distance to the nearest of four equidistant levels is | ||x - c| - s| - s/2 | with c in their middle, to
+//           the nearest of -s, 0, s it is s/2 - ||x| - s/2|: 6 operations, 6.7 cycles; a scalar addition takes the
+//           absolute value of its operand for free.
+//   3, 4 bits: y = x / s + const is rounded at 2^-16 by a fused multiply-add whose result lies in [128, 256): the low 16
+//           bits are the distance to the nearest code as a signed fraction.  Its absolute value (the smaller of it and its
+//           complement, one unit off where it is negative) is summed by dp2a: 7.4 cycles.  Needs codes within their
+//           range (no_clip), scales that are not zero and a zero-point of at most 64 scales.
+template <int BITS> struct QuickErr {
+  F2 nc, inv_a, off_a, inv_s;               // pairs for the two operands of add()
+  float2 s_a, h_a, h_s;
+  float2 a = make_float2(0.f, 0.f), t = make_float2(0.f, 0.f);
+  uint32_t ua0 = 0, ua1 = 0, us0 = 0, us1 = 0;
+  static constexpr float kFrac = 192.f;     // 1.5 * 2^7
+  __device__ __forceinline__ QuickErr(const GroupParams& p, const GroupParams& q)
+      : nc(f2(-fmaf(1.5f, p.s_a, p.z_a), -fmaf(1.5f, q.s_a, q.z_a))), inv_a(f2(p.inv_a, q.inv_a)),
+        off_a(f2(fmaf(-p.z_a, p.inv_a, kFrac), fmaf(-q.z_a, q.inv_a, kFrac))), inv_s(f2(p.inv_s, q.inv_s)),
+        s_a(make_float2(p.s_a, q.s_a)), h_a(make_float2(0.5f * p.s_a, 0.5f * q.s_a)), h_s(make_float2(0.5f * p.s_s, 0.5f * q.s_s)) {}
+  // values lo and hi of one group: distances to their nearest codes, in the two halves of a word
+  static __device__ __forceinline__ uint32_t frac_abs(float lo, float hi) {
+    const uint32_t f = __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x5410);
+    return __vminu2(f, ~f);
+  }
+  static __device__ __forceinline__ void acc2(uint32_t& acc, uint32_t f) {
+    asm("dp2a.lo.u32.u32 %0, %1, %2, %0;" : "+r"(acc) : "r"(f), "r"(0x0101));
+  }
+  // x, y: two pairs, the first halves of both belong to one group and the second halves to another (or to the same one)
+  __device__ __forceinline__ void add(F2 x, F2 y) {
+    if constexpr (BITS == 2) {
+      one(x);
+      one(y);
+    } else {
+      const F2 k = f2(kFrac, kFrac);
+      const float2 ax = unf2(fma2(x, inv_a, off_a)), ay = unf2(fma2(y, inv_a, off_a));
+      const float2 sx = unf2(fma2(x, inv_s, k)), sy = unf2(fma2(y, inv_s, k));
+      acc2(ua0, frac_abs(ax.x, ay.x));
+      acc2(ua1, frac_abs(ax.y, ay.y));
+      acc2(us0, frac_abs(sx.x, sy.x));
+      acc2(us1, frac_abs(sx.y, sy.y));
+    }
+  }
+  __device__ __forceinline__ void one(F2 x) {
+    const float2 v = unf2(x), d = unf2(add2(x, nc));
+    a.x += fabsf(fabsf(fabsf(d.x) - s_a.x) - h_a.x);
+    a.y += fabsf(fabsf(fabsf(d.y) - s_a.y) - h_a.y);
+    t.x += fabsf(fabsf(v.x) - h_s.x);
+    t.y += fabsf(fabsf(v.y) - h_s.y);
+  }
+  // (asymmetric - symmetric) error sum of the n values that went into the first / second halves
+  __device__ __forceinline__ float2 difference(float n) const {
+    if constexpr (BITS == 2) return make_float2(a.x - fmaf(n, h_s.x, -t.x), a.y - fmaf(n, h_s.y, -t.y));
+    const float u = 0x1p-16f;
+    return make_float2(u * (s_a.x * (float)ua0 - 2.f * h_s.x * (float)us0), u * (s_a.y * (float)ua1 - 2.f * h_s.y * (float)us1));
+  }
+};
+
+// How far a group's difference of the quick sums and that of PairCoder's can be apart; infinite where the quick sums mean
+// nothing (NaN where the values are not finite: no comparison with it settles anything).  m = largest |x| of the group.
+// 2 bits: a value's rounding errors are below 2^-20 m in each form, those of adding up 32 of them in two chains below
+// 2^-20 m a value; a value beyond the outer symmetric level (whose fp16 scale may be rounded down) counts with the wrong
+// sign.  3, 4 bits: in units of 2^-16 scales a value is off by 1 (complement), 1/2 (constant), 1/2 (rounding) and 1/8
+// (reciprocal scales, the other form's own roundings).
+template <int BITS>
+__device__ __forceinline__ float quick_bound(const GroupParams& p, const Bounds& b, float mn, float mx, int G) {
+  const float m = fmaxf(fabsf(mn), fabsf(mx)), n = (float)G;
+  if constexpr (BITS == 2)
+    return n * (m * 0x1p-18f + 2.f * fmaxf(0.f, m - p.s_s));
+  else
+    return b.no_clip && p.s_a > 0.f && p.s_s > 0.f && fabsf(p.z_a) * p.inv_a < 60.f ? n * 3.f * 0x1p-16f * (p.s_a + p.s_s) : INFINITY;
+}
+// 1: asymmetric, 0: symmetric, -1: the quick sums do not tell
+__device__ __forceinline__ int quick_mode(float difference, float bound) {
+  return difference > bound ? 0 : difference < -bound ? 1 : -1;
 }
 
 __device__ __forceinline__ float min3(float a, float b, float c) {
@@ -166,6 +240,10 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   float r;
   asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
   return r;
+}
+// low bytes of four code words as the four bytes of one word
+__device__ __forceinline__ uint32_t bytes4(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  return __byte_perm(__byte_perm(a, b, 0x0040), __byte_perm(c, d, 0x0040), 0x5410);
 }
 
 // 3-bit codes in byte order (see row_pos_i8_3 / block_pos_i8_3): four codes in the bytes of w become the 2-bit plane's
@@ -305,24 +383,37 @@ quantize_rows_prefill_kernel(const __grid_constant__ Layout L, const __half* __r
       const Bounds bd(mul2, p, mn, mx);               // the same for all lanes of a group
       bool asym = S.mode == 1;
       if (S.mode == 2) {
-        const PairCoder pc(mul2, p, bd, p, bd);
-        float2 ea = make_float2(0.f, 0.f), es = make_float2(0.f, 0.f);
-        auto sums = [&](auto clamp) {
+        int quick = -1;
+        if (L.sym_variant == 0) {               // (the literal formula clips the tails of every group)
+          QuickErr<BITS> qe(p, p);
 #pragma unroll
-          for (int e = 0; e < kSeg / 2; ++e) {
-            const float2 a = pc.template err_asym<decltype(clamp)::value>(x[e]), s = pc.template err_sym<decltype(clamp)::value>(x[e]);
-            ea.x += fabsf(a.x); ea.y += fabsf(a.y);
-            es.x += fabsf(s.x); es.y += fabsf(s.y);
-          }
-        };
-        if (bd.no_clip) sums(std::false_type{});
-        else sums(std::true_type{});
-        float a = ea.x + ea.y, s = es.x + es.y;
-        for (int o = 1; o < gl; o <<= 1) {
-          a += __shfl_xor_sync(0xffffffffu, a, o);
-          s += __shfl_xor_sync(0xffffffffu, s, o);
+          for (int e = 0; e < kSeg / 2; e += 2) qe.add(x[e], x[e + 1]);
+          const float2 d2 = qe.difference((float)(kSeg / 2));
+          float d = d2.x + d2.y;
+          for (int o = 1; o < gl; o <<= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+          quick = quick_mode(d, quick_bound<BITS>(p, bd, mn, mx, L.G));      // the same in all lanes of a group
         }
-        asym = a < s;
+        asym = quick > 0;
+        if (__any_sync(0xffffffffu, quick < 0)) {
+          const PairCoder pc(mul2, p, bd, p, bd);
+          float2 ea = make_float2(0.f, 0.f), es = make_float2(0.f, 0.f);
+          auto sums = [&](auto clamp) {
+#pragma unroll
+            for (int e = 0; e < kSeg / 2; ++e) {
+              const float2 a = pc.template err_asym<decltype(clamp)::value>(x[e]), s = pc.template err_sym<decltype(clamp)::value>(x[e]);
+              ea.x += fabsf(a.x); ea.y += fabsf(a.y);
+              es.x += fabsf(s.x); es.y += fabsf(s.y);
+            }
+          };
+          if (bd.no_clip) sums(std::false_type{});
+          else sums(std::true_type{});
+          float a = ea.x + ea.y, s = es.x + es.y;
+          for (int o = 1; o < gl; o <<= 1) {
+            a += __shfl_xor_sync(0xffffffffu, a, o);
+            s += __shfl_xor_sync(0xffffffffu, s, o);
+          }
+          asym = a < s;
+        }
       }
       uint32_t w8[8];                           // [2 * j + h]: bytes 16 h + 4 j .. + 3 of the segment's bit position
       {
@@ -392,7 +483,11 @@ quantize_rows_prefill_kernel(const __grid_constant__ Layout L, const __half* __r
 // share words of the packed chunk are adjacent lanes, which exchange them and store 16 contiguous bytes each (3-bit:
 // the 1-bit plane's words are shared with the other channel half, a warp away).
 // CTA `part` of `n_parts` takes a contiguous run of all units' groups.
-constexpr int kBlocksSmemWords = 4 * 128 + 4 * 32;      // uint4: statistics of 4 chunks, 1-bit plane words of 4 chunks
+// A warp's 32 tokens x 64 channels come through its own 4 KB of shared memory, requested (cp.async) as soon as the values
+// before them are in registers: read straight from global memory the loads of a group were waited for with nothing else to
+// do, two thirds of the cycles without an instruction.
+constexpr int kBlocksRaw = 8 * 4096 / 16;               // uint4: values of 8 warps
+constexpr int kBlocksSmemWords = kBlocksRaw + 4 * 128 + 4 * 32;      // + statistics of 4 chunks, 1-bit plane words of 4 chunks
 template <int BITS>
 __device__ __forceinline__ void quantize_blocks(const Layout& L, const __half* __restrict__ X, int N, int n_q,
                                                 unsigned char* __restrict__ cache, int part, int n_parts, uint4* smem_q,
@@ -400,23 +495,70 @@ __device__ __forceinline__ void quantize_blocks(const Layout& L, const __half* _
   const Store& S = L.v;
   const int G = L.G, CH = G >> 5, sh = CH >> 1, per_cta = 4 >> sh, n_groups = n_q / G;
   const int tid = threadIdx.x, cp = tid & 63, k4 = tid >> 6, k = k4 & (CH - 1), c0 = 2 * cp;
-  float4* red_m = reinterpret_cast<float4*>(smem_q);                             // [4][64]: min, max of both channels
+  uint4* stats = smem_q + kBlocksRaw;
+  float4* red_m = reinterpret_cast<float4*>(stats);                              // [4][64]: min, max of both channels
   float4* red_e = red_m + 4 * 64;                                                // [4][64]: error sums of both channels
-  uint4* red_h = smem_q + 4 * 128;                                               // [4][32]: 1-bit plane words
+  uint4* red_h = stats + 4 * 128;                                                // [4][32]: 1-bit plane words
+  const int lane = tid & 31;
+  unsigned char* mine = reinterpret_cast<unsigned char*>(smem_q) + (tid >> 5) * 4096;      // this warp's [32 tokens][64 channels]
+  const uint32_t mine_u32 = (uint32_t)__cvta_generic_to_shared(mine);
+  const bool wide = (reinterpret_cast<size_t>(X) & 15) == 0;
   const int m = 4 * (c0 >> 6) + ((c0 >> 1) & 3), gid = (c0 >> 3) & 7;             // fragment coordinates of the pair
-  const long long items = (long long)L.U * n_groups, steps = (items + per_cta - 1) / per_cta;
-  for (long long step = steps * part / n_parts; step < steps * (part + 1) / n_parts; ++step) {
-    long long item = step * per_cta + (k4 >> sh);
-    const bool valid = item < items;                        // the last step may have fewer groups than the CTA takes
+  // Barriers of the warps that exchange something, instead of the whole CTA's: the CH warps with the same channels of a
+  // group (the statistics), the two warps of a chunk (the 1-bit plane).
+  const int my_group = 1 + ((k4 >> sh) << 1) + ((tid >> 5) & 1);
+  auto group_sync = [&]() { asm volatile("barrier.sync %0, %1;" ::"r"(my_group), "r"(32 * CH) : "memory"); };
+  auto group_or = [&](bool p) {
+    int any;
+    asm volatile("{.reg .pred p, q; setp.ne.s32 p, %1, 0; barrier.red.or.pred q, %2, %3, p; selp.s32 %0, 1, 0, q;}"
+                 : "=r"(any) : "r"((int)p), "r"(my_group), "r"(32 * CH) : "memory");
+    return any != 0;
+  };
+  [[maybe_unused]] auto pair_sync = [&]() { asm volatile("barrier.sync %0, 64;" ::"r"(9 + k4) : "memory"); };
+  const int items = L.U * n_groups, steps = (items + per_cta - 1) / per_cta;      // a group is 8 KB at least: 31 bits hold them
+  const int s_begin = (int)((long long)steps * part / n_parts), s_end = (int)((long long)steps * (part + 1) / n_parts);
+  int u = 0, j = 0;                                         // unit and group of this thread's item of the step
+  bool valid = false;
+  auto locate = [&](int step) {
+    int item = step * per_cta + (k4 >> sh);
+    valid = item < items;                                   // the last step may have fewer groups than the CTA takes
     if (!valid) item = items - 1;
-    const int u = (int)(item / n_groups), j = (int)(item - (long long)u * n_groups);
-    const __half* Xu = X + ((size_t)u * N + L.w_sink) * kD + c0;
+    u = item / n_groups;
+    j = item - u * n_groups;
+  };
+  auto request = [&]() {                                    // the warp's values of (u, j), into its shared memory
+    const __half* src = X + ((size_t)u * N + L.w_sink + (size_t)j * G + kSeg * k) * kD + 64 * ((tid >> 5) & 1);
+    if (wide) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int p = i * 32 + lane;                        // 16-byte piece: token p / 8, channels 8 (p % 8) ..
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(mine_u32 + p * 16), "l"(src + (p >> 3) * kD + (p & 7) * 8));
+      }
+    } else {
+#pragma unroll 4
+      for (int i = 0; i < kSeg; ++i)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(mine_u32 + (i * 32 + lane) * 4), "l"(src + i * kD + 2 * lane));
+    }
+  };
+  if (s_begin < s_end) {
+    locate(s_begin);
+    request();
+  }
+  for (int step = s_begin; step < s_end; ++step) {
+    const int u_now = u, j_now = j;
+    const bool valid_now = valid;
     F2 x[kSeg];
     {
       uint32_t raw[kSeg];
-      const __half* src = Xu + ((size_t)j * G + kSeg * k) * kD;
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      __syncwarp();
 #pragma unroll
-      for (int t = 0; t < kSeg; ++t) raw[t] = __ldg(reinterpret_cast<const uint32_t*>(src + (size_t)t * kD));
+      for (int t = 0; t < kSeg; ++t) raw[t] = *reinterpret_cast<const uint32_t*>(mine + t * 128 + lane * 4);
+      __syncwarp();                                         // all lanes have theirs: the next values may come
+      if (step + 1 < s_end) {
+        locate(step + 1);
+        request();
+      }
 #pragma unroll
       for (int t = 0; t < kSeg; ++t) {
         const float2 v = __half22float2(*reinterpret_cast<const __half2*>(&raw[t]));
@@ -436,48 +578,70 @@ __device__ __forceinline__ void quantize_blocks(const Layout& L, const __half* _
       mx.x = max3(mx.x, v.x, w.x); mx.y = max3(mx.y, v.y, w.y);
     }
     if (CH > 1) {
-      __syncthreads();                                       // the previous group's words are no longer read
+      group_sync();                                          // the previous group's words are no longer read
       red_m[k4 * 64 + cp] = make_float4(mn.x, mx.x, mn.y, mx.y);
-      __syncthreads();
+      group_sync();
       for (int kk = 0; kk < CH; ++kk) {
         const float4 o = red_m[(k4 - k + kk) * 64 + cp];
         mn.x = fminf(mn.x, o.x); mx.x = fmaxf(mx.x, o.y);
         mn.y = fminf(mn.y, o.z); mx.y = fmaxf(mx.y, o.w);
       }
-    } else if (BITS == 3) {
-      __syncthreads();
     }
     const GroupParams p0 = seg_params<BITS>(mn.x, mx.x, L.sym_variant), p1 = seg_params<BITS>(mn.y, mx.y, L.sym_variant);
     const Bounds b0(mul2, p0, mn.x, mx.x), b1(mul2, p1, mn.y, mx.y);
     const bool no_clip = b0.no_clip && b1.no_clip;
     bool asym0 = S.mode == 1, asym1 = asym0;
     if (S.mode == 2) {
-      const PairCoder pc(mul2, p0, b0, p1, b1);
-      float2 a0 = make_float2(0.f, 0.f), a1 = a0, s0 = a0, s1 = a0;      // even / odd tokens
-      auto sums = [&](auto clamp) {
-        constexpr bool C = decltype(clamp)::value;
+      bool close = true;
+      if (L.sym_variant == 0) {
+        QuickErr<BITS> qe(p0, p1);
 #pragma unroll
-        for (int t = 0; t < kSeg; t += 2) {
-          const float2 ae = pc.template err_asym<C>(x[t]), ao = pc.template err_asym<C>(x[t + 1]);
-          a0.x += fabsf(ae.x); a0.y += fabsf(ae.y); a1.x += fabsf(ao.x); a1.y += fabsf(ao.y);
-          const float2 se = pc.template err_sym<C>(x[t]), so = pc.template err_sym<C>(x[t + 1]);
-          s0.x += fabsf(se.x); s0.y += fabsf(se.y); s1.x += fabsf(so.x); s1.y += fabsf(so.y);
+        for (int t = 0; t < kSeg; t += 2) qe.add(x[t], x[t + 1]);
+        float2 d = qe.difference((float)kSeg);
+        if (CH > 1) {
+          float2* red_d = reinterpret_cast<float2*>(red_e);         // the first half of the thread's own entry
+          red_d[2 * (k4 * 64 + cp)] = d;
+          group_sync();
+          d = make_float2(0.f, 0.f);
+          for (int kk = 0; kk < CH; ++kk) {
+            const float2 o = red_d[2 * ((k4 - k + kk) * 64 + cp)];
+            d.x += o.x; d.y += o.y;
+          }
         }
-      };
-      if (no_clip) sums(std::false_type{});
-      else sums(std::true_type{});
-      float4 e = make_float4(a0.x + a1.x, s0.x + s1.x, a0.y + a1.y, s0.y + s1.y);
-      if (CH > 1) {
-        red_e[k4 * 64 + cp] = e;
-        __syncthreads();
-        e = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int kk = 0; kk < CH; ++kk) {
-          const float4 o = red_e[(k4 - k + kk) * 64 + cp];
-          e.x += o.x; e.y += o.y; e.z += o.z; e.w += o.w;
-        }
+        const int quick0 = quick_mode(d.x, quick_bound<BITS>(p0, b0, mn.x, mx.x, G));
+        const int quick1 = quick_mode(d.y, quick_bound<BITS>(p1, b1, mn.y, mx.y, G));
+        asym0 = quick0 > 0;
+        asym1 = quick1 > 0;
+        close = quick0 < 0 || quick1 < 0;
       }
-      asym0 = e.x < e.y;
-      asym1 = e.z < e.w;
+      if (CH > 1 ? group_or(close) : (bool)__any_sync(0xffffffffu, close)) {
+        const PairCoder pc(mul2, p0, b0, p1, b1);
+        float2 a0 = make_float2(0.f, 0.f), a1 = a0, s0 = a0, s1 = a0;      // even / odd tokens
+        auto sums = [&](auto clamp) {
+          constexpr bool C = decltype(clamp)::value;
+#pragma unroll
+          for (int t = 0; t < kSeg; t += 2) {
+            const float2 ae = pc.template err_asym<C>(x[t]), ao = pc.template err_asym<C>(x[t + 1]);
+            a0.x += fabsf(ae.x); a0.y += fabsf(ae.y); a1.x += fabsf(ao.x); a1.y += fabsf(ao.y);
+            const float2 se = pc.template err_sym<C>(x[t]), so = pc.template err_sym<C>(x[t + 1]);
+            s0.x += fabsf(se.x); s0.y += fabsf(se.y); s1.x += fabsf(so.x); s1.y += fabsf(so.y);
+          }
+        };
+        if (no_clip) sums(std::false_type{});
+        else sums(std::true_type{});
+        float4 e = make_float4(a0.x + a1.x, s0.x + s1.x, a0.y + a1.y, s0.y + s1.y);
+        if (CH > 1) {
+          red_e[k4 * 64 + cp] = e;
+          group_sync();
+          e = make_float4(0.f, 0.f, 0.f, 0.f);
+          for (int kk = 0; kk < CH; ++kk) {
+            const float4 o = red_e[(k4 - k + kk) * 64 + cp];
+            e.x += o.x; e.y += o.y; e.z += o.z; e.w += o.w;
+          }
+        }
+        asym0 = e.x < e.y;
+        asym1 = e.z < e.w;
+      }
     }
     // codes of token t sit in byte t / 8 of word [2 * (t % 4) + (t % 8) / 4] (see block_pos_i8), at bit position 0 here
     uint32_t w[2][8];
@@ -496,8 +660,8 @@ __device__ __forceinline__ void quantize_blocks(const Layout& L, const __half* _
       if (no_clip) codes(std::false_type{});
       else codes(std::true_type{});
     }
-    const Rec rec = unit_rec(L, cache, u);
-    unsigned char* group = group_ptr(rec, j);
+    const Rec rec = unit_rec(L, cache, u_now);
+    unsigned char* group = group_ptr(rec, j_now);
     uint32_t* chunk = reinterpret_cast<uint32_t*>(group + k * S.chunk_stride + S.code_in_rec);
     if constexpr (BITS == 4) {
       // The two channel pairs cp = 2q, 2q + 1 (adjacent lanes) fill the two nibbles of the same 16 words: after one
@@ -516,7 +680,7 @@ __device__ __forceinline__ void quantize_blocks(const Layout& L, const __half* _
             const uint32_t give = pos ? w[rh][2 * jj + half] : w[rh][2 * (2 + jj) + half];
             f4[2 * half + rh] = keep | __shfl_xor_sync(0xffffffffu, give, 1);
           }
-        if (valid) *reinterpret_cast<uint4*>(chunk + W * 128 + (4 * gid + 2 * pos + jj) * 4) = make_uint4(f4[0], f4[1], f4[2], f4[3]);
+        if (valid_now) *reinterpret_cast<uint4*>(chunk + W * 128 + (4 * gid + 2 * pos + jj) * 4) = make_uint4(f4[0], f4[1], f4[2], f4[3]);
       }
     } else {
       // The four channel pairs cp = 4q .. 4q+3 (adjacent lanes) fill the four bit positions of the same 16 words:
@@ -539,23 +703,24 @@ __device__ __forceinline__ void quantize_blocks(const Layout& L, const __half* _
           lo[2 * i + rh] = l << (2 * pos);
         }
       quad_reduce_scatter<4>(lo, pos, out);
-      if (valid) *reinterpret_cast<uint4*>(chunk + W * 128 + (4 * gid + pos) * 4) = make_uint4(out[0], out[1], out[2], out[3]);
+      if (valid_now) *reinterpret_cast<uint4*>(chunk + W * 128 + (4 * gid + pos) * 4) = make_uint4(out[0], out[1], out[2], out[3]);
       if constexpr (BITS == 3) {
         // 1-bit plane: the words of lane group gid hold the bits of both halves W of the channels, which two warps
         // of this chunk's 64 threads computed: the second hands its words to the first through shared memory
         uint4* hx = red_h + k4 * 32 + (cp & 31);
         quad_reduce_scatter<4>(hi, pos, out);
         const uint4 mine = make_uint4(out[0], out[1], out[2], out[3]);
+        pair_sync();                                        // the words before these have been read
         if (W == 1) *hx = mine;
-        __syncthreads();
-        if (W == 0 && valid) {
+        pair_sync();
+        if (W == 0 && valid_now) {
           const uint4 o = *hx;
           *reinterpret_cast<uint4*>(chunk + 256 + (4 * gid + pos) * 4) =
               make_uint4(mine.x | o.x, mine.y | o.y, mine.z | o.z, mine.w | o.w);
         }
       }
     }
-    if (k == 0 && valid) {
+    if (k == 0 && valid_now) {
       store_meta(group + S.meta_in_rec, block_meta_index(c0), S.meta_bytes, group_meta(p0, asym0));
       store_meta(group + S.meta_in_rec, block_meta_index(c0 + 1), S.meta_bytes, group_meta(p1, asym1));
     }

@@ -96,6 +96,30 @@ def test_prefill_edges(kb, vb, G, N, batch, heads, norm, variant, shift):
         K, V = np.ascontiguousarray(K[..., ::-1, :]), np.ascontiguousarray(V[..., ::-1, :])
 
 
+# Groups whose mode the quantisers' quick error sums cannot tell (both errors zero or equal: zero and constant runs, two
+# levels) among ordinary ones, with values from a pointer that is only 4-byte aligned (no windows, whose copies need 16).
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("G", [32, 64, 128])
+def test_prefill_groups_with_equal_errors(bits, G):
+    torch = _torch()
+    N, heads = 5 * 128, 3      # (no remainder: nothing of V in a window)
+    w = synth.tiny(n_tokens=N, group=G, k_bits=bits, v_bits=bits, batch=1, n_kv_heads=heads, n_q_heads=heads, w_sink=0, w_recent=0)
+    K, V = synth.kv_all(w)
+    for X in (K, V):
+        X[:, 0, 100:300] = 0
+        X[:, 1, :, 40:72] = 0
+        X[:, 2, 256:] = np.where(X[:, 2, 256:] > 0, np.float16(2), np.float16(-2))
+    V[:, 1, :, 5] = 1.5
+    oc = O.from_workload(w, max_tokens=N + 300)
+    oc.prefill(K, V)
+    gc = gpu_cache(w)
+    shifted = torch.empty(V.size + 8, dtype=torch.float16, device="cuda")
+    shifted[2:2 + V.size] = dev(V).reshape(-1)
+    for v in (dev(V), shifted[2:2 + V.size].view(V.shape)):
+        gc.innerq_quantize_prefill(dev(K), v)
+        P.assert_export_equal(gc.innerq_cache_export(), oc.export(), O.INNER, G, True, True)
+
+
 # The fp16 windows: fewer tokens than the sink holds, nothing but windows, windows of no, one and many tokens, and unit
 # counts at which a thread's next piece is units further on or less than a unit's pieces away.
 @pytest.mark.parametrize("grouping", [O.INNER, O.OUTER, O.FP16])
