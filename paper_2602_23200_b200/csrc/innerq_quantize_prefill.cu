@@ -16,6 +16,7 @@
 // half-precision pair) instruction occupies its pipe and the issue for two cycles, as two scalar ones do; it saves
 // instruction fetches and registers, not time.
 #include <algorithm>
+#include <atomic>
 #include <type_traits>
 
 #include "innerq_device.cuh"
@@ -274,10 +275,20 @@ template <int NH> __device__ __forceinline__ void quad_reduce_scatter(const uint
   }
 }
 
-// Key norm of one channel from the partial maxima [U][n_part][128]: sqrt(max |K|), 0 -> 1 (Section "Per-channel
-// Normalization of K").
-__device__ __forceinline__ float key_norm(const float* __restrict__ absmax, int n_part, int u, int c) {
-  const float* p = absmax + (size_t)u * n_part * kD + c;
+// How prefill_first_kernel divides the keys for their maxima: slices of 128 rows (per_unit of them), `ctas` CTAs with a
+// contiguous share each, which leave one row of 128 partial maxima per unit they meet, in that unit's `stride` rows.
+struct MaxShares {
+  int per_unit, ctas, stride;
+  __host__ __device__ int total(int U) const { return U * per_unit; }
+  __host__ __device__ int begin(int U, int cta) const { return (int)((long long)total(U) * cta / ctas); }
+  __host__ __device__ int cta_of(int U, int slice) const {      // whose share holds the slice
+    return (int)(((long long)(slice + 1) * ctas + total(U) - 1) / total(U)) - 1;
+  }
+};
+// Key norm of one channel from the partial maxima: sqrt(max |K|), 0 -> 1 (Section "Per-channel Normalization of K").
+__device__ __forceinline__ float key_norm(const float* __restrict__ absmax, const MaxShares& ms, int U, int u, int c) {
+  const float* p = absmax + (size_t)u * ms.stride * kD + c;
+  const int n_part = ms.cta_of(U, (u + 1) * ms.per_unit - 1) - ms.cta_of(U, u * ms.per_unit) + 1;
   float m = 0.f;
 #pragma unroll 8
   for (int i = 0; i < n_part; ++i) m = fmaxf(m, __ldcg(p + (size_t)i * kD));
@@ -299,12 +310,12 @@ __device__ __forceinline__ unsigned char* chunk_ptr(const Rec& rec, const Store&
 // (Through shared memory with an atomic OR per word instead: 22 more shared-memory operations per 32 values.)
 // CTA x of the grid takes the x-th part of all units' batches (a contiguous run, so every CTA ends at the same time
 // whatever the number of units), unit by unit.
-// NORM: the unit's key norm comes from `absmax`, n_part partial maxima per unit that prefill_first_kernel wrote; every
+// NORM: the unit's key norm comes from `absmax`, the partial maxima that prefill_first_kernel wrote; every
 // unit's norm is stored once.  The launch may start before that kernel has ended (griddepcontrol.wait).
 template <int BITS, bool NORM>
 __global__ void __launch_bounds__(128, kRowsCtasPerSm)
 quantize_rows_prefill_kernel(const __grid_constant__ Layout L, const __half* __restrict__ X, int N, int n_q,
-                             unsigned char* __restrict__ cache, const float* __restrict__ absmax, int n_part, float neg_zero) {
+                             unsigned char* __restrict__ cache, const float* __restrict__ absmax, const MaxShares ms, float neg_zero) {
   const Mul2 mul2(neg_zero);
   const Store& S = L.k;
   constexpr int RW = 4 * BITS;                // 32-bit words per packed row
@@ -316,7 +327,7 @@ quantize_rows_prefill_kernel(const __grid_constant__ Layout L, const __half* __r
   if constexpr (NORM) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     float* norm = reinterpret_cast<float*>(cache + L.norm_off);
-    for (int u = blockIdx.x; u < L.U; u += gridDim.x) norm[(size_t)u * kD + threadIdx.x] = key_norm(absmax, n_part, u, threadIdx.x);
+    for (int u = blockIdx.x; u < L.U; u += gridDim.x) norm[(size_t)u * kD + threadIdx.x] = key_norm(absmax, ms, L.U, u, threadIdx.x);
   }
   const int n_batches = (n_q + 7) >> 3;
   const long long total = (long long)L.U * n_batches;
@@ -329,7 +340,7 @@ quantize_rows_prefill_kernel(const __grid_constant__ Layout L, const __half* __r
     at = (long long)(u + 1) * n_batches;
     if constexpr (NORM) {
       __syncthreads();                          // the previous unit's norms are no longer read
-      inv_s[(threadIdx.x >> 5) * 36 + (threadIdx.x & 31)] = __fdiv_rn(1.0f, key_norm(absmax, n_part, u, threadIdx.x));
+      inv_s[(threadIdx.x >> 5) * 36 + (threadIdx.x & 31)] = __fdiv_rn(1.0f, key_norm(absmax, ms, L.U, u, threadIdx.x));
       __syncthreads();
     }
     const Rec rec = unit_rec(L, cache, u);
@@ -482,20 +493,88 @@ quantize_rows_prefill_kernel(const __grid_constant__ Layout L, const __half* __r
 // channels of one token.  The two channels are the two row halves of one MMA fragment row pair, and the pairs that
 // share words of the packed chunk are adjacent lanes, which exchange them and store 16 contiguous bytes each (3-bit:
 // the 1-bit plane's words are shared with the other channel half, a warp away).
-// CTA `part` of `n_parts` takes a contiguous run of all units' groups.
+// CTA `part` of `n_parts` takes a contiguous run of all units' groups, and between reading a step's values and working on
+// them a slice of the keys for their maxima (KeyMax).
 // A warp's 32 tokens x 64 channels come through its own 4 KB of shared memory, requested (cp.async) as soon as the values
 // before them are in registers: read straight from global memory the loads of a group were waited for with nothing else to
 // do, two thirds of the cycles without an instruction.
-constexpr int kBlocksRaw = 8 * 4096 / 16;               // uint4: values of 8 warps
-constexpr int kBlocksSmemWords = kBlocksRaw + 4 * 128 + 4 * 32;      // + statistics of 4 chunks, 1-bit plane words of 4 chunks
+constexpr int kStage = 8 * 4096 / 16;                   // uint4: a step's values, or a slice of keys, of 8 warps
+constexpr int kStats = 4 * 128 + 4 * 32;                // statistics of 4 chunks, 1-bit plane words of 4 chunks
+constexpr int kFirstSmem = (2 * kStage + kStats) * 16;  // bytes of prefill_first_kernel: values, keys, statistics
+
+// Maxima of |K| per channel over a CTA's share of the keys, a slice of 128 rows at a time: 16 lanes of 8 channels each, 16
+// rows per warp, through 4 KB of shared memory that nobody but the lane which requested a piece reads.
+struct KeyMax {
+  const __half* K;
+  float* out;
+  MaxShares ms;
+  int N, U, cta, at, end;
+  uint4* stage;
+  __half2 m[4];
+  __device__ __forceinline__ KeyMax(const __half* K_, float* out_, const MaxShares& s, int N_, int U_, int cta_, uint4* stage_)
+      : K(K_), out(out_), ms(s), N(N_), U(U_), cta(cta_), stage(stage_) {
+    at = end = 0;
+    if (cta < ms.ctas) { at = ms.begin(U, cta); end = ms.begin(U, cta + 1); }
+    clear();
+    if (at < end) request();
+  }
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) m[i] = __float2half2_rn(0.f);
+  }
+  __device__ __forceinline__ void request() const {
+    const int u = at / ms.per_unit, r0 = (at - u * ms.per_unit) * 128 + (threadIdx.x >> 5) * 16 + ((threadIdx.x >> 4) & 1);
+    const __half* src = K + (size_t)u * N * kD + (threadIdx.x & 15) * 8;
+    const uint32_t to = (uint32_t)__cvta_generic_to_shared(stage + (threadIdx.x >> 5) * 256 + (threadIdx.x & 31));
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + i * 512), "l"(src + (size_t)min(r0 + 2 * i, N - 1) * kD) : "memory");
+  }
+  // the slice that has arrived (cp.async.wait_all); requests the next one
+  __device__ __forceinline__ void take() {
+    if (at >= end) return;
+    const uint4* mine = stage + (threadIdx.x >> 5) * 256 + (threadIdx.x & 31);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const uint4 v = mine[i * 32];
+      const __half2* h = reinterpret_cast<const __half2*>(&v);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) m[k] = __hmax2(m[k], __habs2(h[k]));
+    }
+    const int u = at / ms.per_unit;
+    ++at;
+    if (at >= end || at == (u + 1) * ms.per_unit) flush(u);
+    if (at < end) request();
+  }
+  __device__ __forceinline__ void flush(int u) {        // the unit's maxima of this CTA: one row
+    float* red = reinterpret_cast<float*>(stage);       // [16][kD]
+    const int cg = threadIdx.x & 15, rg = threadIdx.x >> 4;
+    __syncthreads();                                    // everyone has taken the last slice
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      red[rg * kD + cg * 8 + 2 * i] = __low2float(m[i]);
+      red[rg * kD + cg * 8 + 2 * i + 1] = __high2float(m[i]);
+    }
+    __syncthreads();
+    if (threadIdx.x < kD) {
+      float v = 0.f;
+#pragma unroll
+      for (int i = 0; i < 16; ++i) v = fmaxf(v, red[i * kD + threadIdx.x]);
+      out[((size_t)u * ms.stride + cta - ms.cta_of(U, u * ms.per_unit)) * kD + threadIdx.x] = v;
+    }
+    __syncthreads();
+    clear();
+  }
+};
+
 template <int BITS>
 __device__ __forceinline__ void quantize_blocks(const Layout& L, const __half* __restrict__ X, int N, int n_q,
                                                 unsigned char* __restrict__ cache, int part, int n_parts, uint4* smem_q,
-                                                Mul2 mul2) {
+                                                KeyMax& keys, Mul2 mul2) {
   const Store& S = L.v;
   const int G = L.G, CH = G >> 5, sh = CH >> 1, per_cta = 4 >> sh, n_groups = n_q / G;
   const int tid = threadIdx.x, cp = tid & 63, k4 = tid >> 6, k = k4 & (CH - 1), c0 = 2 * cp;
-  uint4* stats = smem_q + kBlocksRaw;
+  uint4* stats = smem_q + 2 * kStage;
   float4* red_m = reinterpret_cast<float4*>(stats);                              // [4][64]: min, max of both channels
   float4* red_e = red_m + 4 * 64;                                                // [4][64]: error sums of both channels
   uint4* red_h = stats + 4 * 128;                                                // [4][32]: 1-bit plane words
@@ -516,7 +595,11 @@ __device__ __forceinline__ void quantize_blocks(const Layout& L, const __half* _
   };
   [[maybe_unused]] auto pair_sync = [&]() { asm volatile("barrier.sync %0, 64;" ::"r"(9 + k4) : "memory"); };
   const int items = L.U * n_groups, steps = (items + per_cta - 1) / per_cta;      // a group is 8 KB at least: 31 bits hold them
-  const int s_begin = (int)((long long)steps * part / n_parts), s_end = (int)((long long)steps * (part + 1) / n_parts);
+  int s_begin = 0, s_end = 0;
+  if (part >= 0 && part < n_parts) {
+    s_begin = (int)((long long)steps * part / n_parts);
+    s_end = (int)((long long)steps * (part + 1) / n_parts);
+  }
   int u = 0, j = 0;                                         // unit and group of this thread's item of the step
   bool valid = false;
   auto locate = [&](int step) {
@@ -532,12 +615,12 @@ __device__ __forceinline__ void quantize_blocks(const Layout& L, const __half* _
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const int p = i * 32 + lane;                        // 16-byte piece: token p / 8, channels 8 (p % 8) ..
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(mine_u32 + p * 16), "l"(src + (p >> 3) * kD + (p & 7) * 8));
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(mine_u32 + p * 16), "l"(src + (p >> 3) * kD + (p & 7) * 8) : "memory");
       }
     } else {
 #pragma unroll 4
       for (int i = 0; i < kSeg; ++i)
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(mine_u32 + (i * 32 + lane) * 4), "l"(src + i * kD + 2 * lane));
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(mine_u32 + (i * 32 + lane) * 4), "l"(src + i * kD + 2 * lane) : "memory");
     }
   };
   if (s_begin < s_end) {
@@ -559,6 +642,7 @@ __device__ __forceinline__ void quantize_blocks(const Layout& L, const __half* _
         locate(step + 1);
         request();
       }
+      keys.take();
 #pragma unroll
       for (int t = 0; t < kSeg; ++t) {
         const float2 v = __half22float2(*reinterpret_cast<const __half2*>(&raw[t]));
@@ -725,47 +809,13 @@ __device__ __forceinline__ void quantize_blocks(const Layout& L, const __half* _
       store_meta(group + S.meta_in_rec, block_meta_index(c0 + 1), S.meta_bytes, group_meta(p1, asym1));
     }
   }
-}
-
-// ------------------------------------------------------------------ key maxima, windows, counts
-// Part `part` of n_part of unit u's rows: maxima of |K| per channel, kept as floats.  One CTA of 256 threads: 16 lanes
-// of 8 channels each, 16 rows at a time.
-__device__ __forceinline__ void key_absmax_part(const __half* __restrict__ K, int N, int u, int part, int n_part,
-                                                float* __restrict__ out, float* red) {
-  const int t0 = (int)((long long)N * part / n_part), t1 = (int)((long long)N * (part + 1) / n_part);
-  const int cg = threadIdx.x & 15, rg = threadIdx.x >> 4;
-  const uint4* base = reinterpret_cast<const uint4*>(K + (size_t)u * N * kD) + cg;
-  __half2 m[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) m[i] = __float2half2_rn(0.f);
-  auto take = [&](const uint4& v) {
-    const __half2* h = reinterpret_cast<const __half2*>(&v);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) m[i] = __hmax2(m[i], __habs2(h[i]));
-  };
-  int t = t0 + rg;
-  for (; t + 16 * 7 < t1; t += 16 * 8) {      // eight rows per thread in flight
-    uint4 v[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = __ldg(base + (size_t)(t + 16 * i) * 16);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) take(v[i]);
-  }
-  for (; t < t1; t += 16) take(__ldg(base + (size_t)t * 16));
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    red[rg * kD + cg * 8 + 2 * i] = __low2float(m[i]);
-    red[rg * kD + cg * 8 + 2 * i + 1] = __high2float(m[i]);
-  }
-  __syncthreads();
-  if (threadIdx.x < kD) {
-    float v = 0.f;
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v = fmaxf(v, red[i * kD + threadIdx.x]);
-    out[((size_t)u * n_part + part) * kD + threadIdx.x] = v;
+  while (keys.at < keys.end) {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    keys.take();
   }
 }
 
+// ------------------------------------------------------------------ windows, counts
 // The fp16 windows of both tensors and the counts that the decode kernel compares with its own N (see append_publish), and
 // the norms (1) unless the key quantiser computes them.  CTA `part` of `n_parts`, 256 threads.  Bound by memory latency in
 // this kernel's two CTAs per SM: kCopies 16-byte pieces are in flight per thread, and stepping from piece to piece takes no
@@ -818,31 +868,24 @@ __device__ __forceinline__ void copy_windows(const Layout& L, const Counts& cn, 
   }
 }
 
-// First of the two launches of an inner-grouped prefill: everything that does not need the key norms.  Roles [0, n_max)
-// take the key maxima (n_part per unit), the next n_val the value groups, the rest the windows.  The first two are dealt
-// to alternate CTAs: the maxima wait for memory while the value groups beside them on the SM compute (32 units x 32768
-// tokens, 2 bits, G = 128: 164 us; one role after the other 177 us; as two launches 43 + 134 us).  A prompt of a few
-// hundred tokens is bound by its launches, not by its kernels: ten of them (clear, maxima, norms, two quantisers, four
-// window copies, counts) took 38.9 us for 512 tokens of 8 heads (3 bits, symmetric; calls through the binding, one after
-// the other), the two take 10.2 us.
+// First of the two launches of an inner-grouped prefill: everything that does not need the key norms.  CTAs [0, ms.ctas)
+// take the key maxima, CTAs [v0, v0 + n_val) the value groups, CTAs [w0, w0 + n_win) the windows.  A prompt that fills the
+// GPU gives all CTAs of one wave a share of all three: the maxima's keys arrive while the value groups are worked on, every
+// load but a CTA's first is requested a step ahead (32 units x 16384 tokens, 2 bits, G = 128: 78 us as CTAs of several
+// roles, four waves of them).  A short one spreads the roles over CTAs of their own; it is bound by its launches, not by its
+// kernels: ten of them (clear, maxima, norms, two quantisers, four window copies, counts) took 38.9 us for 512 tokens of 8
+// heads (3 bits, symmetric; calls through the binding, one after the other), the two take 10.2 us.
 template <int VBITS>
 __global__ void __launch_bounds__(256, 2)
 prefill_first_kernel(const __grid_constant__ Layout L, const Counts cn, const __half* __restrict__ K,
-                     const __half* __restrict__ V, unsigned char* __restrict__ cache, float* __restrict__ absmax, int n_part,
-                     int n_max, int n_val, float neg_zero) {
-  __shared__ uint4 smem[kBlocksSmemWords];
-  static_assert(sizeof(smem) >= 16 * kD * sizeof(float), "the maxima's reduction fits");
+                     const __half* __restrict__ V, unsigned char* __restrict__ cache, float* __restrict__ absmax,
+                     const MaxShares ms, int v0, int n_val, int w0, int n_win, float neg_zero) {
+  extern __shared__ uint4 first_smem[];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  int b = blockIdx.x;
-  const int pairs = n_max < n_val ? n_max : n_val;
-  if (b < 2 * pairs) b = (b & 1) ? n_max + (b >> 1) : b >> 1;
-  else if (b < n_max + n_val) b = n_max > n_val ? b - pairs : n_max + (b - n_max);
-  if (b < n_max)
-    key_absmax_part(K, cn.N, b / n_part, b % n_part, n_part, absmax, reinterpret_cast<float*>(smem));
-  else if (b < n_max + n_val)
-    quantize_blocks<VBITS>(L, V, cn.N, cn.n_qv, cache, b - n_max, n_val, smem, Mul2(neg_zero));
-  else
-    copy_windows(L, cn, K, V, cache, n_max == 0, b - n_max - n_val, gridDim.x - n_max - n_val);
+  const int b = blockIdx.x;
+  KeyMax keys(K, absmax, ms, cn.N, L.U, b, first_smem + kStage);
+  if (b >= w0 && b < w0 + n_win) copy_windows(L, cn, K, V, cache, ms.ctas == 0, b - w0, n_win);
+  quantize_blocks<VBITS>(L, V, cn.N, cn.n_qv, cache, b - v0, n_val, first_smem, keys, Mul2(neg_zero));
 }
 
 // The same for a cache that has nothing else to do here: empty, unquantised (everything goes to the sink array) or
@@ -877,8 +920,8 @@ int window_ctas(const Layout& L, const Counts& cn) {      // about four 16-byte 
 }
 
 template <int KBITS>
-int launch_rows(const Layout& L, const Counts& cn, const __half* K, unsigned char* cache, const float* absmax, int n_part,
-                cudaStream_t st) {
+int launch_rows(const Layout& L, const Counts& cn, const __half* K, unsigned char* cache, const float* absmax,
+                const MaxShares& ms, cudaStream_t st) {
   // one wave of CTAs, each with at least two batches of 8 rows per warp; with norms at least one CTA (it stores them)
   const long long batches = (long long)L.U * ((cn.n_qk + 7) / 8);
   if (batches == 0 && !absmax) return 0;
@@ -890,8 +933,8 @@ int launch_rows(const Layout& L, const Counts& cn, const __half* K, unsigned cha
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = absmax ? 1 : 0;
   const cudaError_t e =
-      absmax ? cudaLaunchKernelEx(&cfg, quantize_rows_prefill_kernel<KBITS, true>, L, K, cn.N, cn.n_qk, cache, absmax, n_part, -0.f)
-             : cudaLaunchKernelEx(&cfg, quantize_rows_prefill_kernel<KBITS, false>, L, K, cn.N, cn.n_qk, cache, absmax, n_part, -0.f);
+      absmax ? cudaLaunchKernelEx(&cfg, quantize_rows_prefill_kernel<KBITS, true>, L, K, cn.N, cn.n_qk, cache, absmax, ms, -0.f)
+             : cudaLaunchKernelEx(&cfg, quantize_rows_prefill_kernel<KBITS, false>, L, K, cn.N, cn.n_qk, cache, absmax, ms, -0.f);
   return e == cudaSuccess ? 1 : -1;
 }
 
@@ -907,20 +950,37 @@ int launch_prefill_windows(const Layout& L, const Counts& cn, unsigned char* cac
 int launch_prefill_inner(const Layout& L, const Counts& cn, unsigned char* cache, unsigned char* ws, const __half* K,
                          const __half* V, cudaStream_t st) {
   float* absmax = L.k_normalize ? reinterpret_cast<float*>(ws + L.ws_partial_off) : nullptr;
-  // key maxima: about four CTAs per SM, at least 64 rows each; their results go where the decode keeps its split
-  // partials, which has max_splits rows of more than 128 floats per unit
+  // key maxima: their results go where the decode keeps its split partials, max_splits rows of more than 128 floats per unit
   static_assert(kPartialStride >= kD, "a row of partial maxima fits a split partial");
-  const int n_part = absmax ? clamp_int((cn.N + 63) / 64, 1, clamp_int((4 * 148 + L.U - 1) / L.U, 1, L.max_splits)) : 0;
-  const int n_max = n_part * L.U;
+  const int wave = 2 * 148;
+  MaxShares ms = {(cn.N + 127) / 128, 0, 0};
+  // a unit meets at most ceil(ctas / U) + 1 CTAs
+  if (absmax) ms.ctas = clamp_int(std::min<long long>((long long)L.U * ms.per_unit, (long long)L.U * (L.max_splits - 1)), 1, wave);
+  ms.stride = (ms.ctas + L.U - 1) / L.U + 1;
   const long long steps = cn.n_qv > 0 ? ((long long)L.U * (cn.n_qv / L.G) * (L.G / kChunk) + 3) / 4 : 0;
-  const int n_val = clamp_int(steps, 0, 148 * 8);
-  const int grid = n_max + n_val + window_ctas(L, cn);
-  auto first = L.v.bits == 2 ? prefill_first_kernel<2> : L.v.bits == 3 ? prefill_first_kernel<3> : prefill_first_kernel<4>;
-  first<<<grid, 256, 0, st>>>(L, cn, K, V, cache, absmax, n_part, n_max, n_val, -0.f);
+  int v0 = 0, n_val = clamp_int(steps, 0, wave), w0 = 0, n_win = window_ctas(L, cn), grid;
+  if (std::min(ms.ctas, n_val) + n_win <= wave && ms.ctas + n_val + n_win <= 2 * wave && std::max(ms.ctas, n_val) < wave) {
+    v0 = ms.ctas;                             // roles apart
+    w0 = v0 + n_val;
+    grid = w0 + n_win;
+  } else {
+    if (n_win > wave) w0 = std::max(ms.ctas, n_val);      // long windows: CTAs of their own
+    else n_win = std::max(ms.ctas, n_val);
+    grid = std::max(std::max(ms.ctas, n_val), w0 + n_win);
+  }
+  auto go = [&](auto kernel, std::atomic<unsigned long long>& configured) {
+    if (!opt_in_dynamic_smem(kernel, kFirstSmem, configured)) return false;
+    kernel<<<grid, 256, kFirstSmem, st>>>(L, cn, K, V, cache, absmax, ms, v0, n_val, w0, n_win, -0.f);
+    return true;
+  };
+  static std::atomic<unsigned long long> configured[3];
+  if (!(L.v.bits == 2   ? go(prefill_first_kernel<2>, configured[0])
+        : L.v.bits == 3 ? go(prefill_first_kernel<3>, configured[1])
+                        : go(prefill_first_kernel<4>, configured[2]))) return -1;
   if (cudaGetLastError() != cudaSuccess) return -1;
-  const int rows = L.k.bits == 2   ? launch_rows<2>(L, cn, K, cache, absmax, n_part, st)
-                   : L.k.bits == 3 ? launch_rows<3>(L, cn, K, cache, absmax, n_part, st)
-                                   : launch_rows<4>(L, cn, K, cache, absmax, n_part, st);
+  const int rows = L.k.bits == 2   ? launch_rows<2>(L, cn, K, cache, absmax, ms, st)
+                   : L.k.bits == 3 ? launch_rows<3>(L, cn, K, cache, absmax, ms, st)
+                                   : launch_rows<4>(L, cn, K, cache, absmax, ms, st);
   return rows < 0 ? -1 : 1 + rows;
 }
 
