@@ -56,6 +56,21 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
   return d;
 }
 
+// ---- distributed shared memory of a cluster of CTAs
+__device__ __forceinline__ void cluster_arrive_wait() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t own, uint32_t rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(own), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ float ld_cluster(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+  return v;
+}
+
 constexpr int kMagicS = 0x4B400000;          // bits of 1.5 * 2^23: signed sums |S| < 2^22
 constexpr float kMagicSf = 12582912.0f;
 constexpr int kMagicU = 0x4B000000;          // bits of 2^23: unsigned sums S < 2^23
@@ -1080,8 +1095,6 @@ __device__ __forceinline__ void decode_i8_body(const Layout& L, const Counts& cn
       for (int m = 0; m < 8; ++m) { out_acc[m][0] *= up; out_acc[m][1] *= up; }
     }
 
-    // the partials and tickets written below are also shared with the previous decode
-    dep_wait();
     if (failed) {
       // a copy never arrived: flag it for the host and contribute nothing
       if (lane == 0) atomicExch(reinterpret_cast<unsigned int*>(a.ws + L.ws_ticket_off) + L.U, 1u);
@@ -1124,6 +1137,11 @@ __device__ __forceinline__ void decode_i8_body(const Layout& L, const Counts& cn
     __syncthreads();
     const int prow0 = at_end().x, nh_end = at_end().y;
     float* partials = a.partials;
+    float* mine_part = wres + (size_t)kWarps * kHeads * (kD + 2);      // a.cluster: [head][kD + 2], read by the cluster
+    // The partials and tickets in global memory, and the result, are shared with the previous decode.  Everything up to
+    // here is done while that may still be running: in a chain of calls of the same cache the wait is the start of what
+    // each call adds (8 KV heads x 1001 tokens, r 4: 6.0 us a call with the wait before the combine).
+    if (!a.cluster) dep_wait();
     for (int i = tid; i < nh_end * kD; i += kThreads) {
       const int h = i >> 7, c = i & (kD - 1);
       float M = -INFINITY;
@@ -1137,15 +1155,55 @@ __device__ __forceinline__ void decode_i8_body(const Layout& L, const Counts& cn
         num = fmaf(r_[c], wgt, num);
         den = fmaf(r_[kD + 1], wgt, den);
       }
-      float* P = partials + ((size_t)(prow0 + h) * a.part_stride + split) * kPartialStride;
+      float* P = a.cluster ? mine_part + h * (kD + 2) : partials + ((size_t)(prow0 + h) * a.part_stride + split) * kPartialStride;
       P[c] = num;
       if (c == 0) { P[kD] = M; P[kD + 1] = den; }
     }
   }
 
+  const int4 end = at_end();
+  if (a.cluster) {
+    // ---------------- cross-CTA merge in the cluster: every CTA reads a share of all parts ---------------
+    const uint32_t part0 = smem_u32(reinterpret_cast<float*>(smem) + (size_t)kWarps * kHeads * (kD + 2));
+    cluster_arrive_wait();         // all parts are written
+    dep_wait();
+    for (int i = split * kThreads + tid; i < end.y * kD; i += n_parts * kThreads) {
+      const int h = i >> 7, c = i & (kD - 1);
+      float M = -INFINITY, num = 0.f, den = 0.f;
+#pragma unroll 1
+      for (int p0 = 0; p0 < n_parts; p0 += 8) {
+        float m[8], l[8], v[8], m_new = M;
+#pragma unroll
+        for (int p = 0; p < 8; ++p) {
+          m[p] = -INFINITY;
+          l[p] = v[p] = 0.f;
+          if (p0 + p < n_parts) {
+            const uint32_t P = cluster_addr(part0 + (uint32_t)(h * (kD + 2) * 4), p0 + p);
+            v[p] = ld_cluster(P + 4 * c);
+            m[p] = ld_cluster(P + 4 * kD);
+            l[p] = ld_cluster(P + 4 * kD + 4);
+          }
+        }
+#pragma unroll
+        for (int p = 0; p < 8; ++p) m_new = fmaxf(m_new, m[p]);
+        const float alpha = M == -INFINITY ? 0.f : ex2_approx(M - m_new);
+        M = m_new;
+        num *= alpha;
+        den *= alpha;
+#pragma unroll
+        for (int p = 0; p < 8; ++p) {
+          const float wgt = m[p] == -INFINITY ? 0.f : ex2_approx(m[p] - M);
+          num = fmaf(v[p], wgt, num);
+          den = fmaf(l[p], wgt, den);
+        }
+      }
+      a.out[(size_t)q_row_of(u, end.w, h) * kD + c] = __float2half_rn(num / den);
+    }
+    cluster_arrive_wait();         // nobody leaves while its part is being read
+    return;
+  }
   // ---------------- cross-CTA merge: the last CTA of the unit to arrive combines all parts -----------
   __shared__ unsigned int s_ticket;
-  const int4 end = at_end();
   __syncthreads();                 // all partial writes of this CTA happen-before thread 0's ticket below
   if (tid == 0) {
     // release: publishes the whole CTA's partial (ordered before this thread by the barrier) with the ticket;
@@ -1196,20 +1254,22 @@ int launch_i8_one_p(const Layout& L, const Counts& cn, DecodeArgs a, int n_split
   constexpr int kSmem = SL::kCtaBytes;
   constexpr int RU = SL::kCH;
   static std::atomic<unsigned long long> configured{0};
-  if (!opt_in_dynamic_smem(decode_i8_kernel<KB, VB, G, KM, VM, SPLIT, CPI, PAGED>, kSmem, configured)) return -1;
+  if (!opt_in_dynamic_smem(decode_i8_kernel<KB, VB, G, KM, VM, SPLIT, CPI, PAGED>, kSmem, configured, true)) return -1;
   // a paged cache whose page list fits the parameter space: the kernel that takes the table as a parameter
   [[maybe_unused]] PageIds ids;
   bool table_in_params = false;
   if constexpr (PAGED) {
     static std::atomic<unsigned long long> configured_p{0};
     if (a.pages_host && a.n_pages_host <= kParamPages) {
-      if (!opt_in_dynamic_smem(decode_i8_paged_kernel<KB, VB, G, KM, VM, SPLIT, CPI>, kSmem, configured_p)) return -1;
+      if (!opt_in_dynamic_smem(decode_i8_paged_kernel<KB, VB, G, KM, VM, SPLIT, CPI>, kSmem, configured_p, true)) return -1;
       for (int i = 0; i < a.n_pages_host; ++i) ids.id[i] = a.pages_host[i];
       table_in_params = true;
     }
   }
   const int grid_y = fill_split_args(L, cn, a, RU, false, n_splits, 0);
   fill_reference_args(cn, a, RU, CPI, false);
+  const bool cluster = merges_in_cluster(L.U * a.passes, grid_y);
+  a.cluster = cluster;
   int launches = 0;
   const int rows = L.r * a.n_q, step = SPLIT ? 1 : kHeads, per = a.passes;
   for (int h0 = 0; h0 < rows; h0 += step * per) {
@@ -1219,10 +1279,13 @@ int launch_i8_one_p(const Layout& L, const Counts& cn, DecodeArgs a, int n_split
     // launched as a programmatic dependent of whatever precedes it in the stream (see the kernel's dep_wait)
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid; cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kSmem; cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = attr[1].val.clusterDim.z = 1;
+    attr[1].val.clusterDim.y = grid_y;
+    cfg.attrs = attr; cfg.numAttrs = cluster ? 2 : 1;
     cudaError_t err;
     if constexpr (PAGED) {
       if (a.ablation) return -2;      // the timing instances exist for contiguous caches only
@@ -1232,10 +1295,10 @@ int launch_i8_one_p(const Layout& L, const Counts& cn, DecodeArgs a, int n_split
 #ifdef IQ_WITH_TIMING_INSTANCES      // defined by the translation units of the formats the latency study and the bench time
       static std::atomic<unsigned long long> configured_a1{0}, configured_a2{0};
       if (a.ablation == 1) {
-        if (!opt_in_dynamic_smem(decode_i8_kernel<KB, VB, G, KM, VM, SPLIT, CPI, false, 1>, kSmem, configured_a1)) return -1;
+        if (!opt_in_dynamic_smem(decode_i8_kernel<KB, VB, G, KM, VM, SPLIT, CPI, false, 1>, kSmem, configured_a1, true)) return -1;
         err = cudaLaunchKernelEx(&cfg, decode_i8_kernel<KB, VB, G, KM, VM, SPLIT, CPI, false, 1>, L, cn, a);
       } else {
-        if (!opt_in_dynamic_smem(decode_i8_kernel<KB, VB, G, KM, VM, SPLIT, CPI, false, 2>, kSmem, configured_a2)) return -1;
+        if (!opt_in_dynamic_smem(decode_i8_kernel<KB, VB, G, KM, VM, SPLIT, CPI, false, 2>, kSmem, configured_a2, true)) return -1;
         err = cudaLaunchKernelEx(&cfg, decode_i8_kernel<KB, VB, G, KM, VM, SPLIT, CPI, false, 2>, L, cn, a);
       }
 #else
@@ -1257,7 +1320,7 @@ int launch_i8_batched_p(const Layout& L, SeqTable& T, int n_seqs, int n_splits, 
   constexpr int kSmem = SL::kCtaBytes;
   constexpr int RU = SL::kCH;
   static std::atomic<unsigned long long> configured{0};
-  if (!opt_in_dynamic_smem(decode_i8_batched_kernel<KB, VB, G, KM, VM, SPLIT, CPI, PAGED>, kSmem, configured)) return -1;
+  if (!opt_in_dynamic_smem(decode_i8_batched_kernel<KB, VB, G, KM, VM, SPLIT, CPI, PAGED>, kSmem, configured, true)) return -1;
   long long chunks[kMaxSeqs], longest = 1;
   for (int i = 0; i < n_seqs; ++i) {
     chunks[i] = T.s[i].cn.n_qv / kChunk;
@@ -1282,6 +1345,8 @@ int launch_i8_batched_p(const Layout& L, SeqTable& T, int n_seqs, int n_splits, 
     const int gy = fill_split_args(L, T.s[i].cn, T.s[i].a, RU, false, want, 0);
     if (gy > grid_y) grid_y = gy;
   }
+  const bool cluster = merges_in_cluster(n_seqs * L.U, grid_y);
+  for (int i = 0; i < n_seqs; ++i) T.s[i].a.cluster = cluster;
   int launches = 0;
   const dim3 grid(n_seqs * L.U, grid_y);
   const int step = SPLIT ? 1 : kHeads;
@@ -1289,10 +1354,13 @@ int launch_i8_batched_p(const Layout& L, SeqTable& T, int n_seqs, int n_splits, 
     for (int i = 0; i < n_seqs; ++i) T.s[i].a.head0 = h0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid; cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kSmem; cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = attr[1].val.clusterDim.z = 1;
+    attr[1].val.clusterDim.y = grid_y;
+    cfg.attrs = attr; cfg.numAttrs = cluster ? 2 : 1;
     if (cudaLaunchKernelEx(&cfg, decode_i8_batched_kernel<KB, VB, G, KM, VM, SPLIT, CPI, PAGED>, L, T) != cudaSuccess) return -1;
     ++launches;
   }

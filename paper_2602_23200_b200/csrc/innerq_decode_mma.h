@@ -25,6 +25,8 @@ struct DecodeArgs : SplitArgs {
                          // unpack + MMA work of the streaming loop (scores are taken as 0), bit 1 the value side's
   float* partials;       // split partials [rows][part_stride][kPartialStride]: row = global query head (n_q == 1) or
                          // (unit, pass) * 4 + column of the launch (n_q > 1)
+  int cluster;           // the CTAs of a (unit, pass) are a cluster (merges_in_cluster) and merge through distributed shared
+                         // memory; 0: through split partials in global memory and the unit's ticket
   // HOST side only (paged caches): the cache's page list, which the launcher copies into the kernel's parameter
   // space when it fits (PageIds), so that no copy of a CTA waits for a look-up in the table in device memory
   const uint32_t* pages_host;

@@ -13,12 +13,14 @@ namespace iq {
 // More than 48 KB of dynamic shared memory is an opt-in per kernel AND per device: `done` (one per kernel, a bit per
 // device ordinal) remembers where it has been set, so a process that drives several GPUs sets it on each of them.
 template <typename Kernel>
-inline bool opt_in_dynamic_smem(Kernel kernel, int bytes, std::atomic<unsigned long long>& done) {
+inline bool opt_in_dynamic_smem(Kernel kernel, int bytes, std::atomic<unsigned long long>& done, bool clusters = false) {
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
   const unsigned long long bit = 1ull << dev;
   if (done.load(std::memory_order_acquire) & bit) return true;
   if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return false;
+  // clusters of more than the portable 8 CTAs
+  if (clusters && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
   done.fetch_or(bit, std::memory_order_release);
   return true;
 }

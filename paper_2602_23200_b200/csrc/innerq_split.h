@@ -34,6 +34,16 @@ struct SplitArgs {
                          // fill_reference_args
 };
 
+// Whether the CTAs of a unit (and group) are a cluster that merges through distributed shared memory instead of through
+// global memory and a ticket.  That saves three dependent trips to L2 at the end of a launch (8 KV heads x 1001 tokens, r 4,
+// 3-bit keys: 13.3 -> 11.2 us alone, 6.0 -> 4.2 us in a chain), but a cluster starts only when all its CTAs find room in one
+// GPC: a launch that fills the slots then overlaps its neighbours less (32 units x 8 CTAs, 8192 tokens: 9.2 -> 10.6 us in a
+// chain).  So: launches of one CTA per SM at most; 16 CTAs are the most a cluster can have.
+constexpr int kClusterCtas = 16;
+inline bool merges_in_cluster(int n_clusters, int grid_y) {
+  return grid_y <= kClusterCtas && n_clusters * grid_y <= kCtaSlots / 2;
+}
+
 // Partial slots per query head: token-range splits (two waves of CTAs for all units, 64 at most) plus one per 32 tokens of
 // the fp16 tail.
 inline int max_splits_for(int n_units, int w_sink, int w_recent, int G) {
