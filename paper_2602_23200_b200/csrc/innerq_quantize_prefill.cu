@@ -280,9 +280,10 @@ template <int NH> __device__ __forceinline__ void quad_reduce_scatter(const uint
 struct MaxShares {
   int per_unit, ctas, stride;
   __host__ __device__ int total(int U) const { return U * per_unit; }
-  __host__ __device__ int begin(int U, int cta) const { return (int)((long long)total(U) * cta / ctas); }
+  // (products of a slice and a CTA stay below 2^32: a slice is 32 KB of keys)
+  __host__ __device__ int begin(int U, int cta) const { return (int)((uint32_t)total(U) * (uint32_t)cta / (uint32_t)ctas); }
   __host__ __device__ int cta_of(int U, int slice) const {      // whose share holds the slice
-    return (int)(((long long)(slice + 1) * ctas + total(U) - 1) / total(U)) - 1;
+    return (int)(((uint32_t)(slice + 1) * (uint32_t)ctas + (uint32_t)total(U) - 1u) / (uint32_t)total(U)) - 1;
   }
 };
 // Key norm of one channel from the partial maxima: sqrt(max |K|), 0 -> 1 (Section "Per-channel Normalization of K").
@@ -324,6 +325,7 @@ quantize_rows_prefill_kernel(const __grid_constant__ Layout L, const __half* __r
   const int gl = L.G >> 5, sh = gl >> 1;      // lanes per group: 1, 2 or 4, and its logarithm
   // reciprocal key norms: segment rows padded to 36 words, so that the four lanes of a token read different banks
   __shared__ __align__(16) float inv_s[NORM ? 4 * 36 : 4];
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");      // whatever follows waits before it touches anything
   if constexpr (NORM) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     float* norm = reinterpret_cast<float*>(cache + L.norm_off);
@@ -882,6 +884,9 @@ prefill_first_kernel(const __grid_constant__ Layout L, const Counts cn, const __
                      const MaxShares ms, int v0, int n_val, int w0, int n_win, float neg_zero) {
   extern __shared__ uint4 first_smem[];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // a programmatic dependent of whatever comes before it, for its launch to overlap that kernel's end; keys and values may be
+  // that kernel's results, and the cache and workspace what it reads
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int b = blockIdx.x;
   KeyMax keys(K, absmax, ms, cn.N, L.U, b, first_smem + kStage);
   if (b >= w0 && b < w0 + n_win) copy_windows(L, cn, K, V, cache, ms.ctas == 0, b - w0, n_win);
@@ -922,11 +927,11 @@ int window_ctas(const Layout& L, const Counts& cn) {      // about four 16-byte 
 template <int KBITS>
 int launch_rows(const Layout& L, const Counts& cn, const __half* K, unsigned char* cache, const float* absmax,
                 const MaxShares& ms, cudaStream_t st) {
-  // one wave of CTAs, each with at least two batches of 8 rows per warp; with norms at least one CTA (it stores them)
+  // one wave of CTAs, each with at least one batch of 8 rows per warp; with norms at least one CTA (it stores them)
   const long long batches = (long long)L.U * ((cn.n_qk + 7) / 8);
   if (batches == 0 && !absmax) return 0;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(clamp_int((batches + 7) / 8, absmax ? (L.U < 148 ? L.U : 148) : 1, 148 * kRowsCtasPerSm));
+  cfg.gridDim = dim3(clamp_int((batches + 3) / 4, absmax ? (L.U < 148 ? L.U : 148) : 1, 148 * kRowsCtasPerSm));
   cfg.blockDim = dim3(128); cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // see prefill_first_kernel
@@ -970,8 +975,13 @@ int launch_prefill_inner(const Layout& L, const Counts& cn, unsigned char* cache
   }
   auto go = [&](auto kernel, std::atomic<unsigned long long>& configured) {
     if (!opt_in_dynamic_smem(kernel, kFirstSmem, configured)) return false;
-    kernel<<<grid, 256, kFirstSmem, st>>>(L, cn, K, V, cache, absmax, ms, v0, n_val, w0, n_win, -0.f);
-    return true;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(256); cfg.dynamicSmemBytes = kFirstSmem; cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, L, cn, K, V, cache, absmax, ms, v0, n_val, w0, n_win, -0.f) == cudaSuccess;
   };
   static std::atomic<unsigned long long> configured[3];
   if (!(L.v.bits == 2   ? go(prefill_first_kernel<2>, configured[0])
