@@ -320,6 +320,19 @@ __device__ void quantize_block_quarter(const TokSrc& src, const __half* __restri
   }
 }
 
+// Grid row 1 .. 4 of an append that packs a group of value tokens: a quarter of the group's channels.
+__device__ __forceinline__ void append_quarter(const Layout& L, const __half* __restrict__ xv, int N, int u,
+                                               unsigned char* __restrict__ cache, __half* tile, uint32_t* words, int n_parts) {
+  const Store& R = L.v;
+  const int nq_before = n_quantised(kBlock, N - 1, L.w_sink, L.w_recent, L.G);
+  const __half* ring = reinterpret_cast<const __half*>(cache + R.ring_off + (size_t)u * R.ring_stride);
+  TokSrc src{ring, R.ring_cap, L.w_sink};
+  quantize_block_quarter(src, xv, N - 1, L.w_sink + nq_before, L, R, tile, words,
+                         reinterpret_cast<float*>(words + (L.G / kChunk) * 512), unit_rec(L, cache, u), nq_before / L.G,
+                         blockIdx.y - 1);
+  append_publish(L, N, u, cache, n_parts);
+}
+
 // Programmatic dependent launch: the decode that follows may start while this kernel runs (it streams what this
 // kernel cannot write and waits for this kernel's completion before it touches the rest).  This kernel in turn
 // waits for the kernels before it, either before its first global access or, with late_wait (the host knows that
@@ -343,14 +356,7 @@ __global__ void __launch_bounds__(128) append_kernel(Layout L, const __half* __r
   if (blockIdx.y == 0) {
     append_unit(L, k_new + (size_t)u * kD, v_new + (size_t)u * kD, N, u, cache, tile, words, n_parts > 1, n_parts);
   } else {
-    const Store& R = L.v;
-    const int nq_before = n_quantised(kBlock, N - 1, L.w_sink, L.w_recent, L.G);
-    const __half* ring = reinterpret_cast<const __half*>(cache + R.ring_off + (size_t)u * R.ring_stride);
-    TokSrc src{ring, R.ring_cap, L.w_sink};
-    quantize_block_quarter(src, v_new + (size_t)u * kD, N - 1, L.w_sink + nq_before, L, R, tile, words,
-                           reinterpret_cast<float*>(words + (L.G / kChunk) * 512), unit_rec(L, cache, u), nq_before / L.G,
-                           blockIdx.y - 1);
-    append_publish(L, N, u, cache, n_parts);
+    append_quarter(L, v_new + (size_t)u * kD, N, u, cache, tile, words, n_parts);
   }
   // one CTA keeps the kernel alive until its predecessor has ended (the chain of completions); the others leave
   if (late_wait && u == 0 && blockIdx.y == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -362,6 +368,7 @@ struct AppendSeq {
   unsigned char* cache;
   int N;           // token count after this append
   int late_wait;   // as for append_kernel
+  int packs;       // this step packs a group of its value tokens: on the grid's rows 1 .. 4 (see append_kernel)
 };
 struct AppendTable {
   AppendSeq s[kMaxSeqs];
@@ -375,10 +382,17 @@ __global__ void __launch_bounds__(128) append_batched_kernel(const __grid_consta
   uint32_t* words = reinterpret_cast<uint32_t*>(append_smem + (size_t)L.G * kD * 2);
   const int seq = blockIdx.x / L.U, u = blockIdx.x - seq * L.U;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int late_wait = T.s[seq].late_wait;
+  const AppendSeq& e = T.s[seq];
+  const int late_wait = e.late_wait;
+  if (blockIdx.y > 0 && !e.packs) return;
   if (!late_wait) asm volatile("griddepcontrol.wait;" ::: "memory");
-  append_unit(L, k_new + (size_t)blockIdx.x * kD, v_new + (size_t)blockIdx.x * kD, T.s[seq].N, u, T.s[seq].cache, tile, words);
-  if (late_wait) asm volatile("griddepcontrol.wait;" ::: "memory");
+  const __half* xv = v_new + (size_t)blockIdx.x * kD;
+  if (blockIdx.y == 0) {
+    append_unit(L, k_new + (size_t)blockIdx.x * kD, xv, e.N, u, e.cache, tile, words, e.packs, e.packs ? 5 : 1);
+    if (late_wait) asm volatile("griddepcontrol.wait;" ::: "memory");
+  } else {
+    append_quarter(L, xv, e.N, u, e.cache, tile, words, 5);
+  }
 }
 
 // ------------------------------------------------------------------ canonical export
@@ -529,14 +543,16 @@ static size_t append_smem_bytes(const Layout& L) {
   return (size_t)L.G * kD * 2 + (size_t)(L.G / kChunk) * 512 * 4 + 4 * 32 * 2 * 4;      // + the quarters' reduction words
 }
 
+static bool packs_v_group(const Layout& L, int N_after) {
+  return L.v.kind == kBlock && L.v.code_kind == kBlock && N_after - 1 >= L.w_sink &&
+         n_quantised(kBlock, N_after, L.w_sink, L.w_recent, L.G) != n_quantised(kBlock, N_after - 1, L.w_sink, L.w_recent, L.G);
+}
+
 int launch_append(const Layout& L, unsigned char* cache, const __half* k_new, const __half* v_new, int N_after,
                   cudaStream_t st, int late_wait) {
   cudaLaunchConfig_t cfg = {};
   // the step on which a chunk-coded group of G value tokens is packed gets four more CTAs per unit (see append_kernel)
-  const bool v_group = L.v.kind == kBlock && L.v.code_kind == kBlock && N_after - 1 >= L.w_sink &&
-                       n_quantised(kBlock, N_after, L.w_sink, L.w_recent, L.G) !=
-                           n_quantised(kBlock, N_after - 1, L.w_sink, L.w_recent, L.G);
-  cfg.gridDim = dim3(L.U, v_group ? 5 : 1); cfg.blockDim = dim3(128); cfg.dynamicSmemBytes = append_smem_bytes(L); cfg.stream = st;
+  cfg.gridDim = dim3(L.U, packs_v_group(L, N_after) ? 5 : 1); cfg.blockDim = dim3(128); cfg.dynamicSmemBytes = append_smem_bytes(L); cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -548,13 +564,16 @@ int launch_append_batched(const Layout& L, int n, unsigned char* const* caches, 
                           const __half* k_new, const __half* v_new, cudaStream_t st) {
   if (n < 1 || n > kMaxSeqs) return -1;
   AppendTable T;
+  bool any_packs = false;
   for (int i = 0; i < kMaxSeqs; ++i) {
     T.s[i].cache = caches[i < n ? i : 0];
     T.s[i].N = Ns_after[i < n ? i : 0];
     T.s[i].late_wait = late_wait[i < n ? i : 0];
+    T.s[i].packs = packs_v_group(L, T.s[i].N);
+    any_packs = any_packs || T.s[i].packs;
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(n * L.U); cfg.blockDim = dim3(128); cfg.dynamicSmemBytes = append_smem_bytes(L); cfg.stream = st;
+  cfg.gridDim = dim3(n * L.U, any_packs ? 5 : 1); cfg.blockDim = dim3(128); cfg.dynamicSmemBytes = append_smem_bytes(L); cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
