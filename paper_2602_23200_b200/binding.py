@@ -196,9 +196,8 @@ def _dev_ptr(t, name: str, shape, device=None) -> int:
 
 
 class _Fast:
-    """The same two checks for the calls of a decode step, which a model makes per layer and token: at 30 layers the
-    general forms above cost more host time (4-5 us a call of 12) than the kernels take on short contexts.  One look-up per
-    property, in the order that lets a valid tensor through with the fewest; whatever does not pass (a subclass among it)
+    """The same two checks for the calls of a decode step that the extension module (csrc/innerq_step.cpp) has not taken.
+    One look-up per property, in the order that lets a valid tensor through with the fewest; whatever does not pass (a subclass among it)
     goes to the general form, which raises (or accepts) it.  Nothing is remembered from call to call."""
     ready = False
 
@@ -214,6 +213,10 @@ class _Fast:
                 setattr(cls, attr, staticmethod(getattr(torch._C, name)))
         global _ptr_of
         _ptr_of = cls._make_ptr_of(torch.Tensor, torch.float16)
+        from . import _step
+        cls.steps = _step.Steps
+        cls.entries = [C.cast(getattr(lib(), f), C.c_void_p).value for f in
+                       ("innerq_append_token", "innerq_decode_attention", "innerq_quantize_prefill", "innerq_decode_step_host")]
         cls.ready = True
 
     @staticmethod
@@ -308,6 +311,8 @@ class InnerQCache:
         self._out_like = self._ws_buf[:2 * cfg.batch * cfg.n_q_heads * cfg.head_dim].view(torch.float16).view(self._q_shape)
         if not _Fast.ready:
             _Fast.load()
+        # the calls of a step from the current stream, with their checks in native code; None once the handle is gone
+        self._steps = _Fast.steps(h.value, self.device.index, self._kv_shape, self._q_shape, *_Fast.entries)
 
     # ---- paged caches
     def innerq_cache_pages_for(self, n_tokens: int) -> int:
@@ -342,7 +347,7 @@ class InnerQCache:
             self.pool.give_back(self.innerq_cache_release_pages())
 
     def close(self):
-        h, self._h = getattr(self, "_h", None), None
+        h, self._h, self._steps = getattr(self, "_h", None), None, None
         if h and _lib is not None:
             _lib.innerq_cache_destroy(h)
 
@@ -361,6 +366,10 @@ class InnerQCache:
         return self.cfg.batch * self.cfg.n_kv_heads
 
     def innerq_quantize_prefill(self, k, v, stream=None):
+        if stream is None and self._steps is not None:
+            st = self._steps.prefill(k, v)
+            if st <= 0:
+                return _check(st, "innerq_quantize_prefill") if st else None
         batch, heads, dim = self._kv_shape
         n = int(k.shape[2]) if k.dim() == 4 else -1
         shape = (batch, heads, n, dim)
@@ -370,6 +379,10 @@ class InnerQCache:
             _check(st, "innerq_quantize_prefill")
 
     def innerq_append_token(self, k_new, v_new, stream=None):
+        if stream is None and self._steps is not None:
+            st = self._steps.append(k_new, v_new)
+            if st <= 0:
+                return _check(st, "innerq_append_token") if st else None
         device = self.device
         st = _lib.innerq_append_token(self._h, _ptr_of(k_new, "k_new", self._kv_shape, device),
                                       _ptr_of(v_new, "v_new", self._kv_shape, device), _stream_of(stream, device))
@@ -377,6 +390,12 @@ class InnerQCache:
             _check(st, "innerq_append_token")
 
     def innerq_decode_attention(self, q, out=None, stream=None):
+        if stream is None and self._steps is not None:
+            st = self._steps.decode(q, out)
+            if type(st) is not int:
+                return st                      # the result
+            if st < 0:
+                _check(st, "innerq_decode_attention")
         device = self.device
         q_ptr = _ptr_of(q, "q", self._q_shape, device)
         if out is None:
@@ -439,6 +458,10 @@ class InnerQCache:
         """One step (append + decode) from pinned host tensors into a pinned host tensor; enqueues only, the
         caller synchronises the stream before reading `out_host`.  The device staging buffer the C call needs
         is a torch allocation made here on first use."""
+        if stream is None and self._steps is not None and getattr(self, "_staging", None) is not None:
+            st = self._steps.step_host(k_new_host, v_new_host, q_host, out_host, self._staging.data_ptr())
+            if st <= 0:
+                return _check(st, "innerq_decode_step_host") if st else None
         import torch
         c, kv_shape, q_shape = self.cfg, self._kv_shape, self._q_shape
         for t, name, shape in ((k_new_host, "k_new_host", kv_shape), (v_new_host, "v_new_host", kv_shape),

@@ -1,4 +1,5 @@
-"""Builds libinnerq.so (sm_100a) next to this file with nvcc.  Usable as `python -m paper_2602_23200_b200.build`."""
+"""Builds libinnerq.so (sm_100a) next to this file with nvcc, and the extension module _step.so (the host side of a step's
+calls, against torch's headers) with g++.  Usable as `python -m paper_2602_23200_b200.build`."""
 from __future__ import annotations
 
 import os
@@ -8,6 +9,7 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libinnerq.so")
+STEP = os.path.join(HERE, "_step.so")
 # every .cu of csrc/: the C ABI, the quantise kernels, the decode kernels (the fused kernel one file per packed format)
 SOURCES = sorted(f for f in os.listdir(CSRC) if f.endswith(".cu"))
 ARCH = ["-gencode", "arch=compute_100a,code=sm_100a"]
@@ -18,11 +20,27 @@ def _stale() -> bool:
     if not os.path.exists(LIB):
         return True
     t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(HERE, "..", "include", "innerq.h"), __file__]
+    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if not f.endswith((".o", ".cpp"))] + [os.path.join(HERE, "..", "include", "innerq.h"), __file__]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def build_step(force: bool = False) -> str:
+    import sysconfig
+
+    import torch
+    src, t = os.path.join(CSRC, "innerq_step.cpp"), os.path.dirname(torch.__file__)
+    if not force and os.path.exists(STEP) and os.path.getmtime(STEP) >= max(os.path.getmtime(src), os.path.getmtime(__file__)):
+        return STEP
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", "-I" + sysconfig.get_paths()["include"],
+           "-I/usr/local/cuda/include", "-isystem", os.path.join(t, "include"), src, "-o", STEP,
+           "-L" + os.path.join(t, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+    subprocess.run(cmd, check=True)
+    return STEP
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
+    build_step(force)
     if not force and not _stale():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")

@@ -62,6 +62,51 @@ CASES = [
 ]
 
 
+# The merge of the splits: in a cluster (up to 16 CTAs a unit, 148 together; eight parts a round) and through tickets.
+@pytest.mark.parametrize("heads,r,kb,vb,G,N,splits", [
+    (1, 4, 2, 2, 32, 4700, (1, 2, 7, 8, 9, 15, 16, 17)), (1, 1, 2, 2, 32, 4700, (2, 8, 9, 16, 17)),
+    (2, 8, 3, 4, 64, 2400, (1, 3, 8)), (37, 1, 4, 4, 32, 1500, (4, 5)), (37, 2, 4, 2, 32, 1500, (4, 5)),
+])
+def test_merge_of_splits(heads, r, kb, vb, G, N, splits):
+    w = synth.tiny(n_tokens=N, group=G, k_bits=kb, v_bits=vb, batch=1, n_kv_heads=heads, n_q_heads=heads * r)
+    oc, gc, _, _ = run_prefill_both(w)
+    check_decode(w, oc, gc, splits=(0,) + splits)
+
+
+# What the extension module does not take goes to the binding's general forms: a subclass, a stream that is given, tensors
+# that are refused, a cache that has been closed.
+def test_step_calls_outside_the_extension():
+    torch = _torch()
+    w = synth.tiny(n_tokens=200)
+    _, gc, _, _ = run_prefill_both(w)
+    q = dev(synth.query(w, 0))
+    ref = gc.innerq_decode_attention(q)
+    assert torch.equal(gc.innerq_decode_attention(torch.nn.Parameter(q, requires_grad=False)), ref)
+    assert torch.equal(gc.innerq_decode_attention(q, stream=torch.cuda.current_stream()), ref)
+    out = torch.empty_like(ref)
+    assert gc.innerq_decode_attention(q, out) is out and torch.equal(out, ref)
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        other = gc.innerq_decode_attention(q)
+    torch.cuda.synchronize()
+    assert torch.equal(other, ref)
+    k = torch.zeros((w.batch, w.n_kv_heads, 128), dtype=torch.float16, device="cuda")
+    for bad, err in ((q.float(), TypeError), (q.cpu(), TypeError), (q[:, :, ::2], TypeError), (q[:1], ValueError), (None, TypeError)):
+        with pytest.raises(err):
+            gc.innerq_decode_attention(bad)
+    for bad, err in ((k.float(), TypeError), (k[:, :1], (TypeError, ValueError)), (3, TypeError)):
+        with pytest.raises(err):
+            gc.innerq_append_token(k, bad)
+    with pytest.raises(ValueError):
+        gc.innerq_quantize_prefill(torch.zeros((w.batch, w.n_kv_heads + 1, 8, 128), dtype=torch.float16, device="cuda"), k)
+    gc.close()
+    with pytest.raises(Exception):
+        gc.innerq_decode_attention(q)
+    with pytest.raises(Exception):
+        gc.innerq_append_token(k, k)
+
+
 @pytest.mark.parametrize("bits,G,mode,variant,N", CASES)
 def test_prefill_and_decode_inner(bits, G, mode, variant, N):
     w = synth.tiny(n_tokens=N, group=G, k_bits=bits, v_bits=bits, k_mode=mode, v_mode=mode, sym_variant=variant)
