@@ -56,21 +56,6 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
   return d;
 }
 
-// ---- distributed shared memory of a cluster of CTAs
-__device__ __forceinline__ void cluster_arrive_wait() {
-  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-}
-__device__ __forceinline__ uint32_t cluster_addr(uint32_t own, uint32_t rank) {
-  uint32_t r;
-  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(own), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ float ld_cluster(uint32_t addr) {
-  float v;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
-  return v;
-}
-
 constexpr int kMagicS = 0x4B400000;          // bits of 1.5 * 2^23: signed sums |S| < 2^22
 constexpr float kMagicSf = 12582912.0f;
 constexpr int kMagicU = 0x4B000000;          // bits of 2^23: unsigned sums S < 2^23
@@ -1163,42 +1148,11 @@ __device__ __forceinline__ void decode_i8_body(const Layout& L, const Counts& cn
 
   const int4 end = at_end();
   if (a.cluster) {
-    // ---------------- cross-CTA merge in the cluster: every CTA reads a share of all parts ---------------
-    const uint32_t part0 = smem_u32(reinterpret_cast<float*>(smem) + (size_t)kWarps * kHeads * (kD + 2));
+    // ---------------- cross-CTA merge in the cluster ----------------
     cluster_arrive_wait();         // all parts are written
     dep_wait();
-    for (int i = split * kThreads + tid; i < end.y * kD; i += n_parts * kThreads) {
-      const int h = i >> 7, c = i & (kD - 1);
-      float M = -INFINITY, num = 0.f, den = 0.f;
-#pragma unroll 1
-      for (int p0 = 0; p0 < n_parts; p0 += 8) {
-        float m[8], l[8], v[8], m_new = M;
-#pragma unroll
-        for (int p = 0; p < 8; ++p) {
-          m[p] = -INFINITY;
-          l[p] = v[p] = 0.f;
-          if (p0 + p < n_parts) {
-            const uint32_t P = cluster_addr(part0 + (uint32_t)(h * (kD + 2) * 4), p0 + p);
-            v[p] = ld_cluster(P + 4 * c);
-            m[p] = ld_cluster(P + 4 * kD);
-            l[p] = ld_cluster(P + 4 * kD + 4);
-          }
-        }
-#pragma unroll
-        for (int p = 0; p < 8; ++p) m_new = fmaxf(m_new, m[p]);
-        const float alpha = M == -INFINITY ? 0.f : ex2_approx(M - m_new);
-        M = m_new;
-        num *= alpha;
-        den *= alpha;
-#pragma unroll
-        for (int p = 0; p < 8; ++p) {
-          const float wgt = m[p] == -INFINITY ? 0.f : ex2_approx(m[p] - M);
-          num = fmaf(v[p], wgt, num);
-          den = fmaf(l[p], wgt, den);
-        }
-      }
-      a.out[(size_t)q_row_of(u, end.w, h) * kD + c] = __float2half_rn(num / den);
-    }
+    merge_in_cluster(reinterpret_cast<float*>(smem) + (size_t)kWarps * kHeads * (kD + 2), a.out, end.y, n_parts, split,
+                     make_int4(q_row_of(u, end.w, 0), q_row_of(u, end.w, 1), q_row_of(u, end.w, 2), q_row_of(u, end.w, 3)));
     cluster_arrive_wait();         // nobody leaves while its part is being read
     return;
   }

@@ -256,6 +256,60 @@ __device__ __noinline__ void merge_parts(const float* __restrict__ partials, flo
   }
 }
 
+// ---- distributed shared memory of a cluster of CTAs
+__device__ __forceinline__ void cluster_arrive_wait() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t own, uint32_t rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(own), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ float ld_cluster(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+  return v;
+}
+
+// The same merge when the CTAs of the unit are a cluster: parts in their shared memory ([head][kD + 2] at `part`, the same
+// address in every CTA), this CTA (rank `split`) makes its share of the outputs.  Eight parts per round of loads.
+__device__ __noinline__ void merge_in_cluster(const float* part, __half* __restrict__ out, int nh, int n_parts, int split, int4 orow) {
+  const uint32_t part0 = smem_u32(part);
+  for (int i = split * kThreads + threadIdx.x; i < nh * kD; i += n_parts * kThreads) {
+    const int h = i >> 7, c = i & (kD - 1);
+    float M = -INFINITY, num = 0.f, den = 0.f;
+#pragma unroll 1
+    for (int p0 = 0; p0 < n_parts; p0 += 8) {
+      float m[8], l[8], v[8], m_new = M;
+#pragma unroll
+      for (int p = 0; p < 8; ++p) {
+        m[p] = -INFINITY;
+        l[p] = v[p] = 0.f;
+        if (p0 + p < n_parts) {
+          const uint32_t P = cluster_addr(part0 + (uint32_t)(h * (kD + 2) * 4), p0 + p);
+          v[p] = ld_cluster(P + 4 * c);
+          m[p] = ld_cluster(P + 4 * kD);
+          l[p] = ld_cluster(P + 4 * kD + 4);
+        }
+      }
+#pragma unroll
+      for (int p = 0; p < 8; ++p) m_new = fmaxf(m_new, m[p]);
+      const float alpha = M == -INFINITY ? 0.f : ex2_approx(M - m_new);
+      M = m_new;
+      num *= alpha;
+      den *= alpha;
+#pragma unroll
+      for (int p = 0; p < 8; ++p) {
+        const float wgt = m[p] == -INFINITY ? 0.f : ex2_approx(m[p] - M);
+        num = fmaf(v[p], wgt, num);
+        den = fmaf(l[p], wgt, den);
+      }
+    }
+    const int row = h == 0 ? orow.x : h == 1 ? orow.y : h == 2 ? orow.z : orow.w;
+    out[(size_t)row * kD + c] = __float2half_rn(num / den);
+  }
+}
+
 // ---- the kernel -------------------------------------------------------------------------------------
 // CPI = chunks (of 32 tokens) a warp processes per loop iteration: one barrier wait, one soft-max update and
 // one refill per iteration, and CPI*2 independent key accumulator chains in flight.
@@ -1235,8 +1289,6 @@ __device__ __forceinline__ void decode_mma_body(const Layout& L, const Counts& c
         }
     }
 
-    // the partials and tickets written below are also shared with the previous decode
-    dep_wait();
     if (failed) {
       // a copy never arrived: flag it for the host and contribute nothing
       if (lane == 0) atomicExch(reinterpret_cast<unsigned int*>(a.ws + L.ws_ticket_off) + L.U, 1u);
@@ -1296,6 +1348,9 @@ __device__ __forceinline__ void decode_mma_body(const Layout& L, const Counts& c
     __syncthreads();
     const int prow0 = s_end.x, nh_end = s_end.w;
     float* partials = a.partials;
+    float* mine_part = wres + (size_t)kWarps * kHeads * (kD + 2);      // a.cluster: [head][kD + 2], read by the cluster
+    // what is in global memory is shared with the previous decode
+    if (!a.cluster) dep_wait();
     for (int i = tid; i < nh_end * kD; i += kThreads) {
       const int h = i >> 7, c = i & (kD - 1);
       float M = -INFINITY;
@@ -1309,15 +1364,23 @@ __device__ __forceinline__ void decode_mma_body(const Layout& L, const Counts& c
         num = fmaf(r_[c], wgt, num);
         den = fmaf(r_[kD + 1], wgt, den);
       }
-      float* P = partials + ((size_t)(prow0 + h) * a.part_stride + split) * kPartialStride;
+      float* P = a.cluster ? mine_part + h * (kD + 2) : partials + ((size_t)(prow0 + h) * a.part_stride + split) * kPartialStride;
       P[c] = num;
       if (c == 0) { P[kD] = M; P[kD + 1] = den; }
     }
   }
 
+  const int4 end = s_end;
+  if (a.cluster) {
+    // ---------------- cross-CTA merge in the cluster ----------------
+    cluster_arrive_wait();         // all parts are written
+    dep_wait();
+    merge_in_cluster(reinterpret_cast<float*>(smem) + (size_t)kWarps * kHeads * (kD + 2), a.out, end.w, n_parts, split, s_rows);
+    cluster_arrive_wait();         // nobody leaves while its part is being read
+    return;
+  }
   // ---------------- cross-CTA merge: the last CTA of the unit to arrive combines all parts -----------
   __shared__ unsigned int s_ticket;
-  const int4 end = s_end;
   __syncthreads();                 // all partial writes of this CTA happen-before thread 0's ticket below
   if (tid == 0) {
     // release: publishes the whole CTA's partial (ordered before this thread by the barrier) with the ticket;
@@ -1366,18 +1429,20 @@ int launch_one_p(const Layout& L, const Counts& cn, DecodeArgs a, int grid_y, cu
   using SL = StageLayout<KB, VB, G, KM, VM, CPI>;
   constexpr int kSmem = SL::kCtaBytes;
   static std::atomic<unsigned long long> configured{0};
-  if (!opt_in_dynamic_smem(decode_mma_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, PAGED, 0, RENEW>, kSmem, configured)) return -1;
+  if (!opt_in_dynamic_smem(decode_mma_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, PAGED, 0, RENEW>, kSmem, configured, true)) return -1;
   // a paged cache whose page list fits the parameter space: the kernel that takes the table as a parameter
   [[maybe_unused]] PageIds ids;
   bool table_in_params = false;
   if constexpr (PAGED) {
     static std::atomic<unsigned long long> configured_p{0};
     if (a.pages_host && a.n_pages_host <= kParamPages) {
-      if (!opt_in_dynamic_smem(decode_mma_paged_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, RENEW>, kSmem, configured_p)) return -1;
+      if (!opt_in_dynamic_smem(decode_mma_paged_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, RENEW>, kSmem, configured_p, true)) return -1;
       for (int i = 0; i < a.n_pages_host; ++i) ids.id[i] = a.pages_host[i];
       table_in_params = true;
     }
   }
+  const bool cluster = merges_in_cluster(L.U * a.passes, grid_y);
+  a.cluster = cluster;
   int launches = 0;
   const int rows = L.r * a.n_q, step = SPLIT ? 1 : kHeads, per = a.passes;
   for (int h0 = 0; h0 < rows; h0 += step * per) {
@@ -1388,10 +1453,13 @@ int launch_one_p(const Layout& L, const Counts& cn, DecodeArgs a, int grid_y, cu
     // kernel's tail, its first global access waits for it (grid_dependency_wait)
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid; cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kSmem; cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = attr[1].val.clusterDim.z = 1;
+    attr[1].val.clusterDim.y = grid_y;
+    cfg.attrs = attr; cfg.numAttrs = cluster ? 2 : 1;
     cudaError_t err;
     if constexpr (PAGED) {
       if (a.ablation) return -2;      // the timing instances exist for contiguous caches only
@@ -1401,10 +1469,10 @@ int launch_one_p(const Layout& L, const Counts& cn, DecodeArgs a, int grid_y, cu
 #ifdef IQ_WITH_TIMING_INSTANCES      // defined by the translation units of the formats the latency study times
       static std::atomic<unsigned long long> configured_a1{0}, configured_a2{0};
       if (a.ablation == 1) {
-        if (!opt_in_dynamic_smem(decode_mma_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, false, 1>, kSmem, configured_a1)) return -1;
+        if (!opt_in_dynamic_smem(decode_mma_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, false, 1>, kSmem, configured_a1, true)) return -1;
         err = cudaLaunchKernelEx(&cfg, decode_mma_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, false, 1>, L, cn, a);
       } else {
-        if (!opt_in_dynamic_smem(decode_mma_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, false, 2>, kSmem, configured_a2)) return -1;
+        if (!opt_in_dynamic_smem(decode_mma_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, false, 2>, kSmem, configured_a2, true)) return -1;
         err = cudaLaunchKernelEx(&cfg, decode_mma_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, false, 2>, L, cn, a);
       }
 #else
@@ -1427,7 +1495,7 @@ int launch_one_batched_p(const Layout& L, SeqTable& T, int n_seqs, int n_splits,
   constexpr int kSmem = SL::kCtaBytes;
   constexpr int RU = SL::kCH;
   static std::atomic<unsigned long long> configured{0};
-  if (!opt_in_dynamic_smem(decode_mma_batched_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, PAGED>, kSmem, configured)) return -1;
+  if (!opt_in_dynamic_smem(decode_mma_batched_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, PAGED>, kSmem, configured, true)) return -1;
   // Grid rows per sequence: the fewest chunks per row T such that all sequences together, each cut into rows of at
   // most T chunks, need no more than n_splits rows in total (so the longest row, which sets the time, is as short
   // as one wave of CTAs allows, and short sequences hold few CTAs).
@@ -1455,6 +1523,8 @@ int launch_one_batched_p(const Layout& L, SeqTable& T, int n_seqs, int n_splits,
     const int gy = fill_split_args(L, T.s[i].cn, T.s[i].a, RU, OUTER, want, 0);
     if (gy > grid_y) grid_y = gy;
   }
+  const bool cluster = merges_in_cluster(n_seqs * L.U, grid_y);
+  for (int i = 0; i < n_seqs; ++i) T.s[i].a.cluster = cluster;
   int launches = 0;
   const dim3 grid(n_seqs * L.U, grid_y);
   const int step = SPLIT ? 1 : kHeads;
@@ -1462,10 +1532,13 @@ int launch_one_batched_p(const Layout& L, SeqTable& T, int n_seqs, int n_splits,
     for (int i = 0; i < n_seqs; ++i) T.s[i].a.head0 = h0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid; cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kSmem; cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = attr[1].val.clusterDim.z = 1;
+    attr[1].val.clusterDim.y = grid_y;
+    cfg.attrs = attr; cfg.numAttrs = cluster ? 2 : 1;
     if (cudaLaunchKernelEx(&cfg, decode_mma_batched_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, PAGED>, L, T) != cudaSuccess) return -1;
     ++launches;
   }

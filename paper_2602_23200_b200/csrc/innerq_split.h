@@ -37,11 +37,12 @@ struct SplitArgs {
 // Whether the CTAs of a unit (and group) are a cluster that merges through distributed shared memory instead of through
 // global memory and a ticket.  That saves three dependent trips to L2 at the end of a launch (8 KV heads x 1001 tokens, r 4,
 // 3-bit keys: 13.3 -> 11.2 us alone, 6.0 -> 4.2 us in a chain), but a cluster starts only when all its CTAs find room in one
-// GPC: a launch that fills the slots then overlaps its neighbours less (32 units x 8 CTAs, 8192 tokens: 9.2 -> 10.6 us in a
-// chain).  So: launches of one CTA per SM at most; 16 CTAs are the most a cluster can have.
+// GPC: a launch that fills the slots then overlaps its neighbours less (64 units x 4 CTAs, 8192 tokens, 4 bits: 25.4 -> 23.5
+// us alone, 15.3 -> 16.7 in a chain).  So: launches of one CTA per SM at most, with the 16 CTAs that a cluster can have, and
+// pairs, for which one SM's two slots will do (128 units x 8192 tokens, 4 bits: 39.9 -> 36.9 us alone, 26.3 -> 26.0).
 constexpr int kClusterCtas = 16;
 inline bool merges_in_cluster(int n_clusters, int grid_y) {
-  return grid_y <= kClusterCtas && n_clusters * grid_y <= kCtaSlots / 2;
+  return grid_y <= kClusterCtas && n_clusters * grid_y <= (grid_y == 2 ? kCtaSlots : kCtaSlots / 2);
 }
 
 // Partial slots per query head: token-range splits (two waves of CTAs for all units, 64 at most) plus one per 32 tokens of

@@ -62,10 +62,11 @@ CASES = [
 ]
 
 
-# The merge of the splits: in a cluster (up to 16 CTAs a unit, 148 together; eight parts a round) and through tickets.
+# The merge of the splits: in a cluster (up to 16 CTAs a unit, 148 together, or pairs; eight parts a round) and through tickets.
 @pytest.mark.parametrize("heads,r,kb,vb,G,N,splits", [
     (1, 4, 2, 2, 32, 4700, (1, 2, 7, 8, 9, 15, 16, 17)), (1, 1, 2, 2, 32, 4700, (2, 8, 9, 16, 17)),
     (2, 8, 3, 4, 64, 2400, (1, 3, 8)), (37, 1, 4, 4, 32, 1500, (4, 5)), (37, 2, 4, 2, 32, 1500, (4, 5)),
+    (100, 1, 2, 2, 64, 1400, (2, 3)),      # pairs of CTAs that fill the GPU
 ])
 def test_merge_of_splits(heads, r, kb, vb, G, N, splits):
     w = synth.tiny(n_tokens=N, group=G, k_bits=kb, v_bits=vb, batch=1, n_kv_heads=heads, n_q_heads=heads * r)
