@@ -160,6 +160,9 @@ int innerq_cache_n_tokens(const innerq_cache_t* cache);
  * not fill a group stay fp16 in front of the recent window.  0 <= n_tokens <= max_tokens.
  * Uses the workspace (partial maxima of the keys, where a decode keeps its split partials): like two decodes, a prefill
  * and another call on the same workspace must not overlap.
+ * Its kernels let programmatic dependents start early: a kernel of the caller's that is launched as one has to wait
+ * (griddepcontrol.wait) before it reads what a prefill writes; kernels launched in the ordinary way, copies and the calls
+ * of this library need nothing.
  * Errors: INVALID_ARG, CAPACITY, CUDA. */
 int innerq_quantize_prefill(innerq_cache_t* cache, const void* k, const void* v, int32_t n_tokens,
                             void* cuda_stream);

@@ -1152,7 +1152,7 @@ __device__ __forceinline__ void decode_i8_body(const Layout& L, const Counts& cn
     cluster_arrive_wait();         // all parts are written
     dep_wait();
     merge_in_cluster(reinterpret_cast<float*>(smem) + (size_t)kWarps * kHeads * (kD + 2), a.out, end.y, n_parts, split,
-                     make_int4(q_row_of(u, end.w, 0), q_row_of(u, end.w, 1), q_row_of(u, end.w, 2), q_row_of(u, end.w, 3)));
+                     [&](int h) { return q_row_of(u, end.w, h); });
     cluster_arrive_wait();         // nobody leaves while its part is being read
     return;
   }
