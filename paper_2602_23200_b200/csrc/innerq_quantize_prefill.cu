@@ -214,7 +214,10 @@ template <int BITS> struct QuickErr {
 };
 
 // How far a group's difference of the quick sums and that of PairCoder's can be apart; infinite where the quick sums mean
-// nothing (NaN where the values are not finite: no comparison with it settles anything).  m = largest |x| of the group.
+// nothing (infinite or NaN also where a value is infinite: no comparison with it settles anything).  A NaN shows in neither
+// scale nor bound, and 3- and 4-bit sums count it as 0: groups with one get PairCoder's sums, whose NaN makes them symmetric
+// as in the append (see has_nan: the maximum that propagates NaN costs what the other one does).  m = largest |x| of the
+// group.
 // 2 bits: a value's rounding errors are below 2^-20 m in each form, those of adding up 32 of them in two chains below
 // 2^-20 m a value; a value beyond the outer symmetric level (whose fp16 scale may be rounded down) counts with the wrong
 // sign.  3, 4 bits: in units of 2^-16 scales a value is off by 1 (complement), 1/2 (constant), 1/2 (rounding) and 1/8
@@ -240,6 +243,12 @@ __device__ __forceinline__ float min3(float a, float b, float c) {
 __device__ __forceinline__ float max3(float a, float b, float c) {
   float r;
   asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+// the same, but a NaN among the three is the result
+__device__ __forceinline__ float max3_nan(float a, float b, float c) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
   return r;
 }
 // low bytes of four code words as the four bytes of one word
@@ -381,11 +390,19 @@ quantize_rows_prefill_kernel(const __grid_constant__ Layout L, const __half* __r
       float mn, mx;                             // three-input min / max: two values per instruction
       {
         const float2 v = unf2(x[0]);
-        mn = fminf(v.x, v.y); mx = fmaxf(v.x, v.y);
+        mn = fminf(v.x, v.y); mx = max3_nan(v.x, v.x, v.y);
 #pragma unroll
         for (int e = 1; e < kSeg / 2; ++e) {
           const float2 w = unf2(x[e]);
-          mn = min3(mn, w.x, w.y); mx = max3(mx, w.x, w.y);
+          mn = min3(mn, w.x, w.y); mx = max3_nan(mx, w.x, w.y);
+        }
+      }
+      const bool has_nan = __any_sync(0xffffffffu, mx != mx);
+      if (has_nan) {                            // the group's largest number
+#pragma unroll
+        for (int e = 0; e < kSeg / 2; ++e) {
+          const float2 w = unf2(x[e]);
+          mx = max3(mx, w.x, w.y);
         }
       }
       for (int o = 1; o < gl; o <<= 1) {
@@ -407,7 +424,7 @@ quantize_rows_prefill_kernel(const __grid_constant__ Layout L, const __half* __r
           quick = quick_mode(d, quick_bound<BITS>(p, bd, mn, mx, L.G));      // the same in all lanes of a group
         }
         asym = quick > 0;
-        if (__any_sync(0xffffffffu, quick < 0)) {
+        if (__any_sync(0xffffffffu, quick < 0) || has_nan) {
           const PairCoder pc(mul2, p, bd, p, bd);
           float2 ea = make_float2(0.f, 0.f), es = make_float2(0.f, 0.f);
           auto sums = [&](auto clamp) {
@@ -655,13 +672,21 @@ __device__ __forceinline__ void quantize_blocks(const Layout& L, const __half* _
     {
       const float2 v = unf2(x[1]);
       mn.x = fminf(mn.x, v.x); mn.y = fminf(mn.y, v.y);
-      mx.x = fmaxf(mx.x, v.x); mx.y = fmaxf(mx.y, v.y);
+      mx.x = max3_nan(mx.x, mx.x, v.x); mx.y = max3_nan(mx.y, mx.y, v.y);
     }
 #pragma unroll
     for (int t = 2; t < kSeg; t += 2) {
       const float2 v = unf2(x[t]), w = unf2(x[t + 1]);
       mn.x = min3(mn.x, v.x, w.x); mn.y = min3(mn.y, v.y, w.y);
-      mx.x = max3(mx.x, v.x, w.x); mx.y = max3(mx.y, v.y, w.y);
+      mx.x = max3_nan(mx.x, v.x, w.x); mx.y = max3_nan(mx.y, v.y, w.y);
+    }
+    const bool has_nan = __any_sync(0xffffffffu, mx.x != mx.x || mx.y != mx.y);
+    if (has_nan) {                                           // the largest numbers
+#pragma unroll
+      for (int t = 0; t < kSeg; ++t) {
+        const float2 v = unf2(x[t]);
+        mx.x = fmaxf(mx.x, v.x); mx.y = fmaxf(mx.y, v.y);
+      }
     }
     if (CH > 1) {
       group_sync();                                          // the previous group's words are no longer read
@@ -698,7 +723,7 @@ __device__ __forceinline__ void quantize_blocks(const Layout& L, const __half* _
         const int quick1 = quick_mode(d.y, quick_bound<BITS>(p1, b1, mn.y, mx.y, G));
         asym0 = quick0 > 0;
         asym1 = quick1 > 0;
-        close = quick0 < 0 || quick1 < 0;
+        close = quick0 < 0 || quick1 < 0 || has_nan;
       }
       if (CH > 1 ? group_or(close) : (bool)__any_sync(0xffffffffu, close)) {
         const PairCoder pc(mul2, p0, b0, p1, b1);

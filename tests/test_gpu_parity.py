@@ -166,6 +166,35 @@ def test_prefill_groups_with_equal_errors(bits, G):
         P.assert_export_equal(gc.innerq_cache_export(), oc.export(), O.INNER, G, True, True)
 
 
+# A group with a NaN or an infinity among values of one sign (which alone would be asymmetric): no sum tells its mode, it is
+# symmetric, whether a prompt or an append packs it.
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("G", [32, 64, 128])
+def test_prefill_and_append_agree_on_groups_that_are_not_finite(bits, G):
+    N = 4 * 128
+    w = synth.tiny(n_tokens=N + 16, group=G, k_bits=bits, v_bits=bits, batch=1, n_kv_heads=2, n_q_heads=2, w_sink=0, w_recent=16,
+                   k_normalize=0)
+    rng = np.random.default_rng(bits * G)
+    K, V = (rng.uniform(5, 7, (1, 2, N + 16, 128)).astype(np.float16) for _ in range(2))
+    special = [(x, t, c) for x, t in ((np.nan, 3), (-np.nan, 70), (np.inf, 200), (-np.inf, 331)) for c in (0, 37, 65, 126)]
+    for x, t, c in special:
+        K[0, 0, t, c] = V[0, 1, t + c // 2, c] = x
+    K[0, 1, 400, 96:] = np.nan                 # nothing but NaN
+    a, b = gpu_cache(w), gpu_cache(w)
+    a.innerq_quantize_prefill(dev(K), dev(V))
+    b.innerq_quantize_prefill(dev(K[:, :, :0]), dev(V[:, :, :0]))
+    k, v = dev(K.transpose(2, 0, 1, 3)), dev(V.transpose(2, 0, 1, 3))
+    for t in range(N + 16):
+        b.innerq_append_token(k[t], v[t])
+    a, b = a.innerq_cache_export(), b.innerq_cache_export()
+    for name, X in (("k", K[0, :, :N].reshape(2, N, 128 // G, G)), ("v", V[0, :, :N].reshape(2, N // G, G, 128).swapaxes(2, 3))):
+        symmetric = (a[f"{name}_scale"] & 0x8000) == 0
+        assert np.array_equal(symmetric, ~np.isfinite(X).all(-1)), name
+        assert np.array_equal(symmetric, (b[f"{name}_scale"] & 0x8000) == 0), name
+        keep = np.isfinite(X).all(-1)
+        assert np.array_equal(a[f"{name}_scale"][keep], b[f"{name}_scale"][keep]), name
+
+
 # The fp16 windows: fewer tokens than the sink holds, nothing but windows, windows of no, one and many tokens, and unit
 # counts at which a thread's next piece is units further on or less than a unit's pieces away.
 @pytest.mark.parametrize("grouping", [O.INNER, O.OUTER, O.FP16])
