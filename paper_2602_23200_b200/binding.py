@@ -1,4 +1,5 @@
-"""ctypes binding over libinnerq.so: argument marshalling only.
+"""Binding over libinnerq.so: argument marshalling only, by ctypes, and for the calls of a step and a prefill in an extension
+module (csrc/innerq_step.cpp) where that has been built.
 
 Function names mirror the C ABI (include/innerq.h).  PyTorch is used for device memory and
 streams; every step of the path runs in the library's CUDA kernels.  There is no CPU fallback:
@@ -213,8 +214,12 @@ class _Fast:
                 setattr(cls, attr, staticmethod(getattr(torch._C, name)))
         global _ptr_of
         _ptr_of = cls._make_ptr_of(torch.Tensor, torch.float16)
-        from . import _step
-        cls.steps = _step.Steps
+        # the calls of a step in native code; None where the extension module is missing: the general forms make every call
+        try:
+            from . import _step
+            cls.steps = _step.Steps
+        except ImportError:
+            cls.steps = None
         cls.entries = [C.cast(getattr(lib(), f), C.c_void_p).value for f in
                        ("innerq_append_token", "innerq_decode_attention", "innerq_quantize_prefill", "innerq_decode_step_host")]
         cls.ready = True
@@ -312,7 +317,7 @@ class InnerQCache:
         if not _Fast.ready:
             _Fast.load()
         # the calls of a step from the current stream, with their checks in native code; None once the handle is gone
-        self._steps = _Fast.steps(h.value, self.device.index, self._kv_shape, self._q_shape, *_Fast.entries)
+        self._steps = _Fast.steps and _Fast.steps(h.value, self.device.index, self._kv_shape, self._q_shape, *_Fast.entries)
 
     # ---- paged caches
     def innerq_cache_pages_for(self, n_tokens: int) -> int:

@@ -40,9 +40,17 @@ def build_step(force: bool = False) -> str:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    build_step(force)
-    if not force and not _stale():
+    if force or _stale():
+        _build_lib(verbose)
+    try:
+        import torch  # noqa: F401
+    except ImportError:      # the library alone serves callers of its C ABI
         return LIB
+    build_step(force)
+    return LIB
+
+
+def _build_lib(verbose: bool) -> None:
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     flags = list(NVCC_FLAGS)
     if verbose:
@@ -70,7 +78,6 @@ def build(force: bool = False, verbose: bool = False) -> str:
             raise RuntimeError("nvcc failed: " + " ".join(cmd))
     cmd = [nvcc, *ARCH, "-shared", "-o", LIB, *objs, "-lcudart"]
     subprocess.run(cmd, check=True)
-    return LIB
 
 
 if __name__ == "__main__":

@@ -3,6 +3,8 @@ header declares, validates arguments, and its packed layout has the paper's effe
 import ctypes as C
 import os
 import re
+import subprocess
+import sys
 
 import pytest
 
@@ -148,3 +150,20 @@ def test_the_short_checks_of_a_step_let_only_tensors_through():
     for t in (torch.zeros(2, 128, dtype=torch.float16), torch.zeros(2, 128), [0.0], None):
         with pytest.raises(TypeError):
             B._ptr_of(t, "q", (2, 128), torch.device("cuda", 0))
+
+
+def test_binding_works_without_the_extension_module(tmp_path):
+    # a tree with the library alone (no _step module, no sources): the general forms make every call
+    pkg = tmp_path / "paper_2602_23200_b200"
+    pkg.mkdir()
+    here = os.path.dirname(B.LIB_PATH)
+    for f in os.listdir(here):
+        if f.endswith(".py") or f == os.path.basename(B.LIB_PATH):
+            os.symlink(os.path.join(here, f), pkg / f)
+    code = ("from paper_2602_23200_b200 import binding as B\n"
+            "B._Fast.load()\n"
+            "assert B._Fast.ready and B._Fast.steps is None\n"
+            f"assert B.LIB_PATH == {str(pkg / 'libinnerq.so')!r}\n")
+    r = subprocess.run([sys.executable, "-c", code], cwd=tmp_path, capture_output=True, text=True,
+                       env={k: v for k, v in os.environ.items() if k != "PYTHONPATH"})
+    assert r.returncode == 0, r.stderr

@@ -686,6 +686,34 @@ def test_result_is_a_plain_contiguous_tensor_whatever_the_query_is():
             assert torch.equal(out, want)
 
 
+def test_general_forms_give_what_the_extension_module_gives():
+    import torch
+    w = synth.tiny(batch=2, n_q_heads=4, n_kv_heads=2, n_tokens=400)
+    K, V = (dev(x) for x in synth.kv_all(w))
+    a, b = gpu_cache(w), gpu_cache(w)
+    assert a._steps is not None
+    b._steps = None
+    host = [torch.empty((2, 4, 128), dtype=torch.float16).pin_memory() for _ in range(2)]
+    for c in (a, b):
+        c.innerq_quantize_prefill(K, V)
+    for step in range(40):
+        k1, v1, q = (torch.from_numpy(x).pin_memory() for x in (*synth.new_token(w, step), synth.query(w, step)))
+        if step % 3 == 2:
+            for c, out in zip((a, b), host):
+                c.innerq_decode_step_host(k1, v1, q, out)
+            torch.cuda.synchronize()
+            assert torch.equal(*host), step
+        else:
+            for c in (a, b):
+                c.innerq_append_token(k1.cuda(), v1.cuda())
+            given = torch.empty((2, 4, 128), dtype=torch.float16, device="cuda")
+            out = a.innerq_decode_attention(q.cuda())
+            assert b.innerq_decode_attention(q.cuda(), given) is given and torch.equal(out, given), step
+            assert torch.equal(a.innerq_decode_attention(q.cuda(), given), b.innerq_decode_attention(q.cuda())), step
+    a, b = a.innerq_cache_export(), b.innerq_cache_export()
+    assert all(np.array_equal(a[key], b[key]) for key in a)
+
+
 def test_batched_calls_argument_checks():
     from paper_2602_23200_b200 import binding as B
     w = synth.tiny(batch=1, n_q_heads=2, n_kv_heads=2, n_tokens=50)
