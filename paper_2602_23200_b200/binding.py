@@ -196,6 +196,31 @@ def _dev_ptr(t, name: str, shape, device=None) -> int:
     return t.data_ptr()
 
 
+def step_path() -> str:
+    """File of the extension module _step for this interpreter and this torch: it is compiled against both, so every pair has
+    its own, and one that was built for another pair is neither loaded nor taken for up to date."""
+    import sysconfig
+
+    import torch
+    abi = int(torch._C._GLIBCXX_USE_CXX11_ABI)
+    return os.path.join(_HERE, f"_step.{sysconfig.get_config_var('SOABI')}-torch{torch.__version__}-abi{abi}.so")
+
+
+def _load_steps():
+    """The calls of a step in native code; None where the extension module is missing: the general forms make every call."""
+    from importlib import machinery, util
+    path = step_path()
+    if not os.path.exists(path):
+        return None
+    loader = machinery.ExtensionFileLoader(f"{__package__}._step", path)
+    try:
+        module = util.module_from_spec(util.spec_from_file_location(loader.name, path, loader=loader))
+        loader.exec_module(module)
+    except ImportError:
+        return None
+    return module.Steps
+
+
 class _Fast:
     """The same two checks for the calls of a decode step that the extension module (csrc/innerq_step.cpp) has not taken.
     One look-up per property, in the order that lets a valid tensor through with the fewest; whatever does not pass (a subclass among it)
@@ -214,12 +239,7 @@ class _Fast:
                 setattr(cls, attr, staticmethod(getattr(torch._C, name)))
         global _ptr_of
         _ptr_of = cls._make_ptr_of(torch.Tensor, torch.float16)
-        # the calls of a step in native code; None where the extension module is missing: the general forms make every call
-        try:
-            from . import _step
-            cls.steps = _step.Steps
-        except ImportError:
-            cls.steps = None
+        cls.steps = _load_steps()
         cls.entries = [C.cast(getattr(lib(), f), C.c_void_p).value for f in
                        ("innerq_append_token", "innerq_decode_attention", "innerq_quantize_prefill", "innerq_decode_step_host")]
         cls.ready = True

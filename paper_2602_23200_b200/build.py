@@ -1,5 +1,5 @@
-"""Builds libinnerq.so (sm_100a) next to this file with nvcc, and the extension module _step.so (the host side of a step's
-calls, against torch's headers) with g++.  Usable as `python -m paper_2602_23200_b200.build`."""
+"""Builds libinnerq.so (sm_100a) next to this file with nvcc, and the extension module _step (the host side of a step's
+calls, against torch's headers; binding.step_path() names its file) with g++.  Usable as `python -m paper_2602_23200_b200.build`."""
 from __future__ import annotations
 
 import os
@@ -9,7 +9,6 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libinnerq.so")
-STEP = os.path.join(HERE, "_step.so")
 # every .cu of csrc/: the C ABI, the quantise kernels, the decode kernels (the fused kernel one file per packed format)
 SOURCES = sorted(f for f in os.listdir(CSRC) if f.endswith(".cu"))
 ARCH = ["-gencode", "arch=compute_100a,code=sm_100a"]
@@ -28,15 +27,17 @@ def build_step(force: bool = False) -> str:
     import sysconfig
 
     import torch
-    src, t = os.path.join(CSRC, "innerq_step.cpp"), os.path.dirname(torch.__file__)
-    if not force and os.path.exists(STEP) and os.path.getmtime(STEP) >= max(os.path.getmtime(src), os.path.getmtime(__file__)):
-        return STEP
+
+    from .binding import step_path
+    src, out, t = os.path.join(CSRC, "innerq_step.cpp"), step_path(), os.path.dirname(torch.__file__)
+    if not force and os.path.exists(out) and os.path.getmtime(out) >= max(os.path.getmtime(src), os.path.getmtime(__file__)):
+        return out
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared",
            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", "-I" + sysconfig.get_paths()["include"],
-           "-I/usr/local/cuda/include", "-isystem", os.path.join(t, "include"), src, "-o", STEP,
+           "-I/usr/local/cuda/include", "-isystem", os.path.join(t, "include"), src, "-o", out,
            "-L" + os.path.join(t, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
     subprocess.run(cmd, check=True)
-    return STEP
+    return out
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

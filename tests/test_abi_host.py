@@ -167,3 +167,26 @@ def test_binding_works_without_the_extension_module(tmp_path):
     r = subprocess.run([sys.executable, "-c", code], cwd=tmp_path, capture_output=True, text=True,
                        env={k: v for k, v in os.environ.items() if k != "PYTHONPATH"})
     assert r.returncode == 0, r.stderr
+
+
+@pytest.mark.parametrize("what,value", [("version", "99.0.0"), ("abi", None), ("python", "cpython-399-x86_64-linux-gnu")])
+def test_extension_module_of_another_torch_or_python_is_not_up_to_date(monkeypatch, what, value):
+    # compiled against the headers of one torch and one interpreter: with another one it is built anew, never loaded
+    import sysconfig
+
+    import torch
+    from paper_2602_23200_b200 import build
+    commands = []
+    monkeypatch.setattr(build.subprocess, "run", lambda cmd, **kw: commands.append(cmd))
+    path = build.build_step()
+    assert not commands and os.path.exists(path)             # this pair's file is there
+    if what == "version":
+        monkeypatch.setattr(torch, "__version__", value)
+    elif what == "abi":
+        monkeypatch.setattr(torch._C, "_GLIBCXX_USE_CXX11_ABI", not torch._C._GLIBCXX_USE_CXX11_ABI)
+    else:
+        get = sysconfig.get_config_var
+        monkeypatch.setattr(sysconfig, "get_config_var", lambda name: value if name == "SOABI" else get(name))
+    other = build.build_step()
+    assert other != path and len(commands) == 1 and other in commands[0]
+    assert B._load_steps() is None
