@@ -53,22 +53,24 @@ void* host_ptr(PyObject* o, const int64_t* shape) {
 bool current(const Steps* s) { return c10::cuda::current_device() == s->device; }
 void* stream_of(const Steps* s) { return c10::cuda::getCurrentCUDAStream((c10::DeviceIndex)s->device).stream(); }
 
-// f's status with the GIL released; exceptions of its checks (a tensor without storage, say) leave the call to binding.py
+// f's status; exceptions (of its checks: a tensor without storage, say) leave the call to binding.py
 template <typename F> PyObject* guarded(F f) {
   long st = kNotHandled;
   try {
     st = f();
   } catch (...) {
+    PyErr_Clear();
     st = kNotHandled;
   }
   return PyLong_FromLong(st);
 }
+// f's status with the GIL released; it is held again whether f returns or throws
 template <typename F> long without_gil(F f) {
-  int st;
-  Py_BEGIN_ALLOW_THREADS
-  st = f();
-  Py_END_ALLOW_THREADS
-  return st;
+  struct Released {
+    PyThreadState* state = PyEval_SaveThread();
+    ~Released() { PyEval_RestoreThread(state); }
+  } released;
+  return f();
 }
 
 PyObject* steps_append(PyObject* self, PyObject* const* a, Py_ssize_t n) {

@@ -714,6 +714,30 @@ def test_general_forms_give_what_the_extension_module_gives():
     assert all(np.array_equal(a[key], b[key]) for key in a)
 
 
+def test_exception_behind_the_extension_module_leaves_the_interpreter_whole(tmp_path):
+    # an entry point that throws: the call is left to the general forms, with the interpreter's lock held again
+    import subprocess
+    import sys
+    (tmp_path / "boom.cpp").write_text('#include <stdexcept>\nextern "C" int boom() { throw std::runtime_error("boom"); }\n')
+    so = str(tmp_path / "boom.so")
+    subprocess.run(["g++", "-shared", "-fPIC", "-o", so, str(tmp_path / "boom.cpp")], check=True)
+    code = f"""
+import ctypes, torch
+from paper_2602_23200_b200 import binding as B
+boom = ctypes.cast(ctypes.CDLL({so!r}).boom, ctypes.c_void_p).value
+kv, q = (1, 2, 128), (1, 4, 128)
+steps = B._load_steps()(0, torch.cuda.current_device(), kv, q, boom, boom, boom, boom)
+k, query = (torch.zeros(s, dtype=torch.float16, device="cuda") for s in (kv, q))
+for _ in range(3):
+    got = [steps.append(k, k), steps.decode(query, None), steps.decode(query, query), steps.prefill(k[:, :, None], k[:, :, None]),
+           steps.step_host(k.cpu(), k.cpu(), query.cpu(), query.cpu(), 4096)]
+    assert got == [1] * 5, got
+print("whole")
+"""
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True)
+    assert r.returncode == 0 and r.stdout.strip() == "whole", r.stderr
+
+
 def test_batched_calls_argument_checks():
     from paper_2602_23200_b200 import binding as B
     w = synth.tiny(batch=1, n_q_heads=2, n_kv_heads=2, n_tokens=50)
