@@ -1445,47 +1445,55 @@ int launch_one_p(const Layout& L, const Counts& cn, DecodeArgs a, int grid_y, cu
       table_in_params = true;
     }
   }
-  const bool cluster = merges_in_cluster(L.U * a.passes, grid_y);
-  a.cluster = cluster;
+  static ClusterRoom room;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(L.U * a.passes, grid_y); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kSmem; cfg.stream = st;
+  const bool cluster = merges_in_cluster(L.U * a.passes, grid_y) && room(decode_mma_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, PAGED, 0, RENEW>, cfg, grid_y) > 0;
   int launches = 0;
   const int rows = L.r * a.n_q, step = SPLIT ? 1 : kHeads, per = a.passes;
   for (int h0 = 0; h0 < rows; h0 += step * per) {
     a.head0 = h0;
     a.passes = std::min(per, (rows - h0 + step - 1) / step);
-    const dim3 grid(L.U * a.passes, grid_y);
+    cfg.gridDim = dim3(L.U * a.passes, grid_y);
     // launched as a programmatic dependent of whatever precedes it in the stream: its set-up overlaps that
     // kernel's tail, its first global access waits for it (grid_dependency_wait)
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid; cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kSmem; cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = attr[1].val.clusterDim.z = 1;
     attr[1].val.clusterDim.y = grid_y;
-    cfg.attrs = attr; cfg.numAttrs = cluster ? 2 : 1;
-    cudaError_t err;
-    if constexpr (PAGED) {
-      if (a.ablation) return -2;      // the timing instances exist for contiguous caches only
-      err = table_in_params ? cudaLaunchKernelEx(&cfg, decode_mma_paged_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, RENEW>, L, cn, a, ids)
-                            : cudaLaunchKernelEx(&cfg, decode_mma_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, PAGED, 0, RENEW>, L, cn, a);
-    } else if (a.ablation == 1 || a.ablation == 2) {
+    cfg.attrs = attr;
+    int unsupported = 0;
+    const bool done = launch_merging(cluster, [&](bool in_cluster) {
+      a.cluster = in_cluster;
+      cfg.numAttrs = in_cluster ? 2 : 1;
+      cudaError_t err;
+      if constexpr (PAGED) {
+        if (a.ablation) { unsupported = 1; return false; }      // the timing instances exist for contiguous caches only
+        err = table_in_params ? cudaLaunchKernelEx(&cfg, decode_mma_paged_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, RENEW>, L, cn, a, ids)
+                              : cudaLaunchKernelEx(&cfg, decode_mma_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, PAGED, 0, RENEW>, L, cn, a);
+      } else if (a.ablation == 1 || a.ablation == 2) {
 #ifdef IQ_WITH_TIMING_INSTANCES      // defined by the translation units of the formats the latency study times
-      static std::atomic<unsigned long long> configured_a1{0}, configured_a2{0};
-      if (a.ablation == 1) {
-        if (!opt_in_dynamic_smem(decode_mma_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, false, 1>, kSmem, configured_a1, true)) return -1;
-        err = cudaLaunchKernelEx(&cfg, decode_mma_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, false, 1>, L, cn, a);
-      } else {
-        if (!opt_in_dynamic_smem(decode_mma_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, false, 2>, kSmem, configured_a2, true)) return -1;
-        err = cudaLaunchKernelEx(&cfg, decode_mma_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, false, 2>, L, cn, a);
-      }
+        static std::atomic<unsigned long long> configured_a1{0}, configured_a2{0};
+        if (a.ablation == 1) {
+          if (!opt_in_dynamic_smem(decode_mma_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, false, 1>, kSmem, configured_a1, true)) return false;
+          err = cudaLaunchKernelEx(&cfg, decode_mma_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, false, 1>, L, cn, a);
+        } else {
+          if (!opt_in_dynamic_smem(decode_mma_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, false, 2>, kSmem, configured_a2, true)) return false;
+          err = cudaLaunchKernelEx(&cfg, decode_mma_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, false, 2>, L, cn, a);
+        }
 #else
-      return -2;
+        unsupported = 1;
+        return false;
 #endif
-    } else {
-      err = cudaLaunchKernelEx(&cfg, decode_mma_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, PAGED, 0, RENEW>, L, cn, a);
-    }
-    if (err != cudaSuccess) return -1;
+      } else {
+        err = cudaLaunchKernelEx(&cfg, decode_mma_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, PAGED, 0, RENEW>, L, cn, a);
+      }
+      if (err != cudaSuccess) cudaGetLastError();
+      return err == cudaSuccess;
+    });
+    if (!done) return unsupported ? -2 : -1;
     ++launches;
   }
   return cudaGetLastError() == cudaSuccess ? launches : -1;
@@ -1527,23 +1535,29 @@ int launch_one_batched_p(const Layout& L, SeqTable& T, int n_seqs, int n_splits,
     const int gy = fill_split_args(L, T.s[i].cn, T.s[i].a, RU, OUTER, want, 0);
     if (gy > grid_y) grid_y = gy;
   }
-  const bool cluster = merges_in_cluster(n_seqs * L.U, grid_y);
-  for (int i = 0; i < n_seqs; ++i) T.s[i].a.cluster = cluster;
+  static ClusterRoom room;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(n_seqs * L.U, grid_y); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kSmem; cfg.stream = st;
+  const bool cluster = merges_in_cluster(n_seqs * L.U, grid_y) && room(decode_mma_batched_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, PAGED>, cfg, grid_y) > 0;
   int launches = 0;
-  const dim3 grid(n_seqs * L.U, grid_y);
   const int step = SPLIT ? 1 : kHeads;
   for (int h0 = 0; h0 < L.r; h0 += step) {      // one launch per group of query rows
     for (int i = 0; i < n_seqs; ++i) T.s[i].a.head0 = h0;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid; cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kSmem; cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = attr[1].val.clusterDim.z = 1;
     attr[1].val.clusterDim.y = grid_y;
-    cfg.attrs = attr; cfg.numAttrs = cluster ? 2 : 1;
-    if (cudaLaunchKernelEx(&cfg, decode_mma_batched_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, PAGED>, L, T) != cudaSuccess) return -1;
+    cfg.attrs = attr;
+    const bool done = launch_merging(cluster, [&](bool in_cluster) {
+      for (int i = 0; i < n_seqs; ++i) T.s[i].a.cluster = in_cluster;
+      cfg.numAttrs = in_cluster ? 2 : 1;
+      if (cudaLaunchKernelEx(&cfg, decode_mma_batched_kernel<KB, VB, G, KM, VM, SPLIT, CPI, OUTER, PAGED>, L, T) == cudaSuccess) return true;
+      cudaGetLastError();
+      return false;
+    });
+    if (!done) return -1;
     ++launches;
   }
   return cudaGetLastError() == cudaSuccess ? launches : -1;

@@ -4,9 +4,11 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 
 #include "innerq_layout.h"
+#include "innerq_split.h"
 
 namespace iq {
 
@@ -19,11 +21,39 @@ inline bool opt_in_dynamic_smem(Kernel kernel, int bytes, std::atomic<unsigned l
   const unsigned long long bit = 1ull << dev;
   if (done.load(std::memory_order_acquire) & bit) return true;
   if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return false;
-  // clusters of more than the portable 8 CTAs
-  if (clusters && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
+  // clusters of more than the portable 8 CTAs, where the device has them (see ClusterRoom)
+  if (clusters && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) cudaGetLastError();
   done.fetch_or(bit, std::memory_order_release);
   return true;
 }
+
+// How many clusters of a kernel the device holds at once, by their number of CTAs; 0: it cannot place one (few SMs per GPC, a
+// share of the SMs only).  Asked of the driver once per kernel (which has one of these), device and number; launches that
+// are refused all the same (a stream with fewer SMs than the device) fall back in launch_merging.
+struct ClusterRoom {
+  std::atomic<uint16_t> known[64][kClusterCtas] = {};      // answer + 1
+  template <typename Kernel> int operator()(Kernel kernel, const cudaLaunchConfig_t& like, int ctas) {
+    int dev = -1;
+    if (ctas < 1 || ctas > kClusterCtas || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    std::atomic<uint16_t>& k = known[dev][ctas - 1];
+    int n = (int)k.load(std::memory_order_relaxed) - 1;
+    if (n < 0) {
+      cudaLaunchConfig_t cfg = like;
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = attr[0].val.clusterDim.z = 1;
+      attr[0].val.clusterDim.y = ctas;
+      cfg.attrs = attr; cfg.numAttrs = 1;
+      if (cudaOccupancyMaxActiveClusters(&n, reinterpret_cast<const void*>(kernel), &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        n = 0;
+      }
+      n = std::min(std::max(n, 0), 65534);
+      k.store((uint16_t)(n + 1), std::memory_order_relaxed);
+    }
+    return n;
+  }
+};
 
 struct ExportPtrs {
   uint8_t *k_code, *v_code;

@@ -45,6 +45,11 @@ inline bool merges_in_cluster(int n_clusters, int grid_y) {
   return grid_y <= kClusterCtas && n_clusters * grid_y <= (grid_y == 2 ? kCtaSlots : kCtaSlots / 2);
 }
 
+// Launches a decode: launch(merge in a cluster?) says whether it was accepted.  A cluster that is refused goes without.
+template <typename Launch> inline bool launch_merging(bool cluster, Launch launch) {
+  return (cluster && launch(true)) || launch(false);
+}
+
 // Partial slots per query head: token-range splits (two waves of CTAs for all units, 64 at most) plus one per 32 tokens of
 // the fp16 tail.
 inline int max_splits_for(int n_units, int w_sink, int w_recent, int G) {

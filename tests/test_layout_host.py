@@ -36,3 +36,12 @@ def test_every_launch_has_a_grid_whose_partials_and_tickets_fit(tmp_path):
     subprocess.run(["g++", "-std=c++17", "-O2", "-I", CSRC, "-o", exe, os.path.join(HERE, "host_split_check.cpp")], check=True)
     r = subprocess.run([exe], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout
+
+
+@pytest.mark.skipif(shutil.which("g++") is None, reason="needs a host C++ compiler")
+def test_decode_launches_go_without_a_cluster_that_cannot_be_placed(tmp_path):
+    exe = str(tmp_path / "host_cluster_check")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-I", CSRC, "-I", "/usr/local/cuda/include", "-o", exe,
+                    os.path.join(HERE, "host_cluster_check.cpp")], check=True)
+    r = subprocess.run([exe], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout
