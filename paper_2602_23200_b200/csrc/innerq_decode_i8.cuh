@@ -1225,7 +1225,8 @@ int launch_i8_one_p(const Layout& L, const Counts& cn, DecodeArgs a, int n_split
   static ClusterRoom room;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(L.U * a.passes, grid_y); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kSmem; cfg.stream = st;
-  const bool cluster = merges_in_cluster(L.U * a.passes, grid_y) && room(decode_i8_kernel<KB, VB, G, KM, VM, SPLIT, CPI, PAGED>, cfg, grid_y) > 0;
+  const bool cluster = merges_in_cluster(L, L.U * a.passes, grid_y, std::min(kHeads, L.r * a.n_q), warp_chunks_of(cn, a, false),
+                                         room(decode_i8_kernel<KB, VB, G, KM, VM, SPLIT, CPI, PAGED>, cfg, grid_y));
   int launches = 0;
   const int rows = L.r * a.n_q, step = SPLIT ? 1 : kHeads, per = a.passes;
   for (int h0 = 0; h0 < rows; h0 += step * per) {
@@ -1299,18 +1300,20 @@ int launch_i8_batched_p(const Layout& L, SeqTable& T, int n_seqs, int n_splits, 
     const long long mid = (lo + hi) / 2;
     if (rows_needed(mid) <= budget) hi = mid; else lo = mid + 1;
   }
-  int grid_y = 1;
+  int grid_y = 1, warp_chunks = 0;
   for (int i = 0; i < n_seqs; ++i) {
     int want = chunks[i] > 0 ? (int)((chunks[i] + lo - 1) / lo) : 1;
     if (want > T.s[i].a.row_cap) want = T.s[i].a.row_cap;
     if (want > 128) want = 128;
     const int gy = fill_split_args(L, T.s[i].cn, T.s[i].a, RU, false, want, 0);
     if (gy > grid_y) grid_y = gy;
+    warp_chunks = std::max(warp_chunks, warp_chunks_of(T.s[i].cn, T.s[i].a, false));
   }
   static ClusterRoom room;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(n_seqs * L.U, grid_y); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kSmem; cfg.stream = st;
-  const bool cluster = merges_in_cluster(n_seqs * L.U, grid_y) && room(decode_i8_batched_kernel<KB, VB, G, KM, VM, SPLIT, CPI, PAGED>, cfg, grid_y) > 0;
+  const bool cluster = merges_in_cluster(L, n_seqs * L.U, grid_y, std::min(kHeads, L.r), warp_chunks,
+                                         room(decode_i8_batched_kernel<KB, VB, G, KM, VM, SPLIT, CPI, PAGED>, cfg, grid_y));
   int launches = 0;
   const int step = SPLIT ? 1 : kHeads;
   for (int h0 = 0; h0 < L.r; h0 += step) {      // one launch per group of query rows

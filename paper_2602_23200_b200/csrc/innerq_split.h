@@ -37,12 +37,39 @@ struct SplitArgs {
 // Whether the CTAs of a unit (and group) are a cluster that merges through distributed shared memory instead of through
 // global memory and a ticket.  That saves three dependent trips to L2 at the end of a launch (8 KV heads x 1001 tokens, r 4,
 // 3-bit keys: 13.3 -> 11.2 us alone, 6.0 -> 4.2 us in a chain), but a cluster starts only when all its CTAs find room in one
-// GPC: a launch that fills the slots then overlaps its neighbours less (64 units x 4 CTAs, 8192 tokens, 4 bits: 25.4 -> 23.5
-// us alone, 15.3 -> 16.7 in a chain).  So: launches of one CTA per SM at most, with the 16 CTAs that a cluster can have, and
-// pairs, for which one SM's two slots will do (128 units x 8192 tokens, 4 bits: 39.9 -> 36.9 us alone, 26.3 -> 26.0).
+// GPC: next to the launches before and after it in a chain it may have to wait.  So the rule goes by the chain (a call alone
+// gains 5 to 20 % at nearly every point below).  `room`: most clusters of this size that are resident at once (ClusterRoom);
+// `warp_chunks`: chunks (of 32 tokens) that a warp streams; `rows`: query rows merged, which the ticket's last CTA takes one
+// after the other.  Chain, tickets -> clusters, over some 2500 points (2, 3, 4 bits, G 32, 64, 128):
+//  * Three and four rows, short ranges: as long as the clusters of two launches fit at once.  With room for 14 of 16 CTAs, 7
+//    took 6.3 -> 4.8 us (2 bits) and 6.6 -> 5.4 (4 bits), 8 took 6.5 -> 6.6 and 6.7 -> 7.6; 16 of 8 (room 33) 6.5 -> 5.4 and
+//    6.6 -> 6.1, 18 of them 6.5 -> 6.7 and 6.9 -> 8.1.  Three rows lose where a warp streams much (15 clusters of 9, 4 bits,
+//    G 128: 7.1 -> 7.6).
+//  * Three and four rows, pairs: to the last slot (one SM's two will do), at every length.  128 pairs: 11.7 -> 9.6 us (4 bits,
+//    G 32, 1200 tokens), 26.3 -> 25.7 on average at 8192 tokens.
+//  * Three and four rows, long ranges (a caller's split count): 16 CTAs a unit, 2 bits, 60000 tokens: 32 of them 6.6
+//    -> 5.3, 64 7.8 -> 7.5, 112 9.7 -> 10.6, 128 10.0 -> 13.1.
+//  * Two rows and one (and such three): the ticket costs less and the chain hardly changes (4.5 -> 4.5 us); above 40 CTAs, 80
+//    where a warp streams little, it loses: 64 CTAs of 8, 4 bits, G 64: 4.5 -> 5.1; 112 of 4, 2 bits, G 32: 5.0 -> 5.2; 148:
+//    5.1 -> 6.2.
+//  * Pairs of few rows: one CTA per SM at most (148: 6.2 -> 5.8); one row above that between 5 % faster and 10 % slower
+//    (128 pairs x 16384 tokens, 2 bits, G 32: 32.4 -> 35.1); two rows 10.9 -> 8.9 (148 pairs x 649 tokens), 13.0 -> 12.3 (128 x
+//    2500), but 18.5 -> 18.7 (100 x 8192), and just above one CTA per SM 6.1 -> 6.4.
 constexpr int kClusterCtas = 16;
-inline bool merges_in_cluster(int n_clusters, int grid_y) {
-  return grid_y <= kClusterCtas && n_clusters * grid_y <= (grid_y == 2 ? kCtaSlots : kCtaSlots / 2);
+inline bool merges_in_cluster(const Layout& L, int n_clusters, int grid_y, int rows, int warp_chunks, int room) {
+  if (grid_y > kClusterCtas || n_clusters > room) return false;
+  const int ctas = n_clusters * grid_y;
+  const int streamed = warp_chunks * (L.k.bits + L.v.bits);
+  const bool is_short = warp_chunks <= 6;
+  if (rows >= 4 || (rows == 3 && (grid_y == 2 || streamed <= 16))) return grid_y == 2 || (is_short ? 2 * n_clusters <= room : ctas <= 40);
+  if (grid_y == 2 && rows == 2 && ctas >= 200) return warp_chunks <= 8;
+  return is_short && ctas <= (grid_y == 2 ? kCtaSlots / 2 : grid_y == 1 || streamed <= 8 ? 80 : 40);
+}
+
+// The longest range of a warp, in chunks (see merges_in_cluster).
+inline int warp_chunks_of(const Counts& cn, const SplitArgs& a, bool outer) {
+  const int n_chunks = (outer ? cn.n_qk : cn.n_qv) / kChunk, warps = kSplitWarps * std::max(1, a.n_splits);
+  return (n_chunks + warps - 1) / warps;
 }
 
 // Launches a decode: launch(merge in a cluster?) says whether it was accepted.  A cluster that is refused goes without.

@@ -1,5 +1,5 @@
-// Host check (no GPU, a fake of the CUDA runtime's calls) of what a decode does where a cluster of CTAs cannot be placed: the
-// device says so, or the launch is refused.  Prints one line per failed property and returns 1 if there were any.
+// Host check (no GPU, a fake of the CUDA runtime's calls) of when a decode merges in a cluster of CTAs, and of what it does
+// where one cannot be placed: the device says so, or the launch is refused.  Prints one line per failed property and returns 1 if there were any.
 #include <cstdio>
 #include <vector>
 
@@ -56,6 +56,25 @@ int main() {
         if (!wanted || !takes_cluster) want.push_back(false);
         check(tried == want && ok == ((wanted && takes_cluster) || takes_plain), "launch_merging");
       }
+  // the rule's edges: {bits, clusters, CTAs of one, rows, chunks per warp, room} and whether they merge in the cluster
+  const struct { int bits, n, grid_y, rows, chunks, room; bool want; } edges[] = {
+      {4, 7, 16, 4, 2, 14, true}, {4, 8, 16, 4, 2, 14, false}, {4, 1, 17, 4, 2, 14, false}, {2, 16, 8, 3, 4, 33, true},
+      {2, 17, 8, 3, 4, 33, false}, {2, 6, 8, 4, 6, 33, true}, {2, 5, 8, 4, 7, 33, true}, {2, 6, 8, 4, 7, 33, false},
+      {4, 6, 8, 3, 2, 33, true}, {4, 6, 8, 3, 3, 33, false}, {4, 5, 8, 3, 3, 33, true}, {4, 148, 2, 3, 9, 148, true},                  // short and long
+      {4, 148, 2, 4, 300, 148, true}, {4, 149, 2, 4, 1, 148, false}, {4, 148, 1, 4, 1, 296, true}, {4, 149, 1, 4, 1, 296, false},
+      {2, 1, 2, 4, 1, 0, false}, {2, 1, 1, 1, 1, 0, false},                                                // no room at all
+      {4, 2, 16, 1, 2, 14, true}, {4, 3, 16, 1, 2, 14, false}, {2, 5, 16, 1, 2, 14, true}, {2, 6, 16, 2, 1, 14, false},
+      {2, 2, 16, 2, 7, 14, false}, {4, 80, 1, 2, 4, 296, true}, {4, 81, 1, 2, 4, 296, false},
+      {2, 74, 2, 1, 1, 148, true}, {2, 75, 2, 1, 1, 148, false}, {2, 148, 2, 1, 1, 148, false},
+      {2, 74, 2, 2, 4, 148, true}, {2, 99, 2, 2, 1, 148, false}, {2, 100, 2, 2, 8, 148, true}, {2, 100, 2, 2, 9, 148, false}};
+  for (const auto& e : edges) {
+    Layout L = {};
+    L.k.bits = L.v.bits = e.bits;
+    if (merges_in_cluster(L, e.n, e.grid_y, e.rows, e.chunks, e.room) != e.want) {
+      ++failures;
+      std::printf("FAIL rule: %d bits, %d clusters of %d, %d rows, %d chunks, room %d\n", e.bits, e.n, e.grid_y, e.rows, e.chunks, e.room);
+    }
+  }
   std::printf("%d failure(s)\n", failures);
   return failures != 0;
 }
