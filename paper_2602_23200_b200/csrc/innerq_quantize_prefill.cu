@@ -533,7 +533,7 @@ struct KeyMax {
   __device__ __forceinline__ KeyMax(const __half* K_, float* out_, const MaxShares& s, int N_, int U_, int cta_, uint4* stage_)
       : K(K_), out(out_), ms(s), N(N_), U(U_), cta(cta_), stage(stage_) {
     at = end = 0;
-    if (cta < ms.ctas) { at = ms.begin(U, cta); end = ms.begin(U, cta + 1); }
+    if (cta >= 0 && cta < ms.ctas) { at = ms.begin(U, cta); end = ms.begin(U, cta + 1); }
     clear();
     if (at < end) request();
   }
@@ -895,7 +895,7 @@ __device__ __forceinline__ void copy_windows(const Layout& L, const Counts& cn, 
   }
 }
 
-// First of the two launches of an inner-grouped prefill: everything that does not need the key norms.  CTAs [0, ms.ctas)
+// First of the two launches of an inner-grouped prefill: everything that does not need the key norms.  CTAs [k0, k0 + ms.ctas)
 // take the key maxima, CTAs [v0, v0 + n_val) the value groups, CTAs [w0, w0 + n_win) the windows.  A prompt that fills the
 // GPU gives all CTAs of one wave a share of all three: the maxima's keys arrive while the value groups are worked on, every
 // load but a CTA's first is requested a step ahead (32 units x 16384 tokens, 2 bits, G = 128: 78 us as CTAs of several
@@ -906,14 +906,14 @@ template <int VBITS>
 __global__ void __launch_bounds__(256, 2)
 prefill_first_kernel(const __grid_constant__ Layout L, const Counts cn, const __half* __restrict__ K,
                      const __half* __restrict__ V, unsigned char* __restrict__ cache, float* __restrict__ absmax,
-                     const MaxShares ms, int v0, int n_val, int w0, int n_win, float neg_zero) {
+                     const MaxShares ms, int k0, int v0, int n_val, int w0, int n_win, float neg_zero) {
   extern __shared__ uint4 first_smem[];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // a programmatic dependent of whatever comes before it, for its launch to overlap that kernel's end; keys and values may be
   // that kernel's results, and the cache and workspace what it reads
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int b = blockIdx.x;
-  KeyMax keys(K, absmax, ms, cn.N, L.U, b, first_smem + kStage);
+  KeyMax keys(K, absmax, ms, cn.N, L.U, b - k0, first_smem + kStage);
   if (b >= w0 && b < w0 + n_win) copy_windows(L, cn, K, V, cache, ms.ctas == 0, b - w0, n_win);
   quantize_blocks<VBITS>(L, V, cn.N, cn.n_qv, cache, b - v0, n_val, first_smem, keys, Mul2(neg_zero));
 }
@@ -988,10 +988,16 @@ int launch_prefill_inner(const Layout& L, const Counts& cn, unsigned char* cache
   if (absmax) ms.ctas = clamp_int(std::min<long long>((long long)L.U * ms.per_unit, (long long)L.U * (L.max_splits - 1)), 1, wave);
   ms.stride = (ms.ctas + L.U - 1) / L.U + 1;
   const long long steps = cn.n_qv > 0 ? ((long long)L.U * (cn.n_qv / L.G) * (L.G / kChunk) + 3) / 4 : 0;
-  int v0 = 0, n_val = clamp_int(steps, 0, wave), w0 = 0, n_win = window_ctas(L, cn), grid;
-  if (std::min(ms.ctas, n_val) + n_win <= wave && ms.ctas + n_val + n_win <= 2 * wave && std::max(ms.ctas, n_val) < wave) {
-    v0 = ms.ctas;                             // roles apart
-    w0 = v0 + n_val;
+  int k0 = 0, v0 = 0, n_val = clamp_int(steps, 0, wave), w0 = 0, n_win = window_ctas(L, cn), grid;
+  if (ms.ctas + n_val <= 2 * wave && std::max(ms.ctas, n_val) < wave) {
+    // Roles apart: 32 units x 768 tokens, 4 bits, G = 128 (192 + 128 + 198 CTAs), 17.4 us, together 20.3; x 1001 tokens (256 +
+    // 192 + 187) 16.8 and 19.1; 56 x 576 (280 + 168 + 222) 18.8 and 20.8.  With a full wave of keys it is the slower form: 48 x
+    // 900 tokens, 2 bits, G = 32 (296 + 288): 21.4 and 20.7.  Where the three need more than a wave, the value groups, which
+    // take longest, start first and the windows fill the end: 24 x 900, 4 bits, G = 128 (192 + 144 + 102): keys first 14.1 us,
+    // values first 13.1.
+    if (ms.ctas + n_val + n_win > wave) k0 = n_val;
+    else v0 = ms.ctas;
+    w0 = ms.ctas + n_val;
     grid = w0 + n_win;
   } else {
     if (n_win > wave) w0 = std::max(ms.ctas, n_val);      // long windows: CTAs of their own
@@ -1006,7 +1012,7 @@ int launch_prefill_inner(const Layout& L, const Counts& cn, unsigned char* cache
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, L, cn, K, V, cache, absmax, ms, v0, n_val, w0, n_win, -0.f) == cudaSuccess;
+    return cudaLaunchKernelEx(&cfg, kernel, L, cn, K, V, cache, absmax, ms, k0, v0, n_val, w0, n_win, -0.f) == cudaSuccess;
   };
   static std::atomic<unsigned long long> configured[3];
   if (!(L.v.bits == 2   ? go(prefill_first_kernel<2>, configured[0])

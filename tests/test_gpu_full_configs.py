@@ -318,3 +318,23 @@ def test_config3_shape_sequences_of_different_lengths():
     for c in caches:
         assert c.innerq_read_device_error() == 0
     print(f"config-3 shape, 16 sequences of mixed lengths: worst err/tol {worst:.3f}")
+
+
+# The forms of a prefill's first launch: a CTA per role (one wave; several, the value groups first; windows of many CTAs), and
+# CTAs that take keys, values and windows (with windows of their own CTAs), where units end in the middle of a CTA's share and
+# the last step of the value groups is not full.
+@pytest.mark.parametrize("units,N,w_recent,bits,G", [
+    *((33, 3070, 16, bits, G) for bits in (2, 3, 4) for G in (32, 64, 128)),
+    (24, 333, 16, 3, 32), (33, 777, 16, 2, 32), (33, 777, 16, 3, 64), (29, 1001, 16, 4, 128), (56, 577, 128, 4, 64),
+    (13, 2000, 1500, 2, 64), (41, 2000, 1500, 3, 32)])
+def test_prefill_forms_of_the_first_launch(units, N, w_recent, bits, G):
+    w = synth.tiny(batch=1, n_kv_heads=units, n_q_heads=units, n_tokens=N, group=G, k_bits=bits, v_bits=bits, w_recent=w_recent)
+    K, V = synth.kv_all(w)
+    gc = make_gpu(w, K, V)
+    sample = [0, units // 2, units - 1]
+    P.assert_export_equal(slice_export(gc.innerq_cache_export(), sample), sub_oracle(w, K, V, sample).export(), O.INNER, G)
+    gc.innerq_quantize_prefill(dev(K[:, ::-1]), dev(V[:, ::-1]))          # the same units in reverse, over the first prefill
+    flipped = {k: v[::-1] if isinstance(v, np.ndarray) and v.ndim >= 2 else v for k, v in gc.innerq_cache_export().items()}
+    gc.innerq_quantize_prefill(dev(K), dev(V))
+    for k, v in gc.innerq_cache_export().items():
+        assert np.array_equal(np.asarray(v), np.asarray(flipped[k])), k
