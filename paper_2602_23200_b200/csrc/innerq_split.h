@@ -40,11 +40,13 @@ struct SplitArgs {
 // GPC: next to the launches before and after it in a chain it may have to wait.  So the rule goes by the chain (a call alone
 // gains 5 to 20 % at nearly every point below).  `room`: most clusters of this size that are resident at once (ClusterRoom);
 // `warp_chunks`: chunks (of 32 tokens) that a warp streams; `rows`: query rows merged, which the ticket's last CTA takes one
-// after the other.  Chain, tickets -> clusters, over some 2500 points (2, 3, 4 bits, G 32, 64, 128):
+// after the other.  Chain, tickets -> clusters, over some 2500 points (2, 3, 4 bits, G 32, 64, 128) of decodes, and 1000 of
+// appends and decodes in turn:
 //  * Three and four rows, short ranges: as long as the clusters of two launches fit at once.  With room for 14 of 16 CTAs, 7
 //    took 6.3 -> 4.8 us (2 bits) and 6.6 -> 5.4 (4 bits), 8 took 6.5 -> 6.6 and 6.7 -> 7.6; 16 of 8 (room 33) 6.5 -> 5.4 and
 //    6.6 -> 6.1, 18 of them 6.5 -> 6.7 and 6.9 -> 8.1.  Three rows lose where a warp streams much (15 clusters of 9, 4 bits,
-//    G 128: 7.1 -> 7.6).
+//    G 128: 7.1 -> 7.6).  So do steps with clusters of 3 to 8 above half a CTA per SM: 108 CTAs, 4 bits, G 64: decodes 6.4 ->
+//    6.1 but steps 8.3 -> 9.3.
 //  * Three and four rows, pairs: to the last slot (one SM's two will do), at every length.  128 pairs: 11.7 -> 9.6 us (4 bits,
 //    G 32, 1200 tokens), 26.3 -> 25.7 on average at 8192 tokens.
 //  * Three and four rows, long ranges (a caller's split count): 16 CTAs a unit, 2 bits, 60000 tokens: 32 of them 6.6
@@ -52,6 +54,8 @@ struct SplitArgs {
 //  * Two rows and one (and such three): the ticket costs less and the chain hardly changes (4.5 -> 4.5 us); above 40 CTAs, 80
 //    where a warp streams little, it loses: 64 CTAs of 8, 4 bits, G 64: 4.5 -> 5.1; 112 of 4, 2 bits, G 32: 5.0 -> 5.2; 148:
 //    5.1 -> 6.2.
+//  * One CTA (its merge needs no other): to 48 of them chains and steps gain up to 2 %; 64 units, one row, 4 bits, G 128: steps
+//    11.6 -> 12.0; 128, 2 bits, G 64: decodes 8.1 -> 8.9.
 //  * Pairs of few rows: one CTA per SM at most (148: 6.2 -> 5.8); one row above that between 5 % faster and 10 % slower
 //    (128 pairs x 16384 tokens, 2 bits, G 32: 32.4 -> 35.1); two rows 10.9 -> 8.9 (148 pairs x 649 tokens), 13.0 -> 12.3 (128 x
 //    2500), but 18.5 -> 18.7 (100 x 8192), and just above one CTA per SM 6.1 -> 6.4.
@@ -61,9 +65,13 @@ inline bool merges_in_cluster(const Layout& L, int n_clusters, int grid_y, int r
   const int ctas = n_clusters * grid_y;
   const int streamed = warp_chunks * (L.k.bits + L.v.bits);
   const bool is_short = warp_chunks <= 6;
-  if (rows >= 4 || (rows == 3 && (grid_y == 2 || streamed <= 16))) return grid_y == 2 || (is_short ? 2 * n_clusters <= room : ctas <= 40);
+  if (grid_y == 1) return is_short && ctas <= 48;
+  if (rows >= 4 || (rows == 3 && (grid_y == 2 || streamed <= 16))) {
+    if (grid_y == 2) return true;
+    return is_short ? 2 * n_clusters <= room && (streamed < 16 || grid_y > 8 || ctas <= 72) : ctas <= 40;
+  }
   if (grid_y == 2 && rows == 2 && ctas >= 200) return warp_chunks <= 8;
-  return is_short && ctas <= (grid_y == 2 ? kCtaSlots / 2 : grid_y == 1 || streamed <= 8 ? 80 : 40);
+  return is_short && ctas <= (grid_y == 2 ? kCtaSlots / 2 : streamed <= 8 ? 80 : 40);
 }
 
 // The longest range of a warp, in chunks (see merges_in_cluster).

@@ -58,13 +58,14 @@ int main() {
       }
   // the rule's edges: {bits, clusters, CTAs of one, rows, chunks per warp, room} and whether they merge in the cluster
   const struct { int bits, n, grid_y, rows, chunks, room; bool want; } edges[] = {
-      {4, 7, 16, 4, 2, 14, true}, {4, 8, 16, 4, 2, 14, false}, {4, 1, 17, 4, 2, 14, false}, {2, 16, 8, 3, 4, 33, true},
-      {2, 17, 8, 3, 4, 33, false}, {2, 6, 8, 4, 6, 33, true}, {2, 5, 8, 4, 7, 33, true}, {2, 6, 8, 4, 7, 33, false},
+      {4, 7, 16, 4, 2, 14, true}, {4, 8, 16, 4, 2, 14, false}, {4, 1, 17, 4, 2, 14, false}, {2, 16, 8, 3, 3, 33, true},
+      {2, 17, 8, 3, 3, 33, false}, {2, 6, 8, 4, 6, 33, true}, {2, 5, 8, 4, 7, 33, true}, {2, 6, 8, 4, 7, 33, false},
       {4, 6, 8, 3, 2, 33, true}, {4, 6, 8, 3, 3, 33, false}, {4, 5, 8, 3, 3, 33, true}, {4, 148, 2, 3, 9, 148, true},                  // short and long
-      {4, 148, 2, 4, 300, 148, true}, {4, 149, 2, 4, 1, 148, false}, {4, 148, 1, 4, 1, 296, true}, {4, 149, 1, 4, 1, 296, false},
+      {4, 148, 2, 4, 300, 148, true}, {4, 149, 2, 4, 1, 148, false}, {4, 48, 1, 4, 1, 296, true}, {4, 49, 1, 4, 1, 296, false},
       {2, 1, 2, 4, 1, 0, false}, {2, 1, 1, 1, 1, 0, false},                                                // no room at all
       {4, 2, 16, 1, 2, 14, true}, {4, 3, 16, 1, 2, 14, false}, {2, 5, 16, 1, 2, 14, true}, {2, 6, 16, 2, 1, 14, false},
-      {2, 2, 16, 2, 7, 14, false}, {4, 80, 1, 2, 4, 296, true}, {4, 81, 1, 2, 4, 296, false},
+      {2, 2, 16, 2, 7, 14, false}, {4, 48, 1, 2, 6, 296, true}, {4, 48, 1, 2, 7, 296, false},
+      {4, 9, 8, 4, 2, 33, true}, {4, 10, 8, 4, 2, 33, false}, {4, 10, 9, 4, 2, 30, true},
       {2, 74, 2, 1, 1, 148, true}, {2, 75, 2, 1, 1, 148, false}, {2, 148, 2, 1, 1, 148, false},
       {2, 74, 2, 2, 4, 148, true}, {2, 99, 2, 2, 1, 148, false}, {2, 100, 2, 2, 8, 148, true}, {2, 100, 2, 2, 9, 148, false}};
   for (const auto& e : edges) {
