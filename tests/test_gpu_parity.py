@@ -108,6 +108,37 @@ def test_step_calls_outside_the_extension():
         gc.innerq_append_token(k, k)
 
 
+# The same for the outer-grouped cache: clusters of up to 16 CTAs, tickets with 17, pairs that fill the GPU.
+@pytest.mark.parametrize("heads,r,bits,G,N,splits", [(2, 4, 2, 32, 4200, (0, 1, 2, 9, 15, 16, 17)), (1, 4, 4, 64, 2400, (0, 3, 4)),
+                                                     (100, 4, 4, 32, 700, (0, 2, 3))])
+def test_merge_of_splits_outer(heads, r, bits, G, N, splits):
+    w = synth.tiny(n_tokens=N, group=G, k_bits=bits, v_bits=bits, batch=1, n_kv_heads=heads, n_q_heads=heads * r, grouping=O.OUTER,
+                   k_normalize=0, k_mode=O.ASYM, v_mode=O.ASYM)
+    oc, gc, _, _ = run_prefill_both(w)
+    check_decode(w, oc, gc, splits=splits)
+
+
+# Batched launches that merge in clusters, where the short sequences' CTAs leave before the long ones' have worked.
+@pytest.mark.parametrize("kw", [dict(), dict(k_bits=4, v_bits=4, group=64), dict(n_q_heads=2),
+                                dict(grouping=O.OUTER, k_normalize=0, k_mode=O.ASYM, v_mode=O.ASYM)], ids=["2bit", "4bit_g64", "one_row", "outer"])
+def test_batched_clusters_with_sequences_of_few_rows(kw):
+    from paper_2602_23200_b200 import binding as B
+    base = synth.tiny(**dict(dict(batch=1, n_q_heads=8, n_kv_heads=2), **kw))
+    ws, ocs, gcs = [], [], []
+    for i, n in enumerate([30, 2080, 300, 900]):
+        w = base.with_(n_tokens=n, wid=base.wid + 900 + i)
+        oc, gc, _, _ = run_prefill_both(w, max_tokens=2400)
+        ws.append(w); ocs.append(oc); gcs.append(gc)
+    for order in ([0, 1, 2, 3], [1, 3, 0], [2, 0], [0, 2, 3, 1]):
+        q = np.stack([synth.query(ws[i], 5 + i) for i in order])
+        q_d = dev(q)
+        outs = [B.innerq_decode_attention_batched([gcs[i] for i in order], q_d) for _ in range(3)]
+        for out in outs:
+            for row, i in enumerate(order):
+                P.assert_outputs_close(out[row].cpu().numpy(), ocs[i].decode(q[row]), f"sequence {i} of {order}")
+    assert all(gc.innerq_read_device_error() == 0 for gc in gcs)
+
+
 @pytest.mark.parametrize("bits,G,mode,variant,N", CASES)
 def test_prefill_and_decode_inner(bits, G, mode, variant, N):
     w = synth.tiny(n_tokens=N, group=G, k_bits=bits, v_bits=bits, k_mode=mode, v_mode=mode, sym_variant=variant)
@@ -884,6 +915,65 @@ def test_random_interleaving_of_calls_on_one_stream(seed):
         w = ws[i]
         assert gc.n_tokens == ocs[i].N and gc.innerq_read_device_error() == 0
         P.assert_export_equal(gc.innerq_cache_export(), ocs[i].export(), w.grouping, w.group,
+                              k_hybrid=w.k_mode == O.HYBRID, v_hybrid=w.v_mode == O.HYBRID)
+
+
+@pytest.mark.parametrize("seed", [1, 2, 3, 4])
+def test_prefills_between_steps_on_one_stream(seed):
+    # A prefill's kernels overlap their neighbours (the first is a programmatic dependent of whatever runs before it, the second
+    # lets its dependents start at once): prefills of two prompts each, appends and decodes of three caches in random order and
+    # in the orders where little lies between two calls of a cache, nothing of it synchronised with the host.
+    torch = _torch()
+    rng = np.random.default_rng(100 + seed)
+    specs = [dict(n_q_heads=4, n_kv_heads=4, group=32, k_bits=2, v_bits=2, w_recent=16),
+             dict(n_q_heads=8, n_kv_heads=2, group=64, k_bits=4, v_bits=3, w_recent=24),
+             dict(n_q_heads=4, n_kv_heads=2, group=32, k_bits=2, v_bits=2, w_recent=16, grouping=O.OUTER, k_normalize=0,
+                  k_mode=O.ASYM, v_mode=O.ASYM)]
+    pool, n_prompts = 60, 3
+    ws, ocs, gcs, prompts, toks, qs, on_gpu = [], [], [], [], [], [], []
+    for i, kw in enumerate(specs):
+        lengths = [int(n) for n in rng.integers(30, 2500, n_prompts - 1)] + [4 + kw["w_recent"] + 20 * 32 + 5 * i]
+        w = synth.tiny(batch=1, n_tokens=max(lengths), wid=700 + 10 * seed + i, **kw)
+        K, V = synth.kv_all(w)
+        ws.append(w)
+        ocs.append(O.from_workload(w, max_tokens=w.n_tokens + 300))
+        gcs.append(gpu_cache(w))
+        prompts.append([(np.ascontiguousarray(K[:, :, -n:]), np.ascontiguousarray(V[:, :, -n:])) for n in lengths])
+        toks.append([synth.new_token(w, s) for s in range(pool)])
+        qs.append([synth.query(w, s) for s in range(pool)])
+        on_gpu.append(([(dev(k), dev(v)) for k, v in prompts[i]], dev(np.stack([t[0] for t in toks[i]])),
+                       dev(np.stack([t[1] for t in toks[i]])), dev(np.stack(qs[i]))))
+    ops = [("prefill", i, int(rng.integers(n_prompts))) for i in range(3)]
+    close = ["PA PB aB dB dA", "dA PB aA dA", "PA PA aA dA", "aA dA PA dA aA", "PA aB dB aA dA", "PA PB PC dC dB dA", "dB dA PA aB dB"]
+    for it in range(24):
+        names = dict(zip("ABC", rng.permutation(3)))
+        ops += [({"P": "prefill", "a": "append", "d": "decode"}[c[0]], int(names[c[1]]), int(rng.integers(n_prompts)))
+                for c in str(rng.choice(close)).split()]
+        for _ in range(int(rng.integers(6))):
+            ops.append((str(rng.choice(["append", "append", "decode", "decode", "prefill"])), int(rng.integers(3)),
+                        int(rng.integers(n_prompts))))
+    count = [0, 0, 0]
+    ops = [(op, i, j if op == "prefill" else (count.__setitem__(i, count[i] + 1) or count[i] % pool)) for op, i, j in ops]
+    torch.cuda.synchronize()
+    outs = []
+    for op, i, j in ops:
+        prompt, k, v, q = on_gpu[i]
+        if op == "prefill":
+            gcs[i].innerq_quantize_prefill(*prompt[j])
+        elif op == "append":
+            gcs[i].innerq_append_token(k[j], v[j])
+        outs.append(gcs[i].innerq_decode_attention(q[j]) if op == "decode" else None)
+    torch.cuda.synchronize()
+    for n, ((op, i, j), out) in enumerate(zip(ops, outs)):
+        if op == "prefill":
+            ocs[i].prefill(*prompts[i][j])
+        elif op == "append":
+            ocs[i].append(*toks[i][j])
+        else:
+            P.assert_outputs_close(out.cpu().numpy(), ocs[i].decode(qs[i][j]), f"call {n}, cache {i}")
+    for w, oc, gc in zip(ws, ocs, gcs):
+        assert gc.n_tokens == oc.N and gc.innerq_read_device_error() == 0
+        P.assert_export_equal(gc.innerq_cache_export(), oc.export(), w.grouping, w.group,
                               k_hybrid=w.k_mode == O.HYBRID, v_hybrid=w.v_mode == O.HYBRID)
 
 
