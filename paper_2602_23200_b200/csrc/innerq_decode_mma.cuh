@@ -4,8 +4,8 @@
 // launch shape, pipeline helpers, tail tiles and merge.  The description below is of the inner-grouped form, from
 // which the outer-grouped one differs in where scales and zero-points are applied (see OUTER in the kernel).
 //   q.K^T on packed key rows  ->  online softmax  ->  p.V on packed value chunks, split over token
-//   ranges, fp16 windows and the K/V skew zone as 16-token tiles dealt to the same warps, cross-CTA merge by
-//   the last CTA to finish.
+//   ranges, fp16 windows and the K/V skew zone as 16-token tiles dealt to the same warps, cross-CTA merge in a cluster
+//   through distributed shared memory (merges_in_cluster) or by the last CTA to finish.
 //
 // Work decomposition.  A CTA owns one (batch, KV head) unit and a range of value groups; each of its
 // 8 warps owns a contiguous sub-range and streams it chunk by chunk (32 tokens) through a private ring

@@ -216,8 +216,8 @@ template <int BITS> struct QuickErr {
 // How far a group's difference of the quick sums and that of PairCoder's can be apart; infinite where the quick sums mean
 // nothing (infinite or NaN also where a value is infinite: no comparison with it settles anything).  A NaN shows in neither
 // scale nor bound, and 3- and 4-bit sums count it as 0: groups with one get PairCoder's sums, whose NaN makes them symmetric
-// as in the append (see has_nan: the maximum that propagates NaN costs what the other one does).  m = largest |x| of the
-// group.
+// as in the append (see `nan`: the maximum that propagates NaN costs what the other one does; the check and what it leads to
+// 1 % of a prefill with 2 bits, whose sums show a NaN themselves).  m = largest |x| of the group.
 // 2 bits: a value's rounding errors are below 2^-20 m in each form, those of adding up 32 of them in two chains below
 // 2^-20 m a value; a value beyond the outer symmetric level (whose fp16 scale may be rounded down) counts with the wrong
 // sign.  3, 4 bits: in units of 2^-16 scales a value is off by 1 (complement), 1/2 (constant), 1/2 (rounding) and 1/8
@@ -245,8 +245,9 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
   return r;
 }
-// the same, but a NaN among the three is the result
-__device__ __forceinline__ float max3_nan(float a, float b, float c) {
+// the same; with 3 and 4 bits a NaN among the three is the result
+template <int BITS> __device__ __forceinline__ float max3_nan(float a, float b, float c) {
+  if constexpr (BITS == 2) return max3(a, b, c);
   float r;
   asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
   return r;
@@ -334,7 +335,11 @@ quantize_rows_prefill_kernel(const __grid_constant__ Layout L, const __half* __r
   const int gl = L.G >> 5, sh = gl >> 1;      // lanes per group: 1, 2 or 4, and its logarithm
   // reciprocal key norms: segment rows padded to 36 words, so that the four lanes of a token read different banks
   __shared__ __align__(16) float inv_s[NORM ? 4 * 36 : 4];
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");      // whatever follows waits before it touches anything
+  // What follows may start: a kernel of this cache waits before it touches anything (innerq_quantize_prefill has reset N_safe
+  // and reads_settled; a paged decode looks at its page table before that, which no kernel writes), one of another cache that
+  // does not touches nothing that a prefill writes, and the triggers and waits in between keep the kernels of that cache in
+  // their order.
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if constexpr (NORM) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     float* norm = reinterpret_cast<float*>(cache + L.norm_off);
@@ -390,15 +395,15 @@ quantize_rows_prefill_kernel(const __grid_constant__ Layout L, const __half* __r
       float mn, mx;                             // three-input min / max: two values per instruction
       {
         const float2 v = unf2(x[0]);
-        mn = fminf(v.x, v.y); mx = max3_nan(v.x, v.x, v.y);
+        mn = fminf(v.x, v.y); mx = max3_nan<BITS>(v.x, v.x, v.y);
 #pragma unroll
         for (int e = 1; e < kSeg / 2; ++e) {
           const float2 w = unf2(x[e]);
-          mn = min3(mn, w.x, w.y); mx = max3_nan(mx, w.x, w.y);
+          mn = min3(mn, w.x, w.y); mx = max3_nan<BITS>(mx, w.x, w.y);
         }
       }
-      const bool has_nan = __any_sync(0xffffffffu, mx != mx);
-      if (has_nan) {                            // the group's largest number
+      const bool nan = BITS > 2 && mx != mx;
+      if (nan) {                                // the largest number
 #pragma unroll
         for (int e = 0; e < kSeg / 2; ++e) {
           const float2 w = unf2(x[e]);
@@ -424,7 +429,7 @@ quantize_rows_prefill_kernel(const __grid_constant__ Layout L, const __half* __r
           quick = quick_mode(d, quick_bound<BITS>(p, bd, mn, mx, L.G));      // the same in all lanes of a group
         }
         asym = quick > 0;
-        if (__any_sync(0xffffffffu, quick < 0) || has_nan) {
+        if (__any_sync(0xffffffffu, quick < 0 || nan)) {
           const PairCoder pc(mul2, p, bd, p, bd);
           float2 ea = make_float2(0.f, 0.f), es = make_float2(0.f, 0.f);
           auto sums = [&](auto clamp) {
@@ -672,16 +677,16 @@ __device__ __forceinline__ void quantize_blocks(const Layout& L, const __half* _
     {
       const float2 v = unf2(x[1]);
       mn.x = fminf(mn.x, v.x); mn.y = fminf(mn.y, v.y);
-      mx.x = max3_nan(mx.x, mx.x, v.x); mx.y = max3_nan(mx.y, mx.y, v.y);
+      mx.x = max3_nan<BITS>(mx.x, mx.x, v.x); mx.y = max3_nan<BITS>(mx.y, mx.y, v.y);
     }
 #pragma unroll
     for (int t = 2; t < kSeg; t += 2) {
       const float2 v = unf2(x[t]), w = unf2(x[t + 1]);
       mn.x = min3(mn.x, v.x, w.x); mn.y = min3(mn.y, v.y, w.y);
-      mx.x = max3_nan(mx.x, v.x, w.x); mx.y = max3_nan(mx.y, v.y, w.y);
+      mx.x = max3_nan<BITS>(mx.x, v.x, w.x); mx.y = max3_nan<BITS>(mx.y, v.y, w.y);
     }
-    const bool has_nan = __any_sync(0xffffffffu, mx.x != mx.x || mx.y != mx.y);
-    if (has_nan) {                                           // the largest numbers
+    const bool nan = BITS > 2 && (mx.x != mx.x || mx.y != mx.y);
+    if (nan) {                                               // the largest numbers
 #pragma unroll
       for (int t = 0; t < kSeg; ++t) {
         const float2 v = unf2(x[t]);
@@ -723,7 +728,7 @@ __device__ __forceinline__ void quantize_blocks(const Layout& L, const __half* _
         const int quick1 = quick_mode(d.y, quick_bound<BITS>(p1, b1, mn.y, mx.y, G));
         asym0 = quick0 > 0;
         asym1 = quick1 > 0;
-        close = quick0 < 0 || quick1 < 0 || has_nan;
+        close = quick0 < 0 || quick1 < 0 || nan;
       }
       if (CH > 1 ? group_or(close) : (bool)__any_sync(0xffffffffu, close)) {
         const PairCoder pc(mul2, p0, b0, p1, b1);
