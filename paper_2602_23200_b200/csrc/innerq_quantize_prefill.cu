@@ -216,8 +216,9 @@ template <int BITS> struct QuickErr {
 // How far a group's difference of the quick sums and that of PairCoder's can be apart; infinite where the quick sums mean
 // nothing (infinite or NaN also where a value is infinite: no comparison with it settles anything).  A NaN shows in neither
 // scale nor bound, and 3- and 4-bit sums count it as 0: groups with one get PairCoder's sums, whose NaN makes them symmetric
-// as in the append (see `nan`: the maximum that propagates NaN costs what the other one does; the check and what it leads to
-// 1 % of a prefill with 2 bits, whose sums show a NaN themselves).  m = largest |x| of the group.
+// as in the append (see `nan`: the maximum that propagates NaN costs what the other one does, the branch 1 to 1.5 % of a
+// prefill; parameters that the rare path below makes anew instead cost 4 %).  2-bit sums show a NaN themselves.  m = largest
+// |x| of the group.
 // 2 bits: a value's rounding errors are below 2^-20 m in each form, those of adding up 32 of them in two chains below
 // 2^-20 m a value; a value beyond the outer symmetric level (whose fp16 scale may be rounded down) counts with the wrong
 // sign.  3, 4 bits: in units of 2^-16 scales a value is off by 1 (complement), 1/2 (constant), 1/2 (rounding) and 1/8

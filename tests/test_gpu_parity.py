@@ -226,6 +226,36 @@ def test_prefill_and_append_agree_on_groups_that_are_not_finite(bits, G):
         assert np.array_equal(a[f"{name}_scale"][keep], b[f"{name}_scale"][keep]), name
 
 
+# The same in the modes without a choice, and the literal symmetric formula: a NaN leaves the scale to the group's numbers.
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("mode,variant", [(O.SYM, 0), (O.ASYM, 0), (O.HYBRID, 1)])
+@pytest.mark.parametrize("G", [32, 128])
+def test_prefill_and_append_agree_on_scales_of_groups_with_a_nan(bits, mode, variant, G):
+    N = 3 * 128
+    w = synth.tiny(n_tokens=N + 16, group=G, k_bits=bits, v_bits=bits, batch=1, n_kv_heads=2, n_q_heads=2, w_sink=0, w_recent=16,
+                   k_normalize=0, k_mode=mode, v_mode=mode, sym_variant=variant)
+    rng = np.random.default_rng(bits + G)
+    K, V = (rng.normal(0, 3, (1, 2, N + 16, 128)).astype(np.float16) for _ in range(2))
+    for t, c in ((3, 0), (70, 37), (70, 38), (200, 65), (383, 127)):
+        K[0, t & 1, t, c] = V[0, t & 1, t, c] = np.nan
+    V[0, 0, 128:256, 9] = np.nan               # nothing but NaN
+    a, b = gpu_cache(w), gpu_cache(w)
+    a.innerq_quantize_prefill(dev(K), dev(V))
+    b.innerq_quantize_prefill(dev(K[:, :, :0]), dev(V[:, :, :0]))
+    k, v = dev(K.transpose(2, 0, 1, 3)), dev(V.transpose(2, 0, 1, 3))
+    for t in range(N + 16):
+        b.innerq_append_token(k[t], v[t])
+    a, b = a.innerq_cache_export(), b.innerq_cache_export()
+    for name, X in (("k", K[0, :, :N].reshape(2, N, 128 // G, G)), ("v", V[0, :, :N].reshape(2, N // G, G, 128).swapaxes(2, 3))):
+        nan = np.isnan(X)
+        groups = ~nan.all(-1)
+        if mode == O.HYBRID:                   # (of the others, ones with nearly equal errors may go either way)
+            groups &= nan.any(-1)
+        assert groups.any()
+        for part in ("scale", "zero"):
+            assert np.array_equal(a[f"{name}_{part}"][groups], b[f"{name}_{part}"][groups]), (name, part)
+
+
 # The fp16 windows: fewer tokens than the sink holds, nothing but windows, windows of no, one and many tokens, and unit
 # counts at which a thread's next piece is units further on or less than a unit's pieces away.
 @pytest.mark.parametrize("grouping", [O.INNER, O.OUTER, O.FP16])
