@@ -28,8 +28,8 @@ inline bool opt_in_dynamic_smem(Kernel kernel, int bytes, std::atomic<unsigned l
 }
 
 // How many clusters of a kernel the device holds at once, by their number of CTAs; 0: it cannot place one (few SMs per GPC, a
-// share of the SMs only).  Asked of the driver once per kernel (which has one of these), device and number; launches that
-// are refused all the same (a stream with fewer SMs than the device) fall back in launch_merging.
+// share of the SMs only).  The question is put once per kernel (which has one of these), device and number; launches that are
+// refused all the same (a stream with fewer SMs than the device) fall back in launch_merging.
 struct ClusterRoom {
   std::atomic<uint16_t> known[64][kClusterCtas] = {};      // answer + 1
   template <typename Kernel> int operator()(Kernel kernel, const cudaLaunchConfig_t& like, int ctas) {
